@@ -103,7 +103,8 @@ struct Layout {
     size_t off_layers, off_pt, off_kc, off_vc, off_h, off_feat, off_abuf, off_qkv, off_attn, off_act, off_po, off_ml,
         off_cnt, off_hp, off_dbgd, off_dbgv, off_out, off_S, off_rlog, off_prompt, off_st, off_bar;
     // tensor-core prompt pass (0 bytes each when the shape cannot take it)
-    size_t off_pf_h, off_pf_h2, off_pf_qkv, off_pf_attn, off_pf_gate, off_pf_up, off_pf_hi, off_pf_lo, off_pf_err;
+    size_t off_pf_h, off_pf_x, off_pf_q, off_pf_f, off_pf_rs, off_pf_cs, off_pf_part, off_pf_cnt, off_pf_err;
+    size_t pf_rows, pf_part_bytes;
     size_t off_embed, off_head, off_gfinal;
     std::vector<size_t> off_w[5];     // wqkv, wo, wgate, wup, wdown
     std::vector<size_t> off_g[2];
@@ -181,10 +182,13 @@ Layout make_layout(const kg_config* c, int own_weights, int nctas) {
     L.off_rlog = take(16 * (size_t)(c->max_seq + KG_M_MAX));
     L.off_prompt = take(4 * (size_t)c->max_seq);
     {
-        const size_t R = prefill_tc_shape(c) ? (size_t)PF_ROWS : 0, kmax = F > d ? F : d;
-        L.off_pf_h = take(4 * R * d); L.off_pf_h2 = take(4 * R * d); L.off_pf_qkv = take(4 * R * 3 * d);
-        L.off_pf_attn = take(4 * R * d); L.off_pf_gate = take(4 * R * F); L.off_pf_up = take(4 * R * F);
-        L.off_pf_hi = take(2 * R * kmax); L.off_pf_lo = take(2 * R * kmax); L.off_pf_err = take(R ? 64 + 4 * R : 0);      // error word, then 1/rms per row
+        // rows of a block; planes (hi, then lo) of the GEMM inputs; partial sums of the tiles that are cut along k
+        const size_t R = prefill_tc_shape(c) ? align_up(c->max_seq < PF_ROWS ? c->max_seq : PF_ROWS, 256) : 0;
+        L.pf_rows = R;
+        L.pf_part_bytes = R ? (size_t)nctas * GM_TM * GM_NT_MAX * 4 : 0;
+        L.off_pf_h = take(4 * R * d); L.off_pf_x = take(4 * R * d); L.off_pf_q = take(4 * R * d); L.off_pf_f = take(4 * R * F);
+        L.off_pf_rs = take(4 * R); L.off_pf_cs = take(4 * R * hd); L.off_pf_part = take(L.pf_part_bytes);
+        L.off_pf_cnt = take(R ? 4 * (size_t)nctas : 0); L.off_pf_err = take(R ? 64 : 0);
     }
     for (int k = 0; k < 5; ++k) L.off_w[k].assign(nl + 1, 0);
     for (int k = 0; k < 2; ++k) L.off_g[k].assign(nl + 1, 0);
@@ -234,8 +238,19 @@ __global__ void check_tokens_kernel(const int* toks, int n, int vocab, State* st
 
 }  // namespace
 
+// Tensor maps of the prompt pass, encoded once per model: the weights in boxes of 128 rows (64 for the gate / up pair),
+// the planes [R][K] in boxes of 32 * (i + 1) rows, one set for K = d (x) and one for K = F (f).
+struct PfMaps {
+    CUtensorMap x[2][4], f[2][4];                              // [hi, lo][activation rows per tile / 64 - 1]
+    struct Layer { CUtensorMap qkv, o, gate, up, down; };
+    std::vector<Layer> layer;
+    CUtensorMap adapter_kv;                                    // the k and v rows of the adapter's W_qkv
+    bool ready;
+};
+
 struct kg_model {
     kg_config cfg;
+    PfMaps pf;
     Dev dev;
     Layout lay;
     char* arena;
@@ -317,6 +332,12 @@ static int read_state(kg_model* m, State* out) {
         return out->status;
     }
     return KG_OK;
+}
+
+namespace {
+int prefill_tc(kg_model* m, int n);                 // the tensor-core prompt pass (end of this file)
+bool prefill_tc_ok(const kg_model* m, int n);
+int prefill_tc_init(kg_model* m);
 }
 
 template <typename WT>
@@ -477,6 +498,10 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
         if (r == KG_OK && cuda_failed(cudaStreamSynchronize(s), "weight fill")) r = KG_E_CUDA;
         if (r != KG_OK) { delete m; return r; }
     }
+    {
+        const int r = prefill_tc_init(m);
+        if (r != KG_OK) { delete m; return r; }
+    }
     *out = m;
     return KG_OK;
 }
@@ -497,11 +522,6 @@ extern "C" int kg_reset(kg_model* m) {
     m->prefilled = m->pending = m->ar_used = false;
     m->P_upper = 0;
     return KG_OK;
-}
-
-namespace {
-int prefill_tc(kg_model* m, int n);                 // the tensor-core prompt pass (end of this file)
-bool prefill_tc_ok(const kg_model* m, int n);
 }
 
 static int prefill_common(kg_model* m, int32_t n) {
@@ -857,7 +877,9 @@ extern "C" int kg_debug_skip_barrier_arrival(kg_model* m, int cta) {
 namespace {
 
 constexpr int OP_K_MAX = 32768;               // longest input row the single-operator entry points pack into scratch
-struct OpScratch { size_t off_hp, off_po, off_ml, off_cnt, off_pt, off_xpk, off_ssq, total; };
+constexpr size_t OP_GEMM_PART = 16u << 20;    // partial sums of the GEMM's cut tiles
+constexpr int OP_GEMM_CNT = 1024;             // their arrival counters, then the error word
+struct OpScratch { size_t off_hp, off_po, off_ml, off_cnt, off_pt, off_xpk, off_ssq, off_gemm, off_gcnt, total; };
 OpScratch op_layout() {
     OpScratch s; size_t o = 0;
     auto take = [&](size_t b) { size_t r = o; o = align_up(o + b, 256); return r; };
@@ -867,6 +889,8 @@ OpScratch op_layout() {
     s.off_cnt = take(4 * 256);
     s.off_xpk = take(4 * (size_t)KG_M_MAX * OP_K_MAX);
     s.off_ssq = take(4 * (size_t)KG_M_MAX * 1024);
+    s.off_gemm = take(OP_GEMM_PART);
+    s.off_gcnt = take(4 * (OP_GEMM_CNT + 1));
     s.total = o;
     return s;
 }
@@ -1073,25 +1097,66 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// Tensor map of a row-major bf16 matrix [rows, K] read in boxes of 64 columns x 128 rows with the 128-byte swizzle.
+// Tensor map of a row-major bf16 matrix [rows, K] read in boxes of 64 columns x box_rows rows with the 128-byte swizzle.
 // base is 16-byte aligned and K * 2 a multiple of 16 (checked by the callers' shape test).
-bool make_tmap(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t K) {
+bool make_tmap(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t K, int box_rows) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {K, rows};
     const cuuint64_t strides[1] = {K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)GM_BK, (cuuint32_t)GM_BM};
+    const cuuint32_t box[2] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+int tmap_failed() {
+    std::snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
+    return KG_E_CUDA;
+}
 
-// launched with the consumer warps only (no copy warp: nothing is streamed), which leaves 255 registers per thread
-__global__ void __launch_bounds__(NTHREADS, 1) pf_attention_kernel(const __grid_constant__ Dev D, AttArgs a, int nrows) {
-    extern __shared__ __align__(128) char smem[];
-    Ctx& c = ctx_init(smem, nullptr, nullptr, false);
-    if (D.dm.hd == 128) attention_prefill<128>(D, a, c, nrows);
-    else attention_prefill<64>(D, a, c, nrows);
+// The kernel's warpgroups re-divide the registers of the launch: a budget beyond that pool would block them for ever, so
+// what the launch allocates is checked and never assumed.
+template <int EPI>
+int gemm_attributes() {
+    cudaFuncAttributes fa;
+    CK(cudaFuncGetAttributes(&fa, (const void*)pf_gemm_kernel<EPI>));
+    if ((long long)fa.numRegs * GM_THREADS < 128LL * GM_CTRL_REGS + 32LL * GM_EPI_WARPS * GM_EPI_REGS) {
+        std::snprintf(g_cuda_err, sizeof(g_cuda_err), "GEMM kernel compiled with %d registers per thread: too few for its register budgets", fa.numRegs);
+        return KG_E_INTERNAL;
+    }
+    CK(cudaFuncSetAttribute((const void*)pf_gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, GM_SMEM));
+    return KG_OK;
+}
+
+int prefill_tc_init(kg_model* m) {
+    m->pf.ready = false;
+    if (m->dev.dm.stream == 0 || !prefill_tc_shape(&m->cfg) || encode_tiled_fn() == nullptr) return KG_OK;
+    const uint64_t d = m->cfg.d_model, F = m->cfg.d_ffn, R = m->lay.pf_rows;
+    const int L = m->cfg.n_layers;
+    char* A = m->arena;
+    bool ok = true;
+    for (int p = 0; p < 2; ++p)
+        for (int i = 0; i < 4; ++i) {
+            ok = ok && make_tmap(&m->pf.x[p][i], A + m->lay.off_pf_x + (size_t)p * R * d * 2, R, d, 32 * (i + 1));
+            ok = ok && make_tmap(&m->pf.f[p][i], A + m->lay.off_pf_f + (size_t)p * R * F * 2, R, F, 32 * (i + 1));
+        }
+    m->pf.layer.resize(L);
+    for (int i = 0; i < L; ++i) {
+        const LayerW& lw = m->layers_host[i];
+        PfMaps::Layer& t = m->pf.layer[i];
+        ok = ok && make_tmap(&t.qkv, lw.wqkv, 3 * d, d, GM_TM / 2) && make_tmap(&t.o, lw.wo, d, d, GM_TM / 2) &&
+             make_tmap(&t.gate, lw.wgate, F, d, GM_TM / 4) && make_tmap(&t.up, lw.wup, F, d, GM_TM / 4) && make_tmap(&t.down, lw.wdown, d, F, GM_TM / 2);
+    }
+    ok = ok && make_tmap(&m->pf.adapter_kv, (const __nv_bfloat16*)m->layers_host[L].wqkv + d * d, 2 * d, d, GM_TM / 2);
+    if (!ok) return tmap_failed();
+    int r;
+    if ((r = gemm_attributes<PF_STORE>()) != KG_OK || (r = gemm_attributes<PF_QKV>()) != KG_OK || (r = gemm_attributes<PF_SWIGLU>()) != KG_OK) return r;
+    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<128>::BYTES));
+    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<64>::BYTES));
+    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
+    CK(cudaMemsetAsync(A + m->lay.off_pf_cnt, 0, 4 * (size_t)m->nctas, m->stream));
+    m->pf.ready = true;
+    return KG_OK;
 }
 
 // x_0 from the per-CTA LM-head partials; the sequence state after a prompt of n tokens (one warp)
@@ -1105,78 +1170,113 @@ __global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* 
     }
 }
 
-bool prefill_tc_ok(const kg_model* m, int n) {
-    return m->prefill_mode == 0 && m->dev.dm.stream != 0 && prefill_tc_shape(&m->cfg) && n >= 2 * KG_M_MAX && encode_tiled_fn() != nullptr;
+bool prefill_tc_ok(const kg_model* m, int n) { return m->prefill_mode == 0 && m->pf.ready && n >= 2 * KG_M_MAX; }
+
+// Tile shape and work items of a GEMM of `rows` activation rows and `wtiles` tiles of weight rows on `pairs` CTA pairs.
+// Row tiles: as few as 256 columns allow, all of the same width (a multiple of 64).  The last wave of tiles is cut into S
+// ranges of k, S the one with the shortest estimated time in units of a k block: the waves of ranges, plus what a cut
+// costs (writing the partial sums and reading S of them back, which grows with the tile's columns).
+void gm_plan(GemmArgs& g, int wtiles, int pairs, size_t part_bytes) {
+    g.nrt = (g.rows + GM_NT_MAX - 1) / GM_NT_MAX;
+    g.nt = ((g.rows + g.nrt - 1) / g.nrt + 63) / 64 * 64;
+    const int tiles = wtiles * g.nrt, nkb = g.K / GM_BK;
+    const int rem = tiles % pairs;
+    g.full = tiles - rem;
+    g.S = 1;
+    int best = nkb;
+    for (int S = 2; S <= 16 && rem > 0 && nkb / S >= 4; ++S) {
+        if ((size_t)rem * S * GM_TM * g.nt * 4 > part_bytes) break;
+        const int cost = (rem * S + pairs - 1) / pairs * ((nkb + S - 1) / S) + 4 + S * g.nt / 128;
+        if (cost < best) { best = cost; g.S = S; }
+    }
+    g.items = g.full + rem * g.S;
 }
 
-// C[rows, N] = (resid) + rowscale * planes[rows, K] W[N, K]^T; with W2: also C2 = rowscale * planes W2^T in the same launch
-int pf_gemm(kg_model* m, const void* W, int N, int K, int rows, float* C, const float* resid, const float* rowscale,
-            const void* W2 = nullptr, float* C2 = nullptr) {
-    char* A = m->arena;
-    const int rows_pad = (rows + GM_BM - 1) / GM_BM * GM_BM;
-    CUtensorMap th, tl, tw, tw2;
-    if (!make_tmap(&th, A + m->lay.off_pf_hi, rows_pad, K) || !make_tmap(&tl, A + m->lay.off_pf_lo, rows_pad, K) || !make_tmap(&tw, W, N, K) ||
-        !make_tmap(&tw2, W2 ? W2 : W, N, K)) {
-        std::snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
-        return KG_E_CUDA;
-    }
-    GemmArgs g;
-    g.C = C; g.C2 = C2; g.ldc = N; g.resid = resid; g.ldr = N; g.rowscale = rowscale; g.rows = rows; g.N = N; g.K = K; g.err = (int*)(A + m->lay.off_pf_err);
-    pf_gemm_kernel<<<dim3(N / GM_BN, rows_pad / GM_BM, W2 ? 2 : 1), GM_THREADS, GM_SMEM, m->stream>>>(th, tl, tw, tw2, g);
+template <int EPI>
+int gm_launch(GemmArgs& g, const CUtensorMap& hi, const CUtensorMap& lo, const CUtensorMap& w, const CUtensorMap& w2, int pairs, cudaStream_t s) {
+    const int used = g.items < pairs ? g.items : pairs;
+    pf_gemm_kernel<EPI><<<2 * used, GM_THREADS, GM_SMEM, s>>>(hi, lo, w, w2, g);
     CK(cudaGetLastError());
     return KG_OK;
 }
 
-// The prompt in blocks of PF_ROWS rows, each block through all layers (its K / V are in the caches before the next
-// block attends to them), the adapter's K / V after layer l, the LM head on the last row.
+// The prompt in blocks of at most PF_ROWS rows of about equal size, each block through all layers (its K / V are in the
+// caches before the next block attends to them), the adapter's K / V after layer l, the LM head on the last row.
 int prefill_tc(kg_model* m, int n) {
     typedef __nv_bfloat16 WT;
     const kg_config& c = m->cfg;
     const Dev& D = m->dev;
     cudaStream_t s = m->stream;
     char* A = m->arena;
-    const int d = c.d_model, F = c.d_ffn, L = c.n_layers, H = c.n_heads;
-    float* h = (float*)(A + m->lay.off_pf_h); float* h2 = (float*)(A + m->lay.off_pf_h2);
-    float* qkv = (float*)(A + m->lay.off_pf_qkv); float* attn = (float*)(A + m->lay.off_pf_attn);
-    float* gate = (float*)(A + m->lay.off_pf_gate); float* up = (float*)(A + m->lay.off_pf_up);
-    WT* hi = (WT*)(A + m->lay.off_pf_hi); WT* lo = (WT*)(A + m->lay.off_pf_lo);
-    float* rs = (float*)(A + m->lay.off_pf_err) + 16;               // [PF_ROWS] 1/rms of the rows the planes were made from
-    CK(cudaFuncSetAttribute((const void*)pf_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GM_SMEM));
-    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
-    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
-    CK(cudaMemsetAsync(A + m->lay.off_pf_err, 0, 4, s));
-    const size_t lstride = (size_t)D.dm.n_pages * H * c.page_size * c.head_dim;
-    int r = KG_OK;
-    for (int b0 = 0; b0 < n; b0 += PF_ROWS) {
-        const int rows = n - b0 < PF_ROWS ? n - b0 : PF_ROWS;
-        pf_embed_kernel<WT><<<rows, 256, 0, s>>>(D.prompt + b0, (const WT*)D.embed, c.vocab, d, h);
-        auto qkv_and_append = [&](const LayerW& lw, int li) -> int {
-            pf_norm_split_kernel<<<rows, PF_EW_THREADS, 0, s>>>(h, d, d, lw.g1, c.rms_eps, hi, lo, rs);
-            int rr = pf_gemm(m, lw.wqkv, 3 * d, d, rows, qkv, nullptr, rs);
-            if (rr != KG_OK) return rr;
-            pf_rope_append_kernel<WT><<<dim3(rows, H), 64, 0, s>>>(D, qkv, b0, (WT*)D.kcache + (size_t)li * lstride, (WT*)D.vcache + (size_t)li * lstride);
-            return KG_OK;
+    const int d = c.d_model, F = c.d_ffn, L = c.n_layers, H = c.n_heads, hd = c.head_dim;
+    const size_t R = m->lay.pf_rows;
+    float* h = (float*)(A + m->lay.off_pf_h);
+    WT* xh = (WT*)(A + m->lay.off_pf_x); WT* xl = xh + R * d;
+    WT* qh = (WT*)(A + m->lay.off_pf_q); WT* ql = qh + R * d;
+    WT* fh = (WT*)(A + m->lay.off_pf_f); WT* fl = fh + R * F;
+    float* rs = (float*)(A + m->lay.off_pf_rs);                     // 1/rms of the rows the planes were made from
+    float2* cs = (float2*)(A + m->lay.off_pf_cs);
+    int* err = (int*)(A + m->lay.off_pf_err);
+    const int pairs = m->nctas / 2;
+    CK(cudaMemsetAsync(err, 0, 4, s));
+    const size_t lstride = (size_t)D.dm.n_pages * H * c.page_size * hd;
+    const int nblk = (int)((n + R - 1) / R);
+    const int brows = nblk == 1 ? n : ((n + nblk - 1) / nblk + 63) / 64 * 64;
+    int last = 0;
+    for (int b0 = 0; b0 < n; b0 += brows) {
+        const int rows = n - b0 < brows ? n - b0 : brows;
+        last = rows - 1;
+        pf_embed_kernel<<<rows, 256, 0, s>>>(D.prompt + b0, (const WT*)D.embed, c.vocab, d, h);
+        pf_rope_table_kernel<<<rows, hd / 2, 0, s>>>(D, b0, cs);
+        GemmArgs base{};
+        base.rows = rows; base.err = err; base.part = (float*)(A + m->lay.off_pf_part); base.cnt = (unsigned*)(A + m->lay.off_pf_cnt);
+        auto norm = [&](const float* gain) { pf_norm_split_kernel<<<rows, PF_EW_THREADS, 0, s>>>(h, d, d, gain, c.rms_eps, xh, xl, rs); };
+        auto qkv = [&](const CUtensorMap& w, int li, int sec0) {
+            GemmArgs g = base;
+            g.N = (3 - sec0) * d; g.K = d; g.rowscale = rs; g.hi = qh; g.lo = ql; g.ldp = d; g.hd = hd; g.H = H; g.sec0 = sec0; g.pos0 = b0;
+            g.cs = cs; g.page_table = D.page_table; g.ps_shift = D.dm.ps_shift; g.n_phys = D.dm.n_phys; g.st = D.st;
+            g.kc = (WT*)D.kcache + (size_t)li * lstride; g.vc = (WT*)D.vcache + (size_t)li * lstride;
+            g.qscale = 1.4426950408889634f / std::sqrt((float)hd);
+            gm_plan(g, (g.N + GM_TM - 1) / GM_TM, pairs, m->lay.pf_part_bytes);
+            return gm_launch<PF_QKV>(g, m->pf.x[0][g.nt / 64 - 1], m->pf.x[1][g.nt / 64 - 1], w, w, pairs, s);
+        };
+        auto resid = [&](const CUtensorMap& w, int K) {            // h += planes W^T
+            GemmArgs g = base;
+            g.N = d; g.K = K; g.C = h; g.resid = h; g.ldc = d;
+            gm_plan(g, (d + GM_TM - 1) / GM_TM, pairs, m->lay.pf_part_bytes);
+            const int i = g.nt / 64 - 1;
+            return K == d ? gm_launch<PF_STORE>(g, m->pf.x[0][i], m->pf.x[1][i], w, w, pairs, s)
+                          : gm_launch<PF_STORE>(g, m->pf.f[0][i], m->pf.f[1][i], w, w, pairs, s);
         };
         for (int i = 0; i < L; ++i) {
             const LayerW& lw = m->layers_host[i];
-            if ((r = qkv_and_append(lw, i)) != KG_OK) return r;
-            AttArgs at;
-            at.qkv = qkv; at.M = 0; at.pos0 = b0; at.kc = (WT*)D.kcache + (size_t)i * lstride; at.vc = (WT*)D.vcache + (size_t)i * lstride;
-            at.out = attn; at.opk = nullptr;
-            pf_attention_kernel<<<m->nctas, NTHREADS, SMEM_TOTAL, s>>>(D, at, rows);
-            pf_split_kernel<<<dim3(rows, (d / 4 + PF_EW_THREADS - 1) / PF_EW_THREADS), PF_EW_THREADS, 0, s>>>(attn, d, d, hi, lo);
-            if ((r = pf_gemm(m, lw.wo, d, d, rows, h2, h, nullptr)) != KG_OK) return r;
-            pf_norm_split_kernel<<<rows, PF_EW_THREADS, 0, s>>>(h2, d, d, lw.g2, c.rms_eps, hi, lo, rs);
-            if ((r = pf_gemm(m, lw.wgate, F, d, rows, gate, nullptr, rs, lw.wup, up)) != KG_OK) return r;
-            pf_swiglu_split_kernel<<<dim3(rows, (F / 4 + PF_EW_THREADS - 1) / PF_EW_THREADS), PF_EW_THREADS, 0, s>>>(gate, up, F, hi, lo);
-            if ((r = pf_gemm(m, lw.wdown, d, F, rows, h, h2, nullptr)) != KG_OK) return r;
-            if (i == c.exit_layer - 1 && (r = qkv_and_append(m->layers_host[L], L)) != KG_OK) return r;      // the adapter's K / V
+            const PfMaps::Layer& tm = m->pf.layer[i];
+            int r;
+            norm(lw.g1);
+            if ((r = qkv(tm.qkv, i, 0)) != KG_OK) return r;
+            FaArgs fa;
+            fa.qh = qh; fa.ql = ql; fa.kc = (const WT*)D.kcache + (size_t)i * lstride; fa.vc = (const WT*)D.vcache + (size_t)i * lstride;
+            fa.oh = xh; fa.ol = xl; fa.page_table = D.page_table; fa.ps_shift = D.dm.ps_shift; fa.n_phys = D.dm.n_phys; fa.st = D.st;
+            fa.H = H; fa.pos0 = b0; fa.rows = rows;
+            const int fgrid = (rows + FA_ROWS - 1) / FA_ROWS * H;
+            if (hd == 128) pf_attention_kernel<128><<<fgrid, 256, FaSm<128>::BYTES, s>>>(fa);
+            else pf_attention_kernel<64><<<fgrid, 256, FaSm<64>::BYTES, s>>>(fa);
+            if ((r = resid(tm.o, d)) != KG_OK) return r;
+            norm(lw.g2);
+            GemmArgs g = base;
+            g.N = F; g.K = d; g.rowscale = rs; g.hi = fh; g.lo = fl; g.ldp = F;
+            gm_plan(g, F / (GM_TM / 2), pairs, m->lay.pf_part_bytes);
+            if ((r = gm_launch<PF_SWIGLU>(g, m->pf.x[0][g.nt / 64 - 1], m->pf.x[1][g.nt / 64 - 1], tm.gate, tm.up, pairs, s)) != KG_OK) return r;
+            if ((r = resid(tm.down, F)) != KG_OK) return r;
+            if (i == c.exit_layer - 1) {                              // the adapter's K / V
+                norm(m->layers_host[L].g1);
+                if ((r = qkv(m->pf.adapter_kv, L, 1)) != KG_OK) return r;
+            }
         }
         CK(cudaGetLastError());
     }
     // LM head on the last prompt row (still in h): the decode path's fused head operator on one row
     {
-        const int last = (n - 1) % PF_ROWS;
         pack_rows_kernel<<<m->nctas, 256, 0, s>>>(h + (size_t)last * d, d, 1, d, D.g_final, D.hA_pk, d * 4, D.ssq_hA, m->nctas);
         LinArgs a{};
         a.W = D.head; a.N = c.vocab; a.K = d; a.M = 1; a.x = h + (size_t)last * d; a.ldx = d; a.gain = D.g_final; a.eps = c.rms_eps;
@@ -1184,7 +1284,7 @@ int prefill_tc(kg_model* m, int n) {
         a.epi = EPI_HEAD; a.scale = c.logit_scale; a.head_part = D.head_part;
         a.logits_dbg = c.debug_logits ? D.dbg_verify : nullptr; a.ld_dbg = c.vocab;
         op_linear_kernel<WT><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 1);
-        pf_finish_kernel<<<1, 32, 0, s>>>(D.head_part, m->nctas, D.st, D.out_tokens, n, (const int*)(A + m->lay.off_pf_err));
+        pf_finish_kernel<<<1, 32, 0, s>>>(D.head_part, m->nctas, D.st, D.out_tokens, n, err);
         CK(cudaGetLastError());
     }
     return KG_OK;
@@ -1202,27 +1302,24 @@ extern "C" int kg_op_gemm(const void* W, int32_t N, int32_t K, const float* x, i
                           void* scratch, void* stream) {
     if (!W || !x || !out || !scratch || M < 1 || N < 1 || K < 1) return KG_E_ARG;
     if (!aligned16(W) || !aligned16(x) || !aligned16(resid) || !aligned16(out) || !aligned16(scratch)) return KG_E_ARG;
-    if (N % GM_BN || K % GM_BK) return KG_E_ARG;
-    const int rows_pad = (M + GM_BM - 1) / GM_BM * GM_BM;
+    if (N % (GM_TM / 2) || K % GM_BK) return KG_E_ARG;
+    const int rows_pad = (M + 127) / 128 * 128;
     OpScratch sc = op_layout();
     if ((size_t)rows_pad * K * 4 > 4 * (size_t)KG_M_MAX * S_CAP * 8192) return KG_E_LIMIT;  // both planes live in the split-partial scratch
     if (!encode_tiled_fn()) { std::snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled is not available"); return KG_E_CUDA; }
     cudaStream_t s = (cudaStream_t)stream;
     __nv_bfloat16* hi = (__nv_bfloat16*)((char*)scratch + sc.off_po);
     __nv_bfloat16* lo = hi + (size_t)rows_pad * K;
-    int* err = (int*)((char*)scratch + sc.off_cnt);
-    CK(cudaMemsetAsync(err, 0, 4, s));
-    CK(cudaMemsetAsync(hi, 0, (size_t)rows_pad * K * 4, s));
-    CK(cudaFuncSetAttribute((const void*)pf_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GM_SMEM));
+    const int nctas = sm_count();
+    GemmArgs g{};
+    g.rows = M; g.N = N; g.K = K; g.C = out; g.resid = resid; g.ldc = N;
+    g.part = (float*)((char*)scratch + sc.off_gemm); g.cnt = (unsigned*)((char*)scratch + sc.off_gcnt); g.err = (int*)g.cnt + OP_GEMM_CNT;
+    CK(cudaMemsetAsync(g.cnt, 0, 4 * (OP_GEMM_CNT + 1), s));
+    const int r = gemm_attributes<PF_STORE>();
+    if (r != KG_OK) return r;
+    gm_plan(g, (N + GM_TM - 1) / GM_TM, nctas / 2, nctas <= OP_GEMM_CNT ? OP_GEMM_PART : 0);
     pf_split_kernel<<<dim3(M, (K / 4 + PF_EW_THREADS - 1) / PF_EW_THREADS), PF_EW_THREADS, 0, s>>>(x, K, K, hi, lo);
     CUtensorMap th, tl, tw;
-    if (!make_tmap(&th, hi, rows_pad, K) || !make_tmap(&tl, lo, rows_pad, K) || !make_tmap(&tw, W, N, K)) {
-        std::snprintf(g_cuda_err, sizeof(g_cuda_err), "cuTensorMapEncodeTiled failed");
-        return KG_E_CUDA;
-    }
-    GemmArgs g;
-    g.C = out; g.C2 = nullptr; g.ldc = N; g.resid = resid; g.ldr = N; g.rowscale = nullptr; g.rows = M; g.N = N; g.K = K; g.err = err;
-    pf_gemm_kernel<<<dim3(N / GM_BN, rows_pad / GM_BM), GM_THREADS, GM_SMEM, s>>>(th, tl, tw, tw, g);
-    CK(cudaGetLastError());
-    return KG_OK;
+    if (!make_tmap(&th, hi, M, K, g.nt / 2) || !make_tmap(&tl, lo, M, K, g.nt / 2) || !make_tmap(&tw, W, N, K, GM_TM / 2)) return tmap_failed();
+    return gm_launch<PF_STORE>(g, th, tl, tw, tw, nctas / 2, s);
 }

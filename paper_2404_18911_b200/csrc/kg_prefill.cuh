@@ -1,17 +1,13 @@
 // Prompt processing on the 5th-generation tensor cores.
 //
 // The decode path streams every weight once per <= 16 rows; for a prompt of hundreds of rows that is the wrong
-// trade.  Here a block of up to PF_ROWS prompt rows goes through a layer as real GEMMs: C[rows, N] = A[rows, K] W[N, K]^T
-// with 128 x 128 output tiles, operands brought into shared memory by TMA tensor copies (64-column boxes, 128-byte
-// swizzle), tcgen05.mma issued by one thread with the accumulators in tensor memory, and an epilogue that reads
-// them back with tcgen05.ld.  The activations keep fp32 accuracy the same way as in the decode path: every value
-// is split into two bf16 planes, x = hi + lo, and both planes are multiplied with the bf16 weights into the same
-// fp32 accumulator.  The tensor core's fp32 accumulation rounds toward zero, which biases long chains; every k block
-// of 64 therefore gets a fresh accumulator (four rotate through the 512 tensor-memory columns) that the epilogue
-// warps add to fp32 registers while the next blocks are being multiplied.
+// trade.  Here a block of up to PF_ROWS prompt rows goes through a layer as real GEMMs C[rows, N] = A[rows, K] W[N, K]^T.
+// The activations keep fp32 accuracy the same way as in the decode path: every value is split into two bf16 planes,
+// x = hi + lo, and both planes are multiplied with the bf16 weights into the same fp32 accumulator.
 //
-// Around the GEMMs sit small elementwise kernels (embedding gather, RMSNorm + split into planes, SwiGLU + split,
-// RoPE + KV append) and the tensor-core attention of the decode path run over (row block, head) items.
+// A layer is seven launches: RMSNorm + split into planes, QKV GEMM (epilogue: rotation, K / V rows into the cache, q
+// planes), attention (reads q planes and the cache, writes planes), O GEMM (+ residual), RMSNorm + split, gate / up GEMM
+// (epilogue: SwiGLU into planes), down GEMM (+ residual).
 #pragma once
 
 #include <cuda.h>
@@ -20,30 +16,50 @@
 
 namespace kg {
 
-constexpr int PF_ROWS = 512;            // prompt rows per pass through the layers
-constexpr int GM_BM = 128, GM_BN = 128, GM_BK = 64;
-constexpr int GM_STAGES = 4;
-constexpr int GM_TILE_BYTES = GM_BM * GM_BK * 2;                       // one 128 x 64 bf16 tile: 16 KB
-constexpr int GM_STAGE_BYTES = 3 * GM_TILE_BYTES;                      // A hi, A lo, W
-constexpr int GM_SMEM = GM_STAGES * GM_STAGE_BYTES + 1024 + 256;       // + alignment slack + barriers
-constexpr int GM_THREADS = 320;                                        // warp 0: TMA, warp 1: MMA, warps 2-9: epilogue
-constexpr int GM_EPI_WARPS = 8;                                        // two per tensor-memory lane quadrant, 64 columns each
-constexpr int GM_ACC = 4;                                              // rotating accumulators of 128 columns (= stages)
+constexpr int PF_ROWS = 2048;                  // most prompt rows per pass through the layers
+constexpr int GM_BK = 64;                      // k block: one 128-byte swizzle atom of bf16
+constexpr int GM_CHAIN = 2;                    // k blocks summed by the tensor core before the sum goes to fp32 registers
+constexpr int GM_TM = 256;                     // weight rows per CTA pair (128 in each CTA: the M side of the MMA)
+constexpr int GM_NT_MAX = 256;                 // most activation rows per tile (the N side)
+constexpr int GM_A_BYTES = (GM_TM / 2) * GM_BK * 2;                    // this CTA's weight rows of a k block: 16 KB
+constexpr int GM_RING_BYTES = 192 * 1024;
+constexpr int GM_MAX_STAGES = 8;
+constexpr int GM_MAX_ACC = 4;
+constexpr int GM_EPI_WARPS = 8;                // two per tensor-memory lane quadrant, half of the tile's columns each
+constexpr int GM_THREADS = 128 + 32 * GM_EPI_WARPS;                    // warp 0: TMA, warp 1: MMA, two idle warps, then the epilogue
+constexpr int GM_STAGE_FLOATS = 32 * 32;                               // [32 columns][32 lanes] of one epilogue warp
+constexpr int GM_XCH_BYTES = GM_EPI_WARPS * GM_STAGE_FLOATS * 4;
+constexpr int GM_SMEM = 1024 + GM_RING_BYTES + GM_XCH_BYTES + 256;     // alignment slack, operand ring, epilogue staging, barriers
+static_assert(GM_SMEM <= SMEM_TOTAL, "GEMM shared memory");
+// registers: the first warpgroup needs few, the two epilogue warpgroups keep 128 sums and two batches of accumulator columns
+// per thread; the pool is what the launch allocated (GM_THREADS x 168), a request beyond it would block for ever
+constexpr int GM_CTRL_REGS = 56, GM_EPI_REGS = 216;
+static_assert(GM_THREADS == DECODE_THREADS && 128 * GM_CTRL_REGS + 32 * GM_EPI_WARPS * GM_EPI_REGS <= GM_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
 constexpr unsigned long long GM_WAIT_CLK = 4000000000ull;              // ~2 s: a wait that runs this long gives up
 
+enum { PF_STORE = 0, PF_QKV = 1, PF_SWIGLU = 2 };                      // what the epilogue makes of the products
+
 struct GemmArgs {
-    float* C; int ldc;                  // [rows, N] fp32
-    float* C2;                          // grid.z == 2: the output of the second weight matrix (same shape, same A)
-    const float* resid; int ldr;        // optional: C = resid + rowscale * A W^T
-    const float* rowscale;              // optional: one factor per row (1/rms of the row the planes were made from)
-    int rows;                           // valid rows (the planes hold a multiple of 128, zero beyond)
-    int N, K;                           // multiples of 128 and 64
+    int rows;                           // valid activation rows (rows of the planes beyond them hold anything)
+    int N, K;                           // output features (multiple of 128; PF_SWIGLU: of each matrix) and contraction (of 64)
+    int nt, nrt;                        // activation rows per tile (64, 128, 192 or 256) and row tiles
+    int full, S, items;                 // work items: `full` whole tiles, then every remaining tile cut into S ranges of k
+    const float* rowscale;              // PF_QKV, PF_SWIGLU: one factor per row (1/rms of the row the planes were made from)
+    float* C; const float* resid; int ldc;      // PF_STORE: C = (resid) + product; C may be resid itself
+    __nv_bfloat16* hi; __nv_bfloat16* lo; int ldp;      // PF_SWIGLU: planes of SiLU(gate) * up; PF_QKV: planes of the rotated, scaled q
+    int hd, H, sec0, pos0;              // PF_QKV: sec0 = first section of W's rows (0: q, k, v; 1: k, v only)
+    const float2* cs;                   // PF_QKV: cos, sin [rows][hd / 2]
+    const int* page_table; int ps_shift, n_phys; State* st;
+    __nv_bfloat16* kc; __nv_bfloat16* vc;
+    float qscale;
+    float* part; unsigned* cnt;         // partial sums of the cut tiles, arrival counters (left at zero)
     int* err;                           // set to 1 when a bounded wait expired
 };
 
 // ---- TMA tile copy, tensor memory and tcgen05 MMA ----------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* tmap, int x, int y, uint32_t bar_smem) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+// (one CTA of a pair: the copy lands in this CTA's shared memory and is counted on an mbarrier of either CTA of the pair)
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const CUtensorMap* tmap, int x, int y, uint32_t bar_smem) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst_smem), "l"(tmap), "r"(x), "r"(y), "r"(bar_smem) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -55,27 +71,46 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 constexpr uint32_t UMMA_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
 // Instruction descriptor: fp32 accumulate (bit 4), bf16 A and B (bits 7, 10), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-__device__ __forceinline__ uint32_t umma_idesc_128(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
+__device__ __forceinline__ uint32_t umma_idesc(int m, int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-// D[128 x N] (+)= A[128 x 16] B[N x 16]^T, issued by one thread
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+// D[256 x N] (+)= A[256 x 16] B[N x 16]^T over a CTA pair, issued by one thread of the even CTA: each CTA holds 128 rows
+// of A, N / 2 rows of B and its 128 rows of D
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
     asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate));
 }
-// the mbarrier receives one arrival when every MMA this thread has issued so far has completed
-__device__ __forceinline__ void umma_commit(unsigned long long* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// the mbarrier of both CTAs of the pair receives one arrival when every MMA this thread has issued so far has completed
+__device__ __forceinline__ void umma_commit_pair(unsigned long long* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
+// shared-memory address of the same variable in the even CTA of the pair
+__device__ __forceinline__ uint32_t leader_smem(uint32_t addr) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 // 32 consecutive accumulator columns of this thread's tensor-memory lane (lane = 32 * (warp % 4) + lane id)
-// (asynchronous: tmem_ld_wait() before the values are used)
+// (asynchronous: tmem_ld_wait32() before the values are used)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                  : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// (the values pass through the wait, so that nothing can use them before it)
+__device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) :: "memory");
+}
 
 // bounded wait on an mbarrier phase; on expiry the error word is set and false returned
 __device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity, int* err) {
@@ -92,139 +127,542 @@ __device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity
 }
 
 // ---- the GEMM ------------------------------------------------------------------------------------------------------
-// grid = (N / 128, row tiles, 1 or 2 weight matrices that share A); one 128 x 128 tile of C per CTA.  k block kb uses shared-memory stage kb mod 4 and
-// tensor-memory accumulator kb mod 4: its eight MMAs (four k16-steps, hi and lo plane) start a fresh accumulator, one
-// tcgen05.commit tells the producer that the stage is free and the epilogue warps that the accumulator is complete,
-// and the epilogue warps add it to their fp32 registers (round to nearest) and hand the accumulator back.  No sum
-// therefore passes through more than eight of the tensor core's truncating accumulations.
-__global__ void __launch_bounds__(GM_THREADS, 1) pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
-                                                                const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_w2,
-                                                                const GemmArgs g) {
-    extern __shared__ __align__(128) char smem_raw[];
-    const uint32_t raw = smem_u32(smem_raw);
-    char* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);              // swizzled tiles sit on 1024-byte boundaries
-    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + GM_STAGES * GM_STAGE_BYTES);   // TMA -> MMA: stage filled
-    unsigned long long* mma_done = full + GM_STAGES;      // MMA -> TMA, epilogue: the k block's MMAs have completed
-    unsigned long long* acc_free = mma_done + GM_STAGES;  // epilogue -> MMA: the accumulator has been read (one arrival per warp)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + GM_ACC);
-    static_assert(GM_STAGES == GM_ACC, "a k block's stage and accumulator share one index and one completion barrier");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n0 = blockIdx.x * GM_BN, m0 = blockIdx.y * GM_BM;
+// One CTA pair (cluster of two, cta_group::2) per work item; the grid is persistent (one pair per two SMs).  The weights
+// are the M side of the MMA (256 rows of a pair), the activation rows the N side (nt of them), because the weights are
+// always whole tiles while a prompt may have any number of rows: nt follows the rows, and the accumulator has one weight
+// row per tensor-memory lane.
+//
+// What bounds it: the operands of a k block.  With the activations in two planes a 128 x 128 tile of one CTA needs 48 KB for
+// 4.2 MFLOP (94 bytes per clock and SM at the full MMA rate, more than L2 delivers); the pair's 256 x 256 tile needs 48 KB
+// per CTA for 8.4 MFLOP, since the two CTAs share the activation planes.  With the attention below and the fused epilogues
+// the prompt pass of the 7B shape (1999 tokens) went from 96.9 to 58.5 ms, of the 13B shape (2048 tokens) from 187 to 107 ms.
+//
+// Accumulation.  The tensor core's fp32 accumulation rounds toward zero at every MMA, by an amount that follows the size
+// of the running sum, which biases long chains.  A chain of GM_CHAIN = 2 k blocks multiplies both lo planes first - sums
+// about 2^-9 of the result, whose truncation does not count - and then the hi planes: eight truncations that count per
+// 128 k, where one accumulator per k block with hi and lo in turn takes sixteen (N(0,1) rows, K = 4096, against float64:
+// error 2.459e-6 of the norm and bias -1.06e-7, before 2.465e-6 and -1.41e-7; longer chains lose bits again).  The epilogue warps add every chain to
+// fp32 registers (round to nearest) while the next ones are multiplied; the accumulators rotate through tensor memory.
+//
+// Work items.  Tiles are ordered row tile first, so that the pairs that run at the same time share weight tiles.  The
+// last, incomplete wave of tiles is cut into S ranges of k (gm_plan on the host): each range leaves fp32 partial sums in
+// global memory, and the CTA that arrives last adds them in the order of the ranges and runs the epilogue; nothing waits.
+struct GmItem { int wt, rt, kb0, kb1, s, r; };            // s < 0: a whole tile
+__device__ __forceinline__ GmItem gm_item(const GemmArgs& g, int idx) {
+    GmItem it;
     const int nkb = g.K / GM_BK;
-    const CUtensorMap* tm_wz = blockIdx.z ? &tm_w2 : &tm_w;
-    float* Cz = blockIdx.z ? g.C2 : g.C;
+    int tile = idx;
+    it.kb0 = 0; it.kb1 = nkb; it.s = -1; it.r = 0;
+    if (idx >= g.full && g.S > 1) {
+        const int j = idx - g.full;
+        it.r = j / g.S; it.s = j - it.r * g.S;
+        tile = g.full + it.r;
+        it.kb0 = nkb * it.s / g.S; it.kb1 = nkb * (it.s + 1) / g.S;
+    }
+    it.wt = tile / g.nrt; it.rt = tile - it.wt * g.nrt;
+    return it;
+}
+
+__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const unsigned*>(&v);
+}
+
+// Finished products of 32 columns (activation rows row0 ..) of this warp's 32 weight rows, staged as [column][lane] in
+// `mine` (`theirs`: the partner warp's staging).  The loops run over the staging and not over registers so that the code
+// stays small: as straight-line code over 128 registers the epilogue took 18 us a tile, most of it instruction fetch.
+template <int EPI>
+__device__ __forceinline__ void gm_epilogue(const GemmArgs& g, const float* mine, const float* theirs, int row0, int wt, int rank, int q, int role) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (EPI == PF_STORE) {
+        // four columns at a time, 16 bytes (four features) per lane
+        const int n = wt * GM_TM + rank * (GM_TM / 2) + q * 32 + (lane & 7) * 4, c0 = lane >> 3;
+        if (n >= g.N) return;
+        float4 rv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + i * 4 + c0;
+            rv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (g.resid && row < g.rows) rv[i] = *reinterpret_cast<const float4*>(g.resid + (size_t)row * g.ldc + n);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + i * 4 + c0;
+            const float4 v = *reinterpret_cast<const float4*>(mine + (i * 4 + c0) * 32 + (lane & 7) * 4);
+            if (row < g.rows) *reinterpret_cast<float4*>(g.C + (size_t)row * g.ldc + n) = make_float4(rv[i].x + v.x, rv[i].y + v.y, rv[i].z + v.z, rv[i].w + v.w);
+        }
+    } else {
+        // two columns at a time, two features per lane; of a pair of warps each takes half of the columns
+        const int cl = lane >> 4, fe = (lane & 15) * 2;
+        if constexpr (EPI == PF_SWIGLU) {
+            const int f = wt * (GM_TM / 2) + rank * (GM_TM / 4) + (q & 1) * 32 + fe;
+            const float* ga = role ? theirs : mine;
+            const float* up = role ? mine : theirs;
+#pragma unroll 2
+            for (int i = 0; i < 8; ++i) {
+                const int col = role * 16 + i * 2 + cl, row = row0 + col;
+                const float2 a = *reinterpret_cast<const float2*>(ga + col * 32 + fe), b = *reinterpret_cast<const float2*>(up + col * 32 + fe);
+                if (row < g.rows) {
+                    const float rs = g.rowscale[row];
+                    unsigned hi, lo;
+                    split_hi_lo(make_float2(silu_f(a.x * rs) * (b.x * rs), silu_f(a.y * rs) * (b.y * rs)), hi, lo);
+                    *reinterpret_cast<unsigned*>(g.hi + (size_t)row * g.ldp + f) = hi;
+                    *reinterpret_cast<unsigned*>(g.lo + (size_t)row * g.ldp + f) = lo;
+                }
+            }
+        } else {
+            const int d = g.H * g.hd, half = g.hd >> 1, psm = (1 << g.ps_shift) - 1;
+            const int n0 = wt * GM_TM + rank * (GM_TM / 2);                 // this CTA's 128 rows of W lie in one section
+            if (n0 >= g.N) return;
+            const int s0 = n0 / d, sec = s0 + g.sec0, nh = n0 - s0 * d + q * 32;     // this warp's first row within the section
+            const int hh = nh >> (half == 64 ? 7 : 6), e0 = nh & (g.hd - 1);
+            if (sec == 2) {
+#pragma unroll 4
+                for (int i = 0; i < 16; ++i) {
+                    const int col = i * 2 + cl, row = row0 + col;
+                    const float2 v = *reinterpret_cast<const float2*>(mine + col * 32 + fe);
+                    if (row < g.rows) {
+                        const float rs = g.rowscale[row];
+                        const int pos = g.pos0 + row;
+                        const int page = checked_page(__ldg(g.page_table + (pos >> g.ps_shift)), g.n_phys, g.st, 61);
+                        *reinterpret_cast<unsigned*>(g.vc + ((((size_t)page * g.H + hh) << g.ps_shift) + (pos & psm)) * g.hd + e0 + fe) = pack_bf16(v.x * rs, v.y * rs);
+                    }
+                }
+            } else {
+                // dims e, e + 1 of the first half of the head and their partners half a head further
+                const int e = (e0 & (half - 1)) + fe;
+                const float* xa = role ? theirs : mine;
+                const float* xb = role ? mine : theirs;
+#pragma unroll 2
+                for (int i = 0; i < 8; ++i) {
+                    const int col = role * 16 + i * 2 + cl, row = row0 + col;
+                    const float2 a = *reinterpret_cast<const float2*>(xa + col * 32 + fe), b = *reinterpret_cast<const float2*>(xb + col * 32 + fe);
+                    if (row < g.rows) {
+                        const float rs = g.rowscale[row];
+                        const float4 cs = __ldg(reinterpret_cast<const float4*>(g.cs + (size_t)row * half + e));
+                        const float a0 = a.x * rs, a1 = a.y * rs, b0 = b.x * rs, b1 = b.y * rs;
+                        const float2 r1 = make_float2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
+                        const float2 r2 = make_float2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
+                        if (sec == 0) {
+                            const size_t o = (size_t)row * g.ldp + (size_t)hh * g.hd + e;
+                            unsigned hi, lo;
+                            split_hi_lo(make_float2(r1.x * g.qscale, r1.y * g.qscale), hi, lo);
+                            *reinterpret_cast<unsigned*>(g.hi + o) = hi;
+                            *reinterpret_cast<unsigned*>(g.lo + o) = lo;
+                            split_hi_lo(make_float2(r2.x * g.qscale, r2.y * g.qscale), hi, lo);
+                            *reinterpret_cast<unsigned*>(g.hi + o + half) = hi;
+                            *reinterpret_cast<unsigned*>(g.lo + o + half) = lo;
+                        } else {
+                            const int pos = g.pos0 + row;
+                            const int page = checked_page(__ldg(g.page_table + (pos >> g.ps_shift)), g.n_phys, g.st, 62);
+                            __nv_bfloat16* kr = g.kc + ((((size_t)page * g.H + hh) << g.ps_shift) + (pos & psm)) * g.hd + e;
+                            *reinterpret_cast<unsigned*>(kr) = pack_bf16(r1.x, r1.y);
+                            *reinterpret_cast<unsigned*>(kr + half) = pack_bf16(r2.x, r2.y);
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GM_THREADS, 1)
+pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo, const __grid_constant__ CUtensorMap tm_w,
+               const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ GemmArgs g) {
+    extern __shared__ __align__(128) char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw) & 0xFFFFFFu;                   // offset inside this CTA's window
+    char* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);              // swizzled tiles sit on 1024-byte boundaries
+    float* xch = reinterpret_cast<float*>(smem + GM_RING_BYTES);
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + GM_RING_BYTES + GM_XCH_BYTES);   // even CTA: both CTAs' tiles have landed
+    unsigned long long* empty = full + GM_MAX_STAGES;      // the stage's MMAs have completed
+    unsigned long long* acc_full = empty + GM_MAX_STAGES;  // the accumulator is complete
+    unsigned long long* acc_free = acc_full + GM_MAX_ACC;  // even CTA: both CTAs' epilogue warps have read the accumulator
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + GM_MAX_ACC);
+    int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = blockIdx.x & 1, pair_id = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int stage_bytes = GM_A_BYTES + g.nt * 128;                       // weights, hi plane, lo plane
+    const int nst = min(GM_MAX_STAGES, GM_RING_BYTES / stage_bytes);       // 4 (nt = 256) .. 8: at least a chain's stages and as many ahead
+    const int nacc = g.nt <= 128 ? 4 : 2, acc_cols = g.nt <= 128 ? 128 : 256;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < GM_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&mma_done[i], 1); mbar_init(&acc_free[i], GM_EPI_WARPS); }
+        for (int i = 0; i < GM_MAX_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+        for (int i = 0; i < GM_MAX_ACC; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_free[i], 2 * GM_EPI_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();                                                    // both CTAs' barriers and tensor memory exist
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
-        // ---- TMA producer: A hi, A lo and W boxes of one k block per stage
-        for (int kb = 0; kb < nkb; ++kb) {
-            const int s = kb % GM_STAGES;
-            if (!gm_wait(&mma_done[s], ((unsigned)(kb / GM_STAGES) & 1u) ^ 1u, g.err)) break;
-            const uint32_t dst = smem_u32(smem + s * GM_STAGE_BYTES), bar = smem_u32(&full[s]);
-            mbar_arrive_expect_tx(&full[s], (unsigned)GM_STAGE_BYTES);
-            tma_load_2d(dst, &tm_hi, kb * GM_BK, m0, bar);
-            tma_load_2d(dst + GM_TILE_BYTES, &tm_lo, kb * GM_BK, m0, bar);
-            tma_load_2d(dst + 2 * GM_TILE_BYTES, tm_wz, kb * GM_BK, n0, bar);
-        }
-    } else if (warp == 1 && lane == 0) {
-        // ---- MMA issuer
-        const uint32_t idesc = umma_idesc_128(GM_BN);
-        for (int kb = 0; kb < nkb; ++kb) {
-            const int s = kb % GM_STAGES;
-            const unsigned par = (unsigned)(kb / GM_STAGES) & 1u;
-            if (!gm_wait(&acc_free[s], par ^ 1u, g.err)) break;
-            if (!gm_wait(&full[s], par, g.err)) break;
-            tc_fence_after();
-            const uint32_t a_hi = umma_desc_lo(smem_u32(smem + s * GM_STAGE_BYTES));
-            const uint32_t a_lo = umma_desc_lo(smem_u32(smem + s * GM_STAGE_BYTES + GM_TILE_BYTES));
-            const uint32_t w = umma_desc_lo(smem_u32(smem + s * GM_STAGE_BYTES + 2 * GM_TILE_BYTES));
-            const uint32_t d = tmem + (uint32_t)s * GM_BN;
-#pragma unroll
-            for (int k16 = 0; k16 < GM_BK / 16; ++k16) {
-                umma_bf16(d, a_hi + 2u * k16, w + 2u * k16, idesc, k16 > 0 ? 1u : 0u);
-                umma_bf16(d, a_lo + 2u * k16, w + 2u * k16, idesc, 1u);
-            }
-            umma_commit(&mma_done[s]);
-        }
-    } else if (warp >= 2) {
-        // ---- epilogue: thread = one row of the tile (tensor-memory lane = 32 * (warp % 4) + lane id) and one half of its
-        // columns (warps 2-5: columns 0-63, warps 6-9: 64-127); the 64 sums live in registers
-        const int q = warp & 3;
-        const int ch = ((warp - 2) >> 2) * (GM_BN / 2);
-        const int row = m0 + q * 32 + lane;
-        float acc[GM_BN / 2];
-#pragma unroll
-        for (int i = 0; i < GM_BN / 2; ++i) acc[i] = 0.f;
-        bool ok = true;
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int s = kb % GM_ACC;
-            ok = gm_wait(&mma_done[s], (unsigned)(kb / GM_ACC) & 1u, g.err);
-            if (!ok) break;
-            tc_fence_after();
-            uint32_t v0[32], v1[32];
-            const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(s * GM_BN + ch);
-            tmem_ld32(ta, v0);
-            tmem_ld32(ta + 32u, v1);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) { acc[i] += __uint_as_float(v0[i]); acc[32 + i] += __uint_as_float(v1[i]); }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_free[s]);
-        }
-        if (ok && row < g.rows) {
-            float* dst = Cz + (size_t)row * g.ldc + n0 + ch;
-            if (g.rowscale) {
-                const float rsc = g.rowscale[row];
-#pragma unroll
-                for (int i = 0; i < GM_BN / 2; ++i) acc[i] *= rsc;
-            }
-            if (g.resid) {
-                const float* rs = g.resid + (size_t)row * g.ldr + n0 + ch;
-#pragma unroll
-                for (int i = 0; i < GM_BN / 2; i += 4) {
-                    const float4 r4 = *reinterpret_cast<const float4*>(rs + i);
-                    acc[i] += r4.x; acc[i + 1] += r4.y; acc[i + 2] += r4.z; acc[i + 3] += r4.w;
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GM_CTRL_REGS));
+        if (warp == 0 && lane == 0) {
+            // ---- TMA producer of this CTA's tiles
+            int s = 0; unsigned par = 1u;
+            const int hrow = g.nt >> 1;
+            bool ok = true;
+            for (int idx = pair_id; idx < g.items && ok; idx += npairs) {
+                const GmItem it = gm_item(g, idx);
+                const int y_act = it.rt * g.nt + rank * hrow;
+                for (int kb = it.kb0; kb < it.kb1; ++kb) {
+                    if (!(ok = gm_wait(&empty[s], par, g.err))) break;
+                    if (rank == 0) mbar_arrive_expect_tx(&full[s], (unsigned)(2 * stage_bytes));
+                    const uint32_t dst = smem_u32(smem + s * stage_bytes), bar = leader_smem(smem_u32(&full[s]));
+                    const int x = kb * GM_BK;
+                    if (EPI == PF_SWIGLU) {
+                        const int y = it.wt * (GM_TM / 2) + rank * (GM_TM / 4);
+                        tma_load_2d_pair(dst, &tm_w, x, y, bar);
+                        tma_load_2d_pair(dst + GM_A_BYTES / 2, &tm_w2, x, y, bar);
+                    } else {
+                        tma_load_2d_pair(dst, &tm_w, x, it.wt * GM_TM + rank * (GM_TM / 2), bar);
+                    }
+                    tma_load_2d_pair(dst + GM_A_BYTES, &tm_hi, x, y_act, bar);
+                    tma_load_2d_pair(dst + GM_A_BYTES + hrow * 128, &tm_lo, x, y_act, bar);
+                    if (++s == nst) { s = 0; par ^= 1u; }
                 }
             }
+            // every completion arrives in this CTA's shared memory before it may leave
+            for (int i = 0; i < nst && ok; ++i) {
+                ok = gm_wait(&empty[s], par, g.err);
+                if (++s == nst) { s = 0; par ^= 1u; }
+            }
+        } else if (warp == 1 && lane == 0 && rank == 0) {
+            // ---- MMA issuer of the pair
+            const uint32_t idesc = umma_idesc(GM_TM, g.nt);
+            const uint32_t lo_off = (uint32_t)((g.nt >> 1) * 128) >> 4;          // hi plane -> lo plane, in descriptor units
+            int s = 0, a = 0; unsigned par = 0u, apar = 1u;
+            bool ok = true;
+            for (int idx = pair_id; idx < g.items && ok; idx += npairs) {
+                const GmItem it = gm_item(g, idx);
+                for (int kb = it.kb0; kb < it.kb1 && ok; kb += GM_CHAIN) {
+                    const int nb = min(GM_CHAIN, it.kb1 - kb);
+                    const uint32_t dcol = tmem + (uint32_t)(a * acc_cols);
+                    if (!(ok = gm_wait(&acc_free[a], apar, g.err))) break;
+                    // the lo planes of the chain's k blocks
+                    int sl = s; unsigned pl = par;
+                    for (int b = 0; b < nb && ok; ++b) {
+                        if (!(ok = gm_wait(&full[sl], pl, g.err))) break;
+                        tc_fence_after();
+                        const uint32_t base = smem_u32(smem + sl * stage_bytes);
+                        const uint32_t w = umma_desc_lo(base), x = umma_desc_lo(base + GM_A_BYTES) + lo_off;
 #pragma unroll
-            for (int i = 0; i < GM_BN / 2; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+                        for (int k16 = 0; k16 < GM_BK / 16; ++k16) umma_bf16_pair(dcol, w + 2u * k16, x + 2u * k16, idesc, (k16 > 0 || b > 0) ? 1u : 0u);
+                        if (++sl == nst) { sl = 0; pl ^= 1u; }
+                    }
+                    if (!ok) break;
+                    // the hi planes; a stage is free after its second pass
+                    for (int b = 0; b < nb; ++b) {
+                        const uint32_t base = smem_u32(smem + s * stage_bytes);
+                        const uint32_t w = umma_desc_lo(base), x = umma_desc_lo(base + GM_A_BYTES);
+#pragma unroll
+                        for (int k16 = 0; k16 < GM_BK / 16; ++k16) umma_bf16_pair(dcol, w + 2u * k16, x + 2u * k16, idesc, 1u);
+                        umma_commit_pair(&empty[s]);
+                        if (++s == nst) { s = 0; par ^= 1u; }
+                    }
+                    umma_commit_pair(&acc_full[a]);
+                    if (++a == nacc) { a = 0; apar ^= 1u; }
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GM_EPI_REGS));
+        // ---- epilogue: thread = one weight row (tensor-memory lane 32 * (warp % 4) + lane id) and half of the tile's columns
+        const int ew = warp - 4, q = warp & 3, chalf = ew >> 2, nch = g.nt >> 6;
+        // the partner: the warp with the other half of a rotation (dims e and e + hd / 2) or the up rows of the same features
+        const int pbit = (EPI == PF_QKV && g.hd == 64) ? 1 : 2;
+        const int role = (q & pbit) ? 1 : 0, pair = pbit == 2 ? (q & 1) * 2 + chalf : (q >> 1) * 2 + chalf;
+        float* mine = xch + ew * GM_STAGE_FLOATS;
+        const float* theirs = xch + (ew ^ pbit) * GM_STAGE_FLOATS;
+        int a = 0; unsigned apar = 0u;
+        bool ok = true;                    // after a wait that gave up: the remaining work runs through without waiting (every
+                                           // warp takes every named barrier), on values that nobody will use
+        for (int idx = pair_id; idx < g.items; idx += npairs) {
+            const GmItem it = gm_item(g, idx);
+            float acc[GM_NT_MAX / 2];
+#pragma unroll
+            for (int i = 0; i < GM_NT_MAX / 2; ++i) acc[i] = 0.f;
+            for (int kb = it.kb0; kb < it.kb1; kb += GM_CHAIN) {
+                if (ok) ok = gm_wait(&acc_full[a], apar, g.err);
+                __syncwarp();
+                tc_fence_after();
+                const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * acc_cols + chalf * (g.nt >> 1));
+                // the next 32 columns are on their way while the current ones are added
+                uint32_t v[2][32];
+                tmem_ld32(ta, v[0]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (c < nch) {
+                        tmem_ld_wait32(v[c & 1]);
+                        if (c + 1 < nch) tmem_ld32(ta + 32u * (c + 1), v[(c + 1) & 1]);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(v[c & 1][i]);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(leader_smem(smem_u32(&acc_free[a])));
+                if (++a == nacc) { a = 0; apar ^= 1u; }
+            }
+            const size_t wsize = (size_t)nch * GM_STAGE_FLOATS;            // floats of one warp's products
+            const size_t one = 2 * GM_EPI_WARPS * wsize;                   // ... of one range of k (both CTAs)
+            float* part = g.part + (size_t)it.r * g.S * one + ((size_t)rank * GM_EPI_WARPS + ew) * wsize + lane;
+            bool finish = true;
+            if (it.s >= 0) {
+                // a range of k: partial sums out; the last of the tile's ranges to arrive adds them in the order of the ranges
+                float* dst = part + (size_t)it.s * one;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (c < nch) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) __stcg(dst + (c * 32 + i) * 32, acc[c * 32 + i]);
+                    }
+                }
+                __threadfence();
+                named_sync(5, 32 * GM_EPI_WARPS);
+                if (threadIdx.x == 128) {
+                    unsigned* cn = g.cnt + it.r * 2 + rank;
+                    const int last = atomicAdd(cn, 1u) == (unsigned)(g.S - 1);
+                    if (last) { *cn = 0u; __threadfence(); }
+                    *(volatile int*)last_flag = last;
+                }
+                named_sync(5, 32 * GM_EPI_WARPS);
+                finish = *(volatile int*)last_flag != 0;
+                named_sync(5, 32 * GM_EPI_WARPS);                          // the flag has been read by every warp
+            }
+            if (finish) {
+#pragma unroll 1
+                for (int c = 0; c < nch; ++c) {
+                    if (it.s >= 0) {
+                        float w[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) w[i] = __ldcg(part + (c * 32 + i) * 32);
+                        for (int s = 1; s < g.S; ++s) {
+                            const float* src = part + (size_t)s * one + c * GM_STAGE_FLOATS;
+                            float u[32];                                   // one batch of loads in flight
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) u[i] = __ldcg(src + i * 32);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) w[i] += u[i];
+                        }
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) mine[i * 32 + lane] = w[i];
+                    } else {
+                        switch (c) {
+#define KG_STAGE(C) case C: { _Pragma("unroll") for (int i = 0; i < 32; ++i) mine[i * 32 + lane] = acc[C * 32 + i]; } break
+                            KG_STAGE(0); KG_STAGE(1); KG_STAGE(2); KG_STAGE(3);
+#undef KG_STAGE
+                        }
+                    }
+                    if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
+                    gm_epilogue<EPI>(g, mine, theirs, it.rt * g.nt + chalf * (g.nt >> 1) + c * 32, it.wt, rank, q, role);
+                    if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
+                }
+            }
         }
     }
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+// ---- attention of a block of prompt rows -----------------------------------------------------------------------------
+// One CTA = 128 query rows of one head (8 warps x 16 rows); key tiles of 64 travel cache -> shared memory with cp.async,
+// three tiles in flight, and are read by every warp with ldmatrix.  S = Q K^T and O += P V on mma.sync.m16n8k16 with q
+// and P as bf16 hi + lo, online softmax in the log2 domain (q carries log2(e) / sqrt(hd)).  CTAs with the most keys start first.
+//
+// What bounds it: the tensor instructions (256 per warp and tile).  The rows of a tile share K and V: with 16-row items
+// (the decode path's tiles, 8 keys x 16 rows per step) every key was fetched from L2 and passed through a serial
+// score - exchange - softmax chain once per 16 rows (7B, 1999 rows, one layer: 0.20 ms; with 16-row items about 0.9 ms).
+constexpr int FA_ROWS = 128, FA_KEYS = 64, FA_STAGES = 3;
+template <int HD> struct FaSm { static constexpr int TILE = FA_KEYS * HD * 2, BYTES = FA_STAGES * 2 * TILE; };
+
+__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(unsigned (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+
+struct FaArgs {
+    const __nv_bfloat16* qh; const __nv_bfloat16* ql;    // [rows][d] rotated, scaled q
+    const __nv_bfloat16* kc; const __nv_bfloat16* vc;    // this layer's cache
+    __nv_bfloat16* oh; __nv_bfloat16* ol;                // [rows][d] planes of the output
+    const int* page_table; int ps_shift, n_phys; State* st;
+    int H, pos0, rows;
+};
+
+template <int HD>
+__global__ void __launch_bounds__(256, 1) pf_attention_kernel(const __grid_constant__ FaArgs a) {
+    extern __shared__ __align__(128) char smem_raw[];
+    constexpr int NK = HD / 16, CH = HD / 8;               // k16-steps of a head; 16-byte chunks of a row
+    const uint32_t sm = smem_u32(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int d = a.H * HD, psm = (1 << a.ps_shift) - 1;
+    const int nblk = (a.rows + FA_ROWS - 1) / FA_ROWS;
+    const int rb = nblk - 1 - blockIdx.x / a.H, hh = blockIdx.x % a.H;
+    const int r0 = rb * FA_ROWS, rend = min(a.rows, r0 + FA_ROWS);
+    const int T = a.pos0 + rend;                           // keys any row of the block may see
+    const int ntile = (T + FA_KEYS - 1) / FA_KEYS;
+
+    auto issue = [&](int ti) {
+        const uint32_t kb = sm + (uint32_t)(ti % FA_STAGES) * (2 * FaSm<HD>::TILE), vb = kb + FaSm<HD>::TILE;
+#pragma unroll
+        for (int i = 0; i < FA_KEYS * CH / 256; ++i) {
+            const int id = tid + i * 256, r = id / CH, c = id % CH;
+            const int key = min(ti * FA_KEYS + r, T - 1);
+            const int page = checked_page(__ldg(a.page_table + (key >> a.ps_shift)), a.n_phys, a.st, 63);
+            const size_t src = ((((size_t)page * a.H + hh) << a.ps_shift) + (key & psm)) * HD + c * 8;
+            const uint32_t o = (uint32_t)(r * HD * 2 + ((c ^ (r & 7)) << 4));
+            cp_async16(kb + o, a.kc + src);
+            cp_async16(vb + o, a.vc + src);
+        }
+    };
+    issue(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (ntile > 1) issue(1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+
+    // this warp's 16 rows: q fragments (rows past the end repeat the last row and are not stored)
+    const int wr0 = r0 + warp * 16;
+    const int ra = min(wr0 + g, a.rows - 1), rb8 = min(wr0 + g + 8, a.rows - 1);
+    unsigned qh[NK][4], ql[NK][4];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const size_t o1 = (size_t)ra * d + hh * HD + k * 16 + 2 * t, o2 = (size_t)rb8 * d + hh * HD + k * 16 + 2 * t;
+        qh[k][0] = *reinterpret_cast<const unsigned*>(a.qh + o1); qh[k][1] = *reinterpret_cast<const unsigned*>(a.qh + o2);
+        qh[k][2] = *reinterpret_cast<const unsigned*>(a.qh + o1 + 8); qh[k][3] = *reinterpret_cast<const unsigned*>(a.qh + o2 + 8);
+        ql[k][0] = *reinterpret_cast<const unsigned*>(a.ql + o1); ql[k][1] = *reinterpret_cast<const unsigned*>(a.ql + o2);
+        ql[k][2] = *reinterpret_cast<const unsigned*>(a.ql + o1 + 8); ql[k][3] = *reinterpret_cast<const unsigned*>(a.ql + o2 + 8);
+    }
+    float o[HD / 8][4];
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
+    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
+    const int lim0 = a.pos0 + wr0 + g, lim1 = lim0 + 8;     // last key each of the two rows may see
+    const int wlast = a.pos0 + wr0 + 15;                    // no row of this warp sees a key beyond
+
+    for (int ti = 0; ti < ntile; ++ti) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();                                    // tile ti has landed for everybody; everybody is done with tile ti - 1
+        if (ti + 2 < ntile) issue(ti + 2);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const int key0 = ti * FA_KEYS;
+        if (key0 > wlast || wr0 >= a.rows) continue;
+        const uint32_t kb = sm + (uint32_t)(ti % FA_STAGES) * (2 * FaSm<HD>::TILE), vb = kb + FaSm<HD>::TILE;
+        float s[8][4];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) { s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f; }
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int r = p * 16 + (lane >> 4) * 8 + (lane & 7), c = k * 2 + ((lane >> 3) & 1);
+                unsigned b[4];
+                ldmatrix_x4(b, kb + (uint32_t)(r * HD * 2 + ((c ^ (r & 7)) << 4)));
+                mma_bf16_16816(s[2 * p], qh[k], b[0], b[1]);
+                mma_bf16_16816(s[2 * p + 1], qh[k], b[2], b[3]);
+                mma_bf16_16816(s[2 * p], ql[k], b[0], b[1]);
+                mma_bf16_16816(s[2 * p + 1], ql[k], b[2], b[3]);
+            }
+        }
+        if (key0 + FA_KEYS - 1 > a.pos0 + wr0) {            // the tile crosses the diagonal of this warp's rows
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                const int k0 = key0 + n * 8 + 2 * t;
+                if (k0 > lim0) s[n][0] = -INFINITY;
+                if (k0 + 1 > lim0) s[n][1] = -INFINITY;
+                if (k0 > lim1) s[n][2] = -INFINITY;
+                if (k0 + 1 > lim1) s[n][3] = -INFINITY;
+            }
+        }
+        float x0 = s[0][0], x1 = s[0][2];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) { x0 = fmaxf(x0, fmaxf(s[n][0], s[n][1])); x1 = fmaxf(x1, fmaxf(s[n][2], s[n][3])); }
+        x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 1)); x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 2));
+        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 1)); x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 2));
+        // key 0 is visible to every row, so the maxima are finite from the first tile on
+        const float n0 = fmaxf(m0, x0), n1 = fmaxf(m1, x1);
+        const float c0 = ex2f(m0 - n0), c1 = ex2f(m1 - n1);
+        m0 = n0; m1 = n1;
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            s[n][0] = ex2f(s[n][0] - n0); s[n][1] = ex2f(s[n][1] - n0); s[n][2] = ex2f(s[n][2] - n1); s[n][3] = ex2f(s[n][3] - n1);
+            a0 += s[n][0] + s[n][1]; a1 += s[n][2] + s[n][3];
+        }
+        l0 = l0 * c0 + a0; l1 = l1 * c1 + a1;
+#pragma unroll
+        for (int n = 0; n < HD / 8; ++n) { o[n][0] *= c0; o[n][1] *= c0; o[n][2] *= c1; o[n][3] *= c1; }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            unsigned ph[4], pl[4];
+            split_hi_lo(make_float2(s[2 * kk][0], s[2 * kk][1]), ph[0], pl[0]);
+            split_hi_lo(make_float2(s[2 * kk][2], s[2 * kk][3]), ph[1], pl[1]);
+            split_hi_lo(make_float2(s[2 * kk + 1][0], s[2 * kk + 1][1]), ph[2], pl[2]);
+            split_hi_lo(make_float2(s[2 * kk + 1][2], s[2 * kk + 1][3]), ph[3], pl[3]);
+#pragma unroll
+            for (int n = 0; n < HD / 16; ++n) {
+                const int r = kk * 16 + ((lane >> 3) & 1) * 8 + (lane & 7), c = n * 2 + (lane >> 4);
+                unsigned b[4];
+                ldmatrix_x4_trans(b, vb + (uint32_t)(r * HD * 2 + ((c ^ (r & 7)) << 4)));
+                mma_bf16_16816(o[2 * n], ph, b[0], b[1]);
+                mma_bf16_16816(o[2 * n + 1], ph, b[2], b[3]);
+                mma_bf16_16816(o[2 * n], pl, b[0], b[1]);
+                mma_bf16_16816(o[2 * n + 1], pl, b[2], b[3]);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
+    l1 += __shfl_xor_sync(0xffffffffu, l1, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+    const float i0 = 1.0f / l0, i1 = 1.0f / l1;
+#pragma unroll
+    for (int n = 0; n < HD / 8; ++n) {
+        unsigned hi, lo;
+        const size_t col = (size_t)hh * HD + n * 8 + 2 * t;
+        if (wr0 + g < a.rows) {
+            split_hi_lo(make_float2(o[n][0] * i0, o[n][1] * i0), hi, lo);
+            *reinterpret_cast<unsigned*>(a.oh + (size_t)(wr0 + g) * d + col) = hi;
+            *reinterpret_cast<unsigned*>(a.ol + (size_t)(wr0 + g) * d + col) = lo;
+        }
+        if (wr0 + g + 8 < a.rows) {
+            split_hi_lo(make_float2(o[n][2] * i1, o[n][3] * i1), hi, lo);
+            *reinterpret_cast<unsigned*>(a.oh + (size_t)(wr0 + g + 8) * d + col) = hi;
+            *reinterpret_cast<unsigned*>(a.ol + (size_t)(wr0 + g + 8) * d + col) = lo;
+        }
     }
 }
 
 // ---- elementwise kernels around the GEMMs ----------------------------------------------------------------------------
-__device__ __forceinline__ void split_store(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t i, float v) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    hi[i] = h;
-    lo[i] = __float2bfloat16_rn(v - __bfloat162float(h));
-}
-
-// h[r] = E[token r]
-template <typename WT>
-__global__ void pf_embed_kernel(const int* toks, const WT* E, int V, int d, float* h) {
+// h[r] = E[token r], eight columns per thread (d is a multiple of 128)
+__global__ void __launch_bounds__(256) pf_embed_kernel(const int* toks, const __nv_bfloat16* E, int V, int d, float* h) {
     const int r = blockIdx.x;
     int tok = toks[r];
     if ((unsigned)tok >= (unsigned)V) tok = 0;
-    for (int e = threadIdx.x; e < d; e += blockDim.x) h[(size_t)r * d + e] = wt_to_float<WT>(E[(size_t)tok * d + e]);
+    for (int e = threadIdx.x * 8; e < d; e += 256 * 8) {
+        const uint4 v = *reinterpret_cast<const uint4*>(E + (size_t)tok * d + e);
+        float4* out = reinterpret_cast<float4*>(h + (size_t)r * d + e);
+        out[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+        out[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u), __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
+    }
+}
+
+// cos, sin of every (row, pair of dims) of a block of rows, once for all layers; grid = rows, hd / 2 threads
+__global__ void pf_rope_table_kernel(const __grid_constant__ Dev D, int pos0, float2* cs) {
+    float c, s;
+    rope_cs(D, pos0 + blockIdx.x, threadIdx.x, c, s);
+    cs[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = make_float2(c, s);
 }
 
 // four consecutive values -> four bf16 of each plane (8-byte stores; i is a multiple of 4)
@@ -288,36 +726,6 @@ __global__ void __launch_bounds__(PF_EW_THREADS) pf_split_kernel(const float* x,
     const int r = blockIdx.x;
     const int i = blockIdx.y * PF_EW_THREADS + threadIdx.x;
     if (i < (K >> 2)) split_store4(hi, lo, (size_t)r * K + (size_t)i * 4, *reinterpret_cast<const float4*>(x + (size_t)r * ldx + (size_t)i * 4));
-}
-
-// planes of SiLU(gate) * up; grid = (rows, ceil(F / (4 * PF_EW_THREADS))), F a multiple of 4
-__global__ void __launch_bounds__(PF_EW_THREADS) pf_swiglu_split_kernel(const float* gate, const float* up, int F, __nv_bfloat16* hi, __nv_bfloat16* lo) {
-    const int r = blockIdx.x;
-    const int i = blockIdx.y * PF_EW_THREADS + threadIdx.x;
-    if (i < (F >> 2)) {
-        const size_t o = (size_t)r * F + (size_t)i * 4;
-        const float4 gt = *reinterpret_cast<const float4*>(gate + o);
-        const float4 u = *reinterpret_cast<const float4*>(up + o);
-        split_store4(hi, lo, o, make_float4(silu_f(gt.x) * u.x, silu_f(gt.y) * u.y, silu_f(gt.z) * u.z, silu_f(gt.w) * u.w));
-    }
-}
-
-// K (rotated) and V rows of a block of prompt rows -> cache, rounded to the storage type; grid = (rows, H)
-template <typename WT>
-__global__ void pf_rope_append_kernel(const Dev D, const float* qkv, int pos0, WT* kc, WT* vc) {
-    const int r = blockIdx.x, hh = blockIdx.y, pos = pos0 + r;
-    const int d = D.dm.d, hd = D.dm.hd, half = hd >> 1, H = D.dm.H, ps = D.dm.page_size;
-    const float* src = qkv + (size_t)r * 3 * d + hh * hd;
-    const int page = D.page_table[pos >> D.dm.ps_shift];
-    const size_t base = (((size_t)page * H + hh) * ps + (pos & (ps - 1))) * hd;
-    for (int e = threadIdx.x; e < half; e += blockDim.x) {
-        float cs, sn; rope_cs(D, pos, e, cs, sn);
-        const float k1 = src[d + e], k2 = src[d + e + half];
-        kc[base + e] = float_to_wt<WT>(k1 * cs - k2 * sn);
-        kc[base + e + half] = float_to_wt<WT>(k2 * cs + k1 * sn);
-        vc[base + e] = float_to_wt<WT>(src[2 * d + e]);
-        vc[base + e + half] = float_to_wt<WT>(src[2 * d + e + half]);
-    }
 }
 
 }  // namespace kg
