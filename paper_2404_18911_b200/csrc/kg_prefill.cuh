@@ -31,8 +31,8 @@ constexpr int GM_STAGE_FLOATS = 32 * 32;                               // [32 co
 constexpr int GM_XCH_BYTES = GM_EPI_WARPS * GM_STAGE_FLOATS * 4;
 constexpr int GM_SMEM = 1024 + GM_RING_BYTES + GM_XCH_BYTES + 256;     // alignment slack, operand ring, epilogue staging, barriers
 static_assert(GM_SMEM <= SMEM_TOTAL, "GEMM shared memory");
-// registers: the first warpgroup needs few, the two epilogue warpgroups keep 128 sums and two batches of accumulator columns
-// per thread; the pool is what the launch allocated (GM_THREADS x 168), a request beyond it would block for ever
+// registers: the first warpgroup needs few, the two epilogue warpgroups keep 128 sums and a batch of accumulator columns per
+// thread; the pool is what the launch allocated (GM_THREADS x 168), a request beyond it would block for ever
 constexpr int GM_CTRL_REGS = 56, GM_EPI_REGS = 216;
 static_assert(GM_THREADS == DECODE_THREADS && 128 * GM_CTRL_REGS + 32 * GM_EPI_WARPS * GM_EPI_REGS <= GM_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
 constexpr unsigned long long GM_WAIT_CLK = 4000000000ull;              // ~2 s: a wait that runs this long gives up
@@ -74,11 +74,20 @@ __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr) { return ((sadd
 __device__ __forceinline__ uint32_t umma_idesc(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-// D[256 x N] (+)= A[256 x 16] B[N x 16]^T over a CTA pair, issued by one thread of the even CTA: each CTA holds 128 rows
-// of A, N / 2 rows of B and its 128 rows of D
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+// one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one() {
+    unsigned p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// D[256 x N] (+)= A[256 x 64] B[N x 64]^T over a CTA pair (four k16-steps), issued by one thread of the even CTA: each CTA
+// holds 128 rows of A, N / 2 rows of B and its 128 rows of D
+__device__ __forceinline__ void umma_kblock_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 q, %5, %5;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\tadd.s64 da, da, 2;\n\tadd.s64 db, db, 2;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, q;\n\tadd.s64 da, da, 2;\n\tadd.s64 db, db, 2;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, q;\n\tadd.s64 da, da, 2;\n\tadd.s64 db, db, 2;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, q;\n\t}"
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate));
 }
 // the mbarrier of both CTAs of the pair receives one arrival when every MMA this thread has issued so far has completed
@@ -92,8 +101,11 @@ __device__ __forceinline__ uint32_t leader_smem(uint32_t addr) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
     return r;
 }
+// (no cluster-scope release: what the arrival hands over is tensor memory whose reads have completed, and that fence would
+// stalls while copies are in flight: a drain took 2650 clocks with it and 690 without, and 64 k blocks of a 256 x 256 tile
+// 111,000 and 71,000 clocks, 66,000 being the MMAs alone)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -135,7 +147,7 @@ __device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity
 // What bounds it: the operands of a k block.  With the activations in two planes a 128 x 128 tile of one CTA needs 48 KB for
 // 4.2 MFLOP (94 bytes per clock and SM at the full MMA rate, more than L2 delivers); the pair's 256 x 256 tile needs 48 KB
 // per CTA for 8.4 MFLOP, since the two CTAs share the activation planes.  With the attention below and the fused epilogues
-// the prompt pass of the 7B shape (1999 tokens) went from 96.9 to 58.5 ms, of the 13B shape (2048 tokens) from 187 to 107 ms.
+// the prompt pass of the 7B shape (1999 tokens) went from 96.9 to 52.6 ms, of 77 tokens from 9.2 to 6.3 ms.
 //
 // Accumulation.  The tensor core's fp32 accumulation rounds toward zero at every MMA, by an amount that follows the size
 // of the running sum, which biases long chains.  A chain of GM_CHAIN = 2 k blocks multiplies both lo planes first - sums
@@ -302,8 +314,8 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GM_CTRL_REGS));
-        if (warp == 0 && lane == 0) {
-            // ---- TMA producer of this CTA's tiles
+        if (warp == 0) {
+            // ---- TMA producer of this CTA's tiles (the warp stays together, one lane issues)
             int s = 0; unsigned par = 1u;
             const int hrow = g.nt >> 1;
             bool ok = true;
@@ -312,18 +324,21 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 const int y_act = it.rt * g.nt + rank * hrow;
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     if (!(ok = gm_wait(&empty[s], par, g.err))) break;
-                    if (rank == 0) mbar_arrive_expect_tx(&full[s], (unsigned)(2 * stage_bytes));
-                    const uint32_t dst = smem_u32(smem + s * stage_bytes), bar = leader_smem(smem_u32(&full[s]));
-                    const int x = kb * GM_BK;
-                    if (EPI == PF_SWIGLU) {
-                        const int y = it.wt * (GM_TM / 2) + rank * (GM_TM / 4);
-                        tma_load_2d_pair(dst, &tm_w, x, y, bar);
-                        tma_load_2d_pair(dst + GM_A_BYTES / 2, &tm_w2, x, y, bar);
-                    } else {
-                        tma_load_2d_pair(dst, &tm_w, x, it.wt * GM_TM + rank * (GM_TM / 2), bar);
+                    if (elect_one()) {
+                        if (rank == 0) mbar_arrive_expect_tx(&full[s], (unsigned)(2 * stage_bytes));
+                        const uint32_t dst = smem_u32(smem + s * stage_bytes), bar = leader_smem(smem_u32(&full[s]));
+                        const int x = kb * GM_BK;
+                        if (EPI == PF_SWIGLU) {
+                            const int y = it.wt * (GM_TM / 2) + rank * (GM_TM / 4);
+                            tma_load_2d_pair(dst, &tm_w, x, y, bar);
+                            tma_load_2d_pair(dst + GM_A_BYTES / 2, &tm_w2, x, y, bar);
+                        } else {
+                            tma_load_2d_pair(dst, &tm_w, x, it.wt * GM_TM + rank * (GM_TM / 2), bar);
+                        }
+                        tma_load_2d_pair(dst + GM_A_BYTES, &tm_hi, x, y_act, bar);
+                        tma_load_2d_pair(dst + GM_A_BYTES + hrow * 128, &tm_lo, x, y_act, bar);
                     }
-                    tma_load_2d_pair(dst + GM_A_BYTES, &tm_hi, x, y_act, bar);
-                    tma_load_2d_pair(dst + GM_A_BYTES + hrow * 128, &tm_lo, x, y_act, bar);
+                    __syncwarp();
                     if (++s == nst) { s = 0; par ^= 1u; }
                 }
             }
@@ -332,8 +347,9 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 ok = gm_wait(&empty[s], par, g.err);
                 if (++s == nst) { s = 0; par ^= 1u; }
             }
-        } else if (warp == 1 && lane == 0 && rank == 0) {
-            // ---- MMA issuer of the pair
+        } else if (warp == 1 && rank == 0) {
+            // ---- MMA issuer of the pair.  The warp stays together and one elected lane issues: with a loop that only lane 0 ran,
+            // issuing took 115 clocks per instruction, which made every tile of up to 192 columns issue-bound.
             const uint32_t idesc = umma_idesc(GM_TM, g.nt);
             const uint32_t lo_off = (uint32_t)((g.nt >> 1) * 128) >> 4;          // hi plane -> lo plane, in descriptor units
             int s = 0, a = 0; unsigned par = 0u, apar = 1u;
@@ -351,8 +367,8 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                         tc_fence_after();
                         const uint32_t base = smem_u32(smem + sl * stage_bytes);
                         const uint32_t w = umma_desc_lo(base), x = umma_desc_lo(base + GM_A_BYTES) + lo_off;
-#pragma unroll
-                        for (int k16 = 0; k16 < GM_BK / 16; ++k16) umma_bf16_pair(dcol, w + 2u * k16, x + 2u * k16, idesc, (k16 > 0 || b > 0) ? 1u : 0u);
+                        if (elect_one()) umma_kblock_pair(dcol, w, x, idesc, b > 0 ? 1u : 0u);
+                        __syncwarp();
                         if (++sl == nst) { sl = 0; pl ^= 1u; }
                     }
                     if (!ok) break;
@@ -360,12 +376,14 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                     for (int b = 0; b < nb; ++b) {
                         const uint32_t base = smem_u32(smem + s * stage_bytes);
                         const uint32_t w = umma_desc_lo(base), x = umma_desc_lo(base + GM_A_BYTES);
-#pragma unroll
-                        for (int k16 = 0; k16 < GM_BK / 16; ++k16) umma_bf16_pair(dcol, w + 2u * k16, x + 2u * k16, idesc, 1u);
-                        umma_commit_pair(&empty[s]);
+                        if (elect_one()) {
+                            umma_kblock_pair(dcol, w, x, idesc, 1u);
+                            umma_commit_pair(&empty[s]);
+                            if (b == nb - 1) umma_commit_pair(&acc_full[a]);
+                        }
+                        __syncwarp();
                         if (++s == nst) { s = 0; par ^= 1u; }
                     }
-                    umma_commit_pair(&acc_full[a]);
                     if (++a == nacc) { a = 0; apar ^= 1u; }
                 }
             }
@@ -392,16 +410,14 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 __syncwarp();
                 tc_fence_after();
                 const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * acc_cols + chalf * (g.nt >> 1));
-                // the next 32 columns are on their way while the current ones are added
-                uint32_t v[2][32];
-                tmem_ld32(ta, v[0]);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     if (c < nch) {
-                        tmem_ld_wait32(v[c & 1]);
-                        if (c + 1 < nch) tmem_ld32(ta + 32u * (c + 1), v[(c + 1) & 1]);
+                        uint32_t v[32];
+                        tmem_ld32(ta + 32u * c, v);
+                        tmem_ld_wait32(v);
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(v[c & 1][i]);
+                        for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(v[i]);
                     }
                 }
                 tc_fence_before();
