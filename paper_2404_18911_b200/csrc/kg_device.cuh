@@ -410,7 +410,7 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // Work split.  The CTA owns a contiguous range of "units": output rows, or for the SwiGLU pair
 // gate/up feature pairs.  A stage of the ring holds 8 weight rows (for the pair: the 8 gate rows of
 // a feature group, then in the next stage the 8 up rows of the same features) times one k phase
-// (2048 k-elements when M <= 8, else 1024), i.e. one bulk copy of up to 4 KB per row: the copy
+// (2048 k-elements when M <= 12, else 1024), i.e. one bulk copy of up to 4 KB per row: the copy
 // engine spends a fixed time per copy, and only copies of 2-4 KB and more keep HBM saturated.
 // The stages are visited superchunk (<= 256 accumulator rows) -> phase -> row group, in the same
 // order by the producer warp (which issues the copies) and the consumers.
@@ -421,6 +421,8 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // split x * gain = hi + lo into two bf16 parts:
 //   V = 4  (M <= 4):  columns 0-3 carry hi, columns 4-7 lo of rows 0-3: one MMA per k16-step;
 //   V = 8  (M <= 8):  hi and lo are two MMAs;
+//   V = 12 (M <= 12): the same for rows 0-7, and a third MMA carries hi and lo of rows 8-11 as V = 4 does for rows 0-3
+//                     (7B, KV 512, verify pass of 11 rows: 5.47 ms with the four MMAs on 1024-k phases of V = 16, now 4.46);
 //   V = 16 (M <= 16): two column tiles, hi and lo: four MMAs.
 // Each of the 8 warps owns a fixed slice of the phase's k range; its B fragments are loaded once
 // per phase from the packed activation rows in global memory (L2) and stay in registers for every
@@ -429,10 +431,15 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 template <int V> struct LinGeom {
     static constexpr int NS = V == 16 ? 8 : 16;           // k16-steps per warp and stage
     static constexpr int PLEN = NS * 16 * NWARPS;         // k-elements per phase: 2048 or 1024
-    static constexpr int FR = V == 4 ? 2 : (V == 8 ? 4 : 8);   // B fragment registers per step
+    static constexpr int FR = V == 4 ? 2 : (V == 8 ? 4 : (V == 12 ? 6 : 8));   // B fragment registers per step
     static constexpr int NACC = V == 16 ? 2 : 1;          // column tiles
+    static constexpr int RED_W = V == 16 ? 256 : (V == 12 ? 192 : 128);        // floats of one warp's partial sums of a stage pair
+    static constexpr int MP = V == 12 ? 12 : 16;          // row accumulator columns (activation rows, padded)
+    // partial sums are double-buffered where the work area has room (V = 16: one buffer and one more barrier per pair);
+    // partial sums and row accumulators together take the same space in every variant
+    static constexpr int ACC_OFF = V == 16 ? NWARPS * RED_W : 2 * NWARPS * RED_W;
 };
-constexpr int MP = 16;                                    // accumulator columns (activation rows, padded)
+constexpr int MP_MAX = 16;
 
 struct LinPlan {
     int u0, u1;          // this CTA's units
@@ -445,7 +452,7 @@ __device__ __forceinline__ LinPlan make_plan(const LinArgs& a, int cta, int ncta
     p.u0 = (int)((unsigned)a.N * (unsigned)cta / (unsigned)nctas);          // N * nctas < 2^32 (checked on the host)
     p.u1 = (int)((unsigned)a.N * (unsigned)(cta + 1) / (unsigned)nctas);
     p.sc_units = a.W2 ? SC_ROWS / 2 : SC_ROWS;
-    p.plen = a.M <= 8 ? LinGeom<8>::PLEN : LinGeom<16>::PLEN;
+    p.plen = a.M <= 12 ? LinGeom<12>::PLEN : LinGeom<16>::PLEN;
     p.nph = (a.K + p.plen - 1) / p.plen;
     return p;
 }
@@ -510,30 +517,33 @@ __device__ __forceinline__ void split_hi_lo(float2 v, unsigned& hi, unsigned& lo
 }
 
 // Shared-memory work area of the streamed path (floats, from WORK_OFF).
-constexpr int LW_RED = 0;                                 // [2][NWARPS][16][8] partial sums of a stage pair
-constexpr int LW_ACC = LW_RED + 2 * NWARPS * 128;         // [SC_ROWS][MP] row accumulators
-constexpr int LW_RS = LW_ACC + SC_ROWS * MP;              // [M_MAX] 1/rms of the input rows
+constexpr int LW_RED = 0;                                 // partial sums of a stage pair, then at LinGeom::ACC_OFF the row accumulators [SC_ROWS][MP]
+constexpr int LW_RS = 2 * NWARPS * 128 + SC_ROWS * MP_MAX;   // [M_MAX] 1/rms of the input rows
 constexpr int LW_RSP = LW_RS + M_MAX;                     // [M_MAX][16] partial sums of squares of the input rows
 constexpr int LW_SSW = LW_RSP + M_MAX * 16;               // [NWARPS][M_MAX] sums of squares of the output rows
 constexpr int PRE_NU = 64;                                // residual / gain values are prefetched for up to this many units
 constexpr int LW_PRES = LW_SSW + NWARPS * M_MAX;          // [M_MAX][PRE_NU] residual values
 constexpr int LW_PREG = LW_PRES + M_MAX * PRE_NU;         // [2][PRE_NU] gains of the packed outputs
-constexpr int LW_END = LW_PREG + 2 * PRE_NU;
+constexpr int LW_HS = LW_PREG + 2 * PRE_NU;               // [M_MAX][3] LM head: running maximum, sum, arg max of each row (kept here and not
+                                                          // in registers, which the fragments of the wide variants fill)
+constexpr int LW_END = LW_HS + M_MAX * 3;
 static_assert(LW_END * 4 <= WORK_BYTES, "linear work area too large");
+static_assert(LinGeom<12>::ACC_OFF + SC_ROWS * LinGeom<12>::MP <= LW_RS && LinGeom<16>::ACC_OFF + SC_ROWS * 16 <= LW_RS && LinGeom<8>::ACC_OFF + SC_ROWS * 16 <= LW_RS,
+              "partial sums and accumulators overlap what follows");
 
 __device__ __forceinline__ void cp_async4(void* dst_smem, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
 
 // Epilogue of the streamed path for everything but the LM head: turns the accumulators of nu output
-// units x M rows (acc_s, 1/rms in rs) into fp32 rows, packed copies and per-CTA sums of squares.
+// units x M rows (acc_s with MP columns, 1/rms in rs) into fp32 rows, packed copies and per-CTA sums of squares.
 // Thread (r, m): m = tid mod 2^ceil(log2 M), so that the lanes of a warp that share m can add their
 // squares by shuffles in a fixed order.  Every consumer thread calls it; ssq_acc (threads < M)
 // accumulates over superchunks.
-__device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, int sc0, int nu, bool prefetched, float& ssq_acc) {
+template <int MP>
+__device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const float* acc_s, int sc0, int nu, bool prefetched, float& ssq_acc) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = a.M;
-    const float* acc_s = wk + LW_ACC;
     const float* rs = wk + LW_RS;
     float* ssw = wk + LW_SSW;
     const int sh = M <= 1 ? 0 : (M <= 2 ? 1 : (M <= 4 ? 2 : (M <= 8 ? 3 : 4)));
@@ -579,7 +589,7 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, int sc0, 
 template <int V>
 __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     using G = LinGeom<V>;
-    constexpr int NS = G::NS, FR = G::FR, NACC = G::NACC;
+    constexpr int NS = G::NS, FR = G::FR, NACC = G::NACC, MP = G::MP;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int M = a.M, K = a.K;
@@ -588,15 +598,13 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
 
     float* wk = reinterpret_cast<float*>(c.smem + WORK_OFF);
     float* red = wk + LW_RED;
-    float* acc_s = wk + LW_ACC;
+    float* acc_s = wk + G::ACC_OFF;
     float* rs = wk + LW_RS;
     const char* ring = c.smem + RING_OFF;
     Ctrl* ctl = c.ctl;
     const int nctas = c.nctas, cta = c.cta;
     int slot = c.slot; unsigned phase = c.phase;              // ring cursor, kept in registers here
 
-    HeadStat hs[2];                                                        // EPI_HEAD: this warp tracks rows warp, warp + 8
-    hs[0].zmax = hs[1].zmax = 0.f; hs[0].sum = hs[1].sum = 0.f; hs[0].arg = hs[1].arg = 0;
     bool ok = true;
     int buf = 0;
     float ssq_acc = 0.f;
@@ -628,6 +636,9 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     // this lane's rows of the packed input: V = 4: row g & 3 (hi for g < 4, lo for g >= 4); else rows g (and g + 8)
     const int xrow = V == 4 ? (g & 3) : g;
     const unsigned char* xlane = a.xpk + (size_t)xrow * a.ldpk + (size_t)warp * NS * 64 + t * 16 + (V == 4 ? (g >> 2) * 8 : 0);
+    // V = 12: rows 8 .. 11 (hi for g < 4, lo for g >= 4), seen from xlane
+    const int mrow = 8 + (g & 3);
+    const ptrdiff_t mofs = (ptrdiff_t)((mrow < M ? mrow : 0) - xrow) * (ptrdiff_t)a.ldpk + (g >> 2) * 8;
 
     for (int sc0 = pl.u0; sc0 < pl.u1; sc0 += pl.sc_units) {
         const int sc1 = min(pl.u1, sc0 + pl.sc_units);
@@ -657,6 +668,10 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                             const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row < M ? px + (size_t)(8 * n) * a.ldpk : px - (size_t)xrow * a.ldpk));
                             fr[s][4 * n + 0] = v.x; fr[s][4 * n + 1] = v.y; fr[s][4 * n + 2] = v.z; fr[s][4 * n + 3] = v.w;
                         }
+                        if (V == 12) {
+                            const uint2 w = __ldcg(reinterpret_cast<const uint2*>(px + mofs));
+                            fr[s][FR - 2] = w.x; fr[s][FR - 1] = w.y;
+                        }
                     }
                 }
                 if (pre_pending) { pre_pending = false; epilogue_prefetch(); }
@@ -669,6 +684,7 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
 #pragma unroll
                         for (int n = 0; n < NACC; ++n)
                             if (!(sv && xrow + 8 * n < M)) { fr[s][4 * n + 0] = 0u; fr[s][4 * n + 1] = 0u; fr[s][4 * n + 2] = 0u; fr[s][4 * n + 3] = 0u; }
+                        if (V == 12 && !(sv && mrow < M)) { fr[s][FR - 2] = 0u; fr[s][FR - 1] = 0u; }
                     }
                 }
             }
@@ -679,9 +695,9 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                 const int slot_a = slot;
                 const int slot_b = two ? (slot_a + 1 == RING ? 0 : slot_a + 1) : slot_a;
                 const unsigned phase_b = (two && slot_a + 1 == RING) ? phase ^ 1u : phase;
-                float acc[4][4];
+                float acc[5][4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f; }
+                for (int q = 0; q < 5; ++q) { acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.f; }
                 if (ok) ok = mbar_wait(c, &ctl->full[slot_a], phase, 41);
                 if (ok && two) ok = mbar_wait(c, &ctl->full[slot_b], phase_b, 41);
                 if (ok) {
@@ -702,6 +718,11 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                             } else if (V == 8) {
                                 mma_bf16_16816(acc[(s & 1) * 2], af[s % PD], fr[s][0], fr[s][1]);
                                 mma_bf16_16816(acc[(s & 1) * 2 + 1], af[s % PD], fr[s][2], fr[s][3]);
+                            } else if (V == 12) {
+                                // chains of eight where hi is summed (as V = 8 and V = 16 have them); lo, 2^-9 of it, in one
+                                mma_bf16_16816(acc[s & 1], af[s % PD], fr[s][0], fr[s][1]);
+                                mma_bf16_16816(acc[4], af[s % PD], fr[s][2], fr[s][3]);
+                                mma_bf16_16816(acc[2 + (s & 1)], af[s % PD], fr[s][FR - 2], fr[s][FR - 1]);
                             } else {
                                 mma_bf16_16816(acc[0], af[s % PD], fr[s][0], fr[s][1]);
                                 mma_bf16_16816(acc[1], af[s % PD], fr[s][2], fr[s][3]);
@@ -718,8 +739,20 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                 if (++slot == RING) { slot = 0; phase ^= 1u; }
                 // ---- add the k-slices in warp order into the row accumulators
                 if (V == 16) cta_sync();                     // single partial-sum buffer: the previous pair's sums have been read
-                float* r = red + (size_t)(V == 16 ? 0 : buf) * NWARPS * 128 + (size_t)warp * NACC * 128;
-                if (V == 16) {
+                float* r = red + (size_t)(V == 16 ? 0 : buf) * NWARPS * G::RED_W + (size_t)warp * G::RED_W;
+                if (V == 12) {
+                    // acc[0], acc[1]: hi of rows 0-7 (even, odd steps), acc[4]: lo; acc[2], acc[3]: rows 8-11, hi in columns 0-3 and lo
+                    // in columns 4-7, which sit two lanes further
+                    *reinterpret_cast<float2*>(r + g * MP + 2 * t) = make_float2(acc[0][0] + acc[1][0] + acc[4][0], acc[0][1] + acc[1][1] + acc[4][1]);
+                    *reinterpret_cast<float2*>(r + (g + 8) * MP + 2 * t) = make_float2(acc[0][2] + acc[1][2] + acc[4][2], acc[0][3] + acc[1][3] + acc[4][3]);
+                    float mx[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { mx[i] = acc[2][i] + acc[3][i]; mx[i] += __shfl_xor_sync(0xffffffffu, mx[i], 2); }
+                    if (t < 2) {
+                        *reinterpret_cast<float2*>(r + g * MP + 8 + 2 * t) = make_float2(mx[0], mx[1]);
+                        *reinterpret_cast<float2*>(r + (g + 8) * MP + 8 + 2 * t) = make_float2(mx[2], mx[3]);
+                    }
+                } else if (V == 16) {
                     // acc[0] / acc[1]: hi / lo of columns 0-7; acc[2] / acc[3]: hi / lo of columns 8-15
                     *reinterpret_cast<float2*>(r + g * 8 + 2 * t) = make_float2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
                     *reinterpret_cast<float2*>(r + (g + 8) * 8 + 2 * t) = make_float2(acc[0][2] + acc[1][2], acc[0][3] + acc[1][3]);
@@ -735,7 +768,16 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                 {
                     // element (weight row r16, activation row m) of the pair; for M <= 8 every thread adds a share of the
                     // eight k-slices and a fixed butterfly joins the shares, so that no warp lags behind the others
-                    if (V == 16) {
+                    if (V == 12) {
+                        if (tid < 192) {
+                            const float* rb = red + (size_t)buf * NWARPS * G::RED_W + tid;
+                            float v = 0.f;
+#pragma unroll
+                            for (int w = 0; w < NWARPS; ++w) v += rb[w * G::RED_W];
+                            float* dst = acc_s + (size_t)(si >> 1) * 16 * MP + tid;
+                            *dst = ph == 0 ? v : *dst + v;
+                        }
+                    } else if (V == 16) {
                         const int r16 = tid >> 4, m = tid & 15;
                         const float* rb = red + (m >> 3) * 128 + r16 * 8 + (m & 7);
                         float v = 0.f;
@@ -800,11 +842,17 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                     float e = 0.f;
                     for (int r = lane; r < nu; r += 32) e += expf(acc_s[(size_t)r * MP + m] * f - zm);
                     e = warp_sum(e);
-                    if (nu > 0) head_merge(hs[q], zm, e, im);
+                    if (lane == 0) {                 // this warp tracks rows warp, warp + 8
+                        HeadStat hs; hs.zmax = 0.f; hs.sum = 0.f; hs.arg = 0;
+                        float* st = wk + LW_HS + m * 3;
+                        if (sc0 != pl.u0) { hs.zmax = st[0]; hs.sum = st[1]; hs.arg = __float_as_int(st[2]); }
+                        head_merge(hs, zm, e, im);
+                        st[0] = hs.zmax; st[1] = hs.sum; st[2] = __int_as_float(hs.arg);
+                    }
                 }
             }
         } else {
-            emit_rows(a, wk, sc0, nu, prefetched && sc0 == pl.u0, ssq_acc);
+            emit_rows<MP>(a, wk, acc_s, sc0, nu, prefetched && sc0 == pl.u0, ssq_acc);
         }
         cta_sync();                                  // acc_s is rewritten by the next superchunk / operator
     }
@@ -812,7 +860,10 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int m = warp + q * NWARPS;
-            if (m < M) a.head_part[(size_t)cta * M_MAX + m] = make_float4(hs[q].zmax, hs[q].sum, __int_as_float(hs[q].arg), 0.f);
+            if (m < M) {
+                const float* st = wk + LW_HS + m * 3;
+                a.head_part[(size_t)cta * M_MAX + m] = pl.u0 < pl.u1 ? make_float4(st[0], st[1], st[2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
     }
     if (a.epi != EPI_HEAD && a.ssq_out && tid < M) a.ssq_out[(size_t)tid * nctas + cta] = ssq_acc;
@@ -835,10 +886,10 @@ __device__ __forceinline__ void emit_plain_rows(LinArgs& a, Ctx& c, F value) {
         const int nu = min(SC_ROWS, u1 - sc0);
         for (int idx = tid; idx < nu * a.M; idx += NTHREADS) {
             const int r = idx % nu, m = idx / nu;
-            wk[LW_ACC + (size_t)r * MP + m] = value(m, sc0 + r);
+            wk[LinGeom<8>::ACC_OFF + (size_t)r * MP_MAX + m] = value(m, sc0 + r);
         }
         cta_sync();
-        emit_rows(a, wk, sc0, nu, false, ssq_acc);
+        emit_rows<MP_MAX>(a, wk, wk + LinGeom<8>::ACC_OFF, sc0, nu, false, ssq_acc);
         cta_sync();
     }
     if (a.ssq_out && tid < a.M) a.ssq_out[(size_t)tid * c.nctas + c.cta] = ssq_acc;
@@ -932,7 +983,8 @@ template <typename WT>
 __device__ __forceinline__ bool linear_consumer(const LinArgs* sa, Ctx& c, bool stream, bool publish) {
     if (publish) cta_sync();
     if (stream) {
-        if (sa->M <= 4) lin_consume<4>(*sa, c); else if (sa->M <= 8) lin_consume<8>(*sa, c); else lin_consume<16>(*sa, c);
+        if (sa->M <= 4) lin_consume<4>(*sa, c); else if (sa->M <= 8) lin_consume<8>(*sa, c);
+        else if (sa->M <= 12) lin_consume<12>(*sa, c); else lin_consume<16>(*sa, c);
     } else {
         lin_simple<WT>(*sa, c);
     }
