@@ -22,7 +22,7 @@ def binding():
     return b
 
 
-@pytest.mark.parametrize("shape,n", [(HD64, 32), (HD64, 65), (HD64, 129), (HD64, 257), (HD64, 600), (HD128, 63), (HD128, 64), (HD128, 193), (HD128, 321)])
+@pytest.mark.parametrize("shape,n", [(HD64, 17), (HD128, 16), (HD64, 32), (HD64, 65), (HD64, 129), (HD64, 257), (HD64, 600), (HD128, 63), (HD128, 64), (HD128, 193), (HD128, 321)])
 def test_prompt_pass_against_the_oracle(binding, shape, n):
     """Logits of the last prompt row, then rounds that read every K / V row the pass wrote."""
     from parity_harness import lockstep
