@@ -67,28 +67,22 @@ __global__ void fill_tokens_kernel(int* out, uint64_t base, int count, int vocab
 }
 
 // fp32 rows -> packed rows (scaled by gain) + per-slice sums of squares, sliced over the columns exactly as the
-// CTAs of the decode kernel slice an operator's output (slice c = columns [K c / n, K (c+1) / n)).
+// CTAs of the decode kernel slice an operator's output (slice c = columns [K c / n, K (c+1) / n)).  One warp per row: a slice
+// is a few dozen columns, so that a CTA per row and slice would spend its time in barriers.
 __global__ void pack_rows_kernel(const float* x, int ldx, int M, int K, const float* gain, unsigned char* xpk, int ldpk,
                                  float* ssq, int nslices) {
-    __shared__ float sred[8];
-    const int cta = blockIdx.x;
+    grid_dependents_launch();
+    const int cta = blockIdx.x, lane = threadIdx.x & 31;
     const int k0 = (int)((unsigned)K * (unsigned)cta / (unsigned)nslices), k1 = (int)((unsigned)K * (unsigned)(cta + 1) / (unsigned)nslices);
-    for (int m = 0; m < M; ++m) {
+    for (int m = threadIdx.x >> 5; m < M; m += blockDim.x >> 5) {
         float ss = 0.f;
-        for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+        for (int k = k0 + lane; k < k1; k += 32) {
             const float v = x[(size_t)m * ldx + k];
             ss += v * v;
             pk_store(xpk + (size_t)m * ldpk, k, gain ? v * gain[k] : v);
         }
         ss = warp_sum(ss);
-        if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = ss;
-        __syncthreads();
-        if (threadIdx.x == 0 && ssq) {
-            float t = 0.f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sred[w];
-            ssq[(size_t)m * nslices + cta] = t;
-        }
-        __syncthreads();
+        if (lane == 0 && ssq) ssq[(size_t)m * nslices + cta] = ss;
     }
 }
 
@@ -901,11 +895,19 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(LinArgs a, 
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
     OpTable* t = reinterpret_cast<OpTable*>(c.producer ? c.ctl->tab_prod : c.ctl->tab_cons);
     if (c.producer ? (threadIdx.x & 31) == 0 : threadIdx.x == 0) t->lin[0] = a;
+    // launched while the kernel that packs the rows may still run: the copy warp starts on the weights at once
+    grid_dependents_launch();
+    if (!c.producer) grid_dependency_wait();
     const bool ok = linear_op<WT>(&t->lin[0], c, stream != 0, true);
     if (!ok && c.producer) ring_drain(c);
 }
-__global__ void op_head_final_kernel(const float4* part, int nctas, int M, int* tok, float* p) {
-    if (threadIdx.x < M) { int t; float pp; head_final(part, nctas, threadIdx.x, t, pp); tok[threadIdx.x] = t; p[threadIdx.x] = pp; }
+// one warp per row (one thread per row took 60 us: a chain of a merge per CTA)
+__global__ void op_head_final_kernel(const float4* part, int nctas, int* tok, float* p) {
+    grid_dependency_wait();
+    const int m = threadIdx.x >> 5;
+    int t; float pp;
+    head_final_warp(part, nctas, m, t, pp);
+    if ((threadIdx.x & 31) == 0) { tok[m] = t; p[m] = pp; }
 }
 template <typename WT>
 __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __grid_constant__ Dev D, AttArgs a) {
@@ -917,6 +919,19 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __
         cta_sync();
         attention_op<WT>(D, &t->att, c);
     }
+}
+
+// A launch that may begin before the kernel ahead of it in the stream has finished; the kernel calls grid_dependency_wait()
+// before it touches anything that one writes.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kfn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kfn, P(args)...);
 }
 
 int g_force_simple_ops = 0;
@@ -946,7 +961,8 @@ static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int x
     }
     if (dtype == KG_BF16) {
         if (set_smem(op_linear_kernel<__nv_bfloat16>) != KG_OK) return KG_E_CUDA;
-        op_linear_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, plain ? 0 : 1);
+        if (plain) op_linear_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
+        else CK(launch_dependent(op_linear_kernel<__nv_bfloat16>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a, 1));
     } else {
         if (set_smem(op_linear_kernel<float>) != KG_OK) return KG_E_CUDA;
         op_linear_kernel<float><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
@@ -984,8 +1000,7 @@ extern "C" int kg_op_lm_head(int32_t dtype, const void* W, int32_t V, int32_t K,
     a.logits_dbg = logits; a.ld_dbg = V;
     int r = op_linear_common(dtype, a, (unsigned char*)scratch + sc.off_xpk, OP_K_MAX, (float*)((char*)scratch + sc.off_ssq), (cudaStream_t)stream);
     if (r != KG_OK) return r;
-    op_head_final_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(a.head_part, sm_count(), M, tok, p);
-    CK(cudaGetLastError());
+    CK(launch_dependent(op_head_final_kernel, dim3(1), dim3(32 * M), 0, (cudaStream_t)stream, a.head_part, sm_count(), tok, p));
     return KG_OK;
 }
 
@@ -1037,8 +1052,7 @@ extern "C" int kg_op_lm_head_noalloc(int32_t dtype, const void* W, int32_t V, in
     r = op_linear_common(dtype, a, (unsigned char*)scratch + NOALLOC_OFF_XPK, NOALLOC_MAX_K, (float*)((char*)scratch + NOALLOC_OFF_SSQ),
                          (cudaStream_t)stream);
     if (r != KG_OK) return r;
-    op_head_final_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(a.head_part, sm_count(), M, tok, p);
-    CK(cudaGetLastError());
+    CK(launch_dependent(op_head_final_kernel, dim3(1), dim3(32 * M), 0, (cudaStream_t)stream, a.head_part, sm_count(), tok, p));
     return KG_OK;
 }
 

@@ -251,6 +251,11 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const unsigned (&a
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Programmatic dependent launch: a kernel launched with that attribute may start early; what it reads of its predecessor's
+// results it reads after the wait (a no-op in an ordinary launch).
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1001,18 +1006,7 @@ __device__ __forceinline__ bool linear_op(const LinArgs* sa, Ctx& c, bool stream
     return c.producer ? linear_producer(sa, c, stream, publish) : linear_consumer<WT>(sa, c, stream, publish);
 }
 
-// Merge the per-CTA head partials of row m (identical result in every CTA: fixed order).
-__device__ __forceinline__ void head_final(const float4* part, int nctas, int m, int& tok, float& p) {
-    HeadStat tot; tot.zmax = 0.f; tot.sum = 0.f; tot.arg = 0;
-    for (int cta = 0; cta < nctas; ++cta) {
-        float4 v = __ldcg(part + (size_t)cta * M_MAX + m);
-        head_merge(tot, v.x, v.y, __float_as_int(v.z));
-    }
-    tok = tot.arg;
-    p = 1.0f / tot.sum;
-}
-
-// The same merge by a whole warp: every lane merges the partials of CTAs lane, lane + 32, ... (independent loads, one
+// Merge the per-CTA head partials of row m by a whole warp (identical result in every CTA): every lane merges the partials of CTAs lane, lane + 32, ... (independent loads, one
 // round trip instead of one per CTA), then a butterfly of merges leaves the identical total in every lane (the merge
 // of two partials is the same whichever of the two lanes computes it).
 __device__ __forceinline__ void head_final_warp(const float4* part, int nctas, int m, int& tok, float& p) {
