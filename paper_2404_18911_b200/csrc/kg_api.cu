@@ -2,6 +2,7 @@
 // launches of the persistent decode kernel, small result copies.  No device allocation anywhere.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -936,9 +937,18 @@ cudaError_t launch_dependent(void (*kfn)(P...), dim3 grid, dim3 block, size_t sm
 
 int g_force_simple_ops = 0;
 
-template <typename K>
-int set_smem(K kfn) {
-    return cudaFuncSetAttribute((const void*)kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL) == cudaSuccess ? KG_OK : KG_E_CUDA;
+// Lets kernel KFN use SMEM_TOTAL bytes of shared memory; the attribute belongs to the kernel and the device, so it is set at the
+// first call on each device (bit `device` of `done`; two threads may both set it, to the same value).
+template <auto KFN>
+int set_smem() {
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return KG_E_CUDA;
+    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (bit && (done.load(std::memory_order_relaxed) & bit)) return KG_OK;
+    if (cudaFuncSetAttribute((const void*)KFN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL) != cudaSuccess) return KG_E_CUDA;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return KG_OK;
 }
 
 }  // namespace
@@ -960,11 +970,11 @@ static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int x
         a.xpk = xpk; a.ldpk = a.K * 4; a.ssq_in = a.gain ? ssq : nullptr;
     }
     if (dtype == KG_BF16) {
-        if (set_smem(op_linear_kernel<__nv_bfloat16>) != KG_OK) return KG_E_CUDA;
+        if (set_smem<op_linear_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
         if (plain) op_linear_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
         else CK(launch_dependent(op_linear_kernel<__nv_bfloat16>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a, 1));
     } else {
-        if (set_smem(op_linear_kernel<float>) != KG_OK) return KG_E_CUDA;
+        if (set_smem<op_linear_kernel<float>>() != KG_OK) return KG_E_CUDA;
         op_linear_kernel<float><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
     }
     CK(cudaGetLastError());
@@ -1082,10 +1092,10 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     AttArgs a; a.qkv = qkv; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out;
     const int nctas = sm_count();
     if (dtype == KG_BF16) {
-        if (set_smem(op_attention_kernel<__nv_bfloat16>) != KG_OK) return KG_E_CUDA;
+        if (set_smem<op_attention_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
         op_attention_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
     } else {
-        if (set_smem(op_attention_kernel<float>) != KG_OK) return KG_E_CUDA;
+        if (set_smem<op_attention_kernel<float>>() != KG_OK) return KG_E_CUDA;
         op_attention_kernel<float><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
     }
     CK(cudaGetLastError());
