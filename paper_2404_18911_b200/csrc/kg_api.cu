@@ -94,8 +94,9 @@ inline uint64_t layer_tid(int layer, int k) { return (uint64_t)TID_LAYER_BASE + 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Layout {
-    size_t off_hApk, off_hBpk, off_attnpk, off_actpk, off_featApk, off_featDpk, off_abufpk, off_ssqA, off_ssqB, off_ssqF, off_ssqAb;
-    size_t off_layers, off_pt, off_kc, off_vc, off_h, off_feat, off_abuf, off_qkv, off_attn, off_act, off_po, off_ml,
+    size_t off_hApk, off_featApk, off_featDpk, off_abufpk, off_ssqA, off_ssqF, off_ssqAb, off_xch[2], xch_bytes;
+    int xch_ld;
+    size_t off_layers, off_pt, off_kc, off_vc, off_h, off_feat, off_abuf, off_po, off_ml,
         off_cnt, off_hp, off_dbgd, off_dbgv, off_out, off_S, off_rlog, off_prompt, off_st, off_bar;
     // tensor-core prompt pass (0 bytes each when the shape cannot take it)
     size_t off_pf_h, off_pf_x, off_pf_q, off_pf_f, off_pf_rs, off_pf_cs, off_pf_part, off_pf_cnt, off_pf_err;
@@ -152,18 +153,14 @@ Layout make_layout(const kg_config* c, int own_weights, int nctas) {
     L.off_h = take(4 * KG_M_MAX * d);
     L.off_feat = take(4 * (KG_M_MAX + 1) * d);
     L.off_abuf = take(4 * 2 * d);
-    L.off_qkv = take(4 * KG_M_MAX * 3 * d);
-    L.off_attn = take(4 * KG_M_MAX * d);
-    L.off_act = take(4 * KG_M_MAX * F);
+    L.xch_ld = (int)align_up(5 * d + F + nctas, 4);
+    L.xch_bytes = 4 * (size_t)KG_M_MAX * L.xch_ld;
+    L.off_xch[0] = take(L.xch_bytes); L.off_xch[1] = take(L.xch_bytes);
     L.off_hApk = take(4 * KG_M_MAX * d);
-    L.off_hBpk = take(4 * KG_M_MAX * d);
-    L.off_attnpk = take(4 * KG_M_MAX * d);
-    L.off_actpk = take(4 * KG_M_MAX * F);
     L.off_featApk = take(4 * (KG_M_MAX + 1) * d);
     L.off_featDpk = take(4 * (KG_M_MAX + 1) * d);
     L.off_abufpk = take(4 * 2 * d);
     L.off_ssqA = take(4 * (size_t)KG_M_MAX * nctas);
-    L.off_ssqB = take(4 * (size_t)KG_M_MAX * nctas);
     L.off_ssqF = take(4 * (size_t)(KG_M_MAX + 1) * nctas);
     L.off_ssqAb = take(4 * (size_t)2 * nctas);
     L.off_po = take(4 * (size_t)KG_M_MAX * H * S_CAP * hd);
@@ -433,14 +430,13 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     D.layers = (const LayerW*)P(lay.off_layers); D.page_table = (const int*)P(lay.off_pt);
     D.kcache = P(lay.off_kc); D.vcache = P(lay.off_vc);
     D.h = (float*)P(lay.off_h); D.feat = (float*)P(lay.off_feat); D.abuf = (float*)P(lay.off_abuf);
-    D.qkv = (float*)P(lay.off_qkv); D.attn = (float*)P(lay.off_attn); D.act = (float*)P(lay.off_act);
+    D.xch[0] = (unsigned*)P(lay.off_xch[0]); D.xch[1] = (unsigned*)P(lay.off_xch[1]); D.xch_ld = lay.xch_ld;
     D.att_po = (float*)P(lay.off_po); D.att_ml = (float*)P(lay.off_ml); D.att_cnt = (unsigned*)P(lay.off_cnt);
     D.head_part = (float4*)P(lay.off_hp);
-    D.hA_pk = (unsigned char*)P(lay.off_hApk); D.hB_pk = (unsigned char*)P(lay.off_hBpk);
-    D.attn_pk = (unsigned char*)P(lay.off_attnpk); D.act_pk = (unsigned char*)P(lay.off_actpk);
+    D.hA_pk = (unsigned char*)P(lay.off_hApk);
     D.featA_pk = (unsigned char*)P(lay.off_featApk); D.featD_pk = (unsigned char*)P(lay.off_featDpk);
     D.abuf_pk = (unsigned char*)P(lay.off_abufpk);
-    D.ssq_hA = (float*)P(lay.off_ssqA); D.ssq_hB = (float*)P(lay.off_ssqB);
+    D.ssq_hA = (float*)P(lay.off_ssqA);
     D.ssq_feat = (float*)P(lay.off_ssqF); D.ssq_abuf = (float*)P(lay.off_ssqAb);
     D.dm.stream = (cfg->dtype == KG_BF16 && cfg->d_model % 16 == 0 && cfg->d_ffn % 16 == 0) ? 1 : 0;
     D.dbg_draft = cfg->debug_logits ? (float*)P(lay.off_dbgd) : nullptr;
@@ -484,6 +480,7 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     }
     ok = ok && cudaMemcpyAsync(P(lay.off_pt), pt.data(), sizeof(int) * pt.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
     ok = ok && cudaMemsetAsync(D.st, 0, sizeof(State), s) == cudaSuccess;
+    for (int i = 0; i < 2; ++i) ok = ok && cudaMemsetAsync(D.xch[i], 0xff, lay.xch_bytes, s) == cudaSuccess;      // XCH_EMPTY
     ok = ok && cudaMemsetAsync(D.att_cnt, 0, 4 * cfg->n_heads, s) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(s) == cudaSuccess;    // pt / layers_host are host temporaries
     if (!ok) { delete m; return KG_E_CUDA; }
@@ -967,7 +964,7 @@ static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int x
     if (!plain) {
         if (a.K > xpk_k_max || nctas > 1024) return KG_E_LIMIT;
         pack_rows_kernel<<<nctas, 256, 0, s>>>(a.x, a.ldx, a.M, a.K, a.gain, xpk, a.K * 4, a.gain ? ssq : nullptr, nctas);
-        a.xpk = xpk; a.ldpk = a.K * 4; a.ssq_in = a.gain ? ssq : nullptr;
+        a.xpk = xpk; a.ldpk = a.K * 4; a.ssq_in = a.gain ? ssq : nullptr; a.ld_ssq = nctas;
     }
     if (dtype == KG_BF16) {
         if (set_smem<op_linear_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
@@ -1089,7 +1086,7 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     D.att_po = (float*)((char*)scratch + sc.off_po); D.att_ml = (float*)((char*)scratch + sc.off_ml);
     D.att_cnt = (unsigned*)((char*)scratch + sc.off_cnt);
     CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
-    AttArgs a; a.qkv = qkv; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out;
+    AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
     if (dtype == KG_BF16) {
         if (set_smem<op_attention_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
@@ -1307,7 +1304,7 @@ int prefill_tc(kg_model* m, int n) {
         pack_rows_kernel<<<m->nctas, 256, 0, s>>>(h + (size_t)last * d, d, 1, d, D.g_final, D.hA_pk, d * 4, D.ssq_hA, m->nctas);
         LinArgs a{};
         a.W = D.head; a.N = c.vocab; a.K = d; a.M = 1; a.x = h + (size_t)last * d; a.ldx = d; a.gain = D.g_final; a.eps = c.rms_eps;
-        a.xpk = D.hA_pk; a.ldpk = d * 4; a.ssq_in = D.ssq_hA;
+        a.xpk = D.hA_pk; a.ldpk = d * 4; a.ssq_in = D.ssq_hA; a.ld_ssq = m->nctas;
         a.epi = EPI_HEAD; a.scale = c.logit_scale; a.head_part = D.head_part;
         a.logits_dbg = c.debug_logits ? D.dbg_verify : nullptr; a.ld_dbg = c.vocab;
         op_linear_kernel<WT><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 1);

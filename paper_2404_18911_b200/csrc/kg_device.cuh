@@ -2,7 +2,7 @@
 //
 // Everything here is written as __device__ "operators" that every CTA of a persistent,
 // cooperatively launched grid executes in lock step: each operator splits its work by
-// (cta, nctas) and a grid-wide barrier separates dependent operators.  The same operators are
+// (cta, nctas); its readers poll for the rows it writes, or a grid-wide barrier comes between.  The same operators are
 // also wrapped one-by-one in small kernels for unit tests.
 //
 // A CTA has 8 consumer warps and one producer warp.  The decode step is bound by HBM bandwidth:
@@ -104,18 +104,16 @@ struct Dev {
     float* h;                      // [M_MAX][d] residual stream of the pass
     float* feat;                   // [M_MAX+1][d]: slot 0 = early feature of position P-1, slot 1+j = f_j
     float* abuf;                   // [2][d] adapter output rows
-    float* qkv;                    // [M_MAX][3d]
-    float* attn;                   // [M_MAX][d]
-    float* act;                    // [M_MAX][F]
+    // Rows exchanged inside a layer, two instances used by turns: row m of an instance is xch_ld words long and holds q, k, v
+    // [3d], the attention output [d], the residual stream after attention [d], the SwiGLU output [F] and the sums of squares
+    // of the residual stream [nctas].  All but q, k, v and the sums are packed rows (streamed path) or fp32 rows (plain path).
+    unsigned* xch[2]; int xch_ld;
     // packed copies (streamed path; row = 4 bytes per element) and per-CTA sums of squares [row][nctas]
     unsigned char* hA_pk;          // [M_MAX][d]   residual stream scaled for the next QKV / the LM head
-    unsigned char* hB_pk;          // [M_MAX][d]   residual stream after attention scaled for the SwiGLU pair
-    unsigned char* attn_pk;        // [M_MAX][d]
-    unsigned char* act_pk;         // [M_MAX][F]
     unsigned char* featA_pk;       // [M_MAX+1][d] early features scaled by the adapter's input gain
     unsigned char* featD_pk;       // [M_MAX+1][d] early features scaled by the first deep layer's gain
     unsigned char* abuf_pk;        // [2][d]       adapter output scaled by its last gain
-    float* ssq_hA; float* ssq_hB;  // [M_MAX][nctas]
+    float* ssq_hA;                 // [M_MAX][nctas]
     float* ssq_feat;               // [M_MAX+1][nctas]
     float* ssq_abuf;               // [2][nctas]
     float* att_po;                 // [M_MAX][H][S_CAP][hd] split partial outputs
@@ -346,6 +344,47 @@ __device__ __forceinline__ bool grid_sync(Ctx& c, int where) {
     return *(volatile int*)&c.ctl->sync_ok != 0;
 }
 
+// ------------------------------------------------------------------------------------ exchange inside a layer
+// Between the operators of a layer there is no grid barrier.  A word that has not been written holds XCH_EMPTY, and a
+// reader polls the words that it needs; a word that holds anything else is the value itself, so neither the writer's
+// stores nor the reader's loads need any order among themselves.  XCH_EMPTY is a NaN that no arithmetic produces: results
+// that are NaN come out as 0x7fffffff (fp32) and 0x7fff (bf16), whatever their inputs.
+//
+// A barrier costs the release of the writer's stores - slow while the CTA's weight copies are in flight -, the serialised
+// arrivals, the polling of the counter and then the fetch of the data; the exchange is one store and one polled load.  Four of
+// the five barriers of a layer went this way: 7B, KV 512, verify pass of one row 3.08 -> 2.74 ms, of seven rows 3.60 -> 3.42,
+// greedy step 3.22 -> 2.87, single draft step 0.352 -> 0.328; the fp32 model of four layers (with the plain path's loads issued
+// ahead) 18.1 -> 7.3 ms for 64 tokens.  What was measured on the way: polling a few words before the first full read costs one
+// more round trip (+2 % of a pass), checking each step's words at its MMA brings calls and spills into the inner loop (+17 %).
+//
+// Two instances of the buffers are used by turns, one per layer.  While a layer uses one of them, the other one, which the
+// layer before used, is filled with XCH_EMPTY again; the grid barrier at the end of every layer stands between the last
+// read of an instance and its refill, and between the refill and its next use.
+constexpr unsigned XCH_EMPTY = 0xffffffffu;
+__device__ __forceinline__ unsigned xch_ld1(const unsigned* p) { unsigned v; asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint2 xch_ld2(const void* p) { uint2 v; asm volatile("ld.relaxed.gpu.global.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p)); return v; }
+__device__ __forceinline__ uint4 xch_ld4(const void* p) {
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void xch_st(unsigned* p, unsigned v) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ void xch_stf(float* p, float v) { xch_st(reinterpret_cast<unsigned*>(p), __float_as_uint(v)); }
+__device__ __forceinline__ bool xch_empty(const uint2& v) { return v.x == XCH_EMPTY || v.y == XCH_EMPTY; }
+__device__ __forceinline__ bool xch_empty(const uint4& v) { return v.x == XCH_EMPTY || v.y == XCH_EMPTY || v.z == XCH_EMPTY || v.w == XCH_EMPTY; }
+
+// Called by a thread whose poll came back empty: true = poll again, false = give up (here or elsewhere).  `spins` starts at 0.
+struct XchSpin { unsigned spins; long long t0; };
+__device__ __noinline__ bool xch_check(Ctx& c, long long t0, int where) {
+    if (*(volatile int*)&c.ctl->abort) return false;
+    if ((unsigned long long)(clock64() - t0) > c.wait_clk) { record_timeout(c, where); return false; }
+    return true;
+}
+__device__ __forceinline__ bool xch_again(Ctx& c, XchSpin& sp, int where) {
+    if (sp.spins == 0u) sp.t0 = clock64();
+    return ((++sp.spins) & 31u) != 0u || xch_check(c, sp.t0, where);
+}
+
 // ------------------------------------------------------------------------------------ RoPE
 // cos / sin of pos * theta^(-2i/hd): the angle is formed and reduced to [-pi, pi] in double, the
 // trigonometric functions are evaluated in fp32 on the reduced argument.
@@ -377,6 +416,21 @@ __device__ __forceinline__ void pk_store(unsigned char* row, int k, float v) {
     *reinterpret_cast<__nv_bfloat16*>(p + 8) = l;
 }
 
+// The same for two neighbouring elements k (even), k + 1, as whole words
+__device__ __forceinline__ void pk_store2(unsigned char* row, int k, float v0, float v1) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+    const float2 f = __bfloat1622float2(h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - f.x, v1 - f.y);
+    unsigned* p = reinterpret_cast<unsigned*>(row + pk_off(k));
+    xch_st(p, *reinterpret_cast<const unsigned*>(&h));
+    xch_st(p + 2, *reinterpret_cast<const unsigned*>(&l));
+}
+// Called by whole warps whose neighbouring lanes hold neighbouring elements (k even in even lanes)
+__device__ __forceinline__ void pk_store_lane(unsigned char* row, int k, float v) {
+    const float o = __shfl_xor_sync(0xffffffffu, v, 1);
+    if (!(k & 1)) pk_store2(row, k, v, o);
+}
+
 struct LinArgs {
     const void* W; const void* W2;   // [N, K]; W2 != null: SwiGLU pair (gate, up)
     int N, K;
@@ -384,7 +438,8 @@ struct LinArgs {
     const float* x; int ldx;         // plain path: fp32 rows (written earlier in this kernel)
     const float* gain; float eps;    // RMSNorm gain of the input (null: no norm)
     const unsigned char* xpk; int ldpk;   // streamed path: packed rows, already multiplied by the gain; bytes per row
-    const float* ssq_in;             // streamed path with norm: [M][nctas] partial sums of squares of the input rows
+    const float* ssq_in; int ld_ssq; // streamed path with norm: [M] rows of nctas partial sums of squares of the input rows
+    int poll;                        // 1: the input rows and their sums are exchange words, to be polled
     const float* resid; int ldr;     // EPI_RESID
     float* out; int ldo;             // fp32 output rows (streamed path: nullable)
     int epi;
@@ -392,7 +447,7 @@ struct LinArgs {
     float4* head_part;               // EPI_HEAD: [nctas][M_MAX]
     float* logits_dbg; int ld_dbg;   // EPI_HEAD, optional
     PkOut pk[2]; int ldpk_out;       // streamed path: packed copies of the output rows for the operators that read them
-    float* ssq_out;                  // streamed path: [M][nctas] partial sums of squares of the output rows (nullable)
+    float* ssq_out; int ld_sout;     // streamed path: [M] rows of nctas partial sums of squares of the output rows (nullable)
 };
 
 __device__ __forceinline__ float silu_f(float v) { return v / (1.0f + expf(-v)); }
@@ -446,6 +501,12 @@ template <int V> struct LinGeom {
 };
 constexpr int MP_MAX = 16;
 
+// First of the units (of N) that belong to CTA `cta`: even, so that a packed word has one writer.
+__device__ __forceinline__ int cta_unit(int N, int cta, int nctas) {
+    const int u = 2 * (int)((unsigned)((N + 1) >> 1) * (unsigned)cta / (unsigned)nctas);      // N * nctas < 2^32 (checked on the host)
+    return min(u, N);
+}
+
 struct LinPlan {
     int u0, u1;          // this CTA's units
     int sc_units;        // units per superchunk
@@ -454,8 +515,8 @@ struct LinPlan {
 
 __device__ __forceinline__ LinPlan make_plan(const LinArgs& a, int cta, int nctas) {
     LinPlan p;
-    p.u0 = (int)((unsigned)a.N * (unsigned)cta / (unsigned)nctas);          // N * nctas < 2^32 (checked on the host)
-    p.u1 = (int)((unsigned)a.N * (unsigned)(cta + 1) / (unsigned)nctas);
+    p.u0 = cta_unit(a.N, cta, nctas);
+    p.u1 = cta_unit(a.N, cta + 1, nctas);
     p.sc_units = a.W2 ? SC_ROWS / 2 : SC_ROWS;
     p.plen = a.M <= 12 ? LinGeom<12>::PLEN : LinGeom<16>::PLEN;
     p.nph = (a.K + p.plen - 1) / p.plen;
@@ -524,8 +585,8 @@ __device__ __forceinline__ void split_hi_lo(float2 v, unsigned& hi, unsigned& lo
 // Shared-memory work area of the streamed path (floats, from WORK_OFF).
 constexpr int LW_RED = 0;                                 // partial sums of a stage pair, then at LinGeom::ACC_OFF the row accumulators [SC_ROWS][MP]
 constexpr int LW_RS = 2 * NWARPS * 128 + SC_ROWS * MP_MAX;   // [M_MAX] 1/rms of the input rows
-constexpr int LW_RSP = LW_RS + M_MAX;                     // [M_MAX][16] partial sums of squares of the input rows
-constexpr int LW_SSW = LW_RSP + M_MAX * 16;               // [NWARPS][M_MAX] sums of squares of the output rows
+constexpr int LW_RSP = LW_RS + M_MAX;                     // [16] partial sums of squares of the input rows
+constexpr int LW_SSW = LW_RSP + 16;                       // [NWARPS][M_MAX] sums of squares of the output rows
 constexpr int PRE_NU = 64;                                // residual / gain values are prefetched for up to this many units
 constexpr int LW_PRES = LW_SSW + NWARPS * M_MAX;          // [M_MAX][PRE_NU] residual values
 constexpr int LW_PREG = LW_PRES + M_MAX * PRE_NU;         // [2][PRE_NU] gains of the packed outputs
@@ -543,7 +604,7 @@ __device__ __forceinline__ void cp_async4(void* dst_smem, const void* src) {
 // Epilogue of the streamed path for everything but the LM head: turns the accumulators of nu output
 // units x M rows (acc_s with MP columns, 1/rms in rs) into fp32 rows, packed copies and per-CTA sums of squares.
 // Thread (r, m): m = tid mod 2^ceil(log2 M), so that the lanes of a warp that share m can add their
-// squares by shuffles in a fixed order.  Every consumer thread calls it; ssq_acc (threads < M)
+// squares by shuffles in a fixed order.  Outputs with a packed copy have an even number of features.  Every consumer thread calls it; ssq_acc (threads < M)
 // accumulates over superchunks.
 template <int MP>
 __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const float* acc_s, int sc0, int nu, bool prefetched, float& ssq_acc) {
@@ -555,9 +616,13 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const flo
     const int mp = 1 << sh;
     const int m = tid & (mp - 1);
     float ssl = 0.f;
-    if (m < M) {
-        for (int r = tid >> sh; r < nu; r += NTHREADS >> sh) {
-            float v;
+    // whole warps go round together: two neighbouring rows of W, in lanes mp apart, make one packed word
+    for (int rb = warp * (32 >> sh); rb < nu; rb += NTHREADS >> sh) {
+        const int r = rb + (lane >> sh);
+        const bool valid = r < nu && m < M;
+        const int row = sc0 + r;
+        float v = 0.f;
+        if (valid) {
             if (a.epi == EPI_SWIGLU) {
                 const int srow = (r >> 3) * 16 + (r & 7);
                 v = silu_f(acc_s[(size_t)srow * MP + m] * rs[m]) * (acc_s[(size_t)(srow + 8) * MP + m] * rs[m]);
@@ -566,16 +631,16 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const flo
                 if (a.epi == EPI_RESID)
                     v += prefetched ? wk[LW_PRES + m * PRE_NU + r] : ldcg_f(a.resid + (size_t)m * a.ldr + sc0 + r);
             }
-            const int row = sc0 + r;
-            if (a.out) a.out[(size_t)m * a.ldo + row] = v;
+            if (a.out) xch_stf(a.out + (size_t)m * a.ldo + row, v);
             ssl += v * v;
+        }
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (a.pk[q].ptr) {
-                    float pv = v;
-                    if (a.pk[q].gain) pv *= prefetched ? wk[LW_PREG + q * PRE_NU + r] : __ldg(a.pk[q].gain + row);
-                    pk_store(a.pk[q].ptr + (size_t)m * a.ldpk_out, row, pv);
-                }
+        for (int q = 0; q < 2; ++q) {
+            if (a.pk[q].ptr) {
+                float pv = v;
+                if (valid && a.pk[q].gain) pv *= prefetched ? wk[LW_PREG + q * PRE_NU + r] : __ldg(a.pk[q].gain + row);
+                const float po = __shfl_xor_sync(0xffffffffu, pv, mp);
+                if (valid && !(r & 1)) pk_store2(a.pk[q].ptr + (size_t)m * a.ldpk_out, row, pv, po);
             }
         }
     }
@@ -590,6 +655,9 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const flo
         }
     }
 }
+
+// log2 of the threads that add the sums of squares of one of M rows
+__device__ __forceinline__ int sum_shift(int M) { return M <= 1 ? 8 : (M <= 2 ? 7 : (M <= 4 ? 6 : (M <= 8 ? 5 : 4))); }
 
 template <int V>
 __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
@@ -614,19 +682,12 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     int buf = 0;
     float ssq_acc = 0.f;
 
-    // ---- fetched early, used in the epilogue: the input rows' sums of squares, residual values, output gains.
-    // The requests go out right behind the first phase's fragment loads, which the first MMA waits for.
+    // ---- fetched early, used in the epilogue: residual values, output gains (the requests go out behind the first phase's
+    // fragment loads, which the first MMA waits for)
     const int nu0 = min(pl.u1 - pl.u0, pl.sc_units);
     const bool prefetched = nu0 <= PRE_NU;
     bool pre_pending = true;
     auto epilogue_prefetch = [&]() {
-        if (a.ssq_in) {
-            // thread (m, j) adds the partial sums of CTAs j, j + 16, ... of row m
-            const int m = tid >> 4, j = tid & 15;
-            float part = 0.f;
-            if (m < M) for (int q = j; q < nctas; q += 16) part += ldcg_f(a.ssq_in + (size_t)m * nctas + q);
-            wk[LW_RSP + tid] = part;
-        }
         if (prefetched && a.epi != EPI_HEAD) {
             if (a.epi == EPI_RESID)
                 for (int i = tid; i < M * nu0; i += NTHREADS) cp_async4(wk + LW_PRES + (i / nu0) * PRE_NU + i % nu0, a.resid + (size_t)(i / nu0) * a.ldr + pl.u0 + i % nu0);
@@ -638,13 +699,6 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    // this lane's rows of the packed input: V = 4: row g & 3 (hi for g < 4, lo for g >= 4); else rows g (and g + 8)
-    const int xrow = V == 4 ? (g & 3) : g;
-    const unsigned char* xlane = a.xpk + (size_t)xrow * a.ldpk + (size_t)warp * NS * 64 + t * 16 + (V == 4 ? (g >> 2) * 8 : 0);
-    // V = 12: rows 8 .. 11 (hi for g < 4, lo for g >= 4), seen from xlane
-    const int mrow = 8 + (g & 3);
-    const ptrdiff_t mofs = (ptrdiff_t)((mrow < M ? mrow : 0) - xrow) * (ptrdiff_t)a.ldpk + (g >> 2) * 8;
-
     for (int sc0 = pl.u0; sc0 < pl.u1; sc0 += pl.sc_units) {
         const int sc1 = min(pl.u1, sc0 + pl.sc_units);
         const int nu = sc1 - sc0;
@@ -653,46 +707,53 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
         for (int ph = 0; ph < pl.nph; ++ph) {
             const int p0 = ph * pl.plen, len = min(pl.plen, K - p0);
             const int nsteps = len / 16;
-            // ---- B fragments of this warp's k slice, kept in registers for every row group of the phase
-            // (every load is issued before any is used: steps past the end of the phase and rows >= M re-read valid
-            // data and are zeroed afterwards)
+            // ---- B fragments of this warp's k slice, kept in registers for every row group of the phase.  Every load is issued
+            // before any is used; exchange words are read again until all of them are there.  Rows >= M re-read a valid row: their
+            // columns of the product are never read, and the columns of an MMA do not mix.  Steps past the end of the phase re-read
+            // the last one and are skipped.
             unsigned fr[NS][FR];
+            const int last = nsteps - 1 - warp * NS;             // last valid step of this warp (< 0: none)
             {
-                const int last = nsteps - 1 - warp * NS;         // last valid step of this warp (< 0: none)
-                const unsigned char* pbase = xlane + (size_t)(p0 / 16) * 64;
+                // this lane's rows of the packed input: V = 4: row g & 3 (hi for g < 4, lo for g >= 4); else row g and, mofs bytes
+                // away, V = 12: row 8 + (g & 3) (hi for g < 4, lo for g >= 4), V = 16: row 8 + g (M > 8 here, so that g < M)
+                const int xrow = V == 4 ? (g & 3) : g, mrow = 8 + (V == 12 ? (g & 3) : g);
+                const int mofs = ((mrow < M ? mrow : 0) - xrow) * a.ldpk + (V == 12 ? (g >> 2) * 8 : 0);
+                const unsigned char* pbase = a.xpk + (size_t)(xrow < M ? xrow : 0) * a.ldpk + (size_t)(p0 / 16 + warp * NS) * 64 + t * 16 + (V == 4 ? (g >> 2) * 8 : 0);
+                int lastv = last;
+                XchSpin sp; sp.spins = 0;
+                while (true) {
+                    asm volatile("" : "+l"(pbase), "+r"(lastv));   // keeps the steps' addresses from being formed, and spilled, ahead of the loop
 #pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const unsigned char* px = pbase + (size_t)max(min(s, last), -warp * NS) * 64;
-                    if (V == 4) {
-                        const uint2 v = __ldcg(reinterpret_cast<const uint2*>(xrow < M ? px : px - (size_t)xrow * a.ldpk));
-                        fr[s][0] = v.x; fr[s][1] = v.y;
-                    } else {
-#pragma unroll
-                        for (int n = 0; n < NACC; ++n) {
-                            const int row = xrow + 8 * n;
-                            const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row < M ? px + (size_t)(8 * n) * a.ldpk : px - (size_t)xrow * a.ldpk));
-                            fr[s][4 * n + 0] = v.x; fr[s][4 * n + 1] = v.y; fr[s][4 * n + 2] = v.z; fr[s][4 * n + 3] = v.w;
-                        }
-                        if (V == 12) {
-                            const uint2 w = __ldcg(reinterpret_cast<const uint2*>(px + mofs));
-                            fr[s][FR - 2] = w.x; fr[s][FR - 1] = w.y;
+                    for (int s = 0; s < NS; ++s) {
+                        const unsigned char* px = pbase + (size_t)max(min(s, lastv), -warp * NS) * 64;
+                        if (V == 4) {
+                            const uint2 v = xch_ld2(px);
+                            fr[s][0] = v.x; fr[s][1] = v.y;
+                        } else {
+                            const uint4 v = xch_ld4(px);
+                            fr[s][0] = v.x; fr[s][1] = v.y; fr[s][2] = v.z; fr[s][3] = v.w;
+                            if (V == 16) {
+                                const uint4 w = xch_ld4(px + mofs);
+                                fr[s][FR - 4] = w.x; fr[s][FR - 3] = w.y; fr[s][FR - 2] = w.z; fr[s][FR - 1] = w.w;
+                            }
+                            if (V == 12) {
+                                const uint2 w = xch_ld2(px + mofs);
+                                fr[s][FR - 2] = w.x; fr[s][FR - 1] = w.y;
+                            }
                         }
                     }
-                }
-                if (pre_pending) { pre_pending = false; epilogue_prefetch(); }
+                    if (!a.poll || !ok) break;
+                    bool empty = false;
 #pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const bool sv = s <= last;
-                    if (V == 4) {
-                        if (!(sv && xrow < M)) { fr[s][0] = 0u; fr[s][1] = 0u; }
-                    } else {
+                    for (int s = 0; s < NS; ++s) {
 #pragma unroll
-                        for (int n = 0; n < NACC; ++n)
-                            if (!(sv && xrow + 8 * n < M)) { fr[s][4 * n + 0] = 0u; fr[s][4 * n + 1] = 0u; fr[s][4 * n + 2] = 0u; fr[s][4 * n + 3] = 0u; }
-                        if (V == 12 && !(sv && mrow < M)) { fr[s][FR - 2] = 0u; fr[s][FR - 1] = 0u; }
+                        for (int i = 0; i < FR; ++i) empty |= fr[s][i] == XCH_EMPTY;
                     }
+                    if (!__any_sync(0xffffffffu, empty)) break;
+                    if (!__all_sync(0xffffffffu, xch_again(c, sp, 43))) ok = false;
                 }
             }
+            if (pre_pending) { pre_pending = false; epilogue_prefetch(); }
             // ---- the row groups of this phase, two stages (16 weight rows) at a time
             const uint32_t a_lane = (uint32_t)((lane & 7) * ST_ROW_BYTES + (warp * NS * 16 + (lane >> 4) * 8) * 2);
             for (int si = 0; si < nst; si += 2) {
@@ -717,7 +778,7 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                     for (int s = 0; s < PD; ++s) ldmatrix_x4(af[s], a_base + (uint32_t)s * 32u);
 #pragma unroll
                     for (int s = 0; s < NS; ++s) {
-                        if (warp * NS + s < nsteps) {
+                        if (s <= last) {
                             if (V == 4) {
                                 mma_bf16_16816(acc[s & 3], af[s % PD], fr[s][0], fr[s][1]);
                             } else if (V == 8) {
@@ -813,13 +874,42 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
         }
         // ---- epilogue of this superchunk
         if (sc0 == pl.u0) {
+            // the input rows' sums of squares: 2^rsh threads per row, SSB partial sums of each thread per batch of loads
+            // (requested here and not beside the fragments, which fill the registers: 2 % of a verify pass at M = 1)
+            if (a.ssq_in) {
+                constexpr int SSB = 5;
+                const int rsh = sum_shift(M), rm = tid >> rsh;
+                const unsigned* ssrow = reinterpret_cast<const unsigned*>(a.ssq_in + (size_t)rm * a.ld_ssq);
+                float part = 0.f;
+                for (int q0 = tid & ((1 << rsh) - 1); q0 < nctas; q0 += SSB << rsh) {
+                    unsigned w[SSB];
+                    XchSpin sp; sp.spins = 0;
+                    while (true) {
+                        bool empty = false;
+#pragma unroll
+                        for (int i = 0; i < SSB; ++i) {
+                            const int q = q0 + (i << rsh);
+                            w[i] = rm < M && q < nctas ? xch_ld1(ssrow + q) : 0u;
+                        }
+#pragma unroll
+                        for (int i = 0; i < SSB; ++i) empty |= w[i] == XCH_EMPTY;
+                        if (!a.poll || !empty || !xch_again(c, sp, 44)) break;
+                    }
+#pragma unroll
+                    for (int i = 0; i < SSB; ++i) part += __uint_as_float(w[i]);
+                }
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+                if ((lane & 15) == 0) wk[LW_RSP + (tid >> 4)] = part;      // 16 sums, 16 / mp of each row
+            }
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             cta_sync();
             if (tid < M_MAX) {
                 float r = 1.0f;
                 if (a.ssq_in && tid < M) {
                     float ss = 0.f;
-                    for (int j = 0; j < 16; ++j) ss += wk[LW_RSP + tid * 16 + j];
+                    const int per = 1 << (sum_shift(M) - 4);                          // 16 / mp
+                    for (int j = 0; j < per; ++j) ss += wk[LW_RSP + tid * per + j];
                     r = rsqrtf(ss / (float)K + a.eps);
                 }
                 rs[tid] = r;
@@ -871,7 +961,7 @@ __device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
             }
         }
     }
-    if (a.epi != EPI_HEAD && a.ssq_out && tid < M) a.ssq_out[(size_t)tid * nctas + cta] = ssq_acc;
+    if (a.epi != EPI_HEAD && a.ssq_out && tid < M) xch_stf(a.ssq_out + (size_t)tid * a.ld_sout + cta, ssq_acc);
     c.slot = slot; c.phase = phase;
 }
 
@@ -882,8 +972,7 @@ template <typename F>
 __device__ __forceinline__ void emit_plain_rows(LinArgs& a, Ctx& c, F value) {
     const int tid = threadIdx.x;
     float* wk = reinterpret_cast<float*>(c.smem + WORK_OFF);
-    const int u0 = (int)((unsigned)a.N * (unsigned)c.cta / (unsigned)c.nctas);
-    const int u1 = (int)((unsigned)a.N * (unsigned)(c.cta + 1) / (unsigned)c.nctas);
+    const int u0 = cta_unit(a.N, c.cta, c.nctas), u1 = cta_unit(a.N, c.cta + 1, c.nctas);
     float ssq_acc = 0.f;
     a.epi = EPI_STORE;
     if (tid < M_MAX) wk[LW_RS + tid] = 1.0f;
@@ -897,29 +986,117 @@ __device__ __forceinline__ void emit_plain_rows(LinArgs& a, Ctx& c, F value) {
         emit_rows<MP_MAX>(a, wk, wk + LinGeom<8>::ACC_OFF, sc0, nu, false, ssq_acc);
         cta_sync();
     }
-    if (a.ssq_out && tid < a.M) a.ssq_out[(size_t)tid * c.nctas + c.cta] = ssq_acc;
+    if (a.ssq_out && tid < a.M) xch_stf(a.ssq_out + (size_t)tid * a.ld_sout + c.cta, ssq_acc);
 }
 
-// Plain path for any storage type (fp32 models, odd shapes, and a cross-check of the tensor-core
-// path): activations staged in shared memory as fp32, one output row per warp at a time.
+// Plain path for any storage type (fp32 models, odd shapes, and a cross-check of the tensor-core path): activations staged in
+// shared memory as fp32, one output row per warp at a time.  What bounds it on a small model is latency: the first weights of
+// a warp's row are requested before the activations are waited for, and a row's sums are formed with 16-byte loads.
+constexpr int SIMPLE_PF = 6;                              // 16-byte groups of a weight row per lane and batch: 768 elements
+template <typename WT>
+__device__ __forceinline__ void simple_fetch(const WT* row, int k0, int K, float4 (&w)[SIMPLE_PF]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < SIMPLE_PF; ++j) {
+        const int k = k0 + j * 128 + lane * 4;
+        w[j] = k < K ? load4_cg<WT>(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+template <typename WT, int MB>
+__device__ __forceinline__ void simple_rows(const LinArgs& a, Ctx& c, const float* xs, const float* rs, float4 (&w1)[SIMPLE_PF], float4 (&w2)[SIMPLE_PF], HeadStat& hs) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int M = a.M, K = a.K;
+    const bool dual = a.W2 != nullptr;
+    const int first = c.cta * NWARPS + warp, step = c.nctas * NWARPS;
+    for (int row = first; row < a.N; row += step) {
+        const WT* wr = reinterpret_cast<const WT*>(a.W) + (size_t)row * K;
+        const WT* wr2 = reinterpret_cast<const WT*>(a.W2) + (size_t)row * K;
+        float acc[MB], acc2[MB];
+#pragma unroll
+        for (int m = 0; m < MB; ++m) { acc[m] = 0.f; acc2[m] = 0.f; }
+        for (int k0 = 0; k0 < K; k0 += SIMPLE_PF * 128) {
+            if (row != first || k0 != 0) { simple_fetch<WT>(wr, k0, K, w1); if (dual) simple_fetch<WT>(wr2, k0, K, w2); }
+#pragma unroll
+            for (int j = 0; j < SIMPLE_PF; ++j) {
+                const int k = k0 + j * 128 + lane * 4;
+                if (k < K) {
+#pragma unroll
+                    for (int m = 0; m < MB; ++m) {
+                        if (m < M) {
+                            const float4 x = *reinterpret_cast<const float4*>(xs + (size_t)m * K + k);
+                            acc[m] = fmaf(w1[j].w, x.w, fmaf(w1[j].z, x.z, fmaf(w1[j].y, x.y, fmaf(w1[j].x, x.x, acc[m]))));
+                            if (dual) acc2[m] = fmaf(w2[j].w, x.w, fmaf(w2[j].z, x.z, fmaf(w2[j].y, x.y, fmaf(w2[j].x, x.x, acc2[m]))));
+                        }
+                    }
+                }
+            }
+        }
+        float v = 0.f, v2 = 0.f;                         // lane m takes row m
+#pragma unroll
+        for (int m = 0; m < MB; ++m) {
+            if (m < M) {
+                const float s1 = warp_sum(acc[m]);
+                if (lane == m) v = s1;
+                if (dual) { const float s2 = warp_sum(acc2[m]); if (lane == m) v2 = s2; }
+            }
+        }
+        if (lane < M) {
+            v *= rs[lane];
+            if (a.epi == EPI_HEAD) {
+                v *= a.scale;
+                if (a.logits_dbg) a.logits_dbg[(size_t)lane * a.ld_dbg + row] = v;
+                head_merge(hs, v, 1.0f, row);
+            } else {
+                if (a.epi == EPI_SWIGLU) v = silu_f(v) * (v2 * rs[lane]);
+                if (a.epi == EPI_RESID) v += ldcg_f(a.resid + (size_t)lane * a.ldr + row);
+                xch_stf(a.out + (size_t)lane * a.ldo + row, v);
+            }
+        }
+    }
+}
 template <typename WT>
 __device__ __noinline__ void lin_simple(const LinArgs& a, Ctx& c) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int M = a.M, K = a.K;
-    const WT* W = reinterpret_cast<const WT*>(a.W);
-    const WT* W2 = reinterpret_cast<const WT*>(a.W2);
-    const bool dual = W2 != nullptr;
     char* work = c.smem + RING_OFF;
     float* xs = reinterpret_cast<float*>(work);                          // [M][K]
     float* rs = reinterpret_cast<float*>(work + SIMPLE_XS_BYTES);        // [M_MAX]
     float* wst = rs + M_MAX;                                             // [NWARPS][M_MAX][3] head stats
 
+    float4 w1[SIMPLE_PF], w2[SIMPLE_PF];
+    {
+        const int first = c.cta * NWARPS + warp;
+        const int row = min(first, a.N - 1);
+        simple_fetch<WT>(reinterpret_cast<const WT*>(a.W) + (size_t)row * K, 0, K, w1);
+        if (a.W2) simple_fetch<WT>(reinterpret_cast<const WT*>(a.W2) + (size_t)row * K, 0, K, w2);
+    }
+    cta_sync();                                          // the staging area of the operator before has been read
     for (int m = warp; m < M; m += NWARPS) {
         float ss = 0.f;
-        for (int k = lane; k < K; k += 32) {
-            float v = ldcg_f(a.x + (size_t)m * a.ldx + k);
-            ss += v * v;
-            xs[(size_t)m * K + k] = a.gain ? v * ldcg_f(a.gain + k) : v;
+        for (int k0 = 0; k0 < K; k0 += SIMPLE_PF * 128) {
+            uint4 x[SIMPLE_PF];
+            XchSpin sp; sp.spins = 0;
+            while (true) {
+                bool empty = false;
+#pragma unroll
+                for (int j = 0; j < SIMPLE_PF; ++j) {
+                    const int k = k0 + j * 128 + lane * 4;
+                    x[j] = make_uint4(0u, 0u, 0u, 0u);
+                    if (k < K) x[j] = xch_ld4(a.x + (size_t)m * a.ldx + k);
+                    empty |= xch_empty(x[j]);
+                }
+                if (!a.poll || !empty || !xch_again(c, sp, 46)) break;
+            }
+#pragma unroll
+            for (int j = 0; j < SIMPLE_PF; ++j) {
+                const int k = k0 + j * 128 + lane * 4;
+                if (k < K) {
+                    float4 v = make_float4(__uint_as_float(x[j].x), __uint_as_float(x[j].y), __uint_as_float(x[j].z), __uint_as_float(x[j].w));
+                    ss += (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+                    if (a.gain) { const float4 gv = __ldg(reinterpret_cast<const float4*>(a.gain + k)); v.x *= gv.x; v.y *= gv.y; v.z *= gv.z; v.w *= gv.w; }
+                    *reinterpret_cast<float4*>(xs + (size_t)m * K + k) = v;
+                }
+            }
         }
         ss = warp_sum(ss);
         if (lane == 0) rs[m] = a.gain ? rsqrtf(ss / (float)K + a.eps) : 1.0f;
@@ -927,41 +1104,10 @@ __device__ __noinline__ void lin_simple(const LinArgs& a, Ctx& c) {
     cta_sync();
 
     HeadStat hs; hs.zmax = 0.f; hs.sum = 0.f; hs.arg = 0;               // lane m tracks row m
-    for (long long row = (long long)c.cta * NWARPS + warp; row < a.N; row += (long long)c.nctas * NWARPS) {
-        float acc[M_MAX], acc2[M_MAX];
-#pragma unroll
-        for (int m = 0; m < M_MAX; ++m) { acc[m] = 0.f; acc2[m] = 0.f; }
-        const WT* wr = W + (size_t)row * K;
-        const WT* wr2 = dual ? W2 + (size_t)row * K : nullptr;
-        for (int k = lane; k < K; k += 32) {
-            const float w = wt_to_float<WT>(wr[k]);
-            const float w2 = dual ? wt_to_float<WT>(wr2[k]) : 0.f;
-#pragma unroll
-            for (int m = 0; m < M_MAX; ++m) {
-                if (m < M) {
-                    const float xv = xs[(size_t)m * K + k];
-                    acc[m] = fmaf(w, xv, acc[m]);
-                    if (dual) acc2[m] = fmaf(w2, xv, acc2[m]);
-                }
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < M_MAX; ++m) {
-            if (m < M) {
-                float v = warp_sum(acc[m]) * rs[m];
-                float v2 = dual ? warp_sum(acc2[m]) * rs[m] : 0.f;
-                if (a.epi == EPI_HEAD) {
-                    v *= a.scale;
-                    if (lane == 0 && a.logits_dbg) a.logits_dbg[(size_t)m * a.ld_dbg + row] = v;
-                    if (lane == m) head_merge(hs, v, 1.0f, (int)row);
-                } else if (lane == 0) {
-                    if (a.epi == EPI_SWIGLU) v = silu_f(v) * v2;
-                    if (a.epi == EPI_RESID) v += ldcg_f(a.resid + (size_t)m * a.ldr + row);
-                    a.out[(size_t)m * a.ldo + row] = v;
-                }
-            }
-        }
-    }
+    if (M == 1) simple_rows<WT, 1>(a, c, xs, rs, w1, w2, hs);
+    else if (M <= 4) simple_rows<WT, 4>(a, c, xs, rs, w1, w2, hs);
+    else if (M <= 8) simple_rows<WT, 8>(a, c, xs, rs, w1, w2, hs);
+    else simple_rows<WT, M_MAX>(a, c, xs, rs, w1, w2, hs);
     if (a.epi == EPI_HEAD) {
         if (lane < M) {
             wst[(warp * M_MAX + lane) * 3 + 0] = hs.zmax;
@@ -1029,14 +1175,36 @@ __device__ __forceinline__ void head_final_warp(const float4* part, int nctas, i
 
 // ------------------------------------------------------------------------------------ attention operator
 struct AttArgs {
-    const float* qkv;      // [M][3d] raw q, k, v rows of this pass
+    const float* qkv; int ldq;      // [M] rows of raw q, k, v of this pass
+    int poll;              // 1: q, k, v are exchange words, to be polled
     int M, pos0;           // rows sit at positions pos0 .. pos0+M-1; row i sees keys 0 .. pos0+i
     void* kc; void* vc;    // this layer's cache: [n_pages][H][page_size][hd]
-    float* out;            // [M][d]
-    unsigned char* opk;    // packed copy of out for the output projection (nullable); d * 4 bytes per row
+    float* out; int ldo;   // [M] rows of d (nullable)
+    unsigned char* opk; int ldopk;  // packed copy of out for the output projection (nullable); bytes per row
 };
 
 // The operators of one layer (or of the adapter / the LM head), prepared together.
+// N words of a row, polled until all are there
+template <int N>
+__device__ __forceinline__ void att_read(const AttArgs& a, Ctx& c, const float* const (&p)[N], float (&v)[N]) {
+    XchSpin sp; sp.spins = 0;
+    while (true) {
+        bool empty = false;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const unsigned w = xch_ld1(reinterpret_cast<const unsigned*>(p[i]));
+            v[i] = __uint_as_float(w);
+            empty |= w == XCH_EMPTY;
+        }
+        if (!a.poll || !empty || !xch_again(c, sp, 45)) return;
+    }
+}
+// One element of the output, called by whole warps whose neighbouring lanes hold neighbouring elements
+__device__ __forceinline__ void att_store(const AttArgs& a, int i, int col, float v) {
+    if (a.out) xch_stf(a.out + (size_t)i * a.ldo + col, v);
+    if (a.opk) pk_store_lane(a.opk + (size_t)i * a.ldopk, col, v);
+}
+
 struct OpTable { LinArgs lin[4]; AttArgs att; };
 static_assert(sizeof(OpTable) <= OP_TABLE_BYTES, "operator table too large");
 
@@ -1209,7 +1377,7 @@ __device__ __forceinline__ void att_warp_slice(const Dev& D, const AttArgs& a, i
 // issued before any is used, so that a batch costs one L2 round trip.
 template <int SC, int U>
 __device__ __forceinline__ void att_merge_splits(const Dev& D, const AttArgs& a, int hh, int S, int M) {
-    const int tid = threadIdx.x, H = D.dm.H, hd = D.dm.hd, d = D.dm.d;
+    const int tid = threadIdx.x, H = D.dm.H, hd = D.dm.hd;
     const int total = M * hd;
     for (int idx0 = tid; idx0 < total; idx0 += NTHREADS * U) {
         float2 mlv[U][SC];
@@ -1244,9 +1412,7 @@ __device__ __forceinline__ void att_merge_splits(const Dev& D, const AttArgs& a,
                         num += pov[u][q] * w;
                     }
                 }
-                const float ov = num / den;
-                a.out[(size_t)i * d + hh * hd + e] = ov;
-                if (a.opk) pk_store(a.opk + (size_t)i * d * 4, hh * hd + e, ov);
+                att_store(a, i, hh * hd + e, num / den);
             }
         }
     }
@@ -1259,7 +1425,7 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
     const int M = a.M, pos0 = a.pos0;
     const int T = pos0 + M;
     const int half = hd >> 1;
-    // number of KV splits: the one that leaves the fewest keys on the busiest CTA
+    // number of KV splits: the one that leaves the least work on the busiest CTA
     int S = 1;
     {
         const float inv_ctas = 1.0f / (float)c.nctas;
@@ -1268,7 +1434,8 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
         for (int sc = 1; sc <= S_CAP; ++sc) {
             const int chunk_ = (T + sc - 1) / sc;                                   // sc is a constant after unrolling
             const float waves = ceilf((float)(H * sc) * inv_ctas - 1e-4f);
-            const float cost = waves * (float)(chunk_ + 48);                        // + a fixed cost per item
+            // in steps of 64 keys (8 warps x 8 keys); an item costs about two more, the merge of a split head about three
+            const float cost = waves * (float)((chunk_ + 63) / 64 + 2 + (sc > 1 ? 3 : 0));
             if ((sc == 1 || chunk_ >= 32) && (best < 0.f || cost < best)) { best = cost; S = sc; }
         }
     }
@@ -1287,8 +1454,11 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
         // q rows: RoPE, pre-scaled by 1/sqrt(hd) (loads first: the angle arithmetic runs while they are in flight)
         for (int idx = tid; idx < M * half; idx += NTHREADS) {
             const int i = idx / half, e = idx % half;
-            const float x1 = ldcg_f(a.qkv + (size_t)i * 3 * d + hh * hd + e);
-            const float x2 = ldcg_f(a.qkv + (size_t)i * 3 * d + hh * hd + e + half);
+            const float* src = a.qkv + (size_t)i * a.ldq + hh * hd + e;
+            const float* const p[2] = {src, src + half};
+            float xv[2];
+            att_read<2>(a, c, p, xv);
+            const float x1 = xv[0], x2 = xv[1];
             float cs, sn; rope_cs(D, pos0 + i, e, cs, sn);
             qs[i * HD_MAX + e] = (x1 * cs - x2 * sn) * sc;
             qs[i * HD_MAX + e + half] = (x2 * cs + x1 * sn) * sc;
@@ -1298,9 +1468,11 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
             const int nb = max(kb, pos0), ne = ke;
             for (int idx = tid; idx < (ne - nb) * half; idx += NTHREADS) {
                 const int pos = nb + idx / half, e = idx % half, i = pos - pos0;
-                const float* src = a.qkv + (size_t)i * 3 * d + hh * hd;
-                const float k1 = ldcg_f(src + d + e), k2 = ldcg_f(src + d + e + half);
-                const float v1 = ldcg_f(src + 2 * d + e), v2 = ldcg_f(src + 2 * d + e + half);
+                const float* src = a.qkv + (size_t)i * a.ldq + hh * hd + e;
+                const float* const p[4] = {src + d, src + d + half, src + 2 * d, src + 2 * d + half};
+                float xv[4];
+                att_read<4>(a, c, p, xv);
+                const float k1 = xv[0], k2 = xv[1], v1 = xv[2], v2 = xv[3];
                 const int page = __ldg(D.page_table + (pos >> D.dm.ps_shift));
                 float cs, sn; rope_cs(D, pos, e, cs, sn);
                 const size_t base = (((size_t)page * H + hh) * ps + (pos & (ps - 1))) * hd;
@@ -1344,9 +1516,7 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
                     }
                 }
                 if (S == 1) {
-                    const float ov = num / den;
-                    a.out[(size_t)i * d + hh * hd + e] = ov;
-                    if (a.opk) pk_store(a.opk + (size_t)i * d * 4, hh * hd + e, ov);
+                    att_store(a, i, hh * hd + e, num / den);
                 } else {
                     D.att_po[(((size_t)i * H + hh) * S_CAP + s) * hd + e] = num;
                     if (e == 0) {
@@ -1578,10 +1748,11 @@ __device__ __forceinline__ void att_item(const Dev& D, const AttArgs& a, Ctx& c,
     // all six loads of an element are issued before the first is used.
     for (int idx = tid; idx < M * half; idx += NTHREADS) {
         const int i = idx / half, e = idx % half, pos = pos0 + i;
-        const float* src = a.qkv + (size_t)i * 3 * d + hh * HD + e;
-        const float q1 = ldcg_f(src), q2 = ldcg_f(src + half);
-        const float k1 = ldcg_f(src + d), k2 = ldcg_f(src + d + half);
-        const float v1 = ldcg_f(src + 2 * d), v2 = ldcg_f(src + 2 * d + half);
+        const float* src = a.qkv + (size_t)i * a.ldq + hh * HD + e;
+        const float* const p[6] = {src, src + half, src + d, src + d + half, src + 2 * d, src + 2 * d + half};
+        float xv[6];
+        att_read<6>(a, c, p, xv);
+        const float q1 = xv[0], q2 = xv[1], k1 = xv[2], k2 = xv[3], v1 = xv[4], v2 = xv[5];
         const int page = checked_page(__ldg(D.page_table + (pos >> psh)), D.dm.n_phys, D.st, 52);
         float cs, sn; rope_cs(D, pos, e, cs, sn);
         const float r1 = (q1 * cs - q2 * sn) * qscale, r2 = (q2 * cs + q1 * sn) * qscale;
@@ -1679,9 +1850,7 @@ __device__ __forceinline__ void att_item(const Dev& D, const AttArgs& a, Ctx& c,
                 }
             }
             if (S == 1) {
-                const float ov = num / den;
-                a.out[(size_t)i * d + hh * HD + e] = ov;
-                if (a.opk) pk_store(a.opk + (size_t)i * d * 4, hh * HD + e, ov);
+                att_store(a, i, hh * HD + e, num / den);
             } else {
                 D.att_po[(((size_t)i * H + hh) * S_CAP + s) * HD + e] = num;
                 if (e == 0) {

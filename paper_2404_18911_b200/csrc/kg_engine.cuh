@@ -1,7 +1,7 @@
 // The persistent decode kernel: one cooperative grid (one CTA per SM) runs whole phases of the
 // method - prefill chunks, the draft loop with its on-device exit test, the verify pass, the
-// prefix accept / rollback, or many rounds back to back - with grid barriers between dependent
-// operators and no host involvement.
+// prefix accept / rollback, or many rounds back to back - with exchanges or grid barriers between
+// dependent operators and no host involvement.
 //
 // Every thread of every CTA walks the same operator sequence and holds the same copy of the
 // sequence state.  The consumer warps do the arithmetic and take part in the grid barriers; the
@@ -51,7 +51,17 @@ struct Engine {
         if constexpr (PROD) __syncwarp();    // the lanes have left the previous operator before lane 0 rewrites the table
         return reinterpret_cast<OpTable*>(PROD ? c.ctl->tab_prod : c.ctl->tab_cons);
     }
-    __device__ __forceinline__ bool writer() const { return PROD ? (threadIdx.x & 31) == 0 : threadIdx.x == 0; }
+    // the one thread that writes part `part` of the table: one of another warp for every part, so that they write side by side
+    // (the producer warp, which reads little of the table, has one writer)
+    __device__ __forceinline__ bool writer(int part = 0) const { return PROD ? (threadIdx.x & 31) == 0 : (int)threadIdx.x == 32 * part; }
+    // operator on the weights [N, K] with M rows: all that the producer reads of a LinArgs
+    __device__ __forceinline__ void shape(LinArgs& a, const void* W, const void* W2, int N, int K, int M) const {
+        a.W = W; a.W2 = W2; a.N = N; a.K = K; a.M = M;
+        if constexpr (!PROD) {
+            a.eps = D.dm.eps; a.gain = nullptr; a.ssq_in = nullptr; a.poll = 0; a.resid = nullptr; a.out = nullptr;
+            a.pk[0] = PkOut{nullptr, nullptr}; a.pk[1] = PkOut{nullptr, nullptr}; a.ssq_out = nullptr;
+        }
+    }
     __device__ __forceinline__ bool linear(const LinArgs* a, bool publish) {
         if constexpr (PROD) return linear_producer(a, c, streamed(), publish);
         else return linear_consumer<WT>(a, c, streamed(), publish);
@@ -89,69 +99,109 @@ struct Engine {
         }
         LinArgs a{};
         a.N = d; a.M = M; a.out = D.h; a.ldo = d;
-        a.pk[0] = PkOut{D.layers[0].g1, D.hA_pk}; a.ldpk_out = (int)ldpk(); a.ssq_out = D.ssq_hA;
+        a.pk[0] = PkOut{D.layers[0].g1, D.hA_pk}; a.ldpk_out = (int)ldpk(); a.ssq_out = D.ssq_hA; a.ld_sout = c.nctas;
         emit_plain_rows(a, c, [&](int m, int e) {
             const int tok = safe_token(toks_global ? __ldcg(toks_global + m) : tok_single);
             return wt_to_float<WT>(E[(size_t)tok * d + e]);
         });
     }
 
-    // Arguments of the attention block of layer / adapter `li` on M rows at pos0: [0] q, k, v and [1] the output
-    // projection with its residual, plus the attention itself.
-    __device__ __forceinline__ void fill_attention_block(OpTable* t, const LayerW& lw, int li, int M, int pos0, const ActIn& in,
-                                                         float* o_out, const PkOut& o_pk, float* o_ssq) {
+    // ---- exchange buffers of a layer (see the exchange words in kg_device.cuh)
+    int xp;                 // instance the next layer uses
+    int xused;              // rows of the other instance, the one of the layer before, that hold data
+    __device__ __forceinline__ unsigned* xrow(int off) const { return D.xch[xp] + off; }
+    __device__ __forceinline__ int x_attn() const { return 3 * D.dm.d; }
+    __device__ __forceinline__ int x_h() const { return 4 * D.dm.d; }
+    __device__ __forceinline__ int x_act() const { return 5 * D.dm.d; }
+    __device__ __forceinline__ int x_ssq() const { return 5 * D.dm.d + D.dm.F; }
+    __device__ __forceinline__ void empty_instance(int p) {
+        const int n4 = xused * (D.xch_ld >> 2);
+        uint4* q = reinterpret_cast<uint4*>(D.xch[p]);
+        for (int i = c.cta * NTHREADS + threadIdx.x; i < n4; i += c.nctas * NTHREADS) q[i] = make_uint4(XCH_EMPTY, XCH_EMPTY, XCH_EMPTY, XCH_EMPTY);
+    }
+    // after the attention of a layer: the instance of the layer before is emptied, this one belongs to M rows (not earlier: the
+    // merge of attention's splits releases what this CTA has stored so far)
+    __device__ __forceinline__ void turn_instance(int M) {
+        if constexpr (!PROD) { empty_instance(xp ^ 1); xused = M; xp ^= 1; }
+    }
+
+    // Arguments of the attention block of layer / adapter `li` on M rows at pos0: [0] q, k, v, the attention itself and [1] the
+    // output projection with its residual (where it goes is left to the caller, who fills in the rest with the same writer).
+    __device__ __forceinline__ void fill_attention_block(OpTable* t, const LayerW& lw, int li, int M, int pos0, const ActIn& in) {
         const Dims& dm = D.dm;
-        LinArgs& q = t->lin[0];
-        q = LinArgs{};
-        q.M = M; q.eps = dm.eps;
-        q.W = lw.wqkv; q.N = 3 * dm.d; q.K = dm.d;
-        q.x = in.x; q.ldx = dm.d; q.gain = lw.g1; q.xpk = in.pk; q.ldpk = (int)ldpk(); q.ssq_in = in.ssq;
-        q.epi = EPI_STORE; q.out = D.qkv; q.ldo = 3 * dm.d;
-        AttArgs& at = t->att;
-        at.qkv = D.qkv; at.M = M; at.pos0 = pos0;
-        at.kc = reinterpret_cast<WT*>(D.kcache) + (size_t)li * cache_layer_stride();
-        at.vc = reinterpret_cast<WT*>(D.vcache) + (size_t)li * cache_layer_stride();
-        at.out = D.attn; at.opk = streamed() ? D.attn_pk : nullptr;
-        LinArgs& o = t->lin[1];
-        o = LinArgs{};
-        o.M = M; o.eps = dm.eps;
-        o.W = lw.wo; o.N = dm.d; o.K = dm.d; o.x = D.attn; o.ldx = dm.d;
-        o.xpk = D.attn_pk; o.ldpk = (int)ldpk();
-        o.epi = EPI_RESID; o.resid = in.x; o.ldr = dm.d; o.out = o_out; o.ldo = dm.d;
-        o.pk[0] = o_pk; o.ldpk_out = (int)ldpk(); o.ssq_out = o_ssq;
+        if (writer(0)) {
+            LinArgs& q = t->lin[0];
+            shape(q, lw.wqkv, nullptr, 3 * dm.d, dm.d, M);
+            if constexpr (!PROD) {
+                q.x = in.x; q.ldx = dm.d; q.gain = lw.g1; q.xpk = in.pk; q.ldpk = (int)ldpk(); q.ssq_in = in.ssq; q.ld_ssq = c.nctas;
+                q.epi = EPI_STORE; q.out = reinterpret_cast<float*>(xrow(0)); q.ldo = D.xch_ld;
+            }
+        }
+        if constexpr (!PROD) {
+            if (writer(1)) {
+                AttArgs& at = t->att;
+                at.qkv = reinterpret_cast<const float*>(xrow(0)); at.ldq = D.xch_ld; at.poll = 1; at.M = M; at.pos0 = pos0;
+                at.kc = reinterpret_cast<WT*>(D.kcache) + (size_t)li * cache_layer_stride();
+                at.vc = reinterpret_cast<WT*>(D.vcache) + (size_t)li * cache_layer_stride();
+                at.out = streamed() ? nullptr : reinterpret_cast<float*>(xrow(x_attn())); at.ldo = D.xch_ld;
+                at.opk = streamed() ? reinterpret_cast<unsigned char*>(xrow(x_attn())) : nullptr; at.ldopk = D.xch_ld * 4;
+            }
+        }
+        if (writer(2)) {
+            LinArgs& o = t->lin[1];
+            shape(o, lw.wo, nullptr, dm.d, dm.d, M);
+            if constexpr (!PROD) {
+                o.x = reinterpret_cast<const float*>(xrow(x_attn())); o.ldx = D.xch_ld;
+                o.xpk = reinterpret_cast<const unsigned char*>(xrow(x_attn())); o.ldpk = D.xch_ld * 4; o.poll = 1;
+                o.epi = EPI_RESID; o.resid = in.x; o.ldr = dm.d;
+            }
+        }
     }
 
     // One decoder block on M rows at positions pos0.. (Section 3.1's M^b layers):
     //   h  = x + Wo Attn(RMSNorm(x; g1));   out = h + Wdown(SiLU(Wgate n) * Wup n), n = RMSNorm(h; g2)
+    // The rows between its operators are exchange words; one grid barrier ends the layer.
     __device__ bool run_layer(int li, int M, int pos0, const ActIn& in, const ActOut& out) {
         const Dims& dm = D.dm;
         OpTable* t = table();
-        if (writer()) {
-            const LayerW lw = D.layers[li];
-            fill_attention_block(t, lw, li, M, pos0, in, D.h, PkOut{lw.g2, D.hB_pk}, D.ssq_hB);
+        const LayerW& lw = D.layers[li];
+        // the residual stream after attention: fp32 rows of each CTA's own features, packed rows for everybody (plain path:
+        // fp32 exchange rows for both)
+        float* hx = reinterpret_cast<float*>(xrow(x_h()));
+        fill_attention_block(t, lw, li, M, pos0, in);
+        if constexpr (!PROD) {
+            if (writer(2)) {
+                LinArgs& o = t->lin[1];
+                o.out = streamed() ? D.h : hx; o.ldo = streamed() ? dm.d : D.xch_ld;
+                o.pk[0] = PkOut{lw.g2, reinterpret_cast<unsigned char*>(hx)}; o.ldpk_out = D.xch_ld * 4;
+                o.ssq_out = reinterpret_cast<float*>(xrow(x_ssq())); o.ld_sout = D.xch_ld;
+            }
+        }
+        if (writer(3)) {
             LinArgs& gu = t->lin[2];
-            gu = LinArgs{};
-            gu.M = M; gu.eps = dm.eps;
-            gu.W = lw.wgate; gu.W2 = lw.wup; gu.N = dm.F; gu.K = dm.d; gu.x = D.h; gu.ldx = dm.d; gu.gain = lw.g2;
-            gu.xpk = D.hB_pk; gu.ldpk = (int)ldpk(); gu.ssq_in = D.ssq_hB;
-            gu.epi = EPI_SWIGLU; gu.out = D.act; gu.ldo = dm.F;
-            gu.pk[0] = PkOut{nullptr, D.act_pk}; gu.ldpk_out = dm.F * 4;
+            shape(gu, lw.wgate, lw.wup, dm.F, dm.d, M);
+            if constexpr (!PROD) {
+                gu.x = hx; gu.ldx = D.xch_ld; gu.gain = lw.g2; gu.xpk = reinterpret_cast<const unsigned char*>(hx); gu.ldpk = D.xch_ld * 4;
+                gu.ssq_in = reinterpret_cast<const float*>(xrow(x_ssq())); gu.ld_ssq = D.xch_ld; gu.poll = 1;
+                gu.epi = EPI_SWIGLU; gu.out = streamed() ? nullptr : reinterpret_cast<float*>(xrow(x_act())); gu.ldo = D.xch_ld;
+                gu.pk[0] = PkOut{nullptr, reinterpret_cast<unsigned char*>(xrow(x_act()))}; gu.ldpk_out = D.xch_ld * 4;
+            }
+        }
+        if (writer(4)) {
             LinArgs& dn = t->lin[3];
-            dn = LinArgs{};
-            dn.M = M; dn.eps = dm.eps;
-            dn.W = lw.wdown; dn.N = dm.d; dn.K = dm.F; dn.x = D.act; dn.ldx = dm.F;
-            dn.xpk = D.act_pk; dn.ldpk = dm.F * 4;
-            dn.epi = EPI_RESID; dn.resid = D.h; dn.ldr = dm.d; dn.out = out.x; dn.ldo = dm.d;
-            dn.pk[0] = out.pk[0]; dn.pk[1] = out.pk[1]; dn.ldpk_out = (int)ldpk(); dn.ssq_out = out.ssq;
+            shape(dn, lw.wdown, nullptr, dm.d, dm.F, M);
+            if constexpr (!PROD) {
+                dn.x = reinterpret_cast<const float*>(xrow(x_act())); dn.ldx = D.xch_ld;
+                dn.xpk = reinterpret_cast<const unsigned char*>(xrow(x_act())); dn.ldpk = D.xch_ld * 4; dn.poll = 1;
+                dn.epi = EPI_RESID; dn.resid = streamed() ? D.h : hx; dn.ldr = streamed() ? dm.d : D.xch_ld; dn.out = out.x; dn.ldo = dm.d;
+                dn.pk[0] = out.pk[0]; dn.pk[1] = out.pk[1]; dn.ldpk_out = (int)ldpk(); dn.ssq_out = out.ssq; dn.ld_sout = c.nctas;
+            }
         }
         if (!linear(&t->lin[0], true)) return false;
-        KG_SYNC(10);
         attention(&t->att);
-        KG_SYNC(11);
+        turn_instance(M);
         if (!linear(&t->lin[1], false)) return false;
-        KG_SYNC(12);
         if (!linear(&t->lin[2], false)) return false;
-        KG_SYNC(13);
         if (!linear(&t->lin[3], false)) return false;
         KG_SYNC(14);
         return true;
@@ -162,16 +212,19 @@ struct Engine {
     __device__ bool run_adapter(int M, int pos0, const ActIn& in, bool want_out) {
         const Dims& dm = D.dm;
         OpTable* t = table();
-        if (writer()) {
-            const LayerW lw = D.layers[dm.L];
-            fill_attention_block(t, lw, dm.L, M, pos0, in, D.abuf, PkOut{lw.g2, D.abuf_pk}, D.ssq_abuf);
+        const LayerW& lw = D.layers[dm.L];
+        fill_attention_block(t, lw, dm.L, M, pos0, in);
+        if constexpr (!PROD) {
+            if (writer(2)) {
+                LinArgs& o = t->lin[1];
+                o.out = D.abuf; o.ldo = dm.d;
+                o.pk[0] = PkOut{lw.g2, D.abuf_pk}; o.ldpk_out = (int)ldpk(); o.ssq_out = D.ssq_abuf; o.ld_sout = c.nctas;
+            }
         }
         if (!linear(&t->lin[0], true)) return false;
-        KG_SYNC(20);
         attention(&t->att);
-        KG_SYNC(21);
-        if (!want_out) return true;
-        if (!linear(&t->lin[1], false)) return false;
+        turn_instance(M);
+        if (want_out && !linear(&t->lin[1], false)) return false;
         KG_SYNC(22);
         return true;
     }
@@ -184,12 +237,12 @@ struct Engine {
         OpTable* t = table();
         if (writer()) {
             LinArgs& a = t->lin[0];
-            a = LinArgs{};
-            a.M = M; a.eps = dm.eps;
-            a.W = D.head; a.N = dm.V; a.K = dm.d; a.x = in.x; a.ldx = dm.d; a.gain = gain;
-            a.xpk = in.pk; a.ldpk = (int)ldpk(); a.ssq_in = in.ssq;
-            a.epi = EPI_HEAD; a.scale = dm.logit_scale; a.head_part = D.head_part;
-            a.logits_dbg = dm.debug ? dbg : nullptr; a.ld_dbg = dm.V;
+            shape(a, D.head, nullptr, dm.V, dm.d, M);
+            if constexpr (!PROD) {
+                a.x = in.x; a.ldx = dm.d; a.gain = gain; a.xpk = in.pk; a.ldpk = (int)ldpk(); a.ssq_in = in.ssq; a.ld_ssq = c.nctas;
+                a.epi = EPI_HEAD; a.scale = dm.logit_scale; a.head_part = D.head_part;
+                a.logits_dbg = dm.debug ? dbg : nullptr; a.ld_dbg = dm.V;
+            }
         }
         if (!linear(&t->lin[0], true)) return false;
         if constexpr (PROD) {
@@ -391,8 +444,10 @@ struct Engine {
         // the plain path streams nothing: its producer warp has no part in the launch
         if (PROD && !streamed()) return;
         load_state();
+        xp = 0; xused = 0;                       // a launch finds both exchange instances empty and leaves them so
         const bool ok = run_program();
         if (!ok && PROD) ring_drain(c);
+        if constexpr (!PROD) { if (ok) empty_instance(xp ^ 1); }
     }
 };
 
