@@ -97,9 +97,9 @@ struct Layout {
     size_t off_hApk, off_featApk, off_featDpk, off_abufpk, off_ssqA, off_ssqF, off_ssqAb, off_xch[2], xch_bytes;
     int xch_ld;
     size_t off_layers, off_pt, off_kc, off_vc, off_h, off_feat, off_abuf, off_po, off_ml,
-        off_cnt, off_hp, off_dbgd, off_dbgv, off_out, off_S, off_rlog, off_prompt, off_st, off_bar;
+        off_cnt, off_xp, xp_bytes, off_rope, off_hp, off_dbgd, off_dbgv, off_out, off_S, off_rlog, off_prompt, off_st, off_bar;
     // tensor-core prompt pass (0 bytes each when the shape cannot take it)
-    size_t off_pf_h, off_pf_x, off_pf_q, off_pf_f, off_pf_rs, off_pf_cs, off_pf_part, off_pf_cnt, off_pf_err;
+    size_t off_pf_h, off_pf_x, off_pf_q, off_pf_f, off_pf_rs, off_pf_part, off_pf_cnt, off_pf_err;
     size_t pf_rows, pf_part_bytes;
     size_t off_embed, off_head, off_gfinal;
     std::vector<size_t> off_w[5];     // wqkv, wo, wgate, wup, wdown
@@ -166,6 +166,9 @@ Layout make_layout(const kg_config* c, int own_weights, int nctas) {
     L.off_po = take(4 * (size_t)KG_M_MAX * H * S_CAP * hd);
     L.off_ml = take(4 * (size_t)KG_M_MAX * H * S_CAP * 2);
     L.off_cnt = take(4 * H);
+    L.xp_bytes = c->dtype == KG_BF16 ? 4 * (size_t)KG_M_MAX * H * S_CAP * (hd + 4) : 0;
+    L.off_xp = take(L.xp_bytes);
+    L.off_rope = take(c->dtype == KG_BF16 ? 4 * (size_t)(c->max_seq + KG_M_MAX) * hd : 0);
     L.off_hp = take(sizeof(float4) * (size_t)nctas * KG_M_MAX);
     L.off_dbgd = take(c->debug_logits ? 4 * (size_t)KG_M_MAX * V : 0);
     L.off_dbgv = take(c->debug_logits ? 4 * (size_t)KG_M_MAX * V : 0);
@@ -179,7 +182,7 @@ Layout make_layout(const kg_config* c, int own_weights, int nctas) {
         L.pf_rows = R;
         L.pf_part_bytes = R ? (size_t)nctas * GM_TM * GM_NT_MAX * 4 : 0;
         L.off_pf_h = take(4 * R * d); L.off_pf_x = take(4 * R * d); L.off_pf_q = take(4 * R * d); L.off_pf_f = take(4 * R * F);
-        L.off_pf_rs = take(4 * R); L.off_pf_cs = take(4 * R * hd); L.off_pf_part = take(L.pf_part_bytes);
+        L.off_pf_rs = take(4 * R); L.off_pf_part = take(L.pf_part_bytes);
         L.off_pf_cnt = take(R ? 4 * (size_t)nctas : 0); L.off_pf_err = take(R ? 64 : 0);
     }
     for (int k = 0; k < 5; ++k) L.off_w[k].assign(nl + 1, 0);
@@ -330,6 +333,8 @@ namespace {
 int prefill_tc(kg_model* m, int n);                 // the tensor-core prompt pass (end of this file)
 bool prefill_tc_ok(const kg_model* m, int n);
 int prefill_tc_init(kg_model* m);
+bool make_tmap(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t K, int box_rows);
+int tmap_failed();
 }
 
 template <typename WT>
@@ -480,6 +485,17 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     }
     ok = ok && cudaMemcpyAsync(P(lay.off_pt), pt.data(), sizeof(int) * pt.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
     ok = ok && cudaMemsetAsync(D.st, 0, sizeof(State), s) == cudaSuccess;
+    if (bf) {
+        D.att_xp = (unsigned*)P(lay.off_xp);
+        ok = ok && cudaMemsetAsync(D.att_xp, 0xff, lay.xp_bytes, s) == cudaSuccess;      // XCH_EMPTY
+        rope_table_kernel<<<cfg->max_seq + KG_M_MAX, cfg->head_dim / 2, 0, s>>>(D, (float2*)P(lay.off_rope));
+        D.rope = (const float2*)P(lay.off_rope);
+        ok = ok && cudaGetLastError() == cudaSuccess;
+        const uint64_t rows = (uint64_t)(cfg->n_layers + 1) * D.dm.n_pages * cfg->n_heads * cfg->page_size;
+        const int box = cfg->page_size < 16 ? cfg->page_size : 16;
+        D.dm.ring = D.dm.stream && (cfg->head_dim == 64 || cfg->head_dim == 128) && rows < (1ull << 31) &&
+                    make_tmap(&D.tmk, D.kcache, rows, cfg->head_dim, box) && make_tmap(&D.tmv, D.vcache, rows, cfg->head_dim, box);
+    }
     for (int i = 0; i < 2; ++i) ok = ok && cudaMemsetAsync(D.xch[i], 0xff, lay.xch_bytes, s) == cudaSuccess;      // XCH_EMPTY
     ok = ok && cudaMemsetAsync(D.att_cnt, 0, 4 * cfg->n_heads, s) == cudaSuccess;
     ok = ok && cudaStreamSynchronize(s) == cudaSuccess;    // pt / layers_host are host temporaries
@@ -871,7 +887,7 @@ namespace {
 constexpr int OP_K_MAX = 32768;               // longest input row the single-operator entry points pack into scratch
 constexpr size_t OP_GEMM_PART = 16u << 20;    // partial sums of the GEMM's cut tiles
 constexpr int OP_GEMM_CNT = 1024;             // their arrival counters, then the error word
-struct OpScratch { size_t off_hp, off_po, off_ml, off_cnt, off_pt, off_xpk, off_ssq, off_gemm, off_gcnt, total; };
+struct OpScratch { size_t off_hp, off_po, off_ml, off_cnt, off_xp, off_xpk, off_ssq, off_gemm, off_gcnt, total; };
 OpScratch op_layout() {
     OpScratch s; size_t o = 0;
     auto take = [&](size_t b) { size_t r = o; o = align_up(o + b, 256); return r; };
@@ -879,6 +895,7 @@ OpScratch op_layout() {
     s.off_po = take(4 * (size_t)KG_M_MAX * S_CAP * 8192);
     s.off_ml = take(4 * (size_t)KG_M_MAX * 256 * S_CAP * 2);
     s.off_cnt = take(4 * 256);
+    s.off_xp = take(4 * (size_t)KG_M_MAX * S_CAP * (8192 + 4 * 256));
     s.off_xpk = take(4 * (size_t)KG_M_MAX * OP_K_MAX);
     s.off_ssq = take(4 * (size_t)KG_M_MAX * 1024);
     s.off_gemm = take(OP_GEMM_PART);
@@ -888,15 +905,13 @@ OpScratch op_layout() {
 }
 
 template <typename WT>
-__global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(LinArgs a, int stream) {
+__global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(const __grid_constant__ LinArgs a, int stream) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
-    OpTable* t = reinterpret_cast<OpTable*>(c.producer ? c.ctl->tab_prod : c.ctl->tab_cons);
-    if (c.producer ? (threadIdx.x & 31) == 0 : threadIdx.x == 0) t->lin[0] = a;
     // launched while the kernel that packs the rows may still run: the copy warp starts on the weights at once
     grid_dependents_launch();
     if (!c.producer) grid_dependency_wait();
-    const bool ok = linear_op<WT>(&t->lin[0], c, stream != 0, true);
+    const bool ok = linear_op<WT>(a, c, stream != 0);
     if (!ok && c.producer) ring_drain(c);
 }
 // one warp per row (one thread per row took 60 us: a chain of a merge per CTA)
@@ -912,10 +927,10 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
     if (!c.producer) {
-        OpTable* t = reinterpret_cast<OpTable*>(c.ctl->tab_cons);
-        if (threadIdx.x == 0) t->att = a;
-        cta_sync();
-        attention_op<WT>(D, &t->att, c);
+        if (D.dm.ring) a.plan = ra_plan(a.pos0, D.dm.H, c.nctas);
+        attention_op<WT>(D, a, c, D.dm.ring != 0);
+    } else if (D.dm.ring) {
+        if (!attention_producer(D, ra_plan(a.pos0, D.dm.H, c.nctas), 0, c)) ring_drain(c);
     }
 }
 
@@ -1079,13 +1094,21 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     std::memset(&D, 0, sizeof(D));
     D.dm.H = H; D.dm.hd = hd; D.dm.d = H * hd; D.dm.page_size = page_size; D.dm.theta = theta;
     D.dm.n_pages = (pos0 + M + page_size - 1) / page_size;       // entries of page_table this call may touch
-    D.dm.n_phys = 0x7fffffff;                                    // the caller's cache: its page count is not known here
+    D.dm.n_phys = 0x7fffffff / (H * page_size);                  // the caller's cache: its page count is not known here
     for (D.dm.ps_shift = 0; (1 << D.dm.ps_shift) < page_size; ++D.dm.ps_shift) {}
     for (int i = 0; i < hd / 2; ++i) D.inv_freq[i] = std::pow((double)theta, -2.0 * (double)i / (double)hd);
     D.page_table = page_table;
     D.att_po = (float*)((char*)scratch + sc.off_po); D.att_ml = (float*)((char*)scratch + sc.off_ml);
     D.att_cnt = (unsigned*)((char*)scratch + sc.off_cnt);
-    CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
+    D.dm.ring = dtype == KG_BF16 && hd != 32;
+    if (D.dm.ring) {
+        const int box = page_size < 16 ? page_size : 16;
+        if (!make_tmap(&D.tmk, kc, 0x7fffffff, hd, box) || !make_tmap(&D.tmv, vc, 0x7fffffff, hd, box)) return tmap_failed();
+        D.att_xp = (unsigned*)((char*)scratch + sc.off_xp);
+        CK(cudaMemsetAsync(D.att_xp, 0xff, 4 * (size_t)M * H * S_CAP * (hd + 4), s));      // XCH_EMPTY
+    } else {
+        CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
+    }
     AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
     if (dtype == KG_BF16) {
@@ -1239,7 +1262,6 @@ int prefill_tc(kg_model* m, int n) {
     WT* qh = (WT*)(A + m->lay.off_pf_q); WT* ql = qh + R * d;
     WT* fh = (WT*)(A + m->lay.off_pf_f); WT* fl = fh + R * F;
     float* rs = (float*)(A + m->lay.off_pf_rs);                     // 1/rms of the rows the planes were made from
-    float2* cs = (float2*)(A + m->lay.off_pf_cs);
     int* err = (int*)(A + m->lay.off_pf_err);
     const int pairs = m->nctas / 2;
     CK(cudaMemsetAsync(err, 0, 4, s));
@@ -1251,14 +1273,13 @@ int prefill_tc(kg_model* m, int n) {
         const int rows = n - b0 < brows ? n - b0 : brows;
         last = rows - 1;
         pf_embed_kernel<<<rows, 256, 0, s>>>(D.prompt + b0, (const WT*)D.embed, c.vocab, d, h);
-        pf_rope_table_kernel<<<rows, hd / 2, 0, s>>>(D, b0, cs);
         GemmArgs base{};
         base.rows = rows; base.err = err; base.part = (float*)(A + m->lay.off_pf_part); base.cnt = (unsigned*)(A + m->lay.off_pf_cnt);
         auto norm = [&](const float* gain) { pf_norm_split_kernel<<<rows, PF_EW_THREADS, 0, s>>>(h, d, d, gain, c.rms_eps, xh, xl, rs); };
         auto qkv = [&](const CUtensorMap& w, int li, int sec0) {
             GemmArgs g = base;
             g.N = (3 - sec0) * d; g.K = d; g.rowscale = rs; g.hi = qh; g.lo = ql; g.ldp = d; g.hd = hd; g.H = H; g.sec0 = sec0; g.pos0 = b0;
-            g.cs = cs; g.page_table = D.page_table; g.ps_shift = D.dm.ps_shift; g.n_phys = D.dm.n_phys; g.st = D.st;
+            g.cs = D.rope + (size_t)b0 * (hd / 2); g.page_table = D.page_table; g.ps_shift = D.dm.ps_shift; g.n_phys = D.dm.n_phys; g.st = D.st;
             g.kc = (WT*)D.kcache + (size_t)li * lstride; g.vc = (WT*)D.vcache + (size_t)li * lstride;
             g.qscale = 1.4426950408889634f / std::sqrt((float)hd);
             gm_plan(g, (g.N + GM_TM - 1) / GM_TM, pairs, m->lay.pf_part_bytes);

@@ -15,6 +15,7 @@
 // activation rows (activations split into bf16 hi + lo so that the product keeps fp32 accuracy).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -25,13 +26,13 @@ constexpr int M_MAX = 16;          // rows per pass
 constexpr int NTHREADS = 256;      // consumer threads per CTA
 constexpr int NWARPS = NTHREADS / 32;
 constexpr int BLOCK_THREADS = NTHREADS + 32;   // + the producer warp (warp index NWARPS)
-// The decode kernel is launched with a whole warpgroup behind the consumers (warp NWARPS is the producer, the other
-// three leave at once): registers are handed out per warpgroup, and the producer's warpgroup gives most of its share
-// to the two consumer warpgroups at kernel start (setmaxnreg).  The pool is what the launch allocated: 384 threads x
-// 168 registers = 64512; a request beyond it would block forever, so the budgets below are checked against it.
+// The decode kernel is launched with a whole warpgroup behind the consumers (warp NWARPS copies, the next one is the sequencer, two
+// leave at once): registers are handed out per warpgroup, and that warpgroup gives most of its share to the two consumer
+// warpgroups at kernel start (setmaxnreg).  The pool is what the launch allocated: 384 threads x 168 registers = 64512; a
+// request beyond it would block forever, so the budgets below are checked against it.
 constexpr int DECODE_THREADS = NTHREADS + 128;
 constexpr int LAUNCH_REGS = 168;                  // 65536 / 384, rounded down to the allocation unit of 8
-constexpr int CONSUMER_REGS = 216, PRODUCER_REGS = 56;
+constexpr int CONSUMER_REGS = 216, PRODUCER_REGS = 72;
 static_assert(NTHREADS * CONSUMER_REGS + 128 * PRODUCER_REGS <= DECODE_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
 static_assert(DECODE_THREADS * (LAUNCH_REGS + 8) > 65536, "LAUNCH_REGS is not what a launch of DECODE_THREADS threads gets");
 constexpr int S_CAP = 16;          // most KV splits per head
@@ -45,7 +46,7 @@ constexpr int ST_K = 2048;
 constexpr int ST_ROW_BYTES = ST_K * 2 + 16;
 constexpr int SLOT_BYTES = ST_ROWS * ST_ROW_BYTES;
 constexpr int CTRL_BYTES = 3072;
-constexpr int OP_TABLE_BYTES = 1024;                    // struct OpTable: the operator arguments of one layer
+constexpr int QUEUE = 8;                                // operators in the queue: more than one layer's
 constexpr int RING_OFF = CTRL_BYTES;
 constexpr int WORK_OFF = RING_OFF + RING * SLOT_BYTES;
 constexpr int SMEM_TOTAL = 232448;                      // 227 KB, the most one CTA may own
@@ -72,6 +73,7 @@ struct Dims {
     int max_seq, page_size, n_pages, gamma_max, debug;
     int n_phys;         // physical pages behind the page table (page numbers must lie below it)
     int ps_shift;       // log2(page_size): page sizes are powers of two
+    int ring;           // 1: attention reads K / V tiles from the weight ring (streamed path, bf16 cache, head_dim 64 / 128)
     int stream;         // 1: linear operators take the streamed tensor-core path (bf16, d and F multiples of 16)
 };
 
@@ -96,6 +98,8 @@ struct State {
 };
 
 struct Dev {
+    alignas(64) CUtensorMap tmk;   // the K and V caches as [rows][hd], in boxes of up to 16 rows x 64 dims (dm.ring)
+    alignas(64) CUtensorMap tmv;
     Dims dm;
     const void* embed; const void* head; const float* g_final;
     const LayerW* layers;          // [L+1], index L = adapter
@@ -119,6 +123,8 @@ struct Dev {
     float* att_po;                 // [M_MAX][H][S_CAP][hd] split partial outputs
     float* att_ml;                 // [M_MAX][H][S_CAP][2]  split partial (max, sum)
     unsigned* att_cnt;             // [H] arrival counters
+    unsigned* att_xp;              // ring attention: [M_MAX][H][S_CAP][hd + 4] split partials as exchange words (empty between uses)
+    const float2* rope;            // [max_seq][hd / 2] cos, sin (null: computed where needed)
     float4* head_part;             // [nctas][M_MAX] (zmax, sumexp, argmax bits, -)
     float* dbg_draft; float* dbg_verify;   // [M_MAX][V] each (debug only)
     int* out_tokens; int* S; int* round_log;   // [max_seq], [max_seq], [max_seq][4]
@@ -128,26 +134,7 @@ struct Dev {
     double inv_freq[HD_MAX / 2];   // theta^(-2i/hd)
 };
 
-// Per-CTA control block at the start of shared memory.
-struct Ctrl {
-    unsigned long long full[RING];     // producer -> consumers: slot filled (transaction count)
-    unsigned long long empty[RING];    // consumers -> producer: slot drained (one arrival per consumer warp)
-    unsigned long long mail;           // consumers -> producer: head_tok / head_p hold a new result
-    int abort;                         // a bounded wait of this CTA gave up
-    int sync_ok;
-    int att_last;
-    int head_tok[M_MAX];
-    float head_p[M_MAX];
-    // operator arguments of a whole layer (struct OpTable), written once per layer by one thread of each role and
-    // read by all of its threads (kept here rather than on the per-thread stack, which the small L1 left beside
-    // 227 KB of shared memory cannot hold)
-    alignas(16) unsigned char tab_cons[OP_TABLE_BYTES];
-    alignas(16) unsigned char tab_prod[OP_TABLE_BYTES];
-    // the per-role context (struct Ctx): one copy for the consumers, one for the producer warp
-    alignas(16) unsigned char ctx_cons[128];
-    alignas(16) unsigned char ctx_prod[128];
-};
-static_assert(sizeof(Ctrl) <= CTRL_BYTES - 16, "control block too large");
+struct Ctrl;
 
 // State of one role (consumers / producer warp) of the CTA.  It lives in shared memory: every thread of the role
 // holds the same values, updates are the same in all of them, and between operators they are ordered by the
@@ -161,11 +148,74 @@ struct Ctx {
     char* smem;
     Ctrl* ctl;
     bool grid;                     // false: single-operator test kernel, grid barriers are CTA barriers
-    bool producer;                 // this thread belongs to the producer warp
+    bool producer;                 // this thread belongs to the copy warp
+    int backoff;                   // nanoseconds to sleep between two polls of a shared-memory barrier
     int slot; unsigned phase;      // ring cursor of this thread's role
     unsigned issued;               // producer: stages issued so far
     unsigned mail_phase;           // producer: parity of the next result it waits for
 };
+
+// ------------------------------------------------------------------------------------ operators
+struct PkOut { const float* gain; unsigned char* ptr; };   // packed copy of output rows; gain == null: unscaled
+
+struct LinArgs {
+    const void* W; const void* W2;   // [N, K]; W2 != null: SwiGLU pair (gate, up)
+    int N, K;
+    int M;                           // activation rows
+    const float* x; int ldx;         // plain path: fp32 rows (written earlier in this kernel)
+    const float* gain; float eps;    // RMSNorm gain of the input (null: no norm)
+    const unsigned char* xpk; int ldpk;   // streamed path: packed rows, already multiplied by the gain; bytes per row
+    const float* ssq_in; int ld_ssq; // streamed path with norm: [M] rows of nctas partial sums of squares of the input rows
+    int poll;                        // 1: the input rows and their sums are exchange words, to be polled
+    const float* resid; int ldr;     // EPI_RESID
+    float* out; int ldo;             // fp32 output rows (streamed path: nullable)
+    int epi;
+    float scale;                     // EPI_HEAD: logit scale
+    float4* head_part;               // EPI_HEAD: [nctas][M_MAX]
+    float* logits_dbg; int ld_dbg;   // EPI_HEAD, optional
+    PkOut pk[2]; int ldpk_out;       // streamed path: packed copies of the output rows for the operators that read them
+    float* ssq_out; int ld_sout;     // streamed path: [M] rows of nctas partial sums of squares of the output rows (nullable)
+};
+
+// Cut of a head's old key tiles into splits (ra_plan); pos: the position it was made for
+struct RaPlan { int ntile, S, chunk; int pos; };
+struct AttArgs {
+    RaPlan plan; int row0; // ring attention: cut into splits; first row of this layer's cache in the tensor maps
+    const float* qkv; int ldq;      // [M] rows of raw q, k, v of this pass
+    int poll;              // 1: q, k, v are exchange words, to be polled
+    int M, pos0;           // rows sit at positions pos0 .. pos0+M-1; row i sees keys 0 .. pos0+i
+    void* kc; void* vc;    // this layer's cache: [n_pages][H][page_size][hd]
+    float* out; int ldo;   // [M] rows of d (nullable)
+    unsigned char* opk; int ldopk;  // packed copy of out for the output projection (nullable); bytes per row
+};
+struct EmbedArgs { const int* toks; int tok, M; };        // toks == null: the one token `tok`
+
+enum { OPK_NONE = 0, OPK_LIN = 1, OPK_ATT = 2, OPK_EMBED = 3, OPK_HEAD = 4, OPK_MAIL = 5, OPK_KEEP = 6, OPK_EXIT = 7 };
+// One operator in the queue of the decode kernel.
+struct Op {
+    int kind;
+    int sync;                        // != 0: a grid barrier follows (and this is where it says it timed out)
+    int empty_p, empty_rows;         // OPK_ATT, OPK_EXIT: rows of this exchange instance are emptied afterwards
+    union { LinArgs lin; AttArgs att; EmbedArgs emb; };
+};
+
+// Per-CTA control block at the start of shared memory.
+struct Ctrl {
+    unsigned long long full[RING];     // producer -> consumers: slot filled (transaction count)
+    unsigned long long empty[RING];    // consumers -> producer: slot drained (one arrival per consumer warp)
+    unsigned long long mail;           // consumers -> sequencer: head_tok / head_p hold a new result
+    int abort;                         // a bounded wait of this CTA gave up
+    int sync_ok;
+    int att_last;
+    int head_tok[M_MAX];
+    float head_p[M_MAX];
+    unsigned long long qfull[QUEUE];   // sequencer -> copy warp, consumers: operator written
+    unsigned long long qempty[QUEUE];  // copy warp, consumer warps -> sequencer: operator done
+    Op queue[QUEUE];
+    // the per-role context (struct Ctx): one copy for the consumers, one for the copy warp, one for the sequencer
+    alignas(16) unsigned char ctx[3][128];
+};
+static_assert(sizeof(Ctrl) <= CTRL_BYTES - 16, "control block too large");
 
 // ------------------------------------------------------------------------------------ helpers
 
@@ -179,6 +229,10 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 __device__ __forceinline__ float ldcg_f(const float* p) { return __ldcg(p); }
 __device__ __forceinline__ float2 ldcg_f2(const float* p) { return __ldcg(reinterpret_cast<const float2*>(p)); }
 __device__ __forceinline__ float4 ldcg_f4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
+
+// The thread index, read anew by every operator: the operators are inlined into one loop, and what is computed from an index that
+// the compiler knows to be the same every time round would be kept, and spilled, across all of them.
+__device__ __forceinline__ int tid_here() { int t; asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t)); return t; }
 
 // barrier among the consumer warps only (the producer warp never takes part)
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NTHREADS) : "memory"); }
@@ -229,8 +283,8 @@ __device__ __forceinline__ bool mbar_wait(Ctx& c, unsigned long long* bar, unsig
     const long long t0 = clock64();
     unsigned spins = 0;
     while (!mbar_try_wait(bar, parity)) {
-        // the producer warp shares an issue port with two consumer warps: it backs off instead of spinning
-        if (c.producer) __nanosleep(200);
+        // the copy warp and the sequencer share issue ports with consumer warps: they back off instead of spinning
+        if (c.backoff) __nanosleep(c.backoff);
         if (((++spins) & 63u) == 0u) {
             if (*(volatile int*)&c.ctl->abort) return false;
             if ((unsigned long long)(clock64() - t0) > c.wait_clk) { record_timeout(c, where); return false; }
@@ -291,17 +345,18 @@ __device__ __forceinline__ Ctx& ctx_init(char* smem, State* st, unsigned* bar, b
                                          unsigned long long wait_clk = WAIT_TIMEOUT_CLK, int skip_arrival = 0) {
     static_assert(sizeof(Ctx) <= 128, "context slot too small");
     Ctrl* ctl = reinterpret_cast<Ctrl*>(smem);
-    const bool producer = threadIdx.x >= NTHREADS;
-    Ctx& c = *reinterpret_cast<Ctx*>(producer ? ctl->ctx_prod : ctl->ctx_cons);
-    if (threadIdx.x == 0 || threadIdx.x == NTHREADS) {
+    const int role = threadIdx.x < NTHREADS ? 0 : (threadIdx.x < NTHREADS + 32 ? 1 : 2);       // consumers, copy warp, sequencer
+    Ctx& c = *reinterpret_cast<Ctx*>(ctl->ctx[role]);
+    if (threadIdx.x == 0 || threadIdx.x == NTHREADS || threadIdx.x == NTHREADS + 32) {
         c.cta = blockIdx.x; c.nctas = gridDim.x; c.bar_target = 0; c.st = st; c.bar = bar; c.smem = smem;
         c.wait_clk = wait_clk; c.skip_arrival = skip_arrival;
         c.ctl = ctl; c.grid = grid;
-        c.producer = producer;
+        c.producer = role == 1; c.backoff = role == 0 ? 0 : (role == 1 ? 200 : 40);
         c.slot = 0; c.phase = 0; c.issued = 0; c.mail_phase = 0;
     }
     if (threadIdx.x == 0) {
         for (int i = 0; i < RING; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], NWARPS); }
+        for (int i = 0; i < QUEUE; ++i) { mbar_init(&ctl->qfull[i], 1); mbar_init(&ctl->qempty[i], NWARPS + 1); }
         mbar_init(&ctl->mail, 1);
         ctl->abort = 0; ctl->sync_ok = 1; ctl->att_last = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -369,6 +424,7 @@ __device__ __forceinline__ uint4 xch_ld4(const void* p) {
     return v;
 }
 __device__ __forceinline__ void xch_st(unsigned* p, unsigned v) { asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ void xch_st4(void* p, uint4 v) { asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory"); }
 __device__ __forceinline__ void xch_stf(float* p, float v) { xch_st(reinterpret_cast<unsigned*>(p), __float_as_uint(v)); }
 __device__ __forceinline__ bool xch_empty(const uint2& v) { return v.x == XCH_EMPTY || v.y == XCH_EMPTY; }
 __device__ __forceinline__ bool xch_empty(const uint4& v) { return v.x == XCH_EMPTY || v.y == XCH_EMPTY || v.z == XCH_EMPTY || v.w == XCH_EMPTY; }
@@ -402,7 +458,6 @@ __device__ __forceinline__ void rope_cs(const Dev& D, int pos, int i, float& cs,
 // (elements k, k+1) with x * gain = hi + lo.  This is the B operand fragment order of the MMA, so a
 // consumer lane fetches its fragments with plain 8- or 16-byte loads.  The operator that produces a
 // row writes it once, in this form, for the operator that reads it.
-struct PkOut { const float* gain; unsigned char* ptr; };   // gain == null: unscaled
 
 // byte offset of the hi half of element k inside a packed row; the lo half sits 8 bytes further
 __device__ __forceinline__ size_t pk_off(int k) {
@@ -431,24 +486,6 @@ __device__ __forceinline__ void pk_store_lane(unsigned char* row, int k, float v
     if (!(k & 1)) pk_store2(row, k, v, o);
 }
 
-struct LinArgs {
-    const void* W; const void* W2;   // [N, K]; W2 != null: SwiGLU pair (gate, up)
-    int N, K;
-    int M;                           // activation rows
-    const float* x; int ldx;         // plain path: fp32 rows (written earlier in this kernel)
-    const float* gain; float eps;    // RMSNorm gain of the input (null: no norm)
-    const unsigned char* xpk; int ldpk;   // streamed path: packed rows, already multiplied by the gain; bytes per row
-    const float* ssq_in; int ld_ssq; // streamed path with norm: [M] rows of nctas partial sums of squares of the input rows
-    int poll;                        // 1: the input rows and their sums are exchange words, to be polled
-    const float* resid; int ldr;     // EPI_RESID
-    float* out; int ldo;             // fp32 output rows (streamed path: nullable)
-    int epi;
-    float scale;                     // EPI_HEAD: logit scale
-    float4* head_part;               // EPI_HEAD: [nctas][M_MAX]
-    float* logits_dbg; int ld_dbg;   // EPI_HEAD, optional
-    PkOut pk[2]; int ldpk_out;       // streamed path: packed copies of the output rows for the operators that read them
-    float* ssq_out; int ld_sout;     // streamed path: [M] rows of nctas partial sums of squares of the output rows (nullable)
-};
 
 __device__ __forceinline__ float silu_f(float v) { return v / (1.0f + expf(-v)); }
 
@@ -608,7 +645,7 @@ __device__ __forceinline__ void cp_async4(void* dst_smem, const void* src) {
 // accumulates over superchunks.
 template <int MP>
 __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const float* acc_s, int sc0, int nu, bool prefetched, float& ssq_acc) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = tid_here(), lane = tid & 31, warp = tid >> 5;
     const int M = a.M;
     const float* rs = wk + LW_RS;
     float* ssw = wk + LW_SSW;
@@ -660,10 +697,10 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const flo
 __device__ __forceinline__ int sum_shift(int M) { return M <= 1 ? 8 : (M <= 2 ? 7 : (M <= 4 ? 6 : (M <= 8 ? 5 : 4))); }
 
 template <int V>
-__device__ __noinline__ void lin_consume(const LinArgs& a, Ctx& c) {
+__device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     using G = LinGeom<V>;
     constexpr int NS = G::NS, FR = G::FR, NACC = G::NACC, MP = G::MP;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = tid_here(), lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int M = a.M, K = a.K;
     const bool dual = a.W2 != nullptr;
@@ -1126,30 +1163,16 @@ __device__ __noinline__ void lin_simple(const LinArgs& a, Ctx& c) {
     cta_sync();
 }
 
-// One linear operator, called by every thread of the CTA; `stream` selects the streamed tensor-core
-// path (bf16 weights, every K a multiple of 16; decided once per model so that the packed activation
-// rows exist wherever they are read).  Consumers return after their part; whether the grid must stop
-// is learnt at the next grid barrier.  The producer returns false when one of its waits gave up.
+// One linear operator, called by every thread of the CTA of a single-operator kernel; `stream` selects the streamed tensor-core
+// path (bf16 weights, every K a multiple of 16).  The copy warp returns false when one of its waits gave up.
 template <typename WT>
-__device__ __forceinline__ bool linear_consumer(const LinArgs* sa, Ctx& c, bool stream, bool publish) {
-    if (publish) cta_sync();
-    if (stream) {
-        if (sa->M <= 4) lin_consume<4>(*sa, c); else if (sa->M <= 8) lin_consume<8>(*sa, c);
-        else if (sa->M <= 12) lin_consume<12>(*sa, c); else lin_consume<16>(*sa, c);
-    } else {
-        lin_simple<WT>(*sa, c);
+__device__ __forceinline__ bool linear_op(const LinArgs& a, Ctx& c, bool stream) {
+    if (c.producer) return !stream || lin_produce(a, c);
+    if (!stream) { lin_simple<WT>(a, c); return true; }
+    if constexpr (sizeof(WT) == 2) {
+        if (a.M <= 4) lin_consume<4>(a, c); else if (a.M <= 8) lin_consume<8>(a, c); else if (a.M <= 12) lin_consume<12>(a, c); else lin_consume<16>(a, c);
     }
     return true;
-}
-__device__ __forceinline__ bool linear_producer(const LinArgs* sa, Ctx& c, bool stream, bool publish) {
-    if (!stream) return true;
-    if (publish) __syncwarp();
-    return lin_produce(*sa, c);
-}
-template <typename WT>
-__device__ __forceinline__ bool linear_op(const LinArgs* sa, Ctx& c, bool stream, bool publish) {
-    // sa points into this role's operator table in shared memory; publish: the table was written just before
-    return c.producer ? linear_producer(sa, c, stream, publish) : linear_consumer<WT>(sa, c, stream, publish);
 }
 
 // Merge the per-CTA head partials of row m by a whole warp (identical result in every CTA): every lane merges the partials of CTAs lane, lane + 32, ... (independent loads, one
@@ -1174,16 +1197,31 @@ __device__ __forceinline__ void head_final_warp(const float4* part, int nctas, i
 }
 
 // ------------------------------------------------------------------------------------ attention operator
-struct AttArgs {
-    const float* qkv; int ldq;      // [M] rows of raw q, k, v of this pass
-    int poll;              // 1: q, k, v are exchange words, to be polled
-    int M, pos0;           // rows sit at positions pos0 .. pos0+M-1; row i sees keys 0 .. pos0+i
-    void* kc; void* vc;    // this layer's cache: [n_pages][H][page_size][hd]
-    float* out; int ldo;   // [M] rows of d (nullable)
-    unsigned char* opk; int ldopk;  // packed copy of out for the output projection (nullable); bytes per row
-};
+constexpr int ATT_TK = 16;                                 // keys per tile
+// Cut of a head's old tiles into splits, the same for the copy warp and the consumers.  The cost of a split count, in steps of
+// one tile per warp (about 0.5 us): the tiles of an item (one step per 8 tiles, and at least the time an SM's share of the HBM
+// bandwidth takes for them, 0.4 steps a tile), two steps of fixed work, three more for the merge of a head that is split.
+// (Made once per position and not per layer: the 16 candidates took 2.4 us a layer in a rolled loop with divisions.)
+__device__ __noinline__ RaPlan ra_plan(int pos0, int H, int nctas) {
+    RaPlan p;
+    p.ntile = (pos0 + ATT_TK - 1) / ATT_TK;
+    p.S = 1;
+    const float inv_ctas = 1.0f / (float)nctas;
+    float best = 0.f;
+    p.pos = pos0;
+#pragma unroll
+    for (int sc = 1; sc <= S_CAP; ++sc) {                  // (constant divisors)
+        const int ch = (p.ntile + sc - 1) / sc;
+        const float waves = ceilf((float)(H * sc) * inv_ctas - 1e-4f);
+        const float cost = waves * (fmaxf((float)((ch + NWARPS - 1) / NWARPS), 0.4f * (float)ch) + 2.f + (sc > 1 ? 3.f : 0.f));
+        if (sc == 1 || (sc <= p.ntile && cost < best)) { best = cost; p.S = sc; }
+    }
+    p.chunk = max(1, (p.ntile + p.S - 1) / p.S);
+    p.S = max(1, (p.ntile + p.chunk - 1) / p.chunk);       // no split without tiles
+    return p;
+}
 
-// The operators of one layer (or of the adapter / the LM head), prepared together.
+
 // N words of a row, polled until all are there
 template <int N>
 __device__ __forceinline__ void att_read(const AttArgs& a, Ctx& c, const float* const (&p)[N], float (&v)[N]) {
@@ -1205,8 +1243,6 @@ __device__ __forceinline__ void att_store(const AttArgs& a, int i, int col, floa
     if (a.opk) pk_store_lane(a.opk + (size_t)i * a.ldopk, col, v);
 }
 
-struct OpTable { LinArgs lin[4]; AttArgs att; };
-static_assert(sizeof(OpTable) <= OP_TABLE_BYTES, "operator table too large");
 
 // Consumer threads only.  One work item = (head, KV split); the eight warps of the CTA cut the item's
 // key range into eight slices and run an online-softmax pass over their slice without any CTA
@@ -1550,63 +1586,49 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
 
 // ---- tensor-core attention (bf16 cache, head_dim 64 or 128) ----------------------------------------------------
 //
-// One pass over the keys for all rows of the pass.  The unit of work is a tile of 16 keys and one group of 8 rows
-// (with more than 8 rows, two units take the same tiles, one row group each: the tile's second reader finds it in
-// L2, so K and V still leave HBM once).  A unit is one warp when head_dim is 64; with head_dim 128 it is a pair of
-// warps that own 64 dims each, which keeps a warp's share of K, V and the output small enough to hold two tiles in
-// registers.  Everything a tile needs travels global memory -> registers -> tensor core:
-//   S = K Q^T   m16n8k16, keys on the M side, rows on the N side.  A lane loads 16 bytes (8 dims) of two key rows;
-//               which dims sit at which k position of the instruction does not matter for a dot product as long as
-//               the Q fragment (read from shared memory, rotated, pre-scaled, split into bf16 hi + lo) uses the same
-//               assignment, so no transposition is needed.  The two warps of a pair add their halves of the dot
-//               products through shared memory (one named barrier per tile); both then hold the same scores.
-//   online softmax in the log2 domain on the accumulator fragment (a lane holds 2 keys x 2 rows; the row maximum is
-//               a butterfly over the 8 lanes that share the rows; the row sum is reduced once, at the end).
-//   O^T = V^T P^T   m16n8k16, dims on the M side, keys on the contraction side.  A lane loads 16 bytes of four key
-//               rows and pairs equal dims of two keys with byte permutes; P (bf16 hi + lo) moves from the accumulator
-//               layout into the B layout with movmatrix.  The M position -> key assignment of the first product is
-//               chosen so that this transposition lands every key where the permuted V fragment expects it.
+// One work item = (head, KV split).  The keys before this pass travel through the weight ring: the copy warp brings tiles of
+// 16 keys (K and V, 64-dim boxes with the 128-byte swizzle) into the slots between the stages of W_qkv and W_o.  They do not
+// depend on this pass, so they are on their way while q, k and v are still being formed; with loads into registers a tile cost
+// a DRAM latency and one tile per warp was in flight (2.3 TB/s on long caches).  The rows of this pass are one more tile, which
+// the last split of a head forms in shared memory from q, k, v and appends to the cache.
+//
+// A warp takes whole tiles (tile j of an item: warp j mod 8):
+//   S = K Q^T      m16n8k16, keys on the M side (ldmatrix), rows on the N side (fragments in shared memory, rotated, pre-scaled by
+//                  log2(e) / sqrt(hd), split into bf16 hi + lo)
+//   online softmax in the log2 domain on the accumulator fragment (a lane holds 2 keys x 2 rows)
+//   O^T = V^T P^T  dims on the M side (ldmatrix.trans), keys on the contraction side; P (hi + lo) moves from the accumulator
+//                  layout into the B layout with movmatrix.
+// With more than 8 rows a warp does both groups of 8 rows (R = 2) on the same K and V fragments.
+//
+// Splits of a head: all but the last one leave (max, sum, o) in exchange words, the last one polls them, merges in split order
+// and empties the words again (their next use lies behind the barrier at the layer's end).  It waits for items of lower number
+// only, and every CTA takes its items in rising order, so there is always one that can go on.
 __device__ __forceinline__ unsigned movmatrix_trans(unsigned a) {
     unsigned d;
     asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
     return d;
 }
-__device__ __forceinline__ void mma_bf16_16816r(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+__device__ __forceinline__ void ldmatrix_x4_trans(unsigned (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
-// barrier among the two warps of a pair (ids 2 .. 5; 0 is the whole CTA, 1 the consumer warps)
-__device__ __forceinline__ void pair_sync(int pair) { asm volatile("bar.sync %0, 64;" ::"r"(2 + pair) : "memory"); }
+__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const CUtensorMap* tmap, int x, int y, uint32_t bar_smem) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst_smem), "l"(tmap), "r"(x), "r"(y), "r"(bar_smem) : "memory");
+}
 
-constexpr int ATT_TK = 16;                  // keys per tile
-constexpr int ATT_DW = 64;                  // dims per warp
-struct AttK { uint4 k[2][2]; };             // raw K bits of a tile: key rows mu(g), mu(g) + 2; 8 dims of each 32-dim block
-struct AttV { uint4 v[4]; };                // raw V bits of a tile: key rows 4t .. 4t+3; dims 8g .. 8g+7 of the warp's 64
-struct AttAcc {                             // running state of a unit's rows: lane (g, t) tracks rows 2t, 2t+1
-    float o[4][4];                          // O^T tile e: [0],[1]: dim 8g + 2e, rows 2t, 2t+1; [2],[3]: dim 8g + 2e + 1
-    float m[2], l[2];                       // running maximum (log2 domain) and this lane's share of the running sum
+template <int HD> struct RaGeom {
+    static constexpr int HALF_BYTES = ATT_TK * HD * 2;     // K (or V) of a tile: HD / 64 boxes of 16 rows x 128 bytes
+    static constexpr int TILE_BYTES = 2 * HALF_BYTES;
+    static constexpr int TPS = 32768 / TILE_BYTES;         // tiles per ring slot: 4 or 8
+    static constexpr int QG = HD / 16 * 512;               // Q fragments of 8 rows: {hi b0, b1, lo b0, b1} per lane and k16-step
+    static constexpr int NT_OFF = 8192;                    // the tile of this pass's rows; afterwards the merge buffer
+    static constexpr int MB_OFF = NT_OFF;                  // [warps][ATT_RB][ROW] floats
+    static constexpr int ROW = HD + 4;                     // a row of partial results: o [HD], maximum, sum, padding
 };
-struct AttP { unsigned bh[2], bl[2]; float cf[2]; };    // a tile's probabilities in the B layout (bf16 hi, lo), rescale factors
+static_assert(2 * RaGeom<128>::QG <= RaGeom<128>::NT_OFF && RaGeom<128>::TPS * RaGeom<128>::TILE_BYTES <= SLOT_BYTES, "attention tiles");
+static_assert(RaGeom<128>::MB_OFF + NWARPS * ATT_RB * RaGeom<128>::ROW * 4 <= WORK_BYTES && WORK_OFF % 128 == 0 && SLOT_BYTES % 128 == 0, "attention buffers");
 
-template <int HD> struct AttSm {
-    static constexpr int QS = HD * 2 + 64;                      // bytes per Q row (padded: two rows per shared-memory phase)
-    static constexpr int Q_BYTES = 2 * M_MAX * QS;              // hi plane, lo plane
-    static constexpr int MB_OFF = (Q_BYTES + 15) / 16 * 16;     // merge buffer [units][ATT_RB][ATT_MB_STRIDE] floats; while the
-                                                                // tiles run, the pairs' score exchange [4][2][2][32] float4
-};
-
-// Page-table entries of a window of 32 pages, one per lane; a lane asks for the page of a key by shuffle.
-struct PageWin {
-    int first, pgs;
-    __device__ __forceinline__ void load(const int* page_table, int n_pages, int first_page) {
-        first = first_page;
-        pgs = __ldg(page_table + min(first_page + (int)(threadIdx.x & 31), n_pages - 1));
-    }
-    // every lane calls this with its own key; the keys of one call lie within [first, first + 32) pages
-    __device__ __forceinline__ int page_of(int key, int psh) const { return __shfl_sync(0xffffffffu, pgs, (key >> psh) - first); }
-};
-
-// kc / vc point at the warp's first dim of the head (element offset hh * HD + dim offset is added by the caller per row)
 // A page number outside the cache never becomes an address: the access goes to page 0 and the state word records it.
 __device__ __forceinline__ int checked_page(int pg, int n_pages, State* st, int where) {
     if ((unsigned)pg < (unsigned)n_pages) return pg;
@@ -1614,313 +1636,372 @@ __device__ __forceinline__ int checked_page(int pg, int n_pages, State* st, int 
     return 0;
 }
 
+// Copy warp: the old K / V tiles of this CTA's items.  row0: first row of this layer's cache in the tensor maps.
 template <int HD>
-__device__ __forceinline__ void att_load(AttK& tk, AttV& tv, const __nv_bfloat16* kc, const __nv_bfloat16* vc, const PageWin& pw,
-                                         int H, int hh, int dof, int psh, int psm, int key0, int last_key, int n_pages, State* st) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int mu = 4 * (g >> 1) + (g & 1);
+__device__ __noinline__ bool att_produce(const Dev& D, const RaPlan pl, int row0, Ctx& c) {
+    using G = RaGeom<HD>;
+    const int lane = threadIdx.x & 31;
+    const int H = D.dm.H, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
+    const int bsh = min(psh, 4), per = (HD / 64 * 2) << (4 - bsh);        // a box holds 2^bsh keys; boxes per tile
+    // the rows were written with ordinary stores (by earlier passes, ordered before this point by a grid barrier)
+    asm volatile("fence.proxy.async;" ::: "memory");
+    int slot = c.slot; unsigned phase = c.phase, issued = c.issued;
+    bool ok = true;
+    for (int item = c.cta; item < H * pl.S && ok; item += c.nctas) {
+        const int hh = item / pl.S, tb = item % pl.S * pl.chunk, nt = min(pl.ntile, tb + pl.chunk) - tb;
+        for (int t0 = 0; t0 < nt; t0 += G::TPS) {
+            const int n = min(G::TPS, nt - t0);
+            int w = 1;
+            if (lane == 0) w = mbar_wait(c, &c.ctl->empty[slot], phase ^ 1u, 47) ? 1 : 0;
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (!w) { ok = false; break; }
+            if (lane == 0) mbar_arrive_expect_tx(&c.ctl->full[slot], (unsigned)(n * G::TILE_BYTES));
+            __syncwarp();
+            const uint32_t dst = smem_u32(c.smem + RING_OFF + (size_t)slot * SLOT_BYTES), bar = smem_u32(&c.ctl->full[slot]);
+            for (int op = lane; op < n * per; op += 32) {
+                const int j = op / per, r = op - j * per;
+                const int kv = r & 1, half = HD == 128 ? (r >> 1) & 1 : 0, b = HD == 128 ? r >> 2 : r >> 1;
+                const int key = (tb + t0 + j) * ATT_TK + (b << bsh);
+                const int page = checked_page(__ldg(D.page_table + min(key >> psh, D.dm.n_pages - 1)), D.dm.n_phys, D.st, 51);
+                tma_load_2d(dst + (uint32_t)(j * G::TILE_BYTES + kv * G::HALF_BYTES + half * 2048 + (b << (bsh + 7))), kv ? &D.tmv : &D.tmk,
+                            half * 64, row0 + ((page * H + hh) << psh) + (key & psm), bar);
+            }
+            issued++;
+            if (++slot == RING) { slot = 0; phase ^= 1u; }
+        }
+    }
+    c.slot = slot; c.phase = phase; c.issued = issued;
+    return ok;
+}
+
+// shared-memory address of the 16-byte chunk `ch` of row `row` of a tile's K or V at `base`
+__device__ __forceinline__ uint32_t ra_addr(uint32_t base, int row, int ch) {
+    const uint32_t ra = base + (uint32_t)((ch >> 3) * 2048 + row * 128);
+    return ra + (((uint32_t)ch ^ (ra >> 7)) & 7u) * 16u;
+}
+
+// One tile: keys 0 .. nv - 1 of it are valid; causal: key i is seen by rows >= i only (the tile of this pass's rows).
+template <int HD, int R>
+__device__ __forceinline__ void ra_tile(uint32_t kb, uint32_t vb, uint32_t qf, int nv, bool causal, float (&o)[R][HD / 16][4],
+                                        float (&mx)[R][2], float (&l)[R][2]) {
+    const int lane = tid_here() & 31, g = lane >> 2, t = lane & 3;
+    // hi of even and odd k16-steps, lo: the tensor core truncates at every accumulation, so that chains stay at HD / 32 steps
+    // where it counts (lo is 2^-9 of the sum)
+    float sc[R][3][4];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int key = min(key0 + mu + 2 * r, last_key);
-        const int pg = checked_page(pw.page_of(key, psh), n_pages, st, 50);
-        const __nv_bfloat16* row = kc + ((((size_t)pg * H + hh) << psh) + (key & psm)) * HD + dof + 8 * t;
-        tk.k[r][0] = __ldcg(reinterpret_cast<const uint4*>(row));
-        tk.k[r][1] = __ldcg(reinterpret_cast<const uint4*>(row + 32));
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sc[r][0][i] = sc[r][1][i] = sc[r][2][i] = 0.f;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int key = min(key0 + 4 * t + i, last_key);
-        const int pg = checked_page(pw.page_of(key, psh), n_pages, st, 51);
-        const __nv_bfloat16* row = vc + ((((size_t)pg * H + hh) << psh) + (key & psm)) * HD + dof + 8 * g;
-        tv.v[i] = __ldcg(reinterpret_cast<const uint4*>(row));
+    for (int k = 0; k < HD / 16; ++k) {
+        unsigned a[4];
+        ldmatrix_x4(a, ra_addr(kb, lane & 15, k * 2 + (lane >> 4)));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            uint4 q;
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "r"(qf + (uint32_t)(r * RaGeom<HD>::QG + (k * 32 + lane) * 16)));
+            mma_bf16_16816(sc[r][k & 1], a, q.x, q.y);
+            mma_bf16_16816(sc[r][2], a, q.z, q.w);
+        }
+    }
+    unsigned bh[R][2], bl[R][2];
+    float cf[R][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float s[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s[i] = (sc[r][0][i] + sc[r][1][i]) + sc[r][2][i];
+            const int key = g + (i >> 1) * 8, row = r * 8 + 2 * t + (i & 1);
+            if (key >= nv || (causal && key > row)) s[i] = -INFINITY;
+        }
+        float p[4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float m = fmaxf(s[i], s[2 + i]);
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+            const float mn = fmaxf(mx[r][i], m);
+            cf[r][i] = mx[r][i] == -INFINITY ? 0.f : ex2f(mx[r][i] - mn);
+            p[i] = s[i] == -INFINITY ? 0.f : ex2f(s[i] - mn);
+            p[2 + i] = s[2 + i] == -INFINITY ? 0.f : ex2f(s[2 + i] - mn);
+            l[r][i] = l[r][i] * cf[r][i] + (p[i] + p[2 + i]);
+            mx[r][i] = mn;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            unsigned hi, lo;
+            split_hi_lo(make_float2(p[2 * q], p[2 * q + 1]), hi, lo);
+            bh[r][q] = movmatrix_trans(hi);
+            bl[r][q] = movmatrix_trans(lo);
+        }
+    }
+    // V rows past the valid keys hold anything (0 * NaN would be NaN)
+    const unsigned vm0 = (2 * t < nv ? 0xffffu : 0u) | (2 * t + 1 < nv ? 0xffff0000u : 0u);
+    const unsigned vm1 = (2 * t + 8 < nv ? 0xffffu : 0u) | (2 * t + 9 < nv ? 0xffff0000u : 0u);
+#pragma unroll
+    for (int d = 0; d < HD / 16; ++d) {
+        unsigned v[4];
+        ldmatrix_x4_trans(v, ra_addr(vb, (lane & 7) + (lane >> 4) * 8, d * 2 + ((lane >> 3) & 1)));
+        if (nv < ATT_TK) { v[0] &= vm0; v[1] &= vm0; v[2] &= vm1; v[3] &= vm1; }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            o[r][d][0] *= cf[r][0]; o[r][d][1] *= cf[r][1]; o[r][d][2] *= cf[r][0]; o[r][d][3] *= cf[r][1];
+            mma_bf16_16816(o[r][d], v, bh[r][0], bh[r][1]);
+            mma_bf16_16816(o[r][d], v, bl[r][0], bl[r][1]);
+        }
     }
 }
 
-// This warp's 64 dims of S = K Q^T for one tile: sc[0], sc[1]: key key0 + mu(g), rows 2t, 2t+1; sc[2], sc[3]: key + 2.
-// qw: shared-memory address of the hi plane at this warp's first dim; row stride QS, lo plane M_MAX rows further.
-template <int QS>
-__device__ __forceinline__ void att_scores(const AttK& tk, float (&sc)[4], uint32_t qw, int row0) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const uint32_t qh = qw + (uint32_t)((row0 + g) * QS + 16 * t);
-    const uint32_t ql = qh + (uint32_t)(M_MAX * QS);
-    sc[0] = sc[1] = sc[2] = sc[3] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        uint4 h, l;
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(h.x), "=r"(h.y), "=r"(h.z), "=r"(h.w) : "r"(qh + 64u * j));
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(l.x), "=r"(l.y), "=r"(l.z), "=r"(l.w) : "r"(ql + 64u * j));
-        mma_bf16_16816r(sc, tk.k[0][j].x, tk.k[1][j].x, tk.k[0][j].y, tk.k[1][j].y, h.x, h.y);
-        mma_bf16_16816r(sc, tk.k[0][j].x, tk.k[1][j].x, tk.k[0][j].y, tk.k[1][j].y, l.x, l.y);
-        mma_bf16_16816r(sc, tk.k[0][j].z, tk.k[1][j].z, tk.k[0][j].w, tk.k[1][j].w, h.z, h.w);
-        mma_bf16_16816r(sc, tk.k[0][j].z, tk.k[1][j].z, tk.k[0][j].w, tk.k[1][j].w, l.z, l.w);
-    }
+__device__ __forceinline__ void rope_at(const Dev& D, int pos, int e, int half, float& cs, float& sn) {
+    if (D.rope) { const float2 v = __ldg(D.rope + (size_t)pos * half + e); cs = v.x; sn = v.y; }
+    else rope_cs(D, pos, e, cs, sn);
 }
 
-// Masking, online-softmax update and the probabilities of a tile in the layout the second product reads.
-__device__ __forceinline__ void att_softmax(float (&sc)[4], AttAcc& ac, AttP& pp, int row0, int key0, int ke, int pos0) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int ka = key0 + 4 * (g >> 1) + (g & 1), kb2 = ka + 2;
-    const int lim0 = pos0 + row0 + 2 * t, lim1 = lim0 + 1;            // last key rows 2t / 2t+1 may see
-    if (ka >= ke || ka > lim0) sc[0] = -INFINITY;
-    if (ka >= ke || ka > lim1) sc[1] = -INFINITY;
-    if (kb2 >= ke || kb2 > lim0) sc[2] = -INFINITY;
-    if (kb2 >= ke || kb2 > lim1) sc[3] = -INFINITY;
-    float p[4];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        float mx = fmaxf(sc[r], sc[2 + r]);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-        const float mn = fmaxf(ac.m[r], mx);
-        pp.cf[r] = (ac.m[r] == -INFINITY) ? 0.f : ex2f(ac.m[r] - mn);
-        p[r] = (sc[r] == -INFINITY) ? 0.f : ex2f(sc[r] - mn);
-        p[2 + r] = (sc[2 + r] == -INFINITY) ? 0.f : ex2f(sc[2 + r] - mn);
-        ac.l[r] = ac.l[r] * pp.cf[r] + (p[r] + p[2 + r]);
-        ac.m[r] = mn;
-    }
-    // P as bf16 hi + lo, moved into the B layout: b0 = keys 4t, 4t+1 of row g; b1 = keys 4t+2, 4t+3
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        unsigned hi, lo;
-        split_hi_lo(make_float2(p[2 * q], p[2 * q + 1]), hi, lo);
-        pp.bh[q] = movmatrix_trans(hi);
-        pp.bl[q] = movmatrix_trans(lo);
-    }
-}
-
-// O^T += V^T P^T on this warp's 64 dims
-__device__ __forceinline__ void att_accumulate(const AttV& tv, AttAcc& ac, const AttP& pp) {
-    const unsigned w0[4] = {tv.v[0].x, tv.v[0].y, tv.v[0].z, tv.v[0].w};
-    const unsigned w1[4] = {tv.v[1].x, tv.v[1].y, tv.v[1].z, tv.v[1].w};
-    const unsigned w2[4] = {tv.v[2].x, tv.v[2].y, tv.v[2].z, tv.v[2].w};
-    const unsigned w3[4] = {tv.v[3].x, tv.v[3].y, tv.v[3].z, tv.v[3].w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        // dims 8g + 2e (M rows 0-7 of the instruction) and + 1 (M rows 8-15); keys (4t, 4t+1) then (4t+2, 4t+3)
-        const unsigned a0 = __byte_perm(w0[e], w1[e], 0x5410), a1 = __byte_perm(w0[e], w1[e], 0x7632);
-        const unsigned a2 = __byte_perm(w2[e], w3[e], 0x5410), a3 = __byte_perm(w2[e], w3[e], 0x7632);
-        float (&o)[4] = ac.o[e];
-        o[0] *= pp.cf[0]; o[1] *= pp.cf[1]; o[2] *= pp.cf[0]; o[3] *= pp.cf[1];
-        mma_bf16_16816r(o, a0, a1, a2, a3, pp.bh[0], pp.bh[1]);
-        mma_bf16_16816r(o, a0, a1, a2, a3, pp.bl[0], pp.bl[1]);
-    }
-}
-
-// One work item of the tensor-core attention: head hh, split s of S (chunk_tiles tiles each) of the keys 0 .. pos0 + M - 1
-// for the rows of `a`.  This pass's K / V rows are rotated, rounded and written to the cache by the item whose key range
-// holds them.
-template <int HD>
-__device__ __forceinline__ void att_item(const Dev& D, const AttArgs& a, Ctx& c, int hh, int s, int S, int chunk_tiles) {
+template <int HD, int R>
+__device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, Ctx& c) {
     typedef __nv_bfloat16 WT;
-    constexpr int NSPLIT = HD / ATT_DW;               // warps per unit: 1 (head_dim 64) or 2 (head_dim 128)
-    constexpr int NUNITS = NWARPS / NSPLIT;
+    using G = RaGeom<HD>;
     constexpr int half = HD / 2;
-    constexpr int QS = AttSm<HD>::QS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3;
+    const int tid = tid_here(), lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const int H = D.dm.H, d = D.dm.d, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
     const int M = a.M, pos0 = a.pos0;
-    const int T = pos0 + M;
-    const int ntiles_all = (T + ATT_TK - 1) / ATT_TK;
-    const int R = (M + 7) >> 3;                       // row groups of 8
-    const int nw = NUNITS / R;                        // units that share the tiles of an item (a power of two)
-    const int tpw = (chunk_tiles + nw - 1) / nw;
+    const RaPlan pl = a.plan;
     const float qscale = rsqrtf((float)HD) * 1.4426950408889634f;      // 1/sqrt(hd) and log2(e)
-    WT* kc = reinterpret_cast<WT*>(a.kc);
-    WT* vc = reinterpret_cast<WT*>(a.vc);
-    unsigned char* qs = reinterpret_cast<unsigned char*>(c.smem + WORK_OFF);
-    float* mb = reinterpret_cast<float*>(c.smem + WORK_OFF + AttSm<HD>::MB_OFF);
-    const int unit = warp / NSPLIT, hsel = warp % NSPLIT, dof = hsel * ATT_DW;
-    const int rg = unit % R, tlane = unit / R;
-    const int row0 = rg * 8;
-    const uint32_t qw = smem_u32(qs) + (uint32_t)(dof * 2);
-    // rows >= M of the row groups in use are zero in both planes
-    for (int idx = tid; idx < (8 * R - M) * half; idx += NTHREADS) {
-        const int i = M + idx / half, e = idx % half;
-        reinterpret_cast<unsigned*>(qs + (size_t)i * QS)[e] = 0u;
-        reinterpret_cast<unsigned*>(qs + (size_t)(M_MAX + i) * QS)[e] = 0u;
-    }
-    const int tb = s * chunk_tiles, te = min(ntiles_all, tb + chunk_tiles);
-    const int kb = tb * ATT_TK, ke = min(T, te * ATT_TK);
-    // this pass's rows: q rotated, scaled and split into the bf16 hi / lo planes; k rotated and, with v, rounded and
-    // appended to the cache when the row's position lies in my key range.  One cos / sin pair serves q and k, and
-    // all six loads of an element are issued before the first is used.
-    for (int idx = tid; idx < M * half; idx += NTHREADS) {
-        const int i = idx / half, e = idx % half, pos = pos0 + i;
-        const float* src = a.qkv + (size_t)i * a.ldq + hh * HD + e;
-        const float* const p[6] = {src, src + half, src + d, src + d + half, src + 2 * d, src + 2 * d + half};
-        float xv[6];
-        att_read<6>(a, c, p, xv);
-        const float q1 = xv[0], q2 = xv[1], k1 = xv[2], k2 = xv[3], v1 = xv[4], v2 = xv[5];
-        const int page = checked_page(__ldg(D.page_table + (pos >> psh)), D.dm.n_phys, D.st, 52);
-        float cs, sn; rope_cs(D, pos, e, cs, sn);
-        const float r1 = (q1 * cs - q2 * sn) * qscale, r2 = (q2 * cs + q1 * sn) * qscale;
-        const __nv_bfloat16 h1 = __float2bfloat16_rn(r1), h2 = __float2bfloat16_rn(r2);
-        __nv_bfloat16* ph = reinterpret_cast<__nv_bfloat16*>(qs + (size_t)i * QS);
-        __nv_bfloat16* pl = reinterpret_cast<__nv_bfloat16*>(qs + (size_t)(M_MAX + i) * QS);
-        ph[e] = h1; ph[e + half] = h2;
-        pl[e] = __float2bfloat16_rn(r1 - __bfloat162float(h1)); pl[e + half] = __float2bfloat16_rn(r2 - __bfloat162float(h2));
-        if (pos >= kb && pos < ke) {
-            const size_t base = ((((size_t)page * H + hh) << psh) + (pos & psm)) * HD;
-            kc[base + e] = __float2bfloat16_rn(k1 * cs - k2 * sn);
-            kc[base + e + half] = __float2bfloat16_rn(k2 * cs + k1 * sn);
-            vc[base + e] = __float2bfloat16_rn(v1);
-            vc[base + e + half] = __float2bfloat16_rn(v2);
-        }
-    }
-    AttAcc ac;
+    char* qsm = c.smem + WORK_OFF;
+    char* ntile = c.smem + WORK_OFF + G::NT_OFF;
+    float* mb = reinterpret_cast<float*>(c.smem + WORK_OFF + G::MB_OFF);
+    const uint32_t nt_u = smem_u32(ntile);
+    int slot = c.slot; unsigned phase = c.phase;
+    bool ok = true;
+
+    for (int item = c.cta; item < H * pl.S; item += c.nctas) {
+        const int hh = item / pl.S, s = item - hh * pl.S;
+        const int tb = s * pl.chunk, nt = min(pl.ntile, tb + pl.chunk) - tb;
+        const bool last = s == pl.S - 1;
+        // ---- this pass's rows: q rotated, scaled, split into fragments; in the last split k rotated and, with v, rounded into the
+        // new tile and the cache.  Rows M .. 8 R - 1 of Q and M .. 15 of V are zero.
+        for (int idx0 = tid; idx0 < 8 * R * half; idx0 += 2 * NTHREADS) {
+            float q1[2], q2[2], k1[2], k2[2], v1[2], v2[2], cs[2], sn[2];
+            int pg[2];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) { ac.o[e][0] = ac.o[e][1] = ac.o[e][2] = ac.o[e][3] = 0.f; }
-    ac.m[0] = ac.m[1] = -INFINITY; ac.l[0] = ac.l[1] = 0.f;
-    // this unit's tiles: a contiguous run, so that one window of page-table entries serves many of them
-    int tile = tb + tlane * tpw;
-    const int tend = min(te, tile + tpw);
-    PageWin pw;
-    if (tile < tend) pw.load(D.page_table, D.dm.n_pages, (tile * ATT_TK) >> psh);
-    cta_sync();
-    auto fetch = [&](AttK& tk, AttV& tv, int ti) {
-        const int key0 = ti * ATT_TK, key1 = min(key0 + ATT_TK - 1, T - 1);
-        if ((key1 >> psh) - pw.first >= 32) pw.load(D.page_table, D.dm.n_pages, key0 >> psh);
-        att_load<HD>(tk, tv, kc, vc, pw, H, hh, dof, psh, psm, key0, T - 1, D.dm.n_phys, D.st);
-    };
-    AttP pp;
-    auto step = [&](const AttK& tk, const AttV& tv, int ti) {
-        float sc[4];
-        att_scores<QS>(tk, sc, qw, row0);
-        if constexpr (NSPLIT == 2) {
-            // the pair's halves of the dot products meet in shared memory (two buffers, used alternately)
-            float4* xb = reinterpret_cast<float4*>(mb) + (size_t)((unit * 2 + (ti & 1)) * 2) * 32;
-            xb[hsel * 32 + lane] = make_float4(sc[0], sc[1], sc[2], sc[3]);
-            pair_sync(unit);
-            const float4 ot = xb[(hsel ^ 1) * 32 + lane];
-            sc[0] += ot.x; sc[1] += ot.y; sc[2] += ot.z; sc[3] += ot.w;
-        }
-        att_softmax(sc, ac, pp, row0, ti * ATT_TK, ke, pos0);
-        att_accumulate(tv, ac, pp);
-    };
-    // One register set for K and V (a second one would not fit: the register allocation is shared with the
-    // linear operators).  A tile therefore costs a memory latency; the split count above keeps the run of
-    // tiles per unit short, and the other units and CTAs keep the memory system busy meanwhile.
-    AttK k0;
-    AttV v0;
-    while (tile < tend) {
-        fetch(k0, v0, tile);
-        step(k0, v0, tile);
-        ++tile;
-    }
-    // the row sums: lanes that share rows add their shares in a fixed order
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        ac.l[r] += __shfl_xor_sync(0xffffffffu, ac.l[r], 4);
-        ac.l[r] += __shfl_xor_sync(0xffffffffu, ac.l[r], 8);
-        ac.l[r] += __shfl_xor_sync(0xffffffffu, ac.l[r], 16);
-    }
-    if constexpr (NSPLIT == 2) cta_sync();          // the merge buffer lies over the pairs' exchange buffers
-    // merge the units of a row group through shared memory, four rows at a time
-#pragma unroll
-    for (int rb = 0; rb < M_MAX / ATT_RB; ++rb) {
-        if (rb * ATT_RB >= M) break;
-        const int nr = min(ATT_RB, M - rb * ATT_RB);
-        if (rg == (rb >> 1) && (t >> 1) == (rb & 1)) {
-            const int rl = 2 * (t & 1);
-            float* r0 = mb + ((size_t)tlane * ATT_RB + rl) * ATT_MB_STRIDE;
-            float* r1 = r0 + ATT_MB_STRIDE;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int dd = dof + 8 * g + 2 * e;
-                *reinterpret_cast<float2*>(r0 + dd) = make_float2(ac.o[e][0], ac.o[e][2]);
-                *reinterpret_cast<float2*>(r1 + dd) = make_float2(ac.o[e][1], ac.o[e][3]);
-            }
-            if (g == 0 && hsel == 0) { r0[HD_MAX] = ac.m[0]; r0[HD_MAX + 1] = ac.l[0]; r1[HD_MAX] = ac.m[1]; r1[HD_MAX + 1] = ac.l[1]; }
-        }
-        cta_sync();
-        for (int idx = tid; idx < nr * HD; idx += NTHREADS) {
-            const int r = idx / HD, e = idx % HD, i = rb * ATT_RB + r;
-            float mx = -INFINITY;
-            for (int w = 0; w < nw; ++w) mx = fmaxf(mx, mb[((size_t)w * ATT_RB + r) * ATT_MB_STRIDE + HD_MAX]);
-            float den = 0.f, num = 0.f;
-            for (int w = 0; w < nw; ++w) {
-                const float* row = mb + ((size_t)w * ATT_RB + r) * ATT_MB_STRIDE;
-                const float mw = row[HD_MAX];
-                if (mw != -INFINITY) {
-                    const float wgt = ex2f(mw - mx);
-                    den += row[HD_MAX + 1] * wgt;
-                    num += row[e] * wgt;
+            for (int u = 0; u < 2; ++u) {                  // what does not depend on this pass, before the poll
+                const int idx = idx0 + u * NTHREADS, i = idx / half;
+                cs[u] = sn[u] = 0.f; pg[u] = 0;
+                if (i < M) {
+                    rope_at(D, pos0 + i, idx & (half - 1), half, cs[u], sn[u]);
+                    if (last) pg[u] = __ldg(D.page_table + ((pos0 + i) >> psh));
                 }
             }
-            if (S == 1) {
-                att_store(a, i, hh * HD + e, num / den);
-            } else {
-                D.att_po[(((size_t)i * H + hh) * S_CAP + s) * HD + e] = num;
-                if (e == 0) {
-                    D.att_ml[(((size_t)i * H + hh) * S_CAP + s) * 2 + 0] = mx;
-                    D.att_ml[(((size_t)i * H + hh) * S_CAP + s) * 2 + 1] = den;
+            {
+                XchSpin sp; sp.spins = 0;
+                const float* qkv = a.qkv;
+                while (true) {
+                    bool empty = false;
+                    asm volatile("" : "+l"(qkv));        // (addresses are formed inside the loop, not kept across it)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int idx = idx0 + u * NTHREADS, i = idx / half;
+                        q1[u] = q2[u] = k1[u] = k2[u] = v1[u] = v2[u] = 0.f;
+                        if (i < M) {
+                            const unsigned* src = reinterpret_cast<const unsigned*>(qkv + (size_t)i * a.ldq + hh * HD + (idx & (half - 1)));
+                            unsigned w[6];
+                            w[0] = xch_ld1(src); w[1] = xch_ld1(src + half);
+                            w[2] = w[3] = w[4] = w[5] = 0u;
+                            if (last) { w[2] = xch_ld1(src + d); w[3] = xch_ld1(src + d + half); w[4] = xch_ld1(src + 2 * d); w[5] = xch_ld1(src + 2 * d + half); }
+#pragma unroll
+                            for (int q = 0; q < 6; ++q) empty |= w[q] == XCH_EMPTY;
+                            q1[u] = __uint_as_float(w[0]); q2[u] = __uint_as_float(w[1]); k1[u] = __uint_as_float(w[2]); k2[u] = __uint_as_float(w[3]);
+                            v1[u] = __uint_as_float(w[4]); v2[u] = __uint_as_float(w[5]);
+                        }
+                    }
+                    if (!a.poll || !empty || !xch_again(c, sp, 45)) break;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int idx = idx0 + u * NTHREADS, i = idx / half, e = idx & (half - 1), pos = pos0 + i;
+                if (i >= 8 * R) break;
+                const float r[2] = {(q1[u] * cs[u] - q2[u] * sn[u]) * qscale, (q2[u] * cs[u] + q1[u] * sn[u]) * qscale};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int dim = e + h * half, kk = dim & 15;
+                    char* p = qsm + (i >> 3) * G::QG + (((dim >> 4) * 32) + (i & 7) * 4 + ((kk & 7) >> 1)) * 16 + (kk >> 3) * 4 + (kk & 1) * 2;
+                    const WT hi = __float2bfloat16_rn(r[h]);
+                    *reinterpret_cast<WT*>(p) = hi;
+                    *reinterpret_cast<WT*>(p + 8) = __float2bfloat16_rn(r[h] - __bfloat162float(hi));
+                }
+                if (last) {
+                    const WT kr[2] = {__float2bfloat16_rn(k1[u] * cs[u] - k2[u] * sn[u]), __float2bfloat16_rn(k2[u] * cs[u] + k1[u] * sn[u])};
+                    const WT vr[2] = {__float2bfloat16_rn(v1[u]), __float2bfloat16_rn(v2[u])};
+                    WT* kc = nullptr; WT* vc = nullptr;
+                    if (i < M) {
+                        const int page = checked_page(pg[u], D.dm.n_phys, D.st, 52);
+                        const size_t base = ((((size_t)page * H + hh) << psh) + (pos & psm)) * HD;
+                        kc = reinterpret_cast<WT*>(a.kc) + base; vc = reinterpret_cast<WT*>(a.vc) + base;
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int dim = e + h * half;
+                        const uint32_t off = ra_addr(nt_u, i, dim >> 3) - nt_u + (uint32_t)(dim & 7) * 2;
+                        *reinterpret_cast<WT*>(ntile + off) = kr[h];
+                        *reinterpret_cast<WT*>(ntile + G::HALF_BYTES + off) = vr[h];
+                        if (i < M) { kc[dim] = kr[h]; vc[dim] = vr[h]; }
+                    }
                 }
             }
         }
         cta_sync();
-    }
-    if (S > 1) {
-        // the partials of this CTA are ordered before the counter by the barrier above and the release of the
-        // atomic; the last arriver's acquire orders the counter before its reads of every split's partials
-        if (tid == 0) {
-            unsigned prev;
-            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(D.att_cnt + hh) : "memory");
-            const int last = (prev == (unsigned)(S - 1));
-            c.ctl->att_last = last;
-            if (last) D.att_cnt[hh] = 0u;
-        }
-        cta_sync();
-        if (*(volatile int*)&c.ctl->att_last) {
-            if (S <= 4) att_merge_splits<4, 4>(D, a, hh, S, M);
-            else if (S <= 8) att_merge_splits<8, 2>(D, a, hh, S, M);
-            else att_merge_splits<S_CAP, 1>(D, a, hh, S, M);
-        }
-        cta_sync();
-    }
-}
-
-template <int HD>
-__device__ __noinline__ void attention_mma(const Dev& D, const AttArgs& a, Ctx& c) {
-    constexpr int NUNITS = NWARPS / (HD / ATT_DW);
-    const int H = D.dm.H;
-    const int ntiles_all = (a.pos0 + a.M + ATT_TK - 1) / ATT_TK;
-    const int nw = NUNITS / ((a.M + 7) >> 3);
-    const int nw_sh = 31 - __clz(nw);
-    // KV splits per head.  An item costs its units' tiles (one memory latency each) plus a fixed part, and a head
-    // that is split pays for the merge of its partials through global memory (several dependent round trips, about
-    // as long as three tiles): very short caches stay unsplit.
-    int S = 1;
-    {
-        const float inv_ctas = 1.0f / (float)c.nctas;
-        float best = -1.f;
+        // ---- the tiles
+        float o[R][HD / 16][4], mx[R][2], l[R][2];
 #pragma unroll
-        for (int sc = 1; sc <= S_CAP; ++sc) {
-            const int chunk_ = (ntiles_all + sc - 1) / sc;
-            const int tpw_ = (chunk_ + nw - 1) >> nw_sh;
-            const float waves = ceilf((float)(H * sc) * inv_ctas - 1e-4f);
-            const float cost = waves * (float)(tpw_ + 2 + (sc > 1 ? 3 : 0));
-            if ((sc == 1 || chunk_ >= 2) && (best < 0.f || cost < best)) { best = cost; S = sc; }
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int e = 0; e < HD / 16; ++e) { o[r][e][0] = o[r][e][1] = o[r][e][2] = o[r][e][3] = 0.f; }
+            mx[r][0] = mx[r][1] = -INFINITY; l[r][0] = l[r][1] = 0.f;
+        }
+        const uint32_t qf = smem_u32(qsm);
+        const int nslot = (nt + G::TPS - 1) / G::TPS;
+        // one round per ring slot, and one more for the tile of this pass's rows
+        for (int k = 0; k <= nslot; ++k) {
+            const bool fresh = k == nslot;
+            if (fresh && !last) break;
+            if (!fresh && ok) ok = mbar_wait(c, &c.ctl->full[slot], phase, 48);
+            const int jt = fresh ? nt : k * G::TPS + ((warp - k * G::TPS) & (NWARPS - 1));       // this warp's tile, if it lies in the slot
+            const bool mine = fresh ? warp == (nt & (NWARPS - 1)) : (jt < (k + 1) * G::TPS && jt < nt);
+            if (mine && ok) {
+                const uint32_t kb = fresh ? nt_u : smem_u32(c.smem + RING_OFF + (size_t)slot * SLOT_BYTES) + (uint32_t)((jt - k * G::TPS) * G::TILE_BYTES);
+                ra_tile<HD, R>(kb, kb + G::HALF_BYTES, qf, fresh ? M : min(ATT_TK, pos0 - (tb + jt) * ATT_TK), fresh, o, mx, l);
+            }
+            if (!fresh) {
+                __syncwarp();
+                if (ok && lane == 0) mbar_arrive(&c.ctl->empty[slot]);
+                if (++slot == RING) { slot = 0; phase ^= 1u; }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                l[r][i] += __shfl_xor_sync(0xffffffffu, l[r][i], 4);
+                l[r][i] += __shfl_xor_sync(0xffffffffu, l[r][i], 8);
+                l[r][i] += __shfl_xor_sync(0xffffffffu, l[r][i], 16);
+            }
+        }
+        cta_sync();                                        // the new tile has been read: the merge buffer lies over it
+        // ---- merge of the warps (those without tiles hold zeros and a maximum of -inf), four rows at a time, then of the splits; a
+        // thread takes four neighbouring elements (one element a thread, in rolled loops, took 4.6 us for seven rows)
+        unsigned* xw = D.att_xp;                           // [M_MAX][H][S_CAP][ROW]
+        constexpr int ROW = G::ROW;
+#pragma unroll
+        for (int rb = 0; rb < 2 * R; ++rb) {
+            if (rb * ATT_RB >= M) break;
+            const int nr = min(ATT_RB, M - rb * ATT_RB), r = rb >> 1;
+            if ((t >> 1) == (rb & 1)) {
+                const int rl = 2 * (t & 1);
+                float* r0 = mb + ((size_t)warp * ATT_RB + rl) * ROW;
+                float* r1 = r0 + ROW;
+#pragma unroll
+                for (int e = 0; e < HD / 16; ++e) {
+                    r0[e * 16 + g] = o[r][e][0]; r1[e * 16 + g] = o[r][e][1];
+                    r0[e * 16 + 8 + g] = o[r][e][2]; r1[e * 16 + 8 + g] = o[r][e][3];
+                }
+                if (g == 0) { r0[HD] = mx[r][0]; r0[HD + 1] = l[r][0]; r1[HD] = mx[r][1]; r1[HD + 1] = l[r][1]; }
+            }
+            cta_sync();
+            if (tid < nr * (HD / 4)) {
+                const int rr = tid / (HD / 4), e = tid % (HD / 4) * 4, i = rb * ATT_RB + rr;
+                unsigned* xrow = xw + (((size_t)i * H + hh) * S_CAP) * ROW;
+                // the other splits' words are requested before this one's are added up
+                constexpr int QB = 4;
+                uint4 wo[QB]; uint2 wm[QB];
+                auto request = [&](int q0) {
+                    asm volatile("" : "+l"(xrow));
+#pragma unroll
+                    for (int q = 0; q < QB; ++q)
+                        if (last && q0 + q < s) { wo[q] = xch_ld4(xrow + (q0 + q) * ROW + e); wm[q] = xch_ld2(xrow + (q0 + q) * ROW + HD); }
+                };
+                request(0);
+                const float* row = mb + rr * ROW;
+                float2 ml[NWARPS];
+#pragma unroll
+                for (int w = 0; w < NWARPS; ++w) ml[w] = *reinterpret_cast<const float2*>(row + w * ATT_RB * ROW + HD);
+                float m = ml[0].x, den = 0.f;
+#pragma unroll
+                for (int w = 1; w < NWARPS; ++w) m = fmaxf(m, ml[w].x);
+                float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int w = 0; w < NWARPS; ++w) {
+                    const float f = ml[w].x == -INFINITY ? 0.f : ex2f(ml[w].x - m);
+                    const float4 v = *reinterpret_cast<const float4*>(row + w * ATT_RB * ROW + e);
+                    den += ml[w].y * f;
+                    num.x += v.x * f; num.y += v.y * f; num.z += v.z * f; num.w += v.w * f;
+                }
+                if (!last) {
+                    unsigned* p = xrow + s * ROW;
+                    xch_st4(p + e, make_uint4(__float_as_uint(num.x), __float_as_uint(num.y), __float_as_uint(num.z), __float_as_uint(num.w)));
+                    if (e == 0) { xch_st(p + HD, __float_as_uint(m)); xch_st(p + HD + 1, __float_as_uint(den)); }
+                } else {
+                    for (int q0 = 0; q0 < s; q0 += QB) {
+                        if (q0) request(q0);
+                        XchSpin sp; sp.spins = 0;
+                        while (true) {
+                            bool empty = false;
+#pragma unroll
+                            for (int q = 0; q < QB; ++q) empty |= q0 + q < s && (xch_empty(wo[q]) || xch_empty(wm[q]));
+                            if (!empty || !xch_again(c, sp, 49)) break;
+                            request(q0);
+                        }
+#pragma unroll
+                        for (int q = 0; q < QB; ++q) {
+                            if (q0 + q < s) {
+                                const float om = __uint_as_float(wm[q].x), mn = fmaxf(m, om);
+                                const float f0 = m == -INFINITY ? 0.f : ex2f(m - mn), f1 = om == -INFINITY ? 0.f : ex2f(om - mn);
+                                den = den * f0 + __uint_as_float(wm[q].y) * f1;
+                                num.x = num.x * f0 + __uint_as_float(wo[q].x) * f1; num.y = num.y * f0 + __uint_as_float(wo[q].y) * f1;
+                                num.z = num.z * f0 + __uint_as_float(wo[q].z) * f1; num.w = num.w * f0 + __uint_as_float(wo[q].w) * f1;
+                                m = mn;
+                                xch_st4(xrow + (q0 + q) * ROW + e, make_uint4(XCH_EMPTY, XCH_EMPTY, XCH_EMPTY, XCH_EMPTY));      // this thread alone reads them
+                            }
+                        }
+                    }
+                    num.x /= den; num.y /= den; num.z /= den; num.w /= den;
+                    const int col = hh * HD + e;
+                    if (a.out) *reinterpret_cast<float4*>(a.out + (size_t)i * a.ldo + col) = num;
+                    if (a.opk) { pk_store2(a.opk + (size_t)i * a.ldopk, col, num.x, num.y); pk_store2(a.opk + (size_t)i * a.ldopk, col + 2, num.z, num.w); }
+                }
+            }
+            cta_sync();
+        }
+        if (last && s > 0) {
+            // maxima and sums have been read by every thread of the merge
+            for (int idx = tid; idx < M * s; idx += NTHREADS) {
+                unsigned* p = xw + (((size_t)(idx / s) * H + hh) * S_CAP + idx % s) * ROW + HD;
+                xch_st(p, XCH_EMPTY); xch_st(p + 1, XCH_EMPTY);
+            }
         }
     }
-    const int chunk_tiles = (ntiles_all + S - 1) / S;
-    for (int item = c.cta; item < H * S; item += c.nctas) att_item<HD>(D, a, c, item / S, item % S, S, chunk_tiles);
+    c.slot = slot; c.phase = phase;
 }
 
-static_assert(AttSm<HD_MAX>::MB_OFF + NWARPS * ATT_RB * ATT_MB_STRIDE * 4 <= WORK_BYTES, "tensor-core attention buffers do not fit in the work area");
-static_assert(4 * 2 * 2 * 32 * 16 <= NWARPS * ATT_RB * ATT_MB_STRIDE * 4, "the score exchange does not fit in the merge buffer");
-
+// ring: the tensor-core attention, fed by the copy warp (decided once per model: bf16 streamed path, head_dim 64 or 128)
 template <typename WT>
-__device__ __forceinline__ void attention_op(const Dev& D, const AttArgs* sa, Ctx& c) {
-    // sa points into the consumers' operator table in shared memory
+__device__ __forceinline__ void attention_op(const Dev& D, const AttArgs& a, Ctx& c, bool ring) {
     if constexpr (sizeof(WT) == 2) {
-        if (D.dm.hd == 128) { attention_mma<128>(D, *sa, c); return; }
-        if (D.dm.hd == 64) { attention_mma<64>(D, *sa, c); return; }
+        if (ring) {
+            if (D.dm.hd == 128) { if (a.M <= 8) attention_ring<128, 1>(D, a, c); else attention_ring<128, 2>(D, a, c); }
+            else { if (a.M <= 8) attention_ring<64, 1>(D, a, c); else attention_ring<64, 2>(D, a, c); }
+            return;
+        }
     }
-    if (D.dm.hd == 128) attention_impl<WT, 4>(D, *sa, c);
-    else if (D.dm.hd == 64) attention_impl<WT, 2>(D, *sa, c);
-    else attention_impl<WT, 1>(D, *sa, c);
+    if (D.dm.hd == 128) attention_impl<WT, 4>(D, a, c);
+    else if (D.dm.hd == 64) attention_impl<WT, 2>(D, a, c);
+    else attention_impl<WT, 1>(D, a, c);
+}
+__device__ __forceinline__ bool attention_producer(const Dev& D, const RaPlan& pl, int row0, Ctx& c) {
+    return D.dm.hd == 128 ? att_produce<128>(D, pl, row0, c) : att_produce<64>(D, pl, row0, c);
 }
 
 static_assert((M_MAX * HD_MAX + NWARPS * ATT_RB * ATT_MB_STRIDE + NWARPS * 40) * 4 <= WORK_BYTES, "attention buffers do not fit in the work area");

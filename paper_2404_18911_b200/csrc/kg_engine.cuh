@@ -3,11 +3,17 @@
 // prefix accept / rollback, or many rounds back to back - with exchanges or grid barriers between
 // dependent operators and no host involvement.
 //
-// Every thread of every CTA walks the same operator sequence and holds the same copy of the
-// sequence state.  The consumer warps do the arithmetic and take part in the grid barriers; the
-// producer warp only issues the weight copies of each linear operator, so it runs ahead of the
-// consumers (through barriers and attention) until the next decision that depends on a result
-// (a drafted token, its confidence, the accepted prefix), which it receives through shared memory.
+// Three roles in every CTA, joined by a queue of operators in shared memory:
+//   the sequencer (one thread) walks through the method - layers, draft steps, accept decisions - and writes the arguments of one
+//     operator after the other into the queue.  It runs ahead of the others until the next decision that depends on a result (a
+//     drafted token, its confidence, the accepted prefix), which it receives through shared memory.  Every CTA's sequencer
+//     holds the same copy of the sequence state and comes to the same decisions.
+//   the copy warp streams the weights and the K / V tiles of the operators in the queue;
+//   the eight consumer warps do the arithmetic and take part in the grid barriers.
+// The consumers' loop holds every operator once, inlined.  Before, every thread walked through the method itself and called the
+// operators as functions from a dozen places: they were compiled for the 168 registers of the launch (the warpgroups' own budgets
+// reach inlined code only), what the callers kept across them was spilled - beside 227 KB of shared memory there is hardly any L1,
+// so that a spilled register is an L2 access -, and each layer began with one thread writing its arguments while 255 waited.
 #pragma once
 
 #include "kg_device.cuh"
@@ -25,52 +31,59 @@ struct Program {
     int skip_arrival;   // test hook: 1 + index of a CTA that leaves out its first grid-barrier arrival, so that a wait expires
 };
 
-#define KG_SYNC(where) do { if (!sync(where)) return false; } while (0)
-#define KG_LIN(args) do { if (!linear(args)) return false; } while (0)
-
 // Rows handed from one operator to the next: fp32 rows (residual input, plain path), their packed copy
 // scaled by the reader's norm gain, and the per-CTA sums of squares the reader's RMSNorm needs.
 struct ActIn { const float* x; const unsigned char* pk; const float* ssq; };
 struct ActOut { float* x; PkOut pk[2]; float* ssq; };
 
-// PROD: the instruction stream of the producer warp (it only issues weight copies and follows the control flow) or of
-// the consumer warps; the two are compiled apart because they run with different register budgets.
-template <typename WT, bool PROD>
-struct Engine {
+// linear operators on the streamed tensor-core path / attention from the ring, for this launch
+__device__ __forceinline__ bool launch_streamed(const Dev& D, const Program& pg) { return D.dm.stream != 0 && pg.force_simple == 0; }
+
+// ---- the sequencer (one thread per CTA) ----------------------------------------------------------------------------
+template <typename WT>
+struct Sequencer {
     const Dev& D;
     Ctx& c;
     const Program& pg;
+    const bool streamed;
+    int qi = 0; unsigned qph = 0;      // queue cursor
+    RaPlan plan;                       // of the last attention position
+    int xp = 0;                        // exchange instance the next layer uses
+    int xused = 0;                     // rows of the other instance, the one of the layer before, that hold data
 
-    __device__ Engine(const Dev& d, Ctx& cx, const Program& p) : D(d), c(cx), pg(p) {}
+    __device__ Sequencer(const Dev& d, Ctx& cx, const Program& p) : D(d), c(cx), pg(p), streamed(launch_streamed(d, p)) { plan.pos = -1; }
 
-    // ---- leaf operations: what a thread does depends on its role -------------------------------
-    __device__ __forceinline__ bool streamed() const { return D.dm.stream != 0 && pg.force_simple == 0; }
-    __device__ __forceinline__ bool sync(int where) { if constexpr (PROD) return true; else return grid_sync(c, where); }
-    // this role's operator table in shared memory, and the one thread of the role that fills it
-    __device__ __forceinline__ OpTable* table() const {
-        if constexpr (PROD) __syncwarp();    // the lanes have left the previous operator before lane 0 rewrites the table
-        return reinterpret_cast<OpTable*>(PROD ? c.ctl->tab_prod : c.ctl->tab_cons);
+    // ---- the queue
+    __device__ __forceinline__ Op* begin(int kind) {
+        if (!mbar_wait(c, &c.ctl->qempty[qi], qph ^ 1u, 33)) return nullptr;
+        Op* o = &c.ctl->queue[qi];
+        o->kind = kind; o->sync = 0;
+        return o;
     }
-    // the one thread that writes part `part` of the table: one of another warp for every part, so that they write side by side
-    // (the producer warp, which reads little of the table, has one writer)
-    __device__ __forceinline__ bool writer(int part = 0) const { return PROD ? (threadIdx.x & 31) == 0 : (int)threadIdx.x == 32 * part; }
-    // operator on the weights [N, K] with M rows: all that the producer reads of a LinArgs
-    __device__ __forceinline__ void shape(LinArgs& a, const void* W, const void* W2, int N, int K, int M) const {
-        a.W = W; a.W2 = W2; a.N = N; a.K = K; a.M = M;
-        if constexpr (!PROD) {
-            a.eps = D.dm.eps; a.gain = nullptr; a.ssq_in = nullptr; a.poll = 0; a.resid = nullptr; a.out = nullptr;
-            a.pk[0] = PkOut{nullptr, nullptr}; a.pk[1] = PkOut{nullptr, nullptr}; a.ssq_out = nullptr;
-        }
+    __device__ __forceinline__ void commit() {
+        mbar_arrive(&c.ctl->qfull[qi]);
+        if (++qi == QUEUE) { qi = 0; qph ^= 1u; }
     }
-    __device__ __forceinline__ bool linear(const LinArgs* a, bool publish) {
-        if constexpr (PROD) return linear_producer(a, c, streamed(), publish);
-        else return linear_consumer<WT>(a, c, streamed(), publish);
+    // waits until the consumers have come to the operator that answers
+    __device__ __forceinline__ bool wait_mail() {
+        const unsigned mp = c.mail_phase;
+        c.mail_phase = mp ^ 1u;
+        return mbar_wait(c, &c.ctl->mail, mp, 42);
     }
-    __device__ __forceinline__ void attention(const AttArgs* at) { if constexpr (!PROD) attention_op<WT>(D, at, c); }
+    // operator on the weights [N, K] with M rows
+    __device__ __forceinline__ LinArgs* linear(const void* W, const void* W2, int N, int K, int M) {
+        Op* o = begin(OPK_LIN);
+        if (!o) return nullptr;
+        LinArgs& a = o->lin;
+        a.W = W; a.W2 = W2; a.N = N; a.K = K; a.M = M; a.eps = D.dm.eps;
+        a.gain = nullptr; a.ssq_in = nullptr; a.poll = 0; a.resid = nullptr; a.out = nullptr;
+        a.pk[0] = PkOut{nullptr, nullptr}; a.pk[1] = PkOut{nullptr, nullptr}; a.ssq_out = nullptr;
+        return &a;
+    }
+    __device__ __forceinline__ void commit_sync(int where) { c.ctl->queue[qi].sync = where; commit(); }
 
-    __device__ size_t cache_layer_stride() const {
-        return (size_t)D.dm.n_pages * D.dm.H * D.dm.page_size * D.dm.hd;
-    }
+    // ---- buffers
+    __device__ size_t cache_layer_stride() const { return (size_t)D.dm.n_pages * D.dm.H * D.dm.page_size * D.dm.hd; }
     __device__ __forceinline__ size_t ldpk() const { return (size_t)D.dm.d * 4; }
     __device__ __forceinline__ ActIn act_h() const { return ActIn{D.h, D.hA_pk, D.ssq_hA}; }
     // the residual stream as an output, packed for a reader whose norm gain is `gain`
@@ -79,196 +92,143 @@ struct Engine {
     }
     // norm gain of whatever reads the output of layer i: the next layer, or the LM head after the last one
     __device__ __forceinline__ const float* next_gain(int i) const { return i + 1 < D.dm.L ? D.layers[i + 1].g1 : D.g_final; }
+    // the early-feature slot `slot` as an input of the adapter / of the first deep layer
+    __device__ __forceinline__ ActIn feat_for_adapter(int slot) const {
+        return ActIn{D.feat + (size_t)slot * D.dm.d, D.featA_pk + (size_t)slot * ldpk(), D.ssq_feat + (size_t)slot * c.nctas};
+    }
+    __device__ __forceinline__ ActIn feat_for_deep(int slot) const {
+        return ActIn{D.feat + (size_t)slot * D.dm.d, D.featD_pk + (size_t)slot * ldpk(), D.ssq_feat + (size_t)slot * c.nctas};
+    }
+    // exchange rows of the layer being pushed
+    __device__ __forceinline__ float* xrow(int off) const { return reinterpret_cast<float*>(D.xch[xp] + off); }
+    __device__ __forceinline__ float* x_qkv() const { return xrow(0); }
+    __device__ __forceinline__ float* x_attn() const { return xrow(3 * D.dm.d); }
+    __device__ __forceinline__ float* x_h() const { return xrow(4 * D.dm.d); }
+    __device__ __forceinline__ float* x_act() const { return xrow(5 * D.dm.d); }
+    __device__ __forceinline__ float* x_ssq() const { return xrow(5 * D.dm.d + D.dm.F); }
+    __device__ static __forceinline__ unsigned char* bytes(float* p) { return reinterpret_cast<unsigned char*>(p); }
 
-    // an id outside [0, V) never indexes the embedding table (ids that arrive in device memory are checked by a
-    // kernel of their own, which records the error; here the access is merely kept in bounds)
-    __device__ __forceinline__ int safe_token(int tok) const { return (unsigned)tok < (unsigned)D.dm.V ? tok : 0; }
-
+    // ---- operators
     // h[i] = E[token_i]; packed for layer 0
-    __device__ void embed_rows(const int* toks_global, int tok_single, int M) {
-        if constexpr (PROD) return;
-        const int d = D.dm.d;
-        const WT* E = reinterpret_cast<const WT*>(D.embed);
-        if (!streamed()) {
-            for (int idx = c.cta * NTHREADS + threadIdx.x; idx < M * d; idx += c.nctas * NTHREADS) {
-                const int i = idx / d, e = idx % d;
-                const int tok = safe_token(toks_global ? __ldcg(toks_global + i) : tok_single);
-                D.h[idx] = wt_to_float<WT>(E[(size_t)tok * d + e]);
-            }
-            return;
-        }
-        LinArgs a{};
-        a.N = d; a.M = M; a.out = D.h; a.ldo = d;
-        a.pk[0] = PkOut{D.layers[0].g1, D.hA_pk}; a.ldpk_out = (int)ldpk(); a.ssq_out = D.ssq_hA; a.ld_sout = c.nctas;
-        emit_plain_rows(a, c, [&](int m, int e) {
-            const int tok = safe_token(toks_global ? __ldcg(toks_global + m) : tok_single);
-            return wt_to_float<WT>(E[(size_t)tok * d + e]);
-        });
+    __device__ bool embed_rows(const int* toks, int tok, int M, int where) {
+        Op* o = begin(OPK_EMBED);
+        if (!o) return false;
+        o->emb.toks = toks; o->emb.tok = tok; o->emb.M = M;
+        commit_sync(where);
+        return true;
     }
-
-    // ---- exchange buffers of a layer (see the exchange words in kg_device.cuh)
-    int xp;                 // instance the next layer uses
-    int xused;              // rows of the other instance, the one of the layer before, that hold data
-    __device__ __forceinline__ unsigned* xrow(int off) const { return D.xch[xp] + off; }
-    __device__ __forceinline__ int x_attn() const { return 3 * D.dm.d; }
-    __device__ __forceinline__ int x_h() const { return 4 * D.dm.d; }
-    __device__ __forceinline__ int x_act() const { return 5 * D.dm.d; }
-    __device__ __forceinline__ int x_ssq() const { return 5 * D.dm.d + D.dm.F; }
-    __device__ __forceinline__ void empty_instance(int p) {
-        const int n4 = xused * (D.xch_ld >> 2);
-        uint4* q = reinterpret_cast<uint4*>(D.xch[p]);
-        for (int i = c.cta * NTHREADS + threadIdx.x; i < n4; i += c.nctas * NTHREADS) q[i] = make_uint4(XCH_EMPTY, XCH_EMPTY, XCH_EMPTY, XCH_EMPTY);
-    }
-    // after the attention of a layer: the instance of the layer before is emptied, this one belongs to M rows (not earlier: the
-    // merge of attention's splits releases what this CTA has stored so far)
-    __device__ __forceinline__ void turn_instance(int M) {
-        if constexpr (!PROD) { empty_instance(xp ^ 1); xused = M; xp ^= 1; }
-    }
-
-    // Arguments of the attention block of layer / adapter `li` on M rows at pos0: [0] q, k, v, the attention itself and [1] the
-    // output projection with its residual (where it goes is left to the caller, who fills in the rest with the same writer).
-    __device__ __forceinline__ void fill_attention_block(OpTable* t, const LayerW& lw, int li, int M, int pos0, const ActIn& in) {
+    // q, k, v and the attention of layer / adapter `li` on M rows at pos0
+    __device__ bool attention_block(const LayerW& lw, int li, int M, int pos0, const ActIn& in) {
         const Dims& dm = D.dm;
-        if (writer(0)) {
-            LinArgs& q = t->lin[0];
-            shape(q, lw.wqkv, nullptr, 3 * dm.d, dm.d, M);
-            if constexpr (!PROD) {
-                q.x = in.x; q.ldx = dm.d; q.gain = lw.g1; q.xpk = in.pk; q.ldpk = (int)ldpk(); q.ssq_in = in.ssq; q.ld_ssq = c.nctas;
-                q.epi = EPI_STORE; q.out = reinterpret_cast<float*>(xrow(0)); q.ldo = D.xch_ld;
-            }
-        }
-        if constexpr (!PROD) {
-            if (writer(1)) {
-                AttArgs& at = t->att;
-                at.qkv = reinterpret_cast<const float*>(xrow(0)); at.ldq = D.xch_ld; at.poll = 1; at.M = M; at.pos0 = pos0;
-                at.kc = reinterpret_cast<WT*>(D.kcache) + (size_t)li * cache_layer_stride();
-                at.vc = reinterpret_cast<WT*>(D.vcache) + (size_t)li * cache_layer_stride();
-                at.out = streamed() ? nullptr : reinterpret_cast<float*>(xrow(x_attn())); at.ldo = D.xch_ld;
-                at.opk = streamed() ? reinterpret_cast<unsigned char*>(xrow(x_attn())) : nullptr; at.ldopk = D.xch_ld * 4;
-            }
-        }
-        if (writer(2)) {
-            LinArgs& o = t->lin[1];
-            shape(o, lw.wo, nullptr, dm.d, dm.d, M);
-            if constexpr (!PROD) {
-                o.x = reinterpret_cast<const float*>(xrow(x_attn())); o.ldx = D.xch_ld;
-                o.xpk = reinterpret_cast<const unsigned char*>(xrow(x_attn())); o.ldpk = D.xch_ld * 4; o.poll = 1;
-                o.epi = EPI_RESID; o.resid = in.x; o.ldr = dm.d;
-            }
-        }
+        LinArgs* q = linear(lw.wqkv, nullptr, 3 * dm.d, dm.d, M);
+        if (!q) return false;
+        q->x = in.x; q->ldx = dm.d; q->gain = lw.g1; q->xpk = in.pk; q->ldpk = (int)ldpk(); q->ssq_in = in.ssq; q->ld_ssq = c.nctas;
+        q->epi = EPI_STORE; q->out = x_qkv(); q->ldo = D.xch_ld;
+        commit();
+        if (D.dm.ring && plan.pos != pos0) plan = ra_plan(pos0, dm.H, c.nctas);
+        Op* o = begin(OPK_ATT);
+        if (!o) return false;
+        AttArgs& at = o->att;
+        at.plan = plan;
+        at.qkv = x_qkv(); at.ldq = D.xch_ld; at.poll = 1; at.M = M; at.pos0 = pos0;
+        at.kc = reinterpret_cast<WT*>(D.kcache) + (size_t)li * cache_layer_stride();
+        at.vc = reinterpret_cast<WT*>(D.vcache) + (size_t)li * cache_layer_stride();
+        at.row0 = li * dm.n_pages * dm.H * dm.page_size;
+        at.out = streamed ? nullptr : x_attn(); at.ldo = D.xch_ld;
+        at.opk = streamed ? bytes(x_attn()) : nullptr; at.ldopk = D.xch_ld * 4;
+        // the instance of the layer before is emptied behind the attention (not earlier: nothing else is stored meanwhile)
+        o->empty_p = xp ^ 1; o->empty_rows = xused;
+        commit();
+        return true;
     }
+    // output projection of the attention with its residual
+    __device__ LinArgs* out_proj(const LayerW& lw, int M, const ActIn& in) {
+        LinArgs* o = linear(lw.wo, nullptr, D.dm.d, D.dm.d, M);
+        if (!o) return nullptr;
+        o->x = x_attn(); o->ldx = D.xch_ld; o->xpk = bytes(x_attn()); o->ldpk = D.xch_ld * 4; o->poll = 1;
+        o->epi = EPI_RESID; o->resid = in.x; o->ldr = D.dm.d;
+        return o;
+    }
+    __device__ __forceinline__ void turn_instance(int M) { xused = M; xp ^= 1; }
 
     // One decoder block on M rows at positions pos0.. (Section 3.1's M^b layers):
     //   h  = x + Wo Attn(RMSNorm(x; g1));   out = h + Wdown(SiLU(Wgate n) * Wup n), n = RMSNorm(h; g2)
     // The rows between its operators are exchange words; one grid barrier ends the layer.
-    __device__ bool run_layer(int li, int M, int pos0, const ActIn& in, const ActOut& out) {
+    __device__ bool layer(int li, int M, int pos0, const ActIn& in, const ActOut& out) {
         const Dims& dm = D.dm;
-        OpTable* t = table();
         const LayerW& lw = D.layers[li];
+        if (!attention_block(lw, li, M, pos0, in)) return false;
         // the residual stream after attention: fp32 rows of each CTA's own features, packed rows for everybody (plain path:
         // fp32 exchange rows for both)
-        float* hx = reinterpret_cast<float*>(xrow(x_h()));
-        fill_attention_block(t, lw, li, M, pos0, in);
-        if constexpr (!PROD) {
-            if (writer(2)) {
-                LinArgs& o = t->lin[1];
-                o.out = streamed() ? D.h : hx; o.ldo = streamed() ? dm.d : D.xch_ld;
-                o.pk[0] = PkOut{lw.g2, reinterpret_cast<unsigned char*>(hx)}; o.ldpk_out = D.xch_ld * 4;
-                o.ssq_out = reinterpret_cast<float*>(xrow(x_ssq())); o.ld_sout = D.xch_ld;
-            }
-        }
-        if (writer(3)) {
-            LinArgs& gu = t->lin[2];
-            shape(gu, lw.wgate, lw.wup, dm.F, dm.d, M);
-            if constexpr (!PROD) {
-                gu.x = hx; gu.ldx = D.xch_ld; gu.gain = lw.g2; gu.xpk = reinterpret_cast<const unsigned char*>(hx); gu.ldpk = D.xch_ld * 4;
-                gu.ssq_in = reinterpret_cast<const float*>(xrow(x_ssq())); gu.ld_ssq = D.xch_ld; gu.poll = 1;
-                gu.epi = EPI_SWIGLU; gu.out = streamed() ? nullptr : reinterpret_cast<float*>(xrow(x_act())); gu.ldo = D.xch_ld;
-                gu.pk[0] = PkOut{nullptr, reinterpret_cast<unsigned char*>(xrow(x_act()))}; gu.ldpk_out = D.xch_ld * 4;
-            }
-        }
-        if (writer(4)) {
-            LinArgs& dn = t->lin[3];
-            shape(dn, lw.wdown, nullptr, dm.d, dm.F, M);
-            if constexpr (!PROD) {
-                dn.x = reinterpret_cast<const float*>(xrow(x_act())); dn.ldx = D.xch_ld;
-                dn.xpk = reinterpret_cast<const unsigned char*>(xrow(x_act())); dn.ldpk = D.xch_ld * 4; dn.poll = 1;
-                dn.epi = EPI_RESID; dn.resid = streamed() ? D.h : hx; dn.ldr = streamed() ? dm.d : D.xch_ld; dn.out = out.x; dn.ldo = dm.d;
-                dn.pk[0] = out.pk[0]; dn.pk[1] = out.pk[1]; dn.ldpk_out = (int)ldpk(); dn.ssq_out = out.ssq; dn.ld_sout = c.nctas;
-            }
-        }
-        if (!linear(&t->lin[0], true)) return false;
-        attention(&t->att);
+        float* hres = streamed ? D.h : x_h();
+        const int ldh = streamed ? dm.d : D.xch_ld;
+        LinArgs* o = out_proj(lw, M, in);
+        if (!o) return false;
+        o->out = hres; o->ldo = ldh;
+        o->pk[0] = PkOut{lw.g2, bytes(x_h())}; o->ldpk_out = D.xch_ld * 4;
+        o->ssq_out = x_ssq(); o->ld_sout = D.xch_ld;
+        commit();
+        LinArgs* gu = linear(lw.wgate, lw.wup, dm.F, dm.d, M);
+        if (!gu) return false;
+        gu->x = x_h(); gu->ldx = D.xch_ld; gu->gain = lw.g2; gu->xpk = bytes(x_h()); gu->ldpk = D.xch_ld * 4;
+        gu->ssq_in = x_ssq(); gu->ld_ssq = D.xch_ld; gu->poll = 1;
+        gu->epi = EPI_SWIGLU; gu->out = streamed ? nullptr : x_act(); gu->ldo = D.xch_ld;
+        gu->pk[0] = PkOut{nullptr, bytes(x_act())}; gu->ldpk_out = D.xch_ld * 4;
+        commit();
+        LinArgs* dn = linear(lw.wdown, nullptr, dm.d, dm.F, M);
+        if (!dn) return false;
+        dn->x = x_act(); dn->ldx = D.xch_ld; dn->xpk = bytes(x_act()); dn->ldpk = D.xch_ld * 4; dn->poll = 1;
+        dn->epi = EPI_RESID; dn->resid = hres; dn->ldr = ldh; dn->out = out.x; dn->ldo = dm.d;
+        dn->pk[0] = out.pk[0]; dn->pk[1] = out.pk[1]; dn->ldpk_out = (int)ldpk(); dn->ssq_out = out.ssq; dn->ld_sout = c.nctas;
+        commit_sync(14);
         turn_instance(M);
-        if (!linear(&t->lin[1], false)) return false;
-        if (!linear(&t->lin[2], false)) return false;
-        if (!linear(&t->lin[3], false)) return false;
-        KG_SYNC(14);
+        return true;
+    }
+    // Layers l0 .. l1 - 1 of a pass: `in` feeds the first one, `out` receives the last one's rows.
+    __device__ __forceinline__ bool layers(int l0, int l1, int M, int pos0, const ActIn in, const ActOut out) {
+        for (int i = l0; i < l1; ++i)
+            if (!layer(i, M, pos0, i == l0 ? in : act_h(), i == l1 - 1 ? out : out_h(next_gain(i)))) return false;
         return true;
     }
 
     // Adapter A (Section 3.1, Table 2): a = f + W^A_o Attn(RMSNorm(f; g_in)) on the rows `in` at pos0..;
     // with want_out == false only the adapter's K/V are appended (prefill).
-    __device__ bool run_adapter(int M, int pos0, const ActIn& in, bool want_out) {
-        const Dims& dm = D.dm;
-        OpTable* t = table();
-        const LayerW& lw = D.layers[dm.L];
-        fill_attention_block(t, lw, dm.L, M, pos0, in);
-        if constexpr (!PROD) {
-            if (writer(2)) {
-                LinArgs& o = t->lin[1];
-                o.out = D.abuf; o.ldo = dm.d;
-                o.pk[0] = PkOut{lw.g2, D.abuf_pk}; o.ldpk_out = (int)ldpk(); o.ssq_out = D.ssq_abuf; o.ld_sout = c.nctas;
-            }
+    __device__ bool adapter(int M, int pos0, const ActIn& in, bool want_out) {
+        const LayerW& lw = D.layers[D.dm.L];
+        if (!attention_block(lw, D.dm.L, M, pos0, in)) return false;
+        if (want_out) {
+            LinArgs* o = out_proj(lw, M, in);
+            if (!o) return false;
+            o->out = D.abuf; o->ldo = D.dm.d;
+            o->pk[0] = PkOut{lw.g2, D.abuf_pk}; o->ldpk_out = (int)ldpk(); o->ssq_out = D.ssq_abuf; o->ld_sout = c.nctas;
+            commit_sync(22);
+        } else {
+            if (!begin(OPK_NONE)) return false;
+            commit_sync(21);
         }
-        if (!linear(&t->lin[0], true)) return false;
-        attention(&t->att);
         turn_instance(M);
-        if (want_out && !linear(&t->lin[1], false)) return false;
-        KG_SYNC(22);
         return true;
     }
 
-    // Shared LM head on the rows `in` (norm gain `gain`), then the merged (token, p) per row: the same
-    // values in every thread of every CTA, the producer warp included (it receives them through
-    // shared memory and an mbarrier, which also holds it back until the result exists).
-    __device__ bool run_head(const ActIn& in, int M, const float* gain, float* dbg, int* toks, float* ps) {
+    // Shared LM head on the rows `in` (norm gain `gain`), then the merged (token, p) per row: the same values in every CTA.
+    __device__ __forceinline__ bool head(const ActIn in, int M, const float* gain, float* dbg, int* toks, float* ps) {
         const Dims& dm = D.dm;
-        OpTable* t = table();
-        if (writer()) {
-            LinArgs& a = t->lin[0];
-            shape(a, D.head, nullptr, dm.V, dm.d, M);
-            if constexpr (!PROD) {
-                a.x = in.x; a.ldx = dm.d; a.gain = gain; a.xpk = in.pk; a.ldpk = (int)ldpk(); a.ssq_in = in.ssq; a.ld_ssq = c.nctas;
-                a.epi = EPI_HEAD; a.scale = dm.logit_scale; a.head_part = D.head_part;
-                a.logits_dbg = dm.debug ? dbg : nullptr; a.ld_dbg = dm.V;
-            }
-        }
-        if (!linear(&t->lin[0], true)) return false;
-        if constexpr (PROD) {
-            // held back here until the consumers have the result
-            int ok = 1;
-            const unsigned mp = c.mail_phase;
-            if ((threadIdx.x & 31) == 0) ok = mbar_wait(c, &c.ctl->mail, mp, 42) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if ((threadIdx.x & 31) == 0) c.mail_phase = mp ^ 1u;      // the context is shared by the warp: one lane updates it
-            __syncwarp();
-            if (!ok) return false;
-        } else {
-            if (!grid_sync(c, 30)) return false;
-            for (int m = threadIdx.x >> 5; m < M; m += NWARPS) {           // one warp per row
-                int tk; float p;
-                head_final_warp(D.head_part, c.nctas, m, tk, p);
-                if ((threadIdx.x & 31) == 0) { c.ctl->head_tok[m] = tk; c.ctl->head_p[m] = p; }
-            }
-            cta_sync();
-            if (threadIdx.x == 0) mbar_arrive(&c.ctl->mail);
-        }
+        LinArgs* a = linear(D.head, nullptr, dm.V, dm.d, M);
+        if (!a) return false;
+        a->x = in.x; a->ldx = dm.d; a->gain = gain; a->xpk = in.pk; a->ldpk = (int)ldpk(); a->ssq_in = in.ssq; a->ld_ssq = c.nctas;
+        a->epi = EPI_HEAD; a->scale = dm.logit_scale; a->head_part = D.head_part;
+        a->logits_dbg = dm.debug ? dbg : nullptr; a->ld_dbg = dm.V;
+        commit_sync(30);
+        Op* o = begin(OPK_HEAD);
+        if (!o) return false;
+        o->emb.M = M;
+        commit();
+        if (!wait_mail()) return false;
         for (int i = 0; i < M; ++i) { toks[i] = c.ctl->head_tok[i]; ps[i] = c.ctl->head_p[i]; }
         return true;
     }
 
-    // ---- sequence state, replicated: every thread of every CTA holds the same values -----------
+    // ---- sequence state: the same values in every CTA
     int P, len_A, x0, total, rounds;
     int n_d, n_steps;
     int dtok[M_MAX];
@@ -280,32 +240,18 @@ struct Engine {
         n_d = __ldcg(&D.st->n_d); n_steps = __ldcg(&D.st->n_steps);
         for (int i = 0; i < M_MAX; ++i) { dtok[i] = __ldcg(&D.st->draft_tok[i]); dconf[i] = __ldcg(&D.st->conf[i]); }
     }
-    __device__ bool leader() const { return c.cta == 0 && threadIdx.x == 0; }
-
-    // the early-feature slot `slot` as an input of the adapter / of the first deep layer
-    __device__ __forceinline__ ActIn feat_for_adapter(int slot) const {
-        return ActIn{D.feat + (size_t)slot * D.dm.d, D.featA_pk + (size_t)slot * ldpk(), D.ssq_feat + (size_t)slot * c.nctas};
-    }
-    __device__ __forceinline__ ActIn feat_for_deep(int slot) const {
-        return ActIn{D.feat + (size_t)slot * D.dm.d, D.featD_pk + (size_t)slot * ldpk(), D.ssq_feat + (size_t)slot * c.nctas};
-    }
+    __device__ bool leader() const { return c.cta == 0; }
 
     // early feature of token `tok` at position pos -> feat slot (fp32 and packed for both of its readers)
     __device__ bool shallow_pass(int tok, int pos, int slot) {
         const Dims& dm = D.dm;
-        embed_rows(nullptr, tok, 1);
-        KG_SYNC(1);
-        for (int i = 0; i < dm.l; ++i) {
-            ActOut o = out_h(next_gain(i));
-            if (i == dm.l - 1) {
-                o.x = D.feat + (size_t)slot * dm.d;
-                o.pk[0] = PkOut{D.layers[dm.L].g1, D.featA_pk + (size_t)slot * ldpk()};
-                o.pk[1] = PkOut{D.layers[dm.l].g1, D.featD_pk + (size_t)slot * ldpk()};
-                o.ssq = D.ssq_feat + (size_t)slot * c.nctas;
-            }
-            if (!run_layer(i, 1, pos, act_h(), o)) return false;
-        }
-        return true;
+        if (!embed_rows(nullptr, tok, 1, 1)) return false;
+        ActOut o;
+        o.x = D.feat + (size_t)slot * dm.d;
+        o.pk[0] = PkOut{D.layers[dm.L].g1, D.featA_pk + (size_t)slot * ldpk()};
+        o.pk[1] = PkOut{D.layers[dm.l].g1, D.featD_pk + (size_t)slot * ldpk()};
+        o.ssq = D.ssq_feat + (size_t)slot * c.nctas;
+        return layers(0, dm.l, 1, pos, act_h(), o);
     }
 
     // Draft phase of one round (Section 3.2; Eq. 4; Figure 2).
@@ -318,10 +264,10 @@ struct Engine {
             if (!shallow_pass(cur, P + n_d, 1 + n_d)) return false;                 // f[n_d]
             if (n_d == pg.gamma || stop_after_shallow) break;
             const int MA = P + n_d - len_A + 1;                                     // 1, or 2 when the adapter cache lags
-            if (!run_adapter(MA, len_A, feat_for_adapter(1 + n_d - (MA - 1)), true)) return false;
-            int tk[M_MAX]; float pp[M_MAX];
+            if (!adapter(MA, len_A, feat_for_adapter(1 + n_d - (MA - 1)), true)) return false;
+            int tk[1]; float pp[1];
             const ActIn hin{D.abuf + (size_t)(MA - 1) * dm.d, D.abuf_pk + (size_t)(MA - 1) * ldpk(), D.ssq_abuf + (size_t)(MA - 1) * c.nctas};
-            if (!run_head(hin, 1, D.layers[dm.L].g2, D.dbg_draft + (size_t)n_steps * dm.V, tk, pp)) return false;
+            if (!head(hin, 1, D.layers[dm.L].g2, D.dbg_draft + (size_t)n_steps * dm.V, tk, pp)) return false;
             len_A += MA;
             dconf[n_steps] = pp[0];
             n_steps++;
@@ -344,23 +290,19 @@ struct Engine {
     __device__ bool verify_phase() {
         const Dims& dm = D.dm;
         const int M = n_d + 1;
-        for (int i = dm.l; i < dm.L; ++i)
-            if (!run_layer(i, M, P, (i == dm.l) ? feat_for_deep(1) : act_h(), out_h(next_gain(i)))) return false;
+        if (!layers(dm.l, dm.L, M, P, feat_for_deep(1), out_h(D.g_final))) return false;
         int t[M_MAX]; float pp[M_MAX];
-        if (!run_head(act_h(), M, D.g_final, D.dbg_verify, t, pp)) return false;
+        if (!head(act_h(), M, D.g_final, D.dbg_verify, t, pp)) return false;
         int k = 0;
         while (k < n_d && dtok[k] == t[k]) ++k;
         const int newP = P + k + 1;
         if (len_A > newP) len_A = newP;
-        if (len_A < newP && !PROD) {
+        if (len_A < newP) {
             // the adapter has not seen f[k] (k == n_d): keep it as the feature of position newP-1 (slot 0)
-            const int gtid = c.cta * NTHREADS + threadIdx.x, gn = c.nctas * NTHREADS;
-            const float* src = D.feat + (size_t)(1 + k) * dm.d;
-            for (int e = gtid; e < dm.d; e += gn) D.feat[e] = __ldcg(src + e);
-            const unsigned* psrc = reinterpret_cast<const unsigned*>(D.featA_pk + (size_t)(1 + k) * ldpk());
-            unsigned* pdst = reinterpret_cast<unsigned*>(D.featA_pk);
-            for (int e = gtid; e < dm.d; e += gn) pdst[e] = __ldcg(psrc + e);
-            for (int e = gtid; e < c.nctas; e += gn) D.ssq_feat[e] = __ldcg(D.ssq_feat + (size_t)(1 + k) * c.nctas + e);
+            Op* o = begin(OPK_KEEP);
+            if (!o) return false;
+            o->emb.M = 1 + k;
+            commit();
         }
         if (leader()) {
             State* st = D.st;
@@ -381,22 +323,24 @@ struct Engine {
     __device__ bool prefill() {
         const Dims& dm = D.dm;
         const int n = pg.n;
-        int tk[M_MAX]; float pp[M_MAX];
+        int tk[1]; float pp[1];
         tk[0] = 0;
         for (int c0 = 0; c0 < n; c0 += M_MAX) {
             const int M = min(M_MAX, n - c0);
-            embed_rows(D.prompt + c0, 0, M);
-            KG_SYNC(2);
-            for (int i = 0; i < dm.l; ++i) {
-                ActOut o = out_h(next_gain(i));
-                if (i == dm.l - 1) o.pk[1] = PkOut{D.layers[dm.L].g1, D.featA_pk};    // the adapter reads the same rows
-                if (!run_layer(i, M, c0, act_h(), o)) return false;
-            }
-            if (!run_adapter(M, c0, ActIn{D.h, D.featA_pk, D.ssq_hA}, false)) return false;
-            for (int i = dm.l; i < dm.L; ++i) if (!run_layer(i, M, c0, act_h(), out_h(next_gain(i)))) return false;
+            if (!embed_rows(D.prompt + c0, 0, M, 2)) return false;
+            ActOut o = out_h(next_gain(dm.l - 1));
+            o.pk[1] = PkOut{D.layers[dm.L].g1, D.featA_pk};    // the adapter reads the same rows
+            if (!layers(0, dm.l, M, c0, act_h(), o)) return false;
+            if (!adapter(M, c0, ActIn{D.h, D.featA_pk, D.ssq_hA}, false)) return false;
+            if (!layers(dm.l, dm.L, M, c0, act_h(), out_h(D.g_final))) return false;
             if (c0 + M == n) {
                 const ActIn hin{D.h + (size_t)(M - 1) * dm.d, D.hA_pk + (size_t)(M - 1) * ldpk(), D.ssq_hA + (size_t)(M - 1) * c.nctas};
-                if (!run_head(hin, 1, D.g_final, D.dbg_verify, tk, pp)) return false;
+                if (!head(hin, 1, D.g_final, D.dbg_verify, tk, pp)) return false;
+            } else {
+                // the next chunk attends to this one's rows: the copy warp must not run ahead of the barrier behind them
+                if (!begin(OPK_MAIL)) return false;
+                commit();
+                if (!wait_mail()) return false;
             }
         }
         if (leader()) {
@@ -408,13 +352,11 @@ struct Engine {
     }
 
     __device__ bool ar_decode() {
-        const Dims& dm = D.dm;
-        int tk[M_MAX]; float pp[M_MAX];
+        int tk[1]; float pp[1];
         while (total < pg.n) {
-            embed_rows(nullptr, x0, 1);
-            KG_SYNC(3);
-            for (int i = 0; i < dm.L; ++i) if (!run_layer(i, 1, P, act_h(), out_h(next_gain(i)))) return false;
-            if (!run_head(act_h(), 1, D.g_final, D.dbg_verify, tk, pp)) return false;
+            if (!embed_rows(nullptr, x0, 1, 3)) return false;
+            if (!layers(0, D.dm.L, 1, P, act_h(), out_h(D.g_final))) return false;
+            if (!head(act_h(), 1, D.g_final, D.dbg_verify, tk, pp)) return false;
             if (leader()) {
                 D.out_tokens[total] = tk[0];
                 D.st->P = P + 1; D.st->x0 = tk[0]; D.st->total = total + 1; D.st->len_A = -1;
@@ -425,47 +367,150 @@ struct Engine {
     }
 
     __device__ bool run_program() {
-        switch (pg.kind) {
-            case PROG_PREFILL: return prefill();
-            case PROG_DRAFT: return draft_phase();
-            case PROG_VERIFY: return verify_phase();
-            case PROG_AR: return ar_decode();
-            case PROG_DECODE:
-                while (total < pg.n) {
-                    if (!draft_phase()) return false;
-                    if (!verify_phase()) return false;
-                }
-                return true;
+        if (pg.kind == PROG_PREFILL) return prefill();
+        if (pg.kind == PROG_AR) return ar_decode();
+        const bool draft = pg.kind != PROG_VERIFY, verify = pg.kind != PROG_DRAFT, once = pg.kind != PROG_DECODE;
+        while (once || total < pg.n) {
+            if (draft && !draft_phase()) return false;
+            if (verify && !verify_phase()) return false;
+            if (once) break;
         }
         return true;
     }
 
     __device__ void run() {
-        // the plain path streams nothing: its producer warp has no part in the launch
-        if (PROD && !streamed()) return;
         load_state();
-        xp = 0; xused = 0;                       // a launch finds both exchange instances empty and leaves them so
-        const bool ok = run_program();
-        if (!ok && PROD) ring_drain(c);
-        if constexpr (!PROD) { if (ok) empty_instance(xp ^ 1); }
+        if (!run_program()) return;              // a wait gave up: the abort flag ends the other roles
+        // a launch finds both exchange instances empty and leaves them so
+        Op* o = begin(OPK_EXIT);
+        if (!o) return;
+        o->empty_p = xp ^ 1; o->empty_rows = xused;
+        commit();
     }
 };
 
+// ---- the copy warp ---------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void copy_loop(const Dev& D, Ctx& c, bool streamed) {
+    Ctrl* ctl = c.ctl;
+    const int lane = threadIdx.x & 31;
+    int q = 0; unsigned qph = 0;
+    bool ok = true, done = false;
+    while (ok && !done) {
+        int w = 1;
+        if (lane == 0) w = mbar_wait(c, &ctl->qfull[q], qph, 34) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, w, 0) != 0;
+        if (!ok) break;
+        const Op& op = ctl->queue[q];
+        const int kind = op.kind;
+        if (streamed && kind == OPK_LIN) ok = lin_produce(op.lin, c);
+        else if (streamed && kind == OPK_ATT && D.dm.ring) ok = attention_producer(D, op.att.plan, op.att.row0, c);
+        done = kind == OPK_EXIT;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->qempty[q]);
+        if (++q == QUEUE) { q = 0; qph ^= 1u; }
+    }
+    if (!ok) ring_drain(c);
+}
+
+// ---- the consumer warps ----------------------------------------------------------------------------------------------
+// true when the predicate holds in every consumer thread (a barrier among them)
+__device__ __forceinline__ bool cta_all(bool p) {
+    unsigned r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"((unsigned)p), "n"(NTHREADS) : "memory");
+    return r != 0;
+}
+
 template <typename WT>
-__global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const Program pg) {
+__device__ __forceinline__ void consume_embed(const Dev& D, Ctx& c, const EmbedArgs& e, bool streamed) {
+    const int d = D.dm.d, M = e.M;
+    const int* toks = e.toks; const int tok1 = e.tok;
+    const WT* E = reinterpret_cast<const WT*>(D.embed);
+    // an id outside [0, V) never indexes the embedding table (ids that arrive in device memory are checked by a
+    // kernel of their own, which records the error; here the access is merely kept in bounds)
+    auto row = [&](int m) { const int tok = toks ? __ldcg(toks + m) : tok1; return E + (size_t)((unsigned)tok < (unsigned)D.dm.V ? tok : 0) * d; };
+    if (!streamed) {
+        for (int idx = c.cta * NTHREADS + threadIdx.x; idx < M * d; idx += c.nctas * NTHREADS) D.h[idx] = wt_to_float<WT>(row(idx / d)[idx % d]);
+        return;
+    }
+    LinArgs a{};
+    a.N = d; a.M = M; a.out = D.h; a.ldo = d;
+    a.pk[0] = PkOut{D.layers[0].g1, D.hA_pk}; a.ldpk_out = d * 4; a.ssq_out = D.ssq_hA; a.ld_sout = c.nctas;
+    emit_plain_rows(a, c, [&](int m, int e_) { return wt_to_float<WT>(row(m)[e_]); });
+}
+
+template <typename WT>
+__device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed) {
+    Ctrl* ctl = c.ctl;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int q = 0; unsigned qph = 0;
+    while (true) {
+        if (!cta_all(mbar_wait(c, &ctl->qfull[q], qph, 31))) return;
+        const Op& op = ctl->queue[q];
+        const int kind = op.kind;
+        if (kind == OPK_LIN) {
+            const LinArgs& a = op.lin;
+            if (!streamed) lin_simple<WT>(a, c);
+            else if constexpr (sizeof(WT) == 2) {
+                if (a.M <= 4) lin_consume<4>(a, c); else if (a.M <= 8) lin_consume<8>(a, c); else if (a.M <= 12) lin_consume<12>(a, c); else lin_consume<16>(a, c);
+            }
+        } else if (kind == OPK_ATT) {
+            const AttArgs& a = op.att;
+            attention_op<WT>(D, a, c, streamed && D.dm.ring);
+        } else if (kind == OPK_EMBED) {
+            consume_embed<WT>(D, c, op.emb, streamed);
+        } else if (kind == OPK_HEAD) {
+            const int M = op.emb.M;
+            for (int m = warp; m < M; m += NWARPS) {                       // one warp per row
+                int tk; float p;
+                head_final_warp(D.head_part, c.nctas, m, tk, p);
+                if (lane == 0) { ctl->head_tok[m] = tk; ctl->head_p[m] = p; }
+            }
+            cta_sync();
+            if (tid == 0) mbar_arrive(&ctl->mail);
+        } else if (kind == OPK_MAIL) {
+            if (tid == 0) mbar_arrive(&ctl->mail);                         // (thread 0 polled the grid barrier that came before)
+        } else if (kind == OPK_KEEP) {
+            // early feature of slot emb.M -> slot 0
+            const int s = op.emb.M, d = D.dm.d;
+            const int gtid = c.cta * NTHREADS + tid, gn = c.nctas * NTHREADS;
+            const float* src = D.feat + (size_t)s * d;
+            for (int e = gtid; e < d; e += gn) D.feat[e] = __ldcg(src + e);
+            const unsigned* psrc = reinterpret_cast<const unsigned*>(D.featA_pk + (size_t)s * d * 4);
+            unsigned* pdst = reinterpret_cast<unsigned*>(D.featA_pk);
+            for (int e = gtid; e < d; e += gn) pdst[e] = __ldcg(psrc + e);
+            for (int e = gtid; e < c.nctas; e += gn) D.ssq_feat[e] = __ldcg(D.ssq_feat + (size_t)s * c.nctas + e);
+        }
+        if (kind == OPK_ATT || kind == OPK_EXIT) {
+            const int n4 = op.empty_rows * (D.xch_ld >> 2);
+            uint4* x = reinterpret_cast<uint4*>(D.xch[op.empty_p]);
+            for (int i = c.cta * NTHREADS + tid; i < n4; i += c.nctas * NTHREADS) x[i] = make_uint4(XCH_EMPTY, XCH_EMPTY, XCH_EMPTY, XCH_EMPTY);
+        }
+        const int where = op.sync;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->qempty[q]);
+        if (where && !grid_sync(c, where)) return;
+        if (kind == OPK_EXIT) return;
+        if (++q == QUEUE) { q = 0; qph ^= 1u; }
+    }
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const __grid_constant__ Program pg) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival);
     if (threadIdx.x >= NTHREADS) {
-        // the producer's warpgroup: keeps what the copy loop needs and returns the rest of its registers
+        // the third warpgroup: keeps what the copy loop and the sequencer need and returns the rest of its registers
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PRODUCER_REGS));
-        if (threadIdx.x < BLOCK_THREADS) {
-            Engine<WT, true> eng(D, c, pg);
-            eng.run();
+        const int w = (threadIdx.x - NTHREADS) >> 5;
+        if (w == 0) copy_loop(D, c, launch_streamed(D, pg));
+        else if (w == 1 && (threadIdx.x & 31) == 0) {
+            Sequencer<WT> seq(D, c, pg);
+            seq.run();
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
-        Engine<WT, false> eng(D, c, pg);
-        eng.run();
+        consume_loop<WT>(D, c, launch_streamed(D, pg));
     }
 }
 

@@ -48,7 +48,7 @@ struct GemmArgs {
     float* C; const float* resid; int ldc;      // PF_STORE: C = (resid) + product; C may be resid itself
     __nv_bfloat16* hi; __nv_bfloat16* lo; int ldp;      // PF_SWIGLU: planes of SiLU(gate) * up; PF_QKV: planes of the rotated, scaled q
     int hd, H, sec0, pos0;              // PF_QKV: sec0 = first section of W's rows (0: q, k, v; 1: k, v only)
-    const float2* cs;                   // PF_QKV: cos, sin [rows][hd / 2]
+    const float2* cs;                   // PF_QKV: cos, sin [rows][hd / 2] of the block's positions
     const int* page_table; int ps_shift, n_phys; State* st;
     __nv_bfloat16* kc; __nv_bfloat16* vc;
     float qscale;
@@ -505,11 +505,6 @@ template <int HD> struct FaSm { static constexpr int TILE = FA_KEYS * HD * 2, BY
 __device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
 }
-__device__ __forceinline__ void ldmatrix_x4_trans(unsigned (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-
 struct FaArgs {
     const __nv_bfloat16* qh; const __nv_bfloat16* ql;    // [rows][d] rotated, scaled q
     const __nv_bfloat16* kc; const __nv_bfloat16* vc;    // this layer's cache
@@ -674,10 +669,10 @@ __global__ void __launch_bounds__(256) pf_embed_kernel(const int* toks, const __
     }
 }
 
-// cos, sin of every (row, pair of dims) of a block of rows, once for all layers; grid = rows, hd / 2 threads
-__global__ void pf_rope_table_kernel(const __grid_constant__ Dev D, int pos0, float2* cs) {
+// cos, sin of every (position, pair of dims), once per model; grid = positions, hd / 2 threads
+__global__ void rope_table_kernel(const __grid_constant__ Dev D, float2* cs) {
     float c, s;
-    rope_cs(D, pos0 + blockIdx.x, threadIdx.x, c, s);
+    rope_cs(D, blockIdx.x, threadIdx.x, c, s);
     cs[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = make_float2(c, s);
 }
 

@@ -1,0 +1,52 @@
+"""The attention that reads its keys from the weight ring, at the edges of its tiles, splits and pages, against float64."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2404_18911_b200 import binding as b
+    b.load()
+    return torch, b
+
+
+# no old keys, one key, whole and partial tiles of 16, more than one ring slot, more than one wave of items; both row groups;
+# pages smaller and larger than a tile
+@pytest.mark.parametrize("H,hd", [(3, 128), (40, 128), (5, 64)])
+@pytest.mark.parametrize("M,pos0,ps", [(1, 0, 16), (16, 0, 4), (3, 1, 1), (8, 15, 16), (9, 16, 32), (1, 17, 2), (7, 127, 8), (16, 1040, 16), (2, 3001, 64)])
+def test_attention_ring(env, H, hd, M, pos0, ps):
+    torch, b = env
+    g = torch.Generator(device="cuda").manual_seed(pos0 * 17 + M)
+    T, d = pos0 + M, H * hd
+    pages = (T + ps - 1) // ps + 3
+    # rows that no key lives in hold NaN: nothing of them may reach a result
+    kc, vc = (torch.full((pages, H, ps, hd), float("nan"), device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    table = torch.randperm(pages, generator=g, device="cuda").to(torch.int32)
+    pos = torch.arange(pos0, device="cuda")
+    past = torch.empty(2, pos0, H, hd, device="cuda", dtype=torch.bfloat16).normal_(generator=g)
+    kc[table[pos // ps].long(), :, pos % ps] = past[0]
+    vc[table[pos // ps].long(), :, pos % ps] = past[1]
+    qkv = torch.empty(M, 3 * d, device="cuda").normal_(generator=g)
+    out = b.op_attention(qkv, pos0, H, hd, 10000.0, kc, vc, table, ps)
+    out2 = b.op_attention(qkv, pos0, H, hd, 10000.0, kc, vc, table, ps)      # the appended rows are there already
+    assert torch.equal(out, out2)
+    new = torch.arange(pos0, T, device="cuda")
+    at = table[torch.arange(T, device="cuda") // ps].long()
+    K = kc[at, :, torch.arange(T, device="cuda") % ps].double()
+    V = vc[at, :, torch.arange(T, device="cuda") % ps].double()
+    inv = 10000.0 ** (-2 * torch.arange(hd // 2, device="cuda").double() / hd)
+    cs, sn = torch.cos(new.double()[:, None] * inv)[:, None], torch.sin(new.double()[:, None] * inv)[:, None]
+    rot = lambda x: torch.cat([x[..., :hd // 2] * cs - x[..., hd // 2:] * sn, x[..., hd // 2:] * cs + x[..., :hd // 2] * sn], -1)
+    q, k, v = (qkv.double().reshape(M, 3, H, hd)[:, i] for i in range(3))
+    # the rows written: bf16 of the rotated k and of v (one ulp where the rounding of a float32 rotation falls the other way)
+    assert (K[pos0:] - rot(k)).abs().max() < 2 ** -8 * 8 and torch.equal(V[pos0:], v.to(torch.bfloat16).double())
+    S = torch.einsum("mhd,thd->hmt", rot(q), K) / hd ** 0.5
+    S = S.masked_fill(torch.arange(T, device="cuda")[None, None] > new[None, :, None], float("-inf"))
+    ref = torch.einsum("hmt,thd->mhd", torch.softmax(S, -1), V).reshape(M, d)
+    # q and p keep 17 bits, fp32 sums: about 5e-6 of the norm is seen, at most 7e-5 of the root mean square in one element
+    e = out.double() - ref
+    assert e.norm() / ref.norm() < 2e-5 and e.abs().max() < 3e-4 * ref.square().mean().sqrt().clamp_min(0.05)
