@@ -295,8 +295,17 @@ extern "C" size_t kg_workspace_bytes(const kg_config* cfg, int own_weights) {
     return make_layout(cfg, own_weights, sm_count()).total + 256;
 }
 
-template <typename WT>
-static int launch_program(kg_model* m, const Program& pg) {
+// The decode kernel for a storage type and head size
+static const void* decode_kernel(const kg_config& c) {
+    if (c.dtype == KG_BF16) {
+        if (c.head_dim == 128) return (const void*)kg_persistent_kernel<__nv_bfloat16, 128>;
+        return c.head_dim == 64 ? (const void*)kg_persistent_kernel<__nv_bfloat16, 64> : (const void*)kg_persistent_kernel<__nv_bfloat16, 32>;
+    }
+    if (c.head_dim == 128) return (const void*)kg_persistent_kernel<float, 128>;
+    return c.head_dim == 64 ? (const void*)kg_persistent_kernel<float, 64> : (const void*)kg_persistent_kernel<float, 32>;
+}
+
+static int launch(kg_model* m, const Program& pg) {
     CK(cudaMemsetAsync(m->dev.bar, 0, BAR_BYTES, m->stream));
     Program p = pg;
     p.force_simple = m->force_simple;
@@ -304,11 +313,8 @@ static int launch_program(kg_model* m, const Program& pg) {
     p.skip_arrival = m->skip_arrival;
     m->skip_arrival = 0;
     void* args[] = {(void*)&m->dev, (void*)&p};
-    CK(cudaLaunchCooperativeKernel((const void*)kg_persistent_kernel<WT>, dim3(m->nctas), dim3(DECODE_THREADS), args, m->smem, m->stream));
+    CK(cudaLaunchCooperativeKernel(decode_kernel(m->cfg), dim3(m->nctas), dim3(DECODE_THREADS), args, m->smem, m->stream));
     return KG_OK;
-}
-static int launch(kg_model* m, const Program& pg) {
-    return m->cfg.dtype == KG_BF16 ? launch_program<__nv_bfloat16>(m, pg) : launch_program<float>(m, pg);
 }
 
 static int read_state(kg_model* m, State* out) {
@@ -403,7 +409,7 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     m->smem = SMEM_TOTAL;
 
     const bool bf = cfg->dtype == KG_BF16;
-    const void* kfn = bf ? (const void*)kg_persistent_kernel<__nv_bfloat16> : (const void*)kg_persistent_kernel<float>;
+    const void* kfn = decode_kernel(*cfg);
     if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem) != cudaSuccess) { delete m; return KG_E_CUDA; }
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, DECODE_THREADS, m->smem) != cudaSuccess || occ < 1) { delete m; return KG_E_CUDA; }
@@ -922,13 +928,13 @@ __global__ void op_head_final_kernel(const float4* part, int nctas, int* tok, fl
     head_final_warp(part, nctas, m, t, pp);
     if ((threadIdx.x & 31) == 0) { tok[m] = t; p[m] = pp; }
 }
-template <typename WT>
+template <typename WT, int HD>
 __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __grid_constant__ Dev D, AttArgs a) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
     if (!c.producer) {
         if (D.dm.ring) a.plan = ra_plan(a.pos0, D.dm.H, c.nctas);
-        attention_op<WT>(D, a, c, D.dm.ring != 0);
+        attention_op<WT, HD>(D, a, c, D.dm.ring != 0);
     } else if (D.dm.ring) {
         if (!attention_producer(D, ra_plan(a.pos0, D.dm.H, c.nctas), 0, c)) ring_drain(c);
     }
@@ -1078,6 +1084,13 @@ extern "C" int kg_op_lm_head_noalloc(int32_t dtype, const void* W, int32_t V, in
     return KG_OK;
 }
 
+template <typename WT, int HD>
+static int launch_attention(const Dev& D, const AttArgs& a, int nctas, cudaStream_t s) {
+    if (set_smem<op_attention_kernel<WT, HD>>() != KG_OK) return KG_E_CUDA;
+    op_attention_kernel<WT, HD><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
+    return KG_OK;
+}
+
 extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32_t pos0, int32_t H, int32_t hd,
                                float theta, void* kc, void* vc, const int32_t* page_table, int32_t page_size,
                                float* out, void* scratch, void* stream) {
@@ -1111,13 +1124,9 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     }
     AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
-    if (dtype == KG_BF16) {
-        if (set_smem<op_attention_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
-        op_attention_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
-    } else {
-        if (set_smem<op_attention_kernel<float>>() != KG_OK) return KG_E_CUDA;
-        op_attention_kernel<float><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
-    }
+    const int r = dtype == KG_BF16 ? (hd == 128 ? launch_attention<__nv_bfloat16, 128>(D, a, nctas, s) : hd == 64 ? launch_attention<__nv_bfloat16, 64>(D, a, nctas, s) : launch_attention<__nv_bfloat16, 32>(D, a, nctas, s))
+                                   : (hd == 128 ? launch_attention<float, 128>(D, a, nctas, s) : hd == 64 ? launch_attention<float, 64>(D, a, nctas, s) : launch_attention<float, 32>(D, a, nctas, s));
+    if (r != KG_OK) return r;
     CK(cudaGetLastError());
     return KG_OK;
 }

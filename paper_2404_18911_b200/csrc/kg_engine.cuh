@@ -14,6 +14,8 @@
 // operators as functions from a dozen places: they were compiled for the 168 registers of the launch (the warpgroups' own budgets
 // reach inlined code only), what the callers kept across them was spilled - beside 227 KB of shared memory there is hardly any L1,
 // so that a spilled register is an L2 access -, and each layer began with one thread writing its arguments while 255 waited.
+// 7B, KV 512, with the attention fed by the ring: verify pass of one row 2.74 -> 2.58 ms, of seven rows 3.42 -> 3.19, draft step
+// 0.328 -> 0.300, greedy step 2.87 -> 2.70.
 #pragma once
 
 #include "kg_device.cuh"
@@ -439,7 +441,7 @@ __device__ __forceinline__ void consume_embed(const Dev& D, Ctx& c, const EmbedA
     emit_plain_rows(a, c, [&](int m, int e_) { return wt_to_float<WT>(row(m)[e_]); });
 }
 
-template <typename WT>
+template <typename WT, int HD>
 __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed) {
     Ctrl* ctl = c.ctl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -456,7 +458,7 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
             }
         } else if (kind == OPK_ATT) {
             const AttArgs& a = op.att;
-            attention_op<WT>(D, a, c, streamed && D.dm.ring);
+            attention_op<WT, HD>(D, a, c, streamed && D.dm.ring);
         } else if (kind == OPK_EMBED) {
             consume_embed<WT>(D, c, op.emb, streamed);
         } else if (kind == OPK_HEAD) {
@@ -495,7 +497,8 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
     }
 }
 
-template <typename WT>
+// HD: the head size, compiled apart (with both of them in one kernel 0.9 KB of registers were spilled around the operators)
+template <typename WT, int HD>
 __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const __grid_constant__ Program pg) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival);
@@ -510,7 +513,7 @@ __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const 
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
-        consume_loop<WT>(D, c, launch_streamed(D, pg));
+        consume_loop<WT, HD>(D, c, launch_streamed(D, pg));
     }
 }
 
