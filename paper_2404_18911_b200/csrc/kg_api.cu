@@ -910,15 +910,22 @@ OpScratch op_layout() {
     return s;
 }
 
-template <typename WT>
-__global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(const __grid_constant__ LinArgs a, int stream) {
+// One linear operator as a kernel of its own.  V: the row variant of the streamed tensor-core path (bf16 weights, K a multiple of
+// 16), 0: the plain path; compiled one by one, because all variants in one kernel spill at its 168 registers.
+template <typename WT, int V>
+__global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(const __grid_constant__ LinArgs a) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
-    // launched while the kernel that packs the rows may still run: the copy warp starts on the weights at once
     grid_dependents_launch();
-    if (!c.producer) grid_dependency_wait();
-    const bool ok = linear_op<WT>(a, c, stream != 0);
-    if (!ok && c.producer) ring_drain(c);
+    if constexpr (V == 0) {
+        if (!c.producer) lin_simple<WT>(a, c);
+    } else if (c.producer) {
+        // launched while the kernel that packs the rows may still run: the copy warp starts on the weights at once
+        if (!lin_produce(a, c)) ring_drain(c);
+    } else {
+        grid_dependency_wait();
+        lin_consume<V>(a, c);
+    }
 }
 // one warp per row (one thread per row took 60 us: a chain of a merge per CTA)
 __global__ void op_head_final_kernel(const float4* part, int nctas, int* tok, float* p) {
@@ -928,13 +935,13 @@ __global__ void op_head_final_kernel(const float4* part, int nctas, int* tok, fl
     head_final_warp(part, nctas, m, t, pp);
     if ((threadIdx.x & 31) == 0) { tok[m] = t; p[m] = pp; }
 }
-template <typename WT, int HD>
+template <typename WT, int HD, int R>
 __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __grid_constant__ Dev D, AttArgs a) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
     if (!c.producer) {
         if (D.dm.ring) a.plan = ra_plan(a.pos0, D.dm.H, c.nctas);
-        attention_op<WT, HD>(D, a, c, D.dm.ring != 0);
+        attention_op<WT, HD, R>(D, a, c, D.dm.ring != 0);
     } else if (D.dm.ring) {
         if (!attention_producer(D, ra_plan(a.pos0, D.dm.H, c.nctas), 0, c)) ring_drain(c);
     }
@@ -975,6 +982,19 @@ extern "C" size_t kg_op_scratch_bytes(void) { return op_layout().total; }
 
 extern "C" int kg_debug_force_simple_ops(int on) { g_force_simple_ops = on ? 1 : 0; return KG_OK; }
 
+template <int V>
+static int launch_linear(const LinArgs& a, int nctas, cudaStream_t s) {
+    if (set_smem<op_linear_kernel<__nv_bfloat16, V>>() != KG_OK) return KG_E_CUDA;
+    CK(launch_dependent(op_linear_kernel<__nv_bfloat16, V>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a));
+    return KG_OK;
+}
+template <typename WT>
+static int launch_plain(const LinArgs& a, int nctas, cudaStream_t s) {
+    if (set_smem<op_linear_kernel<WT, 0>>() != KG_OK) return KG_E_CUDA;
+    op_linear_kernel<WT, 0><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
+    return KG_OK;
+}
+
 // xpk / ssq: scratch for the packed copy of the input rows (xpk_k_max = longest row it holds) and their sums of squares
 static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int xpk_k_max, float* ssq, cudaStream_t s) {
     if (dtype != KG_F32 && dtype != KG_BF16) return KG_E_ARG;
@@ -987,14 +1007,11 @@ static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int x
         pack_rows_kernel<<<nctas, 256, 0, s>>>(a.x, a.ldx, a.M, a.K, a.gain, xpk, a.K * 4, a.gain ? ssq : nullptr, nctas);
         a.xpk = xpk; a.ldpk = a.K * 4; a.ssq_in = a.gain ? ssq : nullptr; a.ld_ssq = nctas;
     }
-    if (dtype == KG_BF16) {
-        if (set_smem<op_linear_kernel<__nv_bfloat16>>() != KG_OK) return KG_E_CUDA;
-        if (plain) op_linear_kernel<__nv_bfloat16><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
-        else CK(launch_dependent(op_linear_kernel<__nv_bfloat16>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a, 1));
-    } else {
-        if (set_smem<op_linear_kernel<float>>() != KG_OK) return KG_E_CUDA;
-        op_linear_kernel<float><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 0);
-    }
+    int r;
+    if (dtype == KG_F32) r = launch_plain<float>(a, nctas, s);
+    else if (plain) r = launch_plain<__nv_bfloat16>(a, nctas, s);
+    else r = a.M <= 4 ? launch_linear<4>(a, nctas, s) : a.M <= 8 ? launch_linear<8>(a, nctas, s) : a.M <= 12 ? launch_linear<12>(a, nctas, s) : launch_linear<16>(a, nctas, s);
+    if (r != KG_OK) return r;
     CK(cudaGetLastError());
     return KG_OK;
 }
@@ -1084,10 +1101,10 @@ extern "C" int kg_op_lm_head_noalloc(int32_t dtype, const void* W, int32_t V, in
     return KG_OK;
 }
 
-template <typename WT, int HD>
+template <typename WT, int HD, int R>
 static int launch_attention(const Dev& D, const AttArgs& a, int nctas, cudaStream_t s) {
-    if (set_smem<op_attention_kernel<WT, HD>>() != KG_OK) return KG_E_CUDA;
-    op_attention_kernel<WT, HD><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
+    if (set_smem<op_attention_kernel<WT, HD, R>>() != KG_OK) return KG_E_CUDA;
+    op_attention_kernel<WT, HD, R><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
     return KG_OK;
 }
 
@@ -1124,8 +1141,12 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     }
     AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
-    const int r = dtype == KG_BF16 ? (hd == 128 ? launch_attention<__nv_bfloat16, 128>(D, a, nctas, s) : hd == 64 ? launch_attention<__nv_bfloat16, 64>(D, a, nctas, s) : launch_attention<__nv_bfloat16, 32>(D, a, nctas, s))
-                                   : (hd == 128 ? launch_attention<float, 128>(D, a, nctas, s) : hd == 64 ? launch_attention<float, 64>(D, a, nctas, s) : launch_attention<float, 32>(D, a, nctas, s));
+    typedef __nv_bfloat16 bf;
+    int r;
+    if (dtype == KG_F32) r = hd == 128 ? launch_attention<float, 128, 1>(D, a, nctas, s) : hd == 64 ? launch_attention<float, 64, 1>(D, a, nctas, s) : launch_attention<float, 32, 1>(D, a, nctas, s);
+    else if (hd == 32) r = launch_attention<bf, 32, 1>(D, a, nctas, s);
+    else if (M <= 8) r = hd == 128 ? launch_attention<bf, 128, 1>(D, a, nctas, s) : launch_attention<bf, 64, 1>(D, a, nctas, s);
+    else r = hd == 128 ? launch_attention<bf, 128, 2>(D, a, nctas, s) : launch_attention<bf, 64, 2>(D, a, nctas, s);
     if (r != KG_OK) return r;
     CK(cudaGetLastError());
     return KG_OK;
@@ -1206,7 +1227,7 @@ int prefill_tc_init(kg_model* m) {
     if ((r = gemm_attributes<PF_STORE>()) != KG_OK || (r = gemm_attributes<PF_QKV>()) != KG_OK || (r = gemm_attributes<PF_SWIGLU>()) != KG_OK) return r;
     CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<128>::BYTES));
     CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<64>::BYTES));
-    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
+    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
     CK(cudaMemsetAsync(A + m->lay.off_pf_cnt, 0, 4 * (size_t)m->nctas, m->stream));
     m->pf.ready = true;
     return KG_OK;
@@ -1337,7 +1358,7 @@ int prefill_tc(kg_model* m, int n) {
         a.xpk = D.hA_pk; a.ldpk = d * 4; a.ssq_in = D.ssq_hA; a.ld_ssq = m->nctas;
         a.epi = EPI_HEAD; a.scale = c.logit_scale; a.head_part = D.head_part;
         a.logits_dbg = c.debug_logits ? D.dbg_verify : nullptr; a.ld_dbg = c.vocab;
-        op_linear_kernel<WT><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a, 1);
+        op_linear_kernel<WT, 4><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
         pf_finish_kernel<<<1, 32, 0, s>>>(D.head_part, m->nctas, D.st, D.out_tokens, n, err);
         CK(cudaGetLastError());
     }

@@ -1163,18 +1163,6 @@ __device__ __noinline__ void lin_simple(const LinArgs& a, Ctx& c) {
     cta_sync();
 }
 
-// One linear operator, called by every thread of the CTA of a single-operator kernel; `stream` selects the streamed tensor-core
-// path (bf16 weights, every K a multiple of 16).  The copy warp returns false when one of its waits gave up.
-template <typename WT>
-__device__ __forceinline__ bool linear_op(const LinArgs& a, Ctx& c, bool stream) {
-    if (c.producer) return !stream || lin_produce(a, c);
-    if (!stream) { lin_simple<WT>(a, c); return true; }
-    if constexpr (sizeof(WT) == 2) {
-        if (a.M <= 4) lin_consume<4>(a, c); else if (a.M <= 8) lin_consume<8>(a, c); else if (a.M <= 12) lin_consume<12>(a, c); else lin_consume<16>(a, c);
-    }
-    return true;
-}
-
 // Merge the per-CTA head partials of row m by a whole warp (identical result in every CTA): every lane merges the partials of CTAs lane, lane + 32, ... (independent loads, one
 // round trip instead of one per CTA), then a butterfly of merges leaves the identical total in every lane (the merge
 // of two partials is the same whichever of the two lanes computes it).
@@ -1987,12 +1975,14 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
     c.slot = slot; c.phase = phase;
 }
 
-// ring: the tensor-core attention, fed by the copy warp (decided once per model: bf16 streamed path, head_dim 64 or 128)
-template <typename WT, int HD>
+// ring: the tensor-core attention, fed by the copy warp (decided once per model: bf16 streamed path, head_dim 64 or 128).
+// R: row groups, 1 or 2, or 0 where both may come.
+template <typename WT, int HD, int R = 0>
 __device__ __forceinline__ void attention_op(const Dev& D, const AttArgs& a, Ctx& c, bool ring) {
     if constexpr (sizeof(WT) == 2 && HD >= 64) {
         if (ring) {
-            if (a.M <= 8) attention_ring<HD, 1>(D, a, c); else attention_ring<HD, 2>(D, a, c);
+            if constexpr (R != 0) attention_ring<HD, R>(D, a, c);
+            else if (a.M <= 8) attention_ring<HD, 1>(D, a, c); else attention_ring<HD, 2>(D, a, c);
             return;
         }
     }
