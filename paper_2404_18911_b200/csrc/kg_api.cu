@@ -1272,8 +1272,7 @@ void gm_plan(GemmArgs& g, int wtiles, int pairs, size_t part_bytes) {
 template <int EPI>
 int gm_launch(GemmArgs& g, const CUtensorMap& hi, const CUtensorMap& lo, const CUtensorMap& w, const CUtensorMap& w2, int pairs, cudaStream_t s) {
     const int used = g.items < pairs ? g.items : pairs;
-    pf_gemm_kernel<EPI><<<2 * used, GM_THREADS, GM_SMEM, s>>>(hi, lo, w, w2, g);
-    CK(cudaGetLastError());
+    CK(launch_dependent(pf_gemm_kernel<EPI>, dim3(2 * used), dim3(GM_THREADS), GM_SMEM, s, hi, lo, w, w2, g));
     return KG_OK;
 }
 
@@ -1305,7 +1304,7 @@ int prefill_tc(kg_model* m, int n) {
         pf_embed_kernel<<<rows, 256, 0, s>>>(D.prompt + b0, (const WT*)D.embed, c.vocab, d, h);
         GemmArgs base{};
         base.rows = rows; base.err = err; base.part = (float*)(A + m->lay.off_pf_part); base.cnt = (unsigned*)(A + m->lay.off_pf_cnt);
-        auto norm = [&](const float* gain) { pf_norm_split_kernel<<<rows, PF_EW_THREADS, 0, s>>>(h, d, d, gain, c.rms_eps, xh, xl, rs); };
+        auto norm = [&](const float* gain) { return launch_dependent(pf_norm_split_kernel, dim3(rows), dim3(PF_EW_THREADS), 0, s, h, d, d, gain, c.rms_eps, xh, xl, rs); };
         auto qkv = [&](const CUtensorMap& w, int li, int sec0) {
             GemmArgs g = base;
             g.N = (3 - sec0) * d; g.K = d; g.rowscale = rs; g.hi = qh; g.lo = ql; g.ldp = d; g.hd = hd; g.H = H; g.sec0 = sec0; g.pos0 = b0;
@@ -1327,24 +1326,24 @@ int prefill_tc(kg_model* m, int n) {
             const LayerW& lw = m->layers_host[i];
             const PfMaps::Layer& tm = m->pf.layer[i];
             int r;
-            norm(lw.g1);
+            CK(norm(lw.g1));
             if ((r = qkv(tm.qkv, i, 0)) != KG_OK) return r;
             FaArgs fa;
             fa.qh = qh; fa.ql = ql; fa.kc = (const WT*)D.kcache + (size_t)i * lstride; fa.vc = (const WT*)D.vcache + (size_t)i * lstride;
             fa.oh = xh; fa.ol = xl; fa.page_table = D.page_table; fa.ps_shift = D.dm.ps_shift; fa.n_phys = D.dm.n_phys; fa.st = D.st;
             fa.H = H; fa.pos0 = b0; fa.rows = rows;
             const int fgrid = (rows + FA_ROWS - 1) / FA_ROWS * H;
-            if (hd == 128) pf_attention_kernel<128><<<fgrid, 256, FaSm<128>::BYTES, s>>>(fa);
-            else pf_attention_kernel<64><<<fgrid, 256, FaSm<64>::BYTES, s>>>(fa);
+            if (hd == 128) CK(launch_dependent(pf_attention_kernel<128>, dim3(fgrid), dim3(256), FaSm<128>::BYTES, s, fa));
+            else CK(launch_dependent(pf_attention_kernel<64>, dim3(fgrid), dim3(256), FaSm<64>::BYTES, s, fa));
             if ((r = resid(tm.o, d)) != KG_OK) return r;
-            norm(lw.g2);
+            CK(norm(lw.g2));
             GemmArgs g = base;
             g.N = F; g.K = d; g.rowscale = rs; g.hi = fh; g.lo = fl; g.ldp = F;
             gm_plan(g, F / (GM_TM / 2), pairs, m->lay.pf_part_bytes);
             if ((r = gm_launch<PF_SWIGLU>(g, m->pf.x[0][g.nt / 64 - 1], m->pf.x[1][g.nt / 64 - 1], tm.gate, tm.up, pairs, s)) != KG_OK) return r;
             if ((r = resid(tm.down, F)) != KG_OK) return r;
             if (i == c.exit_layer - 1) {                              // the adapter's K / V
-                norm(m->layers_host[L].g1);
+                CK(norm(m->layers_host[L].g1));
                 if ((r = qkv(m->pf.adapter_kv, L, 1)) != KG_OK) return r;
             }
         }

@@ -5,6 +5,10 @@
 // The activations keep fp32 accuracy the same way as in the decode path: every value is split into two bf16 planes,
 // x = hi + lo, and both planes are multiplied with the bf16 weights into the same fp32 accumulator.
 //
+// Every kernel but the first of a block is launched as a programmatic dependent: it may be set up while the one before still runs and
+// waits (grid_dependency_wait) before it touches that one's results (7B: 77 tokens 6.22 -> 5.63 ms, 17 tokens 5.30 -> 4.60; a model of
+// four layers with d = 512, 32 tokens: 0.31 -> 0.24).
+//
 // A layer is seven launches: RMSNorm + split into planes, QKV GEMM (epilogue: rotation, K / V rows into the cache, q
 // planes), attention (reads q planes and the cache, writes planes), O GEMM (+ residual), RMSNorm + split, gate / up GEMM
 // (epilogue: SwiGLU into planes), down GEMM (+ residual).
@@ -311,6 +315,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
     cluster_sync_all();                                                    // both CTAs' barriers and tensor memory exist
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_dependents_launch();
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GM_CTRL_REGS));
@@ -319,26 +324,40 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
             int s = 0; unsigned par = 1u;
             const int hrow = g.nt >> 1;
             bool ok = true;
+            // the weights do not come from the kernel before: those of the first stages are on their way while it ends
+            auto load_w = [&](const GmItem& it, int kb, int stage) {
+                const uint32_t dst = smem_u32(smem + stage * stage_bytes), bar = leader_smem(smem_u32(&full[stage]));
+                if (rank == 0) mbar_arrive_expect_tx(&full[stage], (unsigned)(2 * stage_bytes));
+                if (EPI == PF_SWIGLU) {
+                    const int y = it.wt * (GM_TM / 2) + rank * (GM_TM / 4);
+                    tma_load_2d_pair(dst, &tm_w, kb * GM_BK, y, bar);
+                    tma_load_2d_pair(dst + GM_A_BYTES / 2, &tm_w2, kb * GM_BK, y, bar);
+                } else {
+                    tma_load_2d_pair(dst, &tm_w, kb * GM_BK, it.wt * GM_TM + rank * (GM_TM / 2), bar);
+                }
+            };
+            int early = 0;
+            {
+                const GmItem it = gm_item(g, pair_id);
+                early = min(nst, it.kb1 - it.kb0);
+                if (elect_one()) for (int i = 0; i < early; ++i) load_w(it, it.kb0 + i, i);
+                __syncwarp();
+            }
+            grid_dependency_wait();
             for (int idx = pair_id; idx < g.items && ok; idx += npairs) {
                 const GmItem it = gm_item(g, idx);
                 const int y_act = it.rt * g.nt + rank * hrow;
                 for (int kb = it.kb0; kb < it.kb1; ++kb) {
                     if (!(ok = gm_wait(&empty[s], par, g.err))) break;
                     if (elect_one()) {
-                        if (rank == 0) mbar_arrive_expect_tx(&full[s], (unsigned)(2 * stage_bytes));
+                        if (early == 0) load_w(it, kb, s);
                         const uint32_t dst = smem_u32(smem + s * stage_bytes), bar = leader_smem(smem_u32(&full[s]));
                         const int x = kb * GM_BK;
-                        if (EPI == PF_SWIGLU) {
-                            const int y = it.wt * (GM_TM / 2) + rank * (GM_TM / 4);
-                            tma_load_2d_pair(dst, &tm_w, x, y, bar);
-                            tma_load_2d_pair(dst + GM_A_BYTES / 2, &tm_w2, x, y, bar);
-                        } else {
-                            tma_load_2d_pair(dst, &tm_w, x, it.wt * GM_TM + rank * (GM_TM / 2), bar);
-                        }
                         tma_load_2d_pair(dst + GM_A_BYTES, &tm_hi, x, y_act, bar);
                         tma_load_2d_pair(dst + GM_A_BYTES + hrow * 128, &tm_lo, x, y_act, bar);
                     }
                     __syncwarp();
+                    if (early > 0) --early;
                     if (++s == nst) { s = 0; par ^= 1u; }
                 }
             }
@@ -390,6 +409,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GM_EPI_REGS));
+        grid_dependency_wait();
         // ---- epilogue: thread = one weight row (tensor-memory lane 32 * (warp % 4) + lane id) and half of the tile's columns
         const int ew = warp - 4, q = warp & 3, chalf = ew >> 2, nch = g.nt >> 6;
         // the partner: the warp with the other half of a rotation (dims e and e + hd / 2) or the up rows of the same features
@@ -539,6 +559,8 @@ __global__ void __launch_bounds__(256, 1) pf_attention_kernel(const __grid_const
             cp_async16(vb + o, a.vc + src);
         }
     };
+    grid_dependents_launch();
+    grid_dependency_wait();
     issue(0);
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (ntile > 1) issue(1);
@@ -697,6 +719,8 @@ constexpr int PF_NORM_V = 8;                  // float4 per thread: rows of up t
 __global__ void __launch_bounds__(PF_EW_THREADS) pf_norm_split_kernel(const float* x, int ldx, int K, const float* gain, float eps,
                                                                       __nv_bfloat16* hi, __nv_bfloat16* lo, float* rs) {
     __shared__ float red[32];
+    grid_dependents_launch();
+    grid_dependency_wait();
     const int r = blockIdx.x;
     const float4* xr = reinterpret_cast<const float4*>(x + (size_t)r * ldx);
     const int n4 = K >> 2;
