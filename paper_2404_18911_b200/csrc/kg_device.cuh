@@ -55,7 +55,7 @@ constexpr int SC_ROWS = 256;                            // rows whose accumulato
 // the plain path never runs beside the streamed one in a launch, so it stages its activations over the ring too
 constexpr int SIMPLE_XS_BYTES = SMEM_TOTAL - RING_OFF - 4096;
 
-constexpr int BAR_RELEASE = 32;                          // word index of the grid barrier's release word (its own 128-byte line)
+constexpr int BAR_STRIDE = 32;                          // words between the two arrival counters (a 128-byte line each)
 constexpr int BAR_BYTES = 256;
 constexpr unsigned long long WAIT_TIMEOUT_CLK = 6000000000ull;   // default budget of a device-side wait: ~3 s at 1.9 GHz
 
@@ -130,7 +130,7 @@ struct Dev {
     int* out_tokens; int* S; int* round_log;   // [max_seq], [max_seq], [max_seq][4]
     const int* prompt;             // device copy of the prompt
     State* st;
-    unsigned* bar;                 // grid barrier arrival counter (zeroed before every launch)
+    unsigned* bar;                 // two grid barrier arrival counters, used by launches in turn
     double inv_freq[HD_MAX / 2];   // theta^(-2i/hd)
 };
 
