@@ -41,8 +41,16 @@ __device__ __forceinline__ float gen_value(uint64_t base, uint64_t i, float scal
 
 template <typename WT>
 __global__ void fill_matrix_kernel(WT* out, uint64_t base, uint64_t count, float scale) {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x)
-        out[i] = float_to_wt<WT>(gen_value(base, i, scale));
+    // 16 bytes of neighbouring values per thread (out is 16-byte aligned)
+    constexpr int N = 16 / sizeof(WT);
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < count / N; j += step) {
+        alignas(16) WT v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = float_to_wt<WT>(gen_value(base, j * N + k, scale));
+        *reinterpret_cast<uint4*>(out + j * N) = *reinterpret_cast<const uint4*>(v);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < count % N) { const uint64_t i = count / N * N + threadIdx.x; out[i] = float_to_wt<WT>(gen_value(base, i, scale)); }
 }
 __global__ void fill_gain_kernel(float* out, uint64_t base, int count, float scale) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
