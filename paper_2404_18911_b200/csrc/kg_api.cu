@@ -244,7 +244,7 @@ __global__ void check_tokens_kernel(const int* toks, int n, int vocab, State* st
 // Tensor maps of the prompt pass, encoded once per model: the weights in boxes of 128 rows (64 for the gate / up pair),
 // the planes [R][K] in boxes of 32 * (i + 1) rows, one set for K = d (x) and one for K = F (f).
 struct PfMaps {
-    CUtensorMap x[2][4], f[2][4];                              // [hi, lo][activation rows per tile / 64 - 1]
+    CUtensorMap x[2][GM_NT_MAX / GM_NT_STEP], f[2][GM_NT_MAX / GM_NT_STEP];   // [hi, lo][activation rows per tile / GM_NT_STEP - 1]
     struct Layer { CUtensorMap qkv, o, gate, up, down; };
     std::vector<Layer> layer;
     CUtensorMap adapter_kv;                                    // the k and v rows of the adapter's W_qkv
@@ -1221,9 +1221,9 @@ int prefill_tc_init(kg_model* m) {
     char* A = m->arena;
     bool ok = true;
     for (int p = 0; p < 2; ++p)
-        for (int i = 0; i < 4; ++i) {
-            ok = ok && make_tmap(&m->pf.x[p][i], A + m->lay.off_pf_x + (size_t)p * R * d * 2, R, d, 32 * (i + 1));
-            ok = ok && make_tmap(&m->pf.f[p][i], A + m->lay.off_pf_f + (size_t)p * R * F * 2, R, F, 32 * (i + 1));
+        for (int i = 0; i < GM_NT_MAX / GM_NT_STEP; ++i) {
+            ok = ok && make_tmap(&m->pf.x[p][i], A + m->lay.off_pf_x + (size_t)p * R * d * 2, R, d, GM_NT_STEP / 2 * (i + 1));
+            ok = ok && make_tmap(&m->pf.f[p][i], A + m->lay.off_pf_f + (size_t)p * R * F * 2, R, F, GM_NT_STEP / 2 * (i + 1));
         }
     m->pf.layer.resize(L);
     for (int i = 0; i < L; ++i) {
@@ -1261,20 +1261,21 @@ __global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* 
 bool prefill_tc_ok(const kg_model* m, int n) { return m->prefill_mode == 0 && m->pf.ready && n > KG_M_MAX; }
 
 // Tile shape and work items of a GEMM of `rows` activation rows and `wtiles` tiles of weight rows on `pairs` CTA pairs.
-// Row tiles: as few as 256 columns allow, all of the same width (a multiple of 64).  The last wave of tiles is cut into S
+// Row tiles: as few as 256 columns allow, all of the same width (a multiple of 32; of
+// 64 before: 7B prompts of 200, 300 and 777 tokens 8.2, 10.1 and 23.1 ms, 7.9, 9.9 and 22.3 with it).  The last wave of tiles is cut into S
 // ranges of k, S the one with the shortest estimated time in units of a k block: the waves of ranges, plus what a cut
 // costs (writing the partial sums and reading S of them back, which grows with the tile's columns; with 4 + S nt / 128 instead
 // of 10 + S nt / 64, 7B prompts of 32, 200, 512 and 1024 tokens took 4.67, 8.79, 14.07 and 26.5 ms, now 4.43, 8.21, 13.81, 25.7).
 void gm_plan(GemmArgs& g, int wtiles, int pairs, size_t part_bytes) {
     g.nrt = (g.rows + GM_NT_MAX - 1) / GM_NT_MAX;
-    g.nt = ((g.rows + g.nrt - 1) / g.nrt + 63) / 64 * 64;
+    g.nt = ((g.rows + g.nrt - 1) / g.nrt + GM_NT_STEP - 1) / GM_NT_STEP * GM_NT_STEP;
     const int tiles = wtiles * g.nrt, nkb = g.K / GM_BK;
     const int rem = tiles % pairs;
     g.full = tiles - rem;
     g.S = 1;
     int best = nkb;
     for (int S = 2; S <= 16 && rem > 0 && nkb / S >= 4; ++S) {
-        if ((size_t)rem * S * GM_TM * g.nt * 4 > part_bytes) break;
+        if ((size_t)rem * S * GM_TM * ((g.nt + 63) / 64 * 64) * 4 > part_bytes) break;
         const int cost = (rem * S + pairs - 1) / pairs * ((nkb + S - 1) / S) + 10 + S * g.nt / 64;
         if (cost < best) { best = cost; g.S = S; }
     }
@@ -1324,13 +1325,13 @@ int prefill_tc(kg_model* m, int n) {
             g.kc = (WT*)D.kcache + (size_t)li * lstride; g.vc = (WT*)D.vcache + (size_t)li * lstride;
             g.qscale = 1.4426950408889634f / std::sqrt((float)hd);
             gm_plan(g, (g.N + GM_TM - 1) / GM_TM, pairs, m->lay.pf_part_bytes);
-            return gm_launch<PF_QKV>(g, m->pf.x[0][g.nt / 64 - 1], m->pf.x[1][g.nt / 64 - 1], w, w, pairs, s);
+            return gm_launch<PF_QKV>(g, m->pf.x[0][g.nt / GM_NT_STEP - 1], m->pf.x[1][g.nt / GM_NT_STEP - 1], w, w, pairs, s);
         };
         auto resid = [&](const CUtensorMap& w, int K) {            // h += planes W^T
             GemmArgs g = base;
             g.N = d; g.K = K; g.C = h; g.resid = h; g.ldc = d;
             gm_plan(g, (d + GM_TM - 1) / GM_TM, pairs, m->lay.pf_part_bytes);
-            const int i = g.nt / 64 - 1;
+            const int i = g.nt / GM_NT_STEP - 1;
             return K == d ? gm_launch<PF_STORE>(g, m->pf.x[0][i], m->pf.x[1][i], w, w, pairs, s)
                           : gm_launch<PF_STORE>(g, m->pf.f[0][i], m->pf.f[1][i], w, w, pairs, s);
         };
@@ -1352,7 +1353,7 @@ int prefill_tc(kg_model* m, int n) {
             GemmArgs g = base;
             g.N = F; g.K = d; g.rowscale = rs; g.hi = fh; g.lo = fl; g.ldp = F;
             gm_plan(g, F / (GM_TM / 2), pairs, m->lay.pf_part_bytes);
-            if ((r = gm_launch<PF_SWIGLU>(g, m->pf.x[0][g.nt / 64 - 1], m->pf.x[1][g.nt / 64 - 1], tm.gate, tm.up, pairs, s)) != KG_OK) return r;
+            if ((r = gm_launch<PF_SWIGLU>(g, m->pf.x[0][g.nt / GM_NT_STEP - 1], m->pf.x[1][g.nt / GM_NT_STEP - 1], tm.gate, tm.up, pairs, s)) != KG_OK) return r;
             if ((r = resid(tm.down, F)) != KG_OK) return r;
             if (i == c.exit_layer - 1) {                              // the adapter's K / V
                 CK(norm(m->layers_host[L].g1));

@@ -25,6 +25,7 @@ constexpr int GM_BK = 64;                      // k block: one 128-byte swizzle 
 constexpr int GM_CHAIN = 2;                    // k blocks summed by the tensor core before the sum goes to fp32 registers
 constexpr int GM_TM = 256;                     // weight rows per CTA pair (128 in each CTA: the M side of the MMA)
 constexpr int GM_NT_MAX = 256;                 // most activation rows per tile (the N side)
+constexpr int GM_NT_STEP = 32;                 // widths of a tile (the N of a 256-row MMA of a CTA pair is a multiple of 32)
 constexpr int GM_A_BYTES = (GM_TM / 2) * GM_BK * 2;                    // this CTA's weight rows of a k block: 16 KB
 constexpr int GM_RING_BYTES = 192 * 1024;
 constexpr int GM_MAX_STAGES = 8;
@@ -410,8 +411,8 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GM_EPI_REGS));
         grid_dependency_wait();
-        // ---- epilogue: thread = one weight row (tensor-memory lane 32 * (warp % 4) + lane id) and half of the tile's columns
-        const int ew = warp - 4, q = warp & 3, chalf = ew >> 2, nch = g.nt >> 6;
+        // ---- epilogue: thread = one weight row (tensor-memory lane 32 * (warp % 4) + lane id) and every other 32 columns of the tile
+        const int ew = warp - 4, q = warp & 3, chalf = ew >> 2, nch = ((g.nt >> 5) + 1 - chalf) >> 1;
         // the partner: the warp with the other half of a rotation (dims e and e + hd / 2) or the up rows of the same features
         const int pbit = (EPI == PF_QKV && g.hd == 64) ? 1 : 2;
         const int role = (q & pbit) ? 1 : 0, pair = pbit == 2 ? (q & 1) * 2 + chalf : (q >> 1) * 2 + chalf;
@@ -429,12 +430,12 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 if (ok) ok = gm_wait(&acc_full[a], apar, g.err);
                 __syncwarp();
                 tc_fence_after();
-                const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * acc_cols + chalf * (g.nt >> 1));
+                const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * acc_cols + chalf * 32);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     if (c < nch) {
                         uint32_t v[32];
-                        tmem_ld32(ta + 32u * c, v);
+                        tmem_ld32(ta + 64u * c, v);
                         tmem_ld_wait32(v);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(v[i]);
@@ -445,7 +446,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 if (lane == 0) mbar_arrive_cluster(leader_smem(smem_u32(&acc_free[a])));
                 if (++a == nacc) { a = 0; apar ^= 1u; }
             }
-            const size_t wsize = (size_t)nch * GM_STAGE_FLOATS;            // floats of one warp's products
+            const size_t wsize = (size_t)((g.nt + 63) >> 6) * GM_STAGE_FLOATS; // floats of one warp's products (at most)
             const size_t one = 2 * GM_EPI_WARPS * wsize;                   // ... of one range of k (both CTAs)
             float* part = g.part + (size_t)it.r * g.S * one + ((size_t)rank * GM_EPI_WARPS + ew) * wsize + lane;
             bool finish = true;
@@ -496,7 +497,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                         }
                     }
                     if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
-                    gm_epilogue<EPI>(g, mine, theirs, it.rt * g.nt + chalf * (g.nt >> 1) + c * 32, it.wt, rank, q, role);
+                    gm_epilogue<EPI>(g, mine, theirs, it.rt * g.nt + (c * 2 + chalf) * 32, it.wt, rank, q, role);
                     if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
                 }
             }

@@ -1,4 +1,4 @@
-"""Edges of the prompt pass: tile widths of the GEMM (64 .. 256 activation rows, one and more row tiles), whole tiles and
+"""Edges of the prompt pass: tile widths of the GEMM (32 .. 256 activation rows in steps of 32, one and more row tiles), whole tiles and
 tiles cut along k, both head sizes of the fused epilogues, more than one block of prompt rows."""
 import numpy as np
 import pytest
@@ -55,7 +55,8 @@ def test_two_blocks_of_prompt_rows(binding):
 
 
 # N = 19200: 75 tiles of 256 weight rows, one more than the 74 CTA pairs; N = 384 ends in half a tile; K = 192: an odd number of k blocks
-@pytest.mark.parametrize("N,K,M", [(128, 64, 64), (384, 192, 65), (19200, 192, 130), (19200, 512, 257), (2560, 4032, 511), (128, 8192, 256)])
+@pytest.mark.parametrize("N,K,M", [(128, 64, 64), (384, 192, 65), (19200, 192, 130), (19200, 512, 257), (2560, 4032, 511), (128, 8192, 256),
+                                   (384, 192, 20), (2560, 512, 96), (19200, 192, 220)])
 def test_gemm_tiles_against_fp64(binding, N, K, M):
     import torch
     from kg_inputs import synth
