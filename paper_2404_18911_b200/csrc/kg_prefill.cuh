@@ -152,7 +152,7 @@ __device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity
 // What bounds it: the operands of a k block.  With the activations in two planes a 128 x 128 tile of one CTA needs 48 KB for
 // 4.2 MFLOP (94 bytes per clock and SM at the full MMA rate, more than L2 delivers); the pair's 256 x 256 tile needs 48 KB
 // per CTA for 8.4 MFLOP, since the two CTAs share the activation planes.  With the attention below and the fused epilogues
-// the prompt pass of the 7B shape (1999 tokens) went from 96.9 to 52.6 ms, of 77 tokens from 9.2 to 6.3 ms.
+// the prompt pass of the 7B shape (1999 tokens) went from 96.9 to 49.9 ms, of 77 tokens from 9.2 to 5.3 ms.
 //
 // Accumulation.  The tensor core's fp32 accumulation rounds toward zero at every MMA, by an amount that follows the size
 // of the running sum, which biases long chains.  A chain of GM_CHAIN = 2 k blocks multiplies both lo planes first - sums
@@ -185,23 +185,73 @@ __device__ __forceinline__ unsigned pack_bf16(float a, float b) {
     return *reinterpret_cast<const unsigned*>(&v);
 }
 
-// Finished products of 32 columns (activation rows row0 ..) of this warp's 32 weight rows, staged as [column][lane] in
-// `mine` (`theirs`: the partner warp's staging).  The loops run over the staging and not over registers so that the code
-// stays small: as straight-line code over 128 registers the epilogue took 18 us a tile, most of it instruction fetch.
+// What the epilogue needs of one activation row: 1 / rms and the row's place in the caches, (physical page * heads) pages of
+// page_size slots + slot.  Lane i keeps that of row i of 32 columns, loaded before the k loop.
+struct GmRow { float rs; int slot; };
 template <int EPI>
-__device__ __forceinline__ void gm_epilogue(const GemmArgs& g, const float* mine, const float* theirs, int row0, int wt, int rank, int q, int role) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (EPI == PF_STORE) {
-        // four columns at a time, 16 bytes (four features) per lane
-        const int n = wt * GM_TM + rank * (GM_TM / 2) + q * 32 + (lane & 7) * 4, c0 = lane >> 3;
-        if (n >= g.N) return;
-        float4 rv[8];
+__device__ __forceinline__ GmRow gm_row(const GemmArgs& g, int row) {
+    GmRow r{0.f, 0};
+    if (EPI == PF_STORE || row >= g.rows) return r;
+    r.rs = g.rowscale[row];
+    if (EPI == PF_QKV) {
+        const int pos = g.pos0 + row;
+        r.slot = ((checked_page(__ldg(g.page_table + (pos >> g.ps_shift)), g.n_phys, g.st, 61) * g.H) << g.ps_shift) + (pos & ((1 << g.ps_shift) - 1));
+    }
+    return r;
+}
+__device__ __forceinline__ void load8(float (&v)[8], const float* p) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+// eight values as bf16, and as bf16 hi + lo planes (16-byte stores)
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&v)[8]) {
+    *reinterpret_cast<uint4*>(p) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+}
+__device__ __forceinline__ void store8_planes(__nv_bfloat16* hi, __nv_bfloat16* lo, const float (&v)[8]) {
+    uint4 h, l;
+    split_hi_lo(make_float2(v[0], v[1]), h.x, l.x); split_hi_lo(make_float2(v[2], v[3]), h.y, l.y);
+    split_hi_lo(make_float2(v[4], v[5]), h.z, l.z); split_hi_lo(make_float2(v[6], v[7]), h.w, l.w);
+    *reinterpret_cast<uint4*>(hi) = h;
+    *reinterpret_cast<uint4*>(lo) = l;
+}
+
+// The global values that the epilogue of 32 columns reads, requested before the staging: PF_STORE the residual (four columns at
+// a time, four features per lane), PF_QKV (cos, sin) of eight dims of this warp's half of the columns.
+template <int EPI>
+__device__ __forceinline__ void gm_request(const GemmArgs& g, float4 (&rv)[8], int row0, int wt, int rank, int q, int role) {
+    const int lane = threadIdx.x & 31, n = wt * GM_TM + rank * (GM_TM / 2) + q * 32;       // this warp's first row of W
+    if (EPI == PF_STORE) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int row = row0 + i * 4 + c0;
+            const int row = row0 + i * 4 + (lane >> 3);
             rv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (g.resid && row < g.rows) rv[i] = *reinterpret_cast<const float4*>(g.resid + (size_t)row * g.ldc + n);
+            if (g.resid && row < g.rows && n < g.N) rv[i] = *reinterpret_cast<const float4*>(g.resid + (size_t)row * g.ldc + n + (lane & 7) * 4);
         }
+    }
+    if (EPI == PF_QKV) {
+        const int half = g.hd >> 1, e = (n & (half - 1)) + (lane & 3) * 8;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = min(row0 + role * 16 + (i >> 2) * 8 + (lane >> 2), g.rows - 1);
+            rv[i] = __ldg(reinterpret_cast<const float4*>(g.cs + (size_t)row * half + e) + (i & 3));
+        }
+    }
+}
+
+// Finished products of 32 columns (activation rows row0 ..) of this warp's 32 weight rows, staged as [column][lane] in
+// `mine` (`theirs`: the partner warp's staging).  A lane takes eight neighbouring features of a column.  What bounds it: the
+// main loop stands still meanwhile (the accumulator columns of at most nacc chains are ahead), so what counts is the chain
+// of dependent steps.  With two features per lane and step, and with the row factors, page numbers and rotations loaded
+// where they were used, a 256 x 256 tile's epilogue took 36,000 (QKV) and 23,000 (SwiGLU) clocks beside a k loop of 64,000;
+// now 16,000 and 13,000 (7B, 77 tokens 5.6 -> 5.3 ms, 1999 tokens 53.2 -> 49.9 ms).  What is left is the latency of the rotations
+// and of the residual and, for SwiGLU, the divisions (about 4,000).
+template <int EPI>
+__device__ __forceinline__ void gm_epilogue(const GemmArgs& g, const float* mine, const float* theirs, int row0, int wt, int rank, int q, int role,
+                                            GmRow gr, const float4 (&rv)[8]) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (EPI == PF_STORE) {
+        const int n = wt * GM_TM + rank * (GM_TM / 2) + q * 32 + (lane & 7) * 4, c0 = lane >> 3;
+        if (n >= g.N) return;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int row = row0 + i * 4 + c0;
@@ -209,73 +259,75 @@ __device__ __forceinline__ void gm_epilogue(const GemmArgs& g, const float* mine
             if (row < g.rows) *reinterpret_cast<float4*>(g.C + (size_t)row * g.ldc + n) = make_float4(rv[i].x + v.x, rv[i].y + v.y, rv[i].z + v.z, rv[i].w + v.w);
         }
     } else {
-        // two columns at a time, two features per lane; of a pair of warps each takes half of the columns
-        const int cl = lane >> 4, fe = (lane & 15) * 2;
+        // of a pair of warps each takes half of the columns
+        const int cl = lane >> 2, fe = (lane & 3) * 8;
         if constexpr (EPI == PF_SWIGLU) {
             const int f = wt * (GM_TM / 2) + rank * (GM_TM / 4) + (q & 1) * 32 + fe;
             const float* ga = role ? theirs : mine;
             const float* up = role ? mine : theirs;
-#pragma unroll 2
-            for (int i = 0; i < 8; ++i) {
-                const int col = role * 16 + i * 2 + cl, row = row0 + col;
-                const float2 a = *reinterpret_cast<const float2*>(ga + col * 32 + fe), b = *reinterpret_cast<const float2*>(up + col * 32 + fe);
-                if (row < g.rows) {
-                    const float rs = g.rowscale[row];
-                    unsigned hi, lo;
-                    split_hi_lo(make_float2(silu_f(a.x * rs) * (b.x * rs), silu_f(a.y * rs) * (b.y * rs)), hi, lo);
-                    *reinterpret_cast<unsigned*>(g.hi + (size_t)row * g.ldp + f) = hi;
-                    *reinterpret_cast<unsigned*>(g.lo + (size_t)row * g.ldp + f) = lo;
-                }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int col = role * 16 + i * 8 + cl, row = row0 + col;
+                float a[8], b[8];
+                load8(a, ga + col * 32 + fe);
+                load8(b, up + col * 32 + fe);
+                const float rs = __shfl_sync(0xffffffffu, gr.rs, col);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] = silu_f(a[k] * rs) * (b[k] * rs);
+                const size_t o = (size_t)row * g.ldp + f;
+                if (row < g.rows) store8_planes(g.hi + o, g.lo + o, a);
             }
         } else {
-            const int d = g.H * g.hd, half = g.hd >> 1, psm = (1 << g.ps_shift) - 1;
+            const int d = g.H * g.hd, half = g.hd >> 1;
             const int n0 = wt * GM_TM + rank * (GM_TM / 2);                 // this CTA's 128 rows of W lie in one section
             if (n0 >= g.N) return;
             const int s0 = n0 / d, sec = s0 + g.sec0, nh = n0 - s0 * d + q * 32;     // this warp's first row within the section
             const int hh = nh >> (half == 64 ? 7 : 6), e0 = nh & (g.hd - 1);
             if (sec == 2) {
-#pragma unroll 4
-                for (int i = 0; i < 16; ++i) {
-                    const int col = i * 2 + cl, row = row0 + col;
-                    const float2 v = *reinterpret_cast<const float2*>(mine + col * 32 + fe);
-                    if (row < g.rows) {
-                        const float rs = g.rowscale[row];
-                        const int pos = g.pos0 + row;
-                        const int page = checked_page(__ldg(g.page_table + (pos >> g.ps_shift)), g.n_phys, g.st, 61);
-                        *reinterpret_cast<unsigned*>(g.vc + ((((size_t)page * g.H + hh) << g.ps_shift) + (pos & psm)) * g.hd + e0 + fe) = pack_bf16(v.x * rs, v.y * rs);
-                    }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int col = i * 8 + cl;
+                    float v[8];
+                    load8(v, mine + col * 32 + fe);
+                    const float rs = __shfl_sync(0xffffffffu, gr.rs, col);
+                    const int slot = __shfl_sync(0xffffffffu, gr.slot, col) + (hh << g.ps_shift);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] *= rs;
+                    if (row0 + col < g.rows) store8(g.vc + (size_t)slot * g.hd + e0 + fe, v);
                 }
             } else {
-                // dims e, e + 1 of the first half of the head and their partners half a head further
+                // dims e .. e + 7 of the first half of the head and their partners half a head further
                 const int e = (e0 & (half - 1)) + fe;
                 const float* xa = role ? theirs : mine;
                 const float* xb = role ? mine : theirs;
-#pragma unroll 2
-                for (int i = 0; i < 8; ++i) {
-                    const int col = role * 16 + i * 2 + cl, row = row0 + col;
-                    const float2 a = *reinterpret_cast<const float2*>(xa + col * 32 + fe), b = *reinterpret_cast<const float2*>(xb + col * 32 + fe);
-                    if (row < g.rows) {
-                        const float rs = g.rowscale[row];
-                        const float4 cs = __ldg(reinterpret_cast<const float4*>(g.cs + (size_t)row * half + e));
-                        const float a0 = a.x * rs, a1 = a.y * rs, b0 = b.x * rs, b1 = b.y * rs;
-                        const float2 r1 = make_float2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
-                        const float2 r2 = make_float2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
-                        if (sec == 0) {
-                            const size_t o = (size_t)row * g.ldp + (size_t)hh * g.hd + e;
-                            unsigned hi, lo;
-                            split_hi_lo(make_float2(r1.x * g.qscale, r1.y * g.qscale), hi, lo);
-                            *reinterpret_cast<unsigned*>(g.hi + o) = hi;
-                            *reinterpret_cast<unsigned*>(g.lo + o) = lo;
-                            split_hi_lo(make_float2(r2.x * g.qscale, r2.y * g.qscale), hi, lo);
-                            *reinterpret_cast<unsigned*>(g.hi + o + half) = hi;
-                            *reinterpret_cast<unsigned*>(g.lo + o + half) = lo;
-                        } else {
-                            const int pos = g.pos0 + row;
-                            const int page = checked_page(__ldg(g.page_table + (pos >> g.ps_shift)), g.n_phys, g.st, 62);
-                            __nv_bfloat16* kr = g.kc + ((((size_t)page * g.H + hh) << g.ps_shift) + (pos & psm)) * g.hd + e;
-                            *reinterpret_cast<unsigned*>(kr) = pack_bf16(r1.x, r1.y);
-                            *reinterpret_cast<unsigned*>(kr + half) = pack_bf16(r2.x, r2.y);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int col = role * 16 + i * 8 + cl, row = row0 + col;
+                    float a[8], b[8];
+                    load8(a, xa + col * 32 + fe);
+                    load8(b, xb + col * 32 + fe);
+                    const float rs = __shfl_sync(0xffffffffu, gr.rs, col);
+                    const int slot = __shfl_sync(0xffffffffu, gr.slot, col) + (hh << g.ps_shift);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 cs = rv[i * 4 + (k >> 1)];
+                        const float c = k & 1 ? cs.z : cs.x, sn = k & 1 ? cs.w : cs.y;
+                        const float xk = a[k] * rs, yk = b[k] * rs;
+                        a[k] = xk * c - yk * sn;
+                        b[k] = yk * c + xk * sn;
+                    }
+                    if (sec == 0) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) { a[k] *= g.qscale; b[k] *= g.qscale; }
+                        const size_t o = (size_t)row * g.ldp + (size_t)hh * g.hd + e;
+                        if (row < g.rows) {
+                            store8_planes(g.hi + o, g.lo + o, a);
+                            store8_planes(g.hi + o + half, g.lo + o + half, b);
                         }
+                    } else if (row < g.rows) {
+                        __nv_bfloat16* kr = g.kc + (size_t)slot * g.hd + e;
+                        store8(kr, a);
+                        store8(kr + half, b);
                     }
                 }
             }
@@ -426,6 +478,9 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
             float acc[GM_NT_MAX / 2];
 #pragma unroll
             for (int i = 0; i < GM_NT_MAX / 2; ++i) acc[i] = 0.f;
+            GmRow gr[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) gr[c] = gm_row<EPI>(g, it.rt * g.nt + (c * 2 + chalf) * 32 + lane);
             for (int kb = it.kb0; kb < it.kb1; kb += GM_CHAIN) {
                 if (ok) ok = gm_wait(&acc_full[a], apar, g.err);
                 __syncwarp();
@@ -472,33 +527,56 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 finish = *(volatile int*)last_flag != 0;
                 named_sync(5, 32 * GM_EPI_WARPS);                          // the flag has been read by every warp
             }
-            if (finish) {
+            // 32 columns at a time through the staging
+            auto staged = [&](int c, const float4 (&rv)[8]) {
+                if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
+                gm_epilogue<EPI>(g, mine, theirs, it.rt * g.nt + (c * 2 + chalf) * 32, it.wt, rank, q, role, c == 0 ? gr[0] : c == 1 ? gr[1] : c == 2 ? gr[2] : gr[3], rv);
+                if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
+            };
+            if (it.s < 0) {
 #pragma unroll 1
                 for (int c = 0; c < nch; ++c) {
-                    if (it.s >= 0) {
-                        float w[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) w[i] = __ldcg(part + (c * 32 + i) * 32);
-                        for (int s = 1; s < g.S; ++s) {
-                            const float* src = part + (size_t)s * one + c * GM_STAGE_FLOATS;
-                            float u[32];                                   // one batch of loads in flight
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) u[i] = __ldcg(src + i * 32);
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) w[i] += u[i];
-                        }
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) mine[i * 32 + lane] = w[i];
-                    } else {
-                        switch (c) {
+                    float4 rv[8];
+                    gm_request<EPI>(g, rv, it.rt * g.nt + (c * 2 + chalf) * 32, it.wt, rank, q, role);
+                    switch (c) {
 #define KG_STAGE(C) case C: { _Pragma("unroll") for (int i = 0; i < 32; ++i) mine[i * 32 + lane] = acc[C * 32 + i]; } break
-                            KG_STAGE(0); KG_STAGE(1); KG_STAGE(2); KG_STAGE(3);
+                        KG_STAGE(0); KG_STAGE(1); KG_STAGE(2); KG_STAGE(3);
 #undef KG_STAGE
+                    }
+                    staged(c, rv);
+                }
+            } else if (finish) {
+#pragma unroll 1
+                for (int c = 0; c < nch; ++c) {
+                    float4 rv[8];
+                    gm_request<EPI>(g, rv, it.rt * g.nt + (c * 2 + chalf) * 32, it.wt, rank, q, role);
+                    float w[32], u[32];                                    // the loads of two ranges in flight (S is at least 2)
+                    const float* src = part + c * GM_STAGE_FLOATS;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) w[i] = __ldcg(src + i * 32);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) u[i] = __ldcg(src + one + i * 32);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) w[i] += u[i];
+#pragma unroll 1
+                    for (int s = 2; s < g.S; s += 2) {
+                        const float* s0 = src + (size_t)s * one;
+                        const bool two = s + 1 < g.S;
+                        float x[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) u[i] = __ldcg(s0 + i * 32);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) x[i] = two ? __ldcg(s0 + one + i * 32) : 0.f;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) w[i] += u[i];
+                        if (two) {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) w[i] += x[i];
                         }
                     }
-                    if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
-                    gm_epilogue<EPI>(g, mine, theirs, it.rt * g.nt + (c * 2 + chalf) * 32, it.wt, rank, q, role);
-                    if (EPI == PF_STORE) __syncwarp(); else named_sync(1 + pair, 64);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) mine[i * 32 + lane] = w[i];
+                    staged(c, rv);
                 }
             }
         }
