@@ -313,8 +313,9 @@ __device__ __forceinline__ void gm_epilogue(const GemmArgs& g, const float* mine
                         const float4 cs = rv[i * 4 + (k >> 1)];
                         const float c = k & 1 ? cs.z : cs.x, sn = k & 1 ? cs.w : cs.y;
                         const float xk = a[k] * rs, yk = b[k] * rs;
-                        a[k] = xk * c - yk * sn;
-                        b[k] = yk * c + xk * sn;
+                        // (which product is rounded is written out: left to the compiler it changed with the surrounding code)
+                        a[k] = fmaf(-yk, sn, xk * c);
+                        b[k] = fmaf(xk, sn, yk * c);
                     }
                     if (sec == 0) {
 #pragma unroll
