@@ -30,7 +30,7 @@ constexpr int GM_A_BYTES = (GM_TM / 2) * GM_BK * 2;                    // this C
 constexpr int GM_RING_BYTES = 192 * 1024;
 constexpr int GM_MAX_STAGES = 8;
 constexpr int GM_MAX_ACC = 4;
-constexpr int GM_EPI_WARPS = 8;                // two per tensor-memory lane quadrant, half of the tile's columns each
+constexpr int GM_EPI_WARPS = 8;                // two per tensor-memory lane quadrant, every other 32 columns of the tile each
 constexpr int GM_THREADS = 128 + 32 * GM_EPI_WARPS;                    // warp 0: TMA, warp 1: MMA, two idle warps, then the epilogue
 constexpr int GM_STAGE_FLOATS = 32 * 32;                               // [32 columns][32 lanes] of one epilogue warp
 constexpr int GM_XCH_BYTES = GM_EPI_WARPS * GM_STAGE_FLOATS * 4;
