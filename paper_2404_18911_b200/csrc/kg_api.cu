@@ -265,7 +265,6 @@ struct kg_model {
     int prefill_mode;              // 0: tensor-core prompt pass when the shape and the prompt allow, 1: always the chunked pass
     unsigned long long wait_clk;   // budget of a device-side wait, in SM clocks
     int skip_arrival;              // test hook, consumed by the next launch
-    int bar_sel;                   // arrival counter of the next decode launch
     cudaEvent_t ev0, ev1;          // timing of the decode loop in kg_generate, created on first use
     int gamma_pending;
     long long P_upper;      // upper bound of the device-side position P
@@ -316,14 +315,12 @@ static const void* decode_kernel(const kg_config& c) {
 
 static int launch(kg_model* m, const Program& pg) {
     Program p = pg;
-    p.bar_sel = m->bar_sel;                      // two arrival counters by turns: a launch zeroes the one of the next (no memset each)
     p.force_simple = m->force_simple;
     p.wait_clk = m->wait_clk;
     p.skip_arrival = m->skip_arrival;
     m->skip_arrival = 0;
     void* args[] = {(void*)&m->dev, (void*)&p};
     CK(cudaLaunchCooperativeKernel(decode_kernel(m->cfg), dim3(m->nctas), dim3(DECODE_THREADS), args, m->smem, m->stream));
-    m->bar_sel ^= 1;                             // only a kernel that runs zeroes the next one's counter
     return KG_OK;
 }
 
@@ -415,7 +412,7 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     m->cfg = *cfg; m->lay = lay; m->arena = base; m->stream = (cudaStream_t)cuda_stream; m->nctas = nctas;
     m->own_weights = own != 0; m->prefilled = m->pending = m->ar_used = m->dead = false;
     m->gamma_pending = 0; m->P_upper = 0; m->force_simple = 0;
-    m->wait_clk = WAIT_TIMEOUT_CLK; m->skip_arrival = 0; m->bar_sel = 0; m->ev0 = m->ev1 = nullptr; m->prefill_mode = 0;
+    m->wait_clk = WAIT_TIMEOUT_CLK; m->skip_arrival = 0; m->ev0 = m->ev1 = nullptr; m->prefill_mode = 0;
     m->smem = SMEM_TOTAL;
 
     const bool bf = cfg->dtype == KG_BF16;

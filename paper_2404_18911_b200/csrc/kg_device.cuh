@@ -55,7 +55,7 @@ constexpr int SC_ROWS = 256;                            // rows whose accumulato
 // the plain path never runs beside the streamed one in a launch, so it stages its activations over the ring too
 constexpr int SIMPLE_XS_BYTES = SMEM_TOTAL - RING_OFF - 4096;
 
-constexpr int BAR_STRIDE = 32;                          // words between the two arrival counters (a 128-byte line each)
+constexpr int BAR_STRIDE = 32;                          // words between the arrival counter and the count of CTAs that have left (a 128-byte line each)
 constexpr int BAR_BYTES = 256;
 constexpr unsigned long long WAIT_TIMEOUT_CLK = 6000000000ull;   // default budget of a device-side wait: ~3 s at 1.9 GHz
 
@@ -130,7 +130,7 @@ struct Dev {
     int* out_tokens; int* S; int* round_log;   // [max_seq], [max_seq], [max_seq][4]
     const int* prompt;             // device copy of the prompt
     State* st;
-    unsigned* bar;                 // two grid barrier arrival counters, used by launches in turn
+    unsigned* bar;                 // grid barrier arrival counter, and the count of CTAs that have left: both zero between launches
     double inv_freq[HD_MAX / 2];   // theta^(-2i/hd)
 };
 
@@ -397,6 +397,13 @@ __device__ __forceinline__ bool grid_sync(Ctx& c, int where) {
     }
     cta_sync();
     return *(volatile int*)&c.ctl->sync_ok != 0;
+}
+
+// Thread 0 of every CTA, behind its last barrier.  A launch finds the arrival counter at zero and leaves it so: the last CTA to
+// come here clears it, when no CTA polls it any more.  (Nothing about it is kept on the host, so that a captured launch can be
+// replayed.)  A launch that gave up leaves the abort bit, which ends every later launch at its first barrier.
+__device__ __forceinline__ void grid_leave(const Ctx& c) {
+    if (atomicInc(c.bar + BAR_STRIDE, (unsigned)c.nctas - 1u) == (unsigned)c.nctas - 1u) *(volatile unsigned*)c.bar = 0u;
 }
 
 // ------------------------------------------------------------------------------------ exchange inside a layer

@@ -31,7 +31,6 @@ struct Program {
     int force_simple;   // 1: route bf16 linears through the plain path (cross-check)
     unsigned long long wait_clk;   // clocks after which a device-side wait gives up (KG_E_TIMEOUT)
     int skip_arrival;   // test hook: 1 + index of a CTA that leaves out its first grid-barrier arrival, so that a wait expires
-    int bar_sel;        // which of the two arrival counters this launch uses; it zeroes the other one for the next launch
 };
 
 // Rows handed from one operator to the next: fp32 rows (residual input, plain path), their packed copy
@@ -493,7 +492,7 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctl->qempty[q]);
         if (where && !grid_sync(c, where)) return;
-        if (kind == OPK_EXIT) return;
+        if (kind == OPK_EXIT) { if (tid == 0) grid_leave(c); return; }
         if (++q == QUEUE) { q = 0; qph ^= 1u; }
     }
 }
@@ -502,8 +501,7 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
 template <typename WT, int HD>
 __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const __grid_constant__ Program pg) {
     extern __shared__ __align__(128) char smem[];
-    Ctx& c = ctx_init(smem, D.st, D.bar + pg.bar_sel * BAR_STRIDE, true, pg.wait_clk, pg.skip_arrival);
-    if (blockIdx.x == 0 && threadIdx.x == 0) D.bar[(pg.bar_sel ^ 1) * BAR_STRIDE] = 0u;
+    Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival);
     if (threadIdx.x >= NTHREADS) {
         // the third warpgroup: keeps what the copy loop and the sequencer need and returns the rest of its registers
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PRODUCER_REGS));
