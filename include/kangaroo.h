@@ -113,7 +113,8 @@ int kg_init_model(const kg_config* cfg, const kg_weights* weights, void* arena_d
                   void* cuda_stream, kg_model** out);
 int kg_free_model(kg_model* m);              /* frees the host handle only */
 
-/* Forget the sequence (KV lengths, round state); weights stay. */
+/* Forget the sequence (KV lengths, round state); weights stay.  A wait that expired (KG_E_TIMEOUT) is not forgotten, even if no call
+ * has read it yet: the next call that synchronises answers it. */
 int kg_reset(kg_model* m);
 
 /* All L layers over the prompt, the adapter's K/V for every prompt position, and

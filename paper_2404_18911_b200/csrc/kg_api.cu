@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cstddef>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -324,10 +325,14 @@ static int launch(kg_model* m, const Program& pg) {
     return KG_OK;
 }
 
+// The part of the state word that a new sequence starts from; an expired wait stays recorded behind it, because such a launch leaves
+// exchange words behind that the next one would take for values.
+constexpr size_t SEQ_STATE_BYTES = offsetof(State, timed_out);
+
 static int read_state(kg_model* m, State* out) {
     CK(cudaMemcpyAsync(out, m->dev.st, sizeof(State), cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
-    if (out->status == ST_TIMEOUT) { m->dead = true; return KG_E_TIMEOUT; }
+    if (out->timed_out) { m->dead = true; return KG_E_TIMEOUT; }
     if (out->status == ST_INTERNAL) {
         std::snprintf(g_cuda_err, sizeof(g_cuda_err), "device-side index check %d failed", out->timeout_where);
         m->dead = true;
@@ -539,7 +544,7 @@ extern "C" int kg_free_model(kg_model* m) {
 extern "C" int kg_reset(kg_model* m) {
     if (!m) return KG_E_ARG;
     if (m->dead) return KG_E_TIMEOUT;
-    CK(cudaMemsetAsync(m->dev.st, 0, sizeof(State), m->stream));
+    CK(cudaMemsetAsync(m->dev.st, 0, SEQ_STATE_BYTES, m->stream));
     CK(cudaMemsetAsync(m->dev.att_cnt, 0, 4 * m->cfg.n_heads, m->stream));
     m->prefilled = m->pending = m->ar_used = false;
     m->P_upper = 0;
@@ -863,7 +868,7 @@ extern "C" int kg_debug_fill_state(kg_model* m, int32_t T, int32_t n_d, uint64_t
         st.pending = 1; st.n_d = n_d; st.n_steps = n_d;
         for (int i = 0; i < n_d; ++i) { st.draft_tok[i] = (int)(mix64(tb + (uint64_t)i) % (uint64_t)c.vocab); st.conf[i] = 1.0f; }
     }
-    CK(cudaMemcpyAsync(m->dev.st, &st, sizeof(State), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(m->dev.st, &st, SEQ_STATE_BYTES, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(m->dev.att_cnt, 0, 4 * c.n_heads, s));
     CK(cudaStreamSynchronize(s));
     m->prefilled = true; m->pending = n_d >= 0; m->ar_used = false; m->gamma_pending = n_d >= 0 ? n_d : 0; m->P_upper = T;
@@ -1246,7 +1251,7 @@ __global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* 
     int tok; float p;
     head_final_warp(part, nctas, 0, tok, p);
     if (threadIdx.x == 0) {
-        if (*gemm_err) { atomicCAS(&st->status, 0, ST_TIMEOUT); st->timeout_where = 60; }      // a wait inside a GEMM gave up
+        if (*gemm_err) { atomicCAS(&st->status, 0, ST_TIMEOUT); st->timeout_where = 60; st->timed_out = 1; }      // a wait inside a GEMM gave up
         st->P = n; st->len_A = n; st->x0 = tok; st->pending = 0; st->total = 1; st->rounds = 0;
         out_tokens[0] = tok;
     }

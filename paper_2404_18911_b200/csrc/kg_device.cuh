@@ -95,6 +95,8 @@ struct State {
     float conf[M_MAX];
     int emitted[M_MAX];
     int target[M_MAX];
+    // the last word: 1 after a wait that gave up, until the model is built anew (exchange words and counters may hold anything)
+    int timed_out;
 };
 
 struct Dev {
@@ -273,6 +275,7 @@ __device__ __forceinline__ void record_timeout(Ctx& c, int where) {
     if (c.st) {
         atomicCAS(&c.st->status, 0, ST_TIMEOUT);
         c.st->timeout_where = where;
+        *(volatile int*)&c.st->timed_out = 1;
     }
     if (c.grid && c.bar) atomicOr(c.bar, BAR_ABORT);
 }

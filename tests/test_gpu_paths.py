@@ -183,6 +183,29 @@ def test_expired_device_wait_returns_timeout_and_leaves_the_context_usable(env):
     o = ko.KangarooOracle(shape, ki.make_weights(shape), np.float64)
     res = lockstep(g2, o, prompt, 24, shape.eta, shape.gamma, 0)
     assert not res["flips"] and res["max_logit_err"] < 2e-2
+    # an expired wait that no call has read yet outlives a reset and a filled state: its launch left exchange words behind that the
+    # next one would take for values
+    for start in ("generate", "fill_state", "bad_id"):
+        g = b.KangarooModel(shape, arena=arena)
+        if start == "bad_id":                               # another error stands in the state word already
+            g.set_wait_budget(5.0)
+            g.skip_barrier_arrival(2)
+            g.prefill_device(torch.tensor([shape.vocab] + prompt[1:], dtype=torch.int32, device="cuda"))
+        else:
+            g.prefill(prompt)
+            g.set_wait_budget(5.0)
+            g.skip_barrier_arrival(1)
+            g.draft(shape.eta, shape.gamma, sync=False)
+        with pytest.raises(b.KgError) as e:
+            if start == "fill_state":
+                g.fill_state(40, 3, 1)
+                g.verify()
+            else:
+                g.generate(prompt, 24, shape.eta, shape.gamma)
+        assert e.value.status == b.KG_E_TIMEOUT, start
+        torch.cuda.synchronize()
+    g = b.KangarooModel(shape, arena=arena)
+    assert g.generate(prompt, 24, shape.eta, shape.gamma)[0] == o.generate(prompt, 24, shape.eta, shape.gamma)
     # the streamed (bf16) path: the producer warp and the weight ring leave their waits too
     from test_gpu_parity import SMALL_BF
     gb = b.KangarooModel(SMALL_BF)
