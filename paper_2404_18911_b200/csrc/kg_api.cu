@@ -1148,10 +1148,8 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
         const int box = page_size < 16 ? page_size : 16;
         if (!make_tmap(&D.tmk, kc, 0x7fffffff, hd, box) || !make_tmap(&D.tmv, vc, 0x7fffffff, hd, box)) return tmap_failed();
         D.att_xp = (unsigned*)((char*)scratch + sc.off_xp);
-        CK(cudaMemsetAsync(D.att_xp, 0xff, 4 * (size_t)M * H * S_CAP * (hd + 4), s));      // XCH_EMPTY
-    } else {
-        CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
     }
+    CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
     AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
     typedef __nv_bfloat16 bf;

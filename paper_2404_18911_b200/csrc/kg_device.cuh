@@ -125,7 +125,7 @@ struct Dev {
     float* att_po;                 // [M_MAX][H][S_CAP][hd] split partial outputs
     float* att_ml;                 // [M_MAX][H][S_CAP][2]  split partial (max, sum)
     unsigned* att_cnt;             // [H] arrival counters
-    unsigned* att_xp;              // ring attention: [M_MAX][H][S_CAP][hd + 4] split partials as exchange words (empty between uses)
+    unsigned* att_xp;              // ring attention: [M_MAX][H][S_CAP][hd + 4] split partials; in the decode kernel exchange words (empty between uses)
     const float2* rope;            // [max_seq][hd / 2] cos, sin (null: computed where needed)
     float4* head_part;             // [nctas][M_MAX] (zmax, sumexp, argmax bits, -)
     float* dbg_draft; float* dbg_verify;   // [M_MAX][V] each (debug only)
@@ -1599,9 +1599,11 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
 //                  layout into the B layout with movmatrix.
 // With more than 8 rows a warp does both groups of 8 rows (R = 2) on the same K and V fragments.
 //
-// Splits of a head: all but the last one leave (max, sum, o) in exchange words, the last one polls them, merges in split order
-// and empties the words again (their next use lies behind the barrier at the layer's end).  It waits for items of lower number
-// only, and every CTA takes its items in rising order, so there is always one that can go on.
+// Splits of a head in the decode kernel (WAIT): all but the last one leave (max, sum, o) in exchange words, the last one polls them,
+// merges in split order and empties the words again (their next use lies behind the barrier at the layer's end).  It waits for items
+// of lower number only, every CTA takes its items in rising order, and the launch is cooperative, so there is always one that can go
+// on.  The single operator is an ordinary launch, whose CTAs may have to wait for an SM: there every split leaves its partial results
+// and counts itself, and whichever comes last merges them, in the same order (att_merge_ring); nobody waits.
 __device__ __forceinline__ unsigned movmatrix_trans(unsigned a) {
     unsigned d;
     asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
@@ -1759,7 +1761,38 @@ __device__ __forceinline__ void rope_at(const Dev& D, int pos, int e, int half, 
     else rope_cs(D, pos, e, cs, sn);
 }
 
-template <int HD, int R>
+// One split's (max, sum, four elements) added to the merge of a row
+__device__ __forceinline__ void ra_add(float& m, float& den, float4& num, float om, float ol, float4 o) {
+    const float mn = fmaxf(m, om);
+    const float f0 = m == -INFINITY ? 0.f : ex2f(m - mn), f1 = om == -INFINITY ? 0.f : ex2f(om - mn);
+    den = den * f0 + ol * f1;
+    num.x = num.x * f0 + o.x * f1; num.y = num.y * f0 + o.y * f1; num.z = num.z * f0 + o.z * f1; num.w = num.w * f0 + o.w * f1;
+    m = mn;
+}
+
+// Single operator: the merge of a head's S partial results by the CTA that came last: the last split's, then the others in order.
+template <int HD>
+__device__ __forceinline__ void att_merge_ring(const Dev& D, const AttArgs& a, int hh, int S) {
+    constexpr int ROW = RaGeom<HD>::ROW, QB = 4;
+    const int tid = tid_here(), H = D.dm.H;
+    for (int idx = tid; idx < a.M * (HD / 4); idx += NTHREADS) {
+        const int i = idx / (HD / 4), e = idx % (HD / 4) * 4;
+        const float* row = reinterpret_cast<const float*>(D.att_xp) + ((size_t)i * H + hh) * S_CAP * ROW;
+        float4 num = ldcg_f4(row + (S - 1) * ROW + e);
+        const float2 ml = ldcg_f2(row + (S - 1) * ROW + HD);
+        float m = ml.x, den = ml.y;
+        for (int q0 = 0; q0 < S - 1; q0 += QB) {
+            float4 wo[QB]; float2 wm[QB];
+#pragma unroll
+            for (int q = 0; q < QB; ++q) { const int s = min(q0 + q, S - 2); wo[q] = ldcg_f4(row + s * ROW + e); wm[q] = ldcg_f2(row + s * ROW + HD); }
+#pragma unroll
+            for (int q = 0; q < QB; ++q) if (q0 + q < S - 1) ra_add(m, den, num, wm[q].x, wm[q].y, wo[q]);
+        }
+        *reinterpret_cast<float4*>(a.out + (size_t)i * a.ldo + hh * HD + e) = make_float4(num.x / den, num.y / den, num.z / den, num.w / den);
+    }
+}
+
+template <int HD, int R, bool WAIT>
 __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, Ctx& c) {
     typedef __nv_bfloat16 WT;
     using G = RaGeom<HD>;
@@ -1920,7 +1953,7 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
                     asm volatile("" : "+l"(xrow));
 #pragma unroll
                     for (int q = 0; q < QB; ++q)
-                        if (last && q0 + q < s) { wo[q] = xch_ld4(xrow + (q0 + q) * ROW + e); wm[q] = xch_ld2(xrow + (q0 + q) * ROW + HD); }
+                        if (WAIT && last && q0 + q < s) { wo[q] = xch_ld4(xrow + (q0 + q) * ROW + e); wm[q] = xch_ld2(xrow + (q0 + q) * ROW + HD); }
                 };
                 request(0);
                 const float* row = mb + rr * ROW;
@@ -1938,12 +1971,12 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
                     den += ml[w].y * f;
                     num.x += v.x * f; num.y += v.y * f; num.z += v.z * f; num.w += v.w * f;
                 }
-                if (!last) {
+                if (WAIT ? !last : pl.S > 1) {
                     unsigned* p = xrow + s * ROW;
                     xch_st4(p + e, make_uint4(__float_as_uint(num.x), __float_as_uint(num.y), __float_as_uint(num.z), __float_as_uint(num.w)));
                     if (e == 0) { xch_st(p + HD, __float_as_uint(m)); xch_st(p + HD + 1, __float_as_uint(den)); }
                 } else {
-                    for (int q0 = 0; q0 < s; q0 += QB) {
+                    for (int q0 = 0; WAIT && q0 < s; q0 += QB) {
                         if (q0) request(q0);
                         XchSpin sp; sp.spins = 0;
                         while (true) {
@@ -1956,12 +1989,8 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
 #pragma unroll
                         for (int q = 0; q < QB; ++q) {
                             if (q0 + q < s) {
-                                const float om = __uint_as_float(wm[q].x), mn = fmaxf(m, om);
-                                const float f0 = m == -INFINITY ? 0.f : ex2f(m - mn), f1 = om == -INFINITY ? 0.f : ex2f(om - mn);
-                                den = den * f0 + __uint_as_float(wm[q].y) * f1;
-                                num.x = num.x * f0 + __uint_as_float(wo[q].x) * f1; num.y = num.y * f0 + __uint_as_float(wo[q].y) * f1;
-                                num.z = num.z * f0 + __uint_as_float(wo[q].z) * f1; num.w = num.w * f0 + __uint_as_float(wo[q].w) * f1;
-                                m = mn;
+                                ra_add(m, den, num, __uint_as_float(wm[q].x), __uint_as_float(wm[q].y),
+                                       make_float4(__uint_as_float(wo[q].x), __uint_as_float(wo[q].y), __uint_as_float(wo[q].z), __uint_as_float(wo[q].w)));
                                 xch_st4(xrow + (q0 + q) * ROW + e, make_uint4(XCH_EMPTY, XCH_EMPTY, XCH_EMPTY, XCH_EMPTY));      // this thread alone reads them
                             }
                         }
@@ -1974,7 +2003,18 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
             }
             cta_sync();
         }
-        if (last && s > 0) {
+        if (!WAIT && pl.S > 1) {
+            // this CTA's partial results are ordered before the counter by the barrier above and the release of the atomic; its
+            // acquire orders the counter before the reads of every split's
+            if (tid == 0) {
+                unsigned prev;
+                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(D.att_cnt + hh) : "memory");
+                c.ctl->att_last = prev == (unsigned)(pl.S - 1);
+            }
+            cta_sync();
+            if (*(volatile int*)&c.ctl->att_last) att_merge_ring<HD>(D, a, hh, pl.S);
+        }
+        if (WAIT && last && s > 0) {
             // maxima and sums have been read by every thread of the merge
             for (int idx = tid; idx < M * s; idx += NTHREADS) {
                 unsigned* p = xw + (((size_t)(idx / s) * H + hh) * S_CAP + idx % s) * ROW + HD;
@@ -1986,13 +2026,13 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
 }
 
 // ring: the tensor-core attention, fed by the copy warp (decided once per model: bf16 streamed path, head_dim 64 or 128).
-// R: row groups, 1 or 2, or 0 where both may come.
+// R: row groups, 1 or 2 (the single operator), or 0 where both may come (the decode kernel).
 template <typename WT, int HD, int R = 0>
 __device__ __forceinline__ void attention_op(const Dev& D, const AttArgs& a, Ctx& c, bool ring) {
     if constexpr (sizeof(WT) == 2 && HD >= 64) {
         if (ring) {
-            if constexpr (R != 0) attention_ring<HD, R>(D, a, c);
-            else if (a.M <= 8) attention_ring<HD, 1>(D, a, c); else attention_ring<HD, 2>(D, a, c);
+            if constexpr (R != 0) attention_ring<HD, R, false>(D, a, c);
+            else if (a.M <= 8) attention_ring<HD, 1, true>(D, a, c); else attention_ring<HD, 2, true>(D, a, c);
             return;
         }
     }

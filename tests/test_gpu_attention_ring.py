@@ -50,3 +50,26 @@ def test_attention_ring(env, H, hd, M, pos0, ps):
     # q and p keep 17 bits, fp32 sums: about 5e-6 of the norm is seen, at most 7e-5 of the root mean square in one element
     e = out.double() - ref
     assert e.norm() / ref.norm() < 2e-5 and e.abs().max() < 3e-4 * ref.square().mean().sqrt().clamp_min(0.05)
+
+
+# heads whose splits run on CTAs of two waves: calls on several streams share the SMs, and a CTA may start when others have ended
+@pytest.mark.parametrize("H,hd,M,pos0", [(40, 128, 7, 3001), (12, 64, 16, 6000)])
+def test_splits_of_calls_that_overlap(env, H, hd, M, pos0):
+    torch, b = env
+    g = torch.Generator(device="cuda").manual_seed(1)
+    pages = (pos0 + M + 15) // 16
+    kc, vc = (torch.empty(pages, H, 16, hd, device="cuda", dtype=torch.bfloat16).normal_(generator=g) for _ in range(2))
+    table = torch.randperm(pages, generator=g, device="cuda").to(torch.int32)
+    qkv = torch.empty(M, 3 * H * hd, device="cuda").normal_(generator=g)
+    ref = b.op_attention(qkv, pos0, H, hd, 10000.0, kc, vc, table, 16)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    state = [(kc.clone(), vc.clone(), b.op_scratch(torch)) for _ in streams]
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(8):
+        for s, (k, v, scratch) in zip(streams, state):
+            with torch.cuda.stream(s):
+                outs.append(b.op_attention(qkv, pos0, H, hd, 10000.0, k, v, table, 16, scratch=scratch))
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, ref) for o in outs)
