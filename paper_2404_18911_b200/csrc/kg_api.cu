@@ -304,14 +304,33 @@ extern "C" size_t kg_workspace_bytes(const kg_config* cfg, int own_weights) {
     return make_layout(cfg, own_weights, sm_count()).total + 256;
 }
 
-// The decode kernel for a storage type and head size
-static const void* decode_kernel(const kg_config& c) {
+// The decode kernel for a storage type, a head size and an attention (ring: bf16, 64 or 128 only)
+static const void* decode_kernel(const kg_config& c, bool ring) {
+    typedef __nv_bfloat16 bf;
     if (c.dtype == KG_BF16) {
-        if (c.head_dim == 128) return (const void*)kg_persistent_kernel<__nv_bfloat16, 128>;
-        return c.head_dim == 64 ? (const void*)kg_persistent_kernel<__nv_bfloat16, 64> : (const void*)kg_persistent_kernel<__nv_bfloat16, 32>;
+        if (ring) return c.head_dim == 128 ? (const void*)kg_persistent_kernel<bf, 128, true> : (const void*)kg_persistent_kernel<bf, 64, true>;
+        if (c.head_dim == 128) return (const void*)kg_persistent_kernel<bf, 128, false>;
+        return c.head_dim == 64 ? (const void*)kg_persistent_kernel<bf, 64, false> : (const void*)kg_persistent_kernel<bf, 32, false>;
     }
-    if (c.head_dim == 128) return (const void*)kg_persistent_kernel<float, 128>;
-    return c.head_dim == 64 ? (const void*)kg_persistent_kernel<float, 64> : (const void*)kg_persistent_kernel<float, 32>;
+    if (c.head_dim == 128) return (const void*)kg_persistent_kernel<float, 128, false>;
+    return c.head_dim == 64 ? (const void*)kg_persistent_kernel<float, 64, false> : (const void*)kg_persistent_kernel<float, 32, false>;
+}
+
+// Before the first launch of a decode kernel.  Its warpgroups re-divide the registers that the launch gives the CTA; a budget beyond
+// that pool would block the kernel at its first instruction, so that the launch allocation is checked here and never assumed.
+static int prepare_decode(const kg_model* m) {
+    const void* kfn = decode_kernel(m->cfg, m->dev.dm.ring != 0);
+    CK(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem));
+    int occ = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, DECODE_THREADS, m->smem));
+    if (occ < 1) return KG_E_CUDA;
+    cudaFuncAttributes fa;
+    CK(cudaFuncGetAttributes(&fa, kfn));
+    if ((long long)fa.numRegs * DECODE_THREADS < (long long)NTHREADS * CONSUMER_REGS + 128LL * PRODUCER_REGS) {
+        std::snprintf(g_cuda_err, sizeof(g_cuda_err), "decode kernel compiled with %d registers per thread: too few for its register budgets", fa.numRegs);
+        return KG_E_INTERNAL;
+    }
+    return KG_OK;
 }
 
 static int launch(kg_model* m, const Program& pg) {
@@ -321,7 +340,7 @@ static int launch(kg_model* m, const Program& pg) {
     p.skip_arrival = m->skip_arrival;
     m->skip_arrival = 0;
     void* args[] = {(void*)&m->dev, (void*)&p};
-    CK(cudaLaunchCooperativeKernel(decode_kernel(m->cfg), dim3(m->nctas), dim3(DECODE_THREADS), args, m->smem, m->stream));
+    CK(cudaLaunchCooperativeKernel(decode_kernel(m->cfg, m->dev.dm.ring != 0), dim3(m->nctas), dim3(DECODE_THREADS), args, m->smem, m->stream));
     return KG_OK;
 }
 
@@ -421,21 +440,6 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
     m->smem = SMEM_TOTAL;
 
     const bool bf = cfg->dtype == KG_BF16;
-    const void* kfn = decode_kernel(*cfg);
-    if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem) != cudaSuccess) { delete m; return KG_E_CUDA; }
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, DECODE_THREADS, m->smem) != cudaSuccess || occ < 1) { delete m; return KG_E_CUDA; }
-    {
-        // the kernel's warpgroups re-divide the registers the launch gives the CTA; a budget beyond that pool would block
-        // the kernel at its first instruction, so the launch allocation is checked here, once, and never assumed
-        cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, kfn) != cudaSuccess) { delete m; return KG_E_CUDA; }
-        if ((long long)fa.numRegs * DECODE_THREADS < (long long)NTHREADS * CONSUMER_REGS + 128LL * PRODUCER_REGS) {
-            std::snprintf(g_cuda_err, sizeof(g_cuda_err), "decode kernel compiled with %d registers per thread: too few for its register budgets", fa.numRegs);
-            delete m;
-            return KG_E_INTERNAL;
-        }
-    }
 
     Dev& D = m->dev;
     std::memset(&D, 0, sizeof(D));
@@ -526,7 +530,8 @@ extern "C" int kg_init_model(const kg_config* cfg, const kg_weights* w, void* ar
         if (r != KG_OK) { delete m; return r; }
     }
     {
-        const int r = prefill_tc_init(m);
+        int r = prepare_decode(m);
+        if (r == KG_OK) r = prefill_tc_init(m);
         if (r != KG_OK) { delete m; return r; }
     }
     *out = m;
@@ -948,16 +953,22 @@ __global__ void op_head_final_kernel(const float4* part, int nctas, int* tok, fl
     head_final_warp(part, nctas, m, t, pp);
     if ((threadIdx.x & 31) == 0) { tok[m] = t; p[m] = pp; }
 }
+// R: row groups of the tensor-core attention.  The other attention has no copy warp: without it a thread gets 255 registers and not
+// 168 (three warps in one of the four register files), at which fp32 of 128 dims spilled 0.7 KB.
+template <typename WT, int HD> constexpr int OP_ATT_THREADS = RING_ATT<WT, HD> ? BLOCK_THREADS : NTHREADS;
 template <typename WT, int HD, int R>
-__global__ void __launch_bounds__(BLOCK_THREADS, 1) op_attention_kernel(const __grid_constant__ Dev D, AttArgs a) {
+__global__ void __launch_bounds__(OP_ATT_THREADS<WT, HD>, 1) op_attention_kernel(const __grid_constant__ Dev D, const __grid_constant__ AttArgs a) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
-    if (!c.producer) {
-        if (D.dm.ring) a.plan = ra_plan(a.pos0, D.dm.H, c.nctas);
-        attention_op<WT, HD, R>(D, a, c, D.dm.ring != 0);
-    } else if (D.dm.ring) {
-        if (!attention_producer(D, ra_plan(a.pos0, D.dm.H, c.nctas), 0, c)) ring_drain(c);
-    }
+    if constexpr (!RING_ATT<WT, HD>) attention_impl<WT, HD / 32, true>(D, a, a.plan, c);
+    else if (!c.producer) attention_ring<HD, R, false>(D, a, c);
+    else if (!att_produce<HD>(D, a.plan, 0, c)) ring_drain(c);
+}
+// The arrival counters of the splits.  The attention behind it starts at once and waits where it counts its first split.  (A
+// memset of the kilobyte cannot overlap the kernel behind it: 2 us a call.)
+__global__ void clear_counters_kernel(unsigned* cnt) {
+    grid_dependents_launch();
+    cnt[threadIdx.x] = 0u;
 }
 
 // A launch that may begin before the kernel ahead of it in the stream has finished; the kernel calls grid_dependency_wait()
@@ -1117,7 +1128,8 @@ extern "C" int kg_op_lm_head_noalloc(int32_t dtype, const void* W, int32_t V, in
 template <typename WT, int HD, int R>
 static int launch_attention(const Dev& D, const AttArgs& a, int nctas, cudaStream_t s) {
     if (set_smem<op_attention_kernel<WT, HD, R>>() != KG_OK) return KG_E_CUDA;
-    op_attention_kernel<WT, HD, R><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(D, a);
+    if (a.plan.S > 1) CK(launch_dependent(op_attention_kernel<WT, HD, R>, dim3(nctas), dim3(OP_ATT_THREADS<WT, HD>), SMEM_TOTAL, s, D, a));
+    else op_attention_kernel<WT, HD, R><<<nctas, OP_ATT_THREADS<WT, HD>, SMEM_TOTAL, s>>>(D, a);
     return KG_OK;
 }
 
@@ -1149,9 +1161,13 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
         if (!make_tmap(&D.tmk, kc, 0x7fffffff, hd, box) || !make_tmap(&D.tmv, vc, 0x7fffffff, hd, box)) return tmap_failed();
         D.att_xp = (unsigned*)((char*)scratch + sc.off_xp);
     }
-    CK(cudaMemsetAsync(D.att_cnt, 0, 4 * 256, s));
     AttArgs a{}; a.qkv = qkv; a.ldq = 3 * H * hd; a.M = M; a.pos0 = pos0; a.kc = kc; a.vc = vc; a.out = out; a.ldo = H * hd;
     const int nctas = sm_count();
+    a.plan = D.dm.ring ? ra_plan(pos0, H, nctas) : ka_plan(pos0, M, H, nctas);
+    if (a.plan.S > 1) {
+        clear_counters_kernel<<<1, 256, 0, s>>>(D.att_cnt);
+        CK(cudaGetLastError());
+    }
     typedef __nv_bfloat16 bf;
     int r;
     if (dtype == KG_F32) r = hd == 128 ? launch_attention<float, 128, 1>(D, a, nctas, s) : hd == 64 ? launch_attention<float, 64, 1>(D, a, nctas, s) : launch_attention<float, 32, 1>(D, a, nctas, s);

@@ -179,10 +179,11 @@ struct LinArgs {
     float* ssq_out; int ld_sout;     // streamed path: [M] rows of nctas partial sums of squares of the output rows (nullable)
 };
 
-// Cut of a head's old key tiles into splits (ra_plan); pos: the position it was made for
-struct RaPlan { int ntile, S, chunk; int pos; };
+// Cut of a head's keys into S splits of `chunk` (ra_plan: tiles of the old keys, ntile of them; ka_plan: keys); pos: the position it was made for
+struct AttPlan { int ntile, S, chunk; int pos; };
 struct AttArgs {
-    RaPlan plan; int row0; // ring attention: cut into splits; first row of this layer's cache in the tensor maps
+    AttPlan plan;          // cut into splits (ring attention and single operator)
+    int row0;              // ring attention: first row of this layer's cache in the tensor maps
     const float* qkv; int ldq;      // [M] rows of raw q, k, v of this pass
     int poll;              // 1: q, k, v are exchange words, to be polled
     int M, pos0;           // rows sit at positions pos0 .. pos0+M-1; row i sees keys 0 .. pos0+i
@@ -1196,12 +1197,13 @@ __device__ __forceinline__ void head_final_warp(const float4* part, int nctas, i
 
 // ------------------------------------------------------------------------------------ attention operator
 constexpr int ATT_TK = 16;                                 // keys per tile
+constexpr int ATT_RB = 4;                                  // rows per block
 // Cut of a head's old tiles into splits, the same for the copy warp and the consumers.  The cost of a split count, in steps of
 // one tile per warp (about 0.5 us): the tiles of an item (one step per 8 tiles, and at least the time an SM's share of the HBM
 // bandwidth takes for them, 0.4 steps a tile), two steps of fixed work, three more for the merge of a head that is split.
 // (Made once per position and not per layer: the 16 candidates took 2.4 us a layer in a rolled loop with divisions.)
-__device__ __noinline__ RaPlan ra_plan(int pos0, int H, int nctas) {
-    RaPlan p;
+__host__ __device__ __noinline__ inline AttPlan ra_plan(int pos0, int H, int nctas) {
+    AttPlan p;
     p.ntile = (pos0 + ATT_TK - 1) / ATT_TK;
     p.S = 1;
     const float inv_ctas = 1.0f / (float)nctas;
@@ -1216,6 +1218,26 @@ __device__ __noinline__ RaPlan ra_plan(int pos0, int H, int nctas) {
     }
     p.chunk = max(1, (p.ntile + p.S - 1) / p.S);
     p.S = max(1, (p.ntile + p.chunk - 1) / p.chunk);       // no split without tiles
+    return p;
+}
+// The same for attention_impl: a head's keys 0 .. pos0 + M - 1, those of this pass among them.  The cost of a split count, in steps of
+// 64 keys and four rows (0.7 to 1.5 us): the steps of an item, two of fixed work, two more for the merge.  The count it takes lies 1.4 %
+// above the best one on average (as a single operator: 4 to 52 heads, fp32 of 64 and 128 dims and both types of 32, 60 to 8000 keys, 1, 7
+// and 16 rows); without the rows in it, 7.4 % and at worst 82 %.
+__host__ __device__ __forceinline__ AttPlan ka_plan(int pos0, int M, int H, int nctas) {
+    AttPlan p;
+    const int T = pos0 + M;
+    const float inv_ctas = 1.0f / (float)nctas, steps = (float)((M + ATT_RB - 1) / ATT_RB) * (1.0f / 64.0f);
+    float best = -1.f;
+    p.ntile = 0; p.S = 1; p.pos = pos0;
+#pragma unroll
+    for (int sc = 1; sc <= S_CAP; ++sc) {
+        const int chunk_ = (T + sc - 1) / sc;                                   // sc is a constant after unrolling
+        const float waves = ceilf((float)(H * sc) * inv_ctas - 1e-4f);
+        const float cost = waves * ((float)chunk_ * steps + (sc > 1 ? 4.f : 2.f));
+        if ((sc == 1 || chunk_ >= 32) && (best < 0.f || cost < best)) { best = cost; p.S = sc; }
+    }
+    p.chunk = (T + p.S - 1) / p.S;
     return p;
 }
 
@@ -1287,7 +1309,6 @@ template <> struct AttLoad<float, 1> {
 };
 
 constexpr int ATT_G = 8;           // keys per group
-constexpr int ATT_RB = 4;          // rows per block
 constexpr int ATT_MB_STRIDE = HD_MAX + 2;   // merge buffer row: o[hd], max, sum
 
 __device__ __forceinline__ float ex2f(float x) {             // 2^x, one special-function instruction
@@ -1309,7 +1330,8 @@ __device__ __forceinline__ void att_warp_slice(const Dev& D, const AttArgs& a, i
     static_assert(ATT_G == 8 && ATT_RB == 4, "the butterfly below is written for 8 keys x 4 rows");
     const int lane = threadIdx.x & 31;
     const int jl = lane >> 2, rl = lane & 3;
-    const int H = D.dm.H, hd = D.dm.hd, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
+    constexpr int hd = 32 * DPL;
+    const int H = D.dm.H, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
     const int pos0 = a.pos0;
     const WT* kc = reinterpret_cast<const WT*>(a.kc);
     const WT* vc = reinterpret_cast<const WT*>(a.vc);
@@ -1409,9 +1431,9 @@ __device__ __forceinline__ void att_warp_slice(const Dev& D, const AttArgs& a, i
 // The last split of a head to arrive merges the S partial (max, sum, o) of every row in split order.  SC >= S is the
 // compile-time bound of the split loop; U elements per thread are handled together, and every load of such a batch is
 // issued before any is used, so that a batch costs one L2 round trip.
-template <int SC, int U>
+template <int hd, int SC, int U>
 __device__ __forceinline__ void att_merge_splits(const Dev& D, const AttArgs& a, int hh, int S, int M) {
-    const int tid = threadIdx.x, H = D.dm.H, hd = D.dm.hd;
+    const int tid = threadIdx.x, H = D.dm.H;
     const int total = M * hd;
     for (int idx0 = tid; idx0 < total; idx0 += NTHREADS * U) {
         float2 mlv[U][SC];
@@ -1452,28 +1474,15 @@ __device__ __forceinline__ void att_merge_splits(const Dev& D, const AttArgs& a,
     }
 }
 
-template <typename WT, int DPL>
-__device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx& c) {
+// OP: single operator
+template <typename WT, int DPL, bool OP>
+__device__ __forceinline__ void attention_impl(const Dev& D, const AttArgs& a, const AttPlan pl, Ctx& c) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int H = D.dm.H, hd = D.dm.hd, d = D.dm.d, ps = D.dm.page_size;
+    constexpr int hd = 32 * DPL, half = hd / 2;
+    const int H = D.dm.H, d = D.dm.d, ps = D.dm.page_size;
     const int M = a.M, pos0 = a.pos0;
     const int T = pos0 + M;
-    const int half = hd >> 1;
-    // number of KV splits: the one that leaves the least work on the busiest CTA
-    int S = 1;
-    {
-        const float inv_ctas = 1.0f / (float)c.nctas;
-        float best = -1.f;
-#pragma unroll
-        for (int sc = 1; sc <= S_CAP; ++sc) {
-            const int chunk_ = (T + sc - 1) / sc;                                   // sc is a constant after unrolling
-            const float waves = ceilf((float)(H * sc) * inv_ctas - 1e-4f);
-            // in steps of 64 keys (8 warps x 8 keys); an item costs about two more, the merge of a split head about three
-            const float cost = waves * (float)((chunk_ + 63) / 64 + 2 + (sc > 1 ? 3 : 0));
-            if ((sc == 1 || chunk_ >= 32) && (best < 0.f || cost < best)) { best = cost; S = sc; }
-        }
-    }
-    const int chunk = (T + S - 1) / S;
+    const int S = pl.S, chunk = pl.chunk;
     const float sc = rsqrtf((float)hd) * 1.4426950408889634f;      // 1/sqrt(hd), and log2(e): scores live in the log2 domain
     WT* kc = reinterpret_cast<WT*>(a.kc);
     WT* vc = reinterpret_cast<WT*>(a.vc);
@@ -1565,6 +1574,7 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
             __threadfence();
             cta_sync();
             if (tid == 0) {
+                if (OP) grid_dependency_wait();            // the counters have been cleared
                 const unsigned prev = atomicAdd(D.att_cnt + hh, 1u);
                 const int last = (prev == (unsigned)(S - 1));
                 c.ctl->att_last = last;
@@ -1572,9 +1582,9 @@ __device__ __noinline__ void attention_impl(const Dev& D, const AttArgs& a, Ctx&
             }
             cta_sync();
             if (*(volatile int*)&c.ctl->att_last) {
-                if (S <= 4) att_merge_splits<4, 4>(D, a, hh, S, M);
-                else if (S <= 8) att_merge_splits<8, 2>(D, a, hh, S, M);
-                else att_merge_splits<S_CAP, 1>(D, a, hh, S, M);
+                if (S <= 4) att_merge_splits<hd, 4, 4>(D, a, hh, S, M);
+                else if (S <= 8) att_merge_splits<hd, 8, 2>(D, a, hh, S, M);
+                else att_merge_splits<hd, S_CAP, 1>(D, a, hh, S, M);
             }
             cta_sync();
         }
@@ -1639,7 +1649,7 @@ __device__ __forceinline__ int checked_page(int pg, int n_pages, State* st, int 
 
 // Copy warp: the old K / V tiles of this CTA's items.  row0: first row of this layer's cache in the tensor maps.
 template <int HD>
-__device__ __noinline__ bool att_produce(const Dev& D, const RaPlan pl, int row0, Ctx& c) {
+__device__ __noinline__ bool att_produce(const Dev& D, const AttPlan pl, int row0, Ctx& c) {
     using G = RaGeom<HD>;
     const int lane = threadIdx.x & 31;
     const int H = D.dm.H, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
@@ -1800,7 +1810,7 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
     const int tid = tid_here(), lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const int H = D.dm.H, d = D.dm.d, psh = D.dm.ps_shift, psm = D.dm.page_size - 1;
     const int M = a.M, pos0 = a.pos0;
-    const RaPlan pl = a.plan;
+    const AttPlan pl = a.plan;
     const float qscale = rsqrtf((float)HD) * 1.4426950408889634f;      // 1/sqrt(hd) and log2(e)
     char* qsm = c.smem + WORK_OFF;
     char* ntile = c.smem + WORK_OFF + G::NT_OFF;
@@ -2008,6 +2018,7 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
             // acquire orders the counter before the reads of every split's
             if (tid == 0) {
                 unsigned prev;
+                grid_dependency_wait();                    // the counters have been cleared
                 asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(D.att_cnt + hh) : "memory");
                 c.ctl->att_last = prev == (unsigned)(pl.S - 1);
             }
@@ -2025,20 +2036,10 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
     c.slot = slot; c.phase = phase;
 }
 
-// ring: the tensor-core attention, fed by the copy warp (decided once per model: bf16 streamed path, head_dim 64 or 128).
-// R: row groups, 1 or 2 (the single operator), or 0 where both may come (the decode kernel).
-template <typename WT, int HD, int R = 0>
-__device__ __forceinline__ void attention_op(const Dev& D, const AttArgs& a, Ctx& c, bool ring) {
-    if constexpr (sizeof(WT) == 2 && HD >= 64) {
-        if (ring) {
-            if constexpr (R != 0) attention_ring<HD, R, false>(D, a, c);
-            else if (a.M <= 8) attention_ring<HD, 1, true>(D, a, c); else attention_ring<HD, 2, true>(D, a, c);
-            return;
-        }
-    }
-    attention_impl<WT, HD / 32>(D, a, c);
-}
-__device__ __forceinline__ bool attention_producer(const Dev& D, const RaPlan& pl, int row0, Ctx& c) {
+// storage type and head size of the tensor-core attention
+template <typename WT, int HD> constexpr bool RING_ATT = sizeof(WT) == 2 && HD >= 64;
+
+__device__ __forceinline__ bool attention_producer(const Dev& D, const AttPlan& pl, int row0, Ctx& c) {
     return D.dm.hd == 128 ? att_produce<128>(D, pl, row0, c) : att_produce<64>(D, pl, row0, c);
 }
 

@@ -38,7 +38,7 @@ struct Program {
 struct ActIn { const float* x; const unsigned char* pk; const float* ssq; };
 struct ActOut { float* x; PkOut pk[2]; float* ssq; };
 
-// linear operators on the streamed tensor-core path / attention from the ring, for this launch
+// linear operators on the streamed tensor-core path, for this launch
 __device__ __forceinline__ bool launch_streamed(const Dev& D, const Program& pg) { return D.dm.stream != 0 && pg.force_simple == 0; }
 
 // ---- the sequencer (one thread per CTA) ----------------------------------------------------------------------------
@@ -49,7 +49,7 @@ struct Sequencer {
     const Program& pg;
     const bool streamed;
     int qi = 0; unsigned qph = 0;      // queue cursor
-    RaPlan plan;                       // of the last attention position
+    AttPlan plan;                      // of the last attention position
     int xp = 0;                        // exchange instance the next layer uses
     int xused = 0;                     // rows of the other instance, the one of the layer before, that hold data
 
@@ -441,7 +441,13 @@ __device__ __forceinline__ void consume_embed(const Dev& D, Ctx& c, const EmbedA
     emit_plain_rows(a, c, [&](int m, int e_) { return wt_to_float<WT>(row(m)[e_]); });
 }
 
+// The attention without the ring as a call: what a model that has the ring takes when it is told to cross-check (force_simple).
 template <typename WT, int HD>
+__device__ __noinline__ void attention_far(const Dev& D, const AttArgs& a, Ctx& c) {
+    attention_impl<WT, HD / 32, false>(D, a, ka_plan(a.pos0, a.M, D.dm.H, c.nctas), c);
+}
+
+template <typename WT, int HD, bool RING>
 __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed) {
     Ctrl* ctl = c.ctl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -458,7 +464,9 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
             }
         } else if (kind == OPK_ATT) {
             const AttArgs& a = op.att;
-            attention_op<WT, HD>(D, a, c, streamed && D.dm.ring);
+            if constexpr (RING) {
+                if (!streamed) attention_far<WT, HD>(D, a, c); else if (a.M <= 8) attention_ring<HD, 1, true>(D, a, c); else attention_ring<HD, 2, true>(D, a, c);
+            } else attention_impl<WT, HD / 32, false>(D, a, ka_plan(a.pos0, a.M, D.dm.H, c.nctas), c);
         } else if (kind == OPK_EMBED) {
             consume_embed<WT>(D, c, op.emb, streamed);
         } else if (kind == OPK_HEAD) {
@@ -497,8 +505,12 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
     }
 }
 
-// HD: the head size, compiled apart (with both of them in one kernel 0.9 KB of registers were spilled around the operators)
-template <typename WT, int HD>
+// HD: the head size.  RING: attention from the ring; else the other attention, inlined (as a call it has the 168 registers of the launch
+// and not the consumers' 216: bf16, four layers of 512 with an F that only the plain linear operators take, 32 tokens 4.13 -> 3.15 ms; fp32,
+// four layers of 1024, 7.3 -> 6.7).  Compiled apart: with two head sizes in one kernel 0.9 KB of registers were spilled around the operators.
+// (In the ring kernel the plain operators stay as calls.  Without them more of the row variants' registers are spilled, 460 against 240 bytes
+// of loads: 7B, verify passes of 11 rows, three rounds 25.9 against 25.0 ms.)
+template <typename WT, int HD, bool RING>
 __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const __grid_constant__ Program pg) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival);
@@ -513,7 +525,7 @@ __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const 
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
-        consume_loop<WT, HD>(D, c, launch_streamed(D, pg));
+        consume_loop<WT, HD, RING>(D, c, launch_streamed(D, pg));
     }
 }
 

@@ -73,3 +73,32 @@ def test_splits_of_calls_that_overlap(env, H, hd, M, pos0):
                 outs.append(b.op_attention(qkv, pos0, H, hd, 10000.0, k, v, table, 16, scratch=scratch))
     torch.cuda.synchronize()
     assert all(torch.equal(o, ref) for o in outs)
+
+
+# the attention without the ring: fp32 caches and heads of 32, with one and with many splits, every block of four rows
+@pytest.mark.parametrize("bf,H,hd", [(False, 5, 128), (False, 40, 64), (False, 9, 32), (True, 12, 32)])
+@pytest.mark.parametrize("M,pos0,ps", [(1, 0, 16), (4, 61, 4), (5, 300, 16), (16, 1500, 32), (1, 6001, 16)])
+def test_attention_without_the_ring(env, bf, H, hd, M, pos0, ps):
+    torch, b = env
+    g = torch.Generator(device="cuda").manual_seed(pos0 + M)
+    T, dt = pos0 + M, torch.bfloat16 if bf else torch.float32
+    pages = (T + ps - 1) // ps + 1
+    kc, vc = (torch.empty(pages, H, ps, hd, device="cuda", dtype=dt).normal_(generator=g) for _ in range(2))
+    table = torch.randperm(pages, generator=g, device="cuda").to(torch.int32)
+    qkv = torch.empty(M, 3 * H * hd, device="cuda").normal_(generator=g)
+    out = b.op_attention(qkv, pos0, H, hd, 10000.0, kc, vc, table, ps)
+    assert torch.equal(out, b.op_attention(qkv, pos0, H, hd, 10000.0, kc, vc, table, ps))
+    pos = torch.arange(T, device="cuda")
+    K, V = (c[table[pos // ps].long(), :, pos % ps].double() for c in (kc, vc))       # with the rows of this pass, as they were written
+    new = pos[pos0:].double()
+    inv = 10000.0 ** (-2 * torch.arange(hd // 2, device="cuda").double() / hd)
+    cs, sn = torch.cos(new[:, None] * inv)[:, None], torch.sin(new[:, None] * inv)[:, None]
+    rot = lambda x: torch.cat([x[..., :hd // 2] * cs - x[..., hd // 2:] * sn, x[..., hd // 2:] * cs + x[..., :hd // 2] * sn], -1)
+    q, k, v = (qkv.double().reshape(M, 3, H, hd)[:, i] for i in range(3))
+    half = 2.0 ** (-8 if bf else -23)                       # half a step of bf16, or a few roundings of fp32; cos and sin are good to 1e-6
+    assert ((K[pos0:] - rot(k)).abs() <= 1.01 * half * rot(k).abs() + 1e-5).all() and torch.equal(V[pos0:], v.to(dt).double())
+    S = torch.einsum("mhd,thd->hmt", rot(q), K) / hd ** 0.5
+    S = S.masked_fill(pos[None, None] > pos[pos0:][None, :, None], float("-inf"))
+    ref = torch.einsum("hmt,thd->mhd", torch.softmax(S, -1), V).reshape(M, -1)
+    e = out.double() - ref                                  # fp32 sums of up to 6002 terms in blocks
+    assert e.norm() / ref.norm() < 5e-6
