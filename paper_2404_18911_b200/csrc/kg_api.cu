@@ -1149,13 +1149,16 @@ extern "C" int kg_op_attention(int32_t dtype, const float* qkv, int32_t M, int32
     std::memset(&D, 0, sizeof(D));
     D.dm.H = H; D.dm.hd = hd; D.dm.d = H * hd; D.dm.page_size = page_size; D.dm.theta = theta;
     D.dm.n_pages = (pos0 + M + page_size - 1) / page_size;       // entries of page_table this call may touch
-    D.dm.n_phys = 0x7fffffff / (H * page_size);                  // the caller's cache: its page count is not known here
+    // the caller's cache: its page count is not known here.  The ring's tensor maps count the rows of all pages in 31 bits
+    const long long page_rows = (long long)H * page_size;
+    D.dm.ring = dtype == KG_BF16 && hd != 32;
+    if (D.dm.ring && page_rows > 0x7fffffff) return KG_E_ARG;
+    D.dm.n_phys = D.dm.ring ? (int)(0x7fffffff / page_rows) : 0x7fffffff;
     for (D.dm.ps_shift = 0; (1 << D.dm.ps_shift) < page_size; ++D.dm.ps_shift) {}
     for (int i = 0; i < hd / 2; ++i) D.inv_freq[i] = std::pow((double)theta, -2.0 * (double)i / (double)hd);
     D.page_table = page_table;
     D.att_po = (float*)((char*)scratch + sc.off_po); D.att_ml = (float*)((char*)scratch + sc.off_ml);
     D.att_cnt = (unsigned*)((char*)scratch + sc.off_cnt);
-    D.dm.ring = dtype == KG_BF16 && hd != 32;
     if (D.dm.ring) {
         const int box = page_size < 16 ? page_size : 16;
         if (!make_tmap(&D.tmk, kc, 0x7fffffff, hd, box) || !make_tmap(&D.tmv, vc, 0x7fffffff, hd, box)) return tmap_failed();

@@ -1,6 +1,8 @@
 """The C-ABI library builds for sm_100a, loads without a GPU and exports every declared symbol."""
 import os
 import re
+import subprocess
+import sys
 
 
 def test_library_exports_every_declared_symbol():
@@ -81,3 +83,18 @@ def test_misaligned_device_pointers_are_refused_before_anything_is_launched():
         h = C.c_void_p()
         assert lib.kg_init_model(C.byref(cfg), C.byref(w), ok, 1 << 40, None, C.byref(h)) == b.KG_E_ARG, field
         assert not h.value
+
+
+def test_attention_operator_counts_the_rows_of_a_page_in_64_bits():
+    """heads x page size of 2^32 and 2^31: the call must answer (here: no device, or too large for the ring), not divide by zero.
+    In a process that sees no GPU, so that nothing can be launched on these pointers."""
+    code = ("import ctypes as C, sys\n"
+            "from paper_2404_18911_b200 import binding as b\n"
+            "lib = b.load(); p = 1 << 20\n"
+            "r = [lib.kg_op_attention(dt, p, 1, 0, H, hd, 10000.0, p, p, p, ps, p, p, None)\n"
+            "     for dt, H, hd, ps in ((b.KG_F32, 256, 32, 1 << 24), (b.KG_BF16, 128, 64, 1 << 25), (b.KG_BF16, 128, 64, 1 << 24))]\n"
+            "print(r, [b.KG_E_CUDA, b.KG_E_ARG, b.KG_E_ARG]); sys.exit(r != [b.KG_E_CUDA, b.KG_E_ARG, b.KG_E_ARG])")
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout, r.stderr[-500:])
