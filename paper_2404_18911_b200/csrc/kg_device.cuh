@@ -1308,6 +1308,13 @@ template <> struct AttLoad<float, 1> {
     static __device__ __forceinline__ void cvt(const Raw& r, float (&v)[1]) { v[0] = r; }
 };
 
+// A page number outside the cache never becomes an address: the access goes to page 0 and the state word records it.
+__device__ __forceinline__ int checked_page(int pg, int n_pages, State* st, int where) {
+    if ((unsigned)pg < (unsigned)n_pages) return pg;
+    if (st) { atomicCAS(&st->status, 0, ST_INTERNAL); st->timeout_where = where; }
+    return 0;
+}
+
 constexpr int ATT_G = 8;           // keys per group
 constexpr int ATT_MB_STRIDE = HD_MAX + 2;   // merge buffer row: o[hd], max, sum
 
@@ -1347,10 +1354,11 @@ __device__ __forceinline__ void att_warp_slice(const Dev& D, const AttArgs& a, i
     // page table entries of a window of keys live in the lanes (lane p holds page first_page + p)
     const int win = max(ATT_G, ((31 << psh) >> 3) << 3);
     int wstart = kb, first_page = kb >> psh;
-    int pgs = __ldg(page_table + min(first_page + lane, D.dm.n_pages - 1));
+    auto pages = [&]() { return checked_page(__ldg(page_table + min(first_page + lane, D.dm.n_pages - 1)), D.dm.n_phys, D.st, 53); };
+    int pgs = pages();
     Raw kr[ATT_G], vr[ATT_G];
     auto issue = [&](int g0) {
-        if (g0 >= wstart + win) { wstart = g0; first_page = g0 >> psh; pgs = __ldg(page_table + min(first_page + lane, D.dm.n_pages - 1)); }
+        if (g0 >= wstart + win) { wstart = g0; first_page = g0 >> psh; pgs = pages(); }
 #pragma unroll
         for (int j = 0; j < ATT_G; ++j) {
             const int pos = min(g0 + j, ke - 1);
@@ -1516,7 +1524,7 @@ __device__ __forceinline__ void attention_impl(const Dev& D, const AttArgs& a, c
                 float xv[4];
                 att_read<4>(a, c, p, xv);
                 const float k1 = xv[0], k2 = xv[1], v1 = xv[2], v2 = xv[3];
-                const int page = __ldg(D.page_table + (pos >> D.dm.ps_shift));
+                const int page = checked_page(__ldg(D.page_table + (pos >> D.dm.ps_shift)), D.dm.n_phys, D.st, 54);
                 float cs, sn; rope_cs(D, pos, e, cs, sn);
                 const size_t base = (((size_t)page * H + hh) * ps + (pos & (ps - 1))) * hd;
                 kc[base + e] = float_to_wt<WT>(k1 * cs - k2 * sn);
@@ -1639,13 +1647,6 @@ template <int HD> struct RaGeom {
 };
 static_assert(2 * RaGeom<128>::QG <= RaGeom<128>::NT_OFF && RaGeom<128>::TPS * RaGeom<128>::TILE_BYTES <= SLOT_BYTES, "attention tiles");
 static_assert(RaGeom<128>::MB_OFF + NWARPS * ATT_RB * RaGeom<128>::ROW * 4 <= WORK_BYTES && WORK_OFF % 128 == 0 && SLOT_BYTES % 128 == 0, "attention buffers");
-
-// A page number outside the cache never becomes an address: the access goes to page 0 and the state word records it.
-__device__ __forceinline__ int checked_page(int pg, int n_pages, State* st, int where) {
-    if ((unsigned)pg < (unsigned)n_pages) return pg;
-    if (st) { atomicCAS(&st->status, 0, ST_INTERNAL); st->timeout_where = where; }
-    return 0;
-}
 
 // Copy warp: the old K / V tiles of this CTA's items.  row0: first row of this layer's cache in the tensor maps.
 template <int HD>

@@ -222,3 +222,35 @@ def test_expired_device_wait_returns_timeout_and_leaves_the_context_usable(env):
     gb2 = b.KangarooModel(SMALL_BF, arena=gb.arena)
     toks, _ = gb2.generate(pb, 16, 0.6, 6)
     assert toks == ref
+
+
+# ---- page numbers outside the cache -----------------------------------------------------------------------------
+
+@pytest.mark.parametrize("case", ["f32", "bf16_plain", "bf16_hd32", "bf16_ring", "prompt_pass"])
+@pytest.mark.parametrize("bad", [1 << 20, -3])
+def test_page_outside_the_cache_is_an_error_not_an_address(env, case, bad):
+    """A page table entry that is overwritten on the host with a number outside the cache: every kernel keeps its accesses inside, and
+    the call reports KG_E_INTERNAL.  bf16_plain: an F that is no multiple of 16, which only the plain linear operators take."""
+    from test_gpu_parity import MICRO_BF, SMALL_BF
+    torch, b = env
+    shape, n = {"f32": (ki.get_config("tiny"), 12), "bf16_plain": (SMALL_BF.with_(d_ffn=1384), 12), "bf16_hd32": (MICRO_BF, 9),
+                "bf16_ring": (SMALL_BF, 12), "prompt_pass": (SMALL_BF.with_(d_ffn=1408), 40)}[case]
+    prompt = ki.make_prompt(shape, n).tolist()
+    g = b.KangarooModel(shape)
+    ref, _ = g.generate(prompt, 8, 0.6, 4)
+    # the table: the identity, on a 256-byte boundary near the arena's start
+    pages = (shape.max_seq + shape.page_size - 1) // shape.page_size
+    base = -g.arena.data_ptr() % 256
+    head = g.arena[base:base + (1 << 16)].view(torch.int32).reshape(-1, 64)
+    want = torch.arange(min(pages, 64), dtype=torch.int32, device="cuda")
+    at = [i for i in range(head.shape[0]) if torch.equal(head[i, :len(want)], want)]
+    assert len(at) == 1
+    table = head[at[0]]
+    table[0] = bad
+    torch.cuda.synchronize()
+    with pytest.raises(b.KgError) as e:
+        g.generate(prompt, 8, 0.6, 4)
+    assert e.value.status == b.KG_E_INTERNAL
+    torch.cuda.synchronize()                                # the context is intact
+    g2 = b.KangarooModel(shape, arena=g.arena)
+    assert g2.generate(prompt, 8, 0.6, 4)[0] == ref
