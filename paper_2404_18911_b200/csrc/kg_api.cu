@@ -71,11 +71,6 @@ __global__ void fill_cache_kernel(WT* cache, const int* page_table, uint64_t bas
         cache[dst] = float_to_wt<WT>(gen_value(base, i, scale));
     }
 }
-__global__ void fill_tokens_kernel(int* out, uint64_t base, int count, int vocab) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-        out[i] = (int)(mix64(base + (uint64_t)i) % (uint64_t)vocab);
-}
-
 // fp32 rows -> packed rows (scaled by gain) + per-slice sums of squares, sliced over the columns exactly as the
 // CTAs of the decode kernel slice an operator's output (slice c = columns [K c / n, K (c+1) / n)).  One warp per row: a slice
 // is a few dozen columns, so that a CTA per row and slice would spend its time in barriers.
@@ -134,8 +129,8 @@ bool valid_config(const kg_config* c) {
     if (c->page_size < 1 || (c->page_size & (c->page_size - 1)) || c->max_seq < 2) return false;       // pages hold a power of two of tokens
     if (c->n_heads > 256) return false;
     if (c->vocab > (1 << 20) || c->d_ffn > (1 << 20)) return false;      // rows x CTAs must fit 32 bits
-    // one launch may run max_seq tokens, each at most 5 (L + 1) + 8 grid barriers of at most 1024 CTAs: the arrival
-    // counter (31 bits beside the abort flag) must hold them all
+    // one launch may run max_seq tokens, each at most L + 5 grid barriers of at most 1024 CTAs: the arrival counter (31 bits
+    // beside the abort flag) must hold them all (the bound counts five barriers a layer)
     if ((long long)c->max_seq * (5LL * (c->n_layers + 1) + 8) * 1024LL >= (1LL << 31)) return false;
     // the plain path stages all rows of an operand in shared memory
     const int kmax = c->d_ffn > c->d_model ? c->d_ffn : c->d_model;
@@ -243,7 +238,7 @@ __global__ void check_tokens_kernel(const int* toks, int n, int vocab, State* st
 }  // namespace
 
 // Tensor maps of the prompt pass, encoded once per model: the weights in boxes of 128 rows (64 for the gate / up pair),
-// the planes [R][K] in boxes of 32 * (i + 1) rows, one set for K = d (x) and one for K = F (f).
+// the planes [R][K] in boxes of 16 * (i + 1) rows (a CTA's half of a tile), one set for K = d (x) and one for K = F (f).
 struct PfMaps {
     CUtensorMap x[2][GM_NT_MAX / GM_NT_STEP], f[2][GM_NT_MAX / GM_NT_STEP];   // [hi, lo][activation rows per tile / GM_NT_STEP - 1]
     struct Layer { CUtensorMap qkv, o, gate, up, down; };
@@ -1275,8 +1270,8 @@ __global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* 
 }
 
 // A prompt of one chunk (at most KG_M_MAX rows) takes the decode kernels, which stream every weight once and need one launch;
-// from two chunks on the GEMMs are faster: 7B, 17 tokens 5.28 against 8.70 ms, a four-layer model with d = 512 0.31 against
-// 0.43 ms.  At 16 tokens it is 5.28 against 5.69 ms there and 0.31 against 0.26 ms here.
+// from two chunks on the GEMMs are faster: 7B, 17 tokens 4.50 against 7.71 ms, 31 tokens 4.49 against 10.18; a four-layer model with
+// d = 512, 17 tokens 0.232 against 0.369 ms.  One chunk of 16 takes 5.13 and 0.231 ms, of 8 tokens 3.35 and 0.218.
 bool prefill_tc_ok(const kg_model* m, int n) { return m->prefill_mode == 0 && m->pf.ready && n > KG_M_MAX; }
 
 // Tile shape and work items of a GEMM of `rows` activation rows and `wtiles` tiles of weight rows on `pairs` CTA pairs.

@@ -47,7 +47,7 @@ enum { PF_STORE = 0, PF_QKV = 1, PF_SWIGLU = 2 };                      // what t
 struct GemmArgs {
     int rows;                           // valid activation rows (rows of the planes beyond them hold anything)
     int N, K;                           // output features (multiple of 128; PF_SWIGLU: of each matrix) and contraction (of 64)
-    int nt, nrt;                        // activation rows per tile (64, 128, 192 or 256) and row tiles
+    int nt, nrt;                        // activation rows per tile (a multiple of 32, at most 256) and row tiles
     int full, S, items;                 // work items: `full` whole tiles, then every remaining tile cut into S ranges of k
     const float* rowscale;              // PF_QKV, PF_SWIGLU: one factor per row (1/rms of the row the planes were made from)
     float* C; const float* resid; int ldc;      // PF_STORE: C = (resid) + product; C may be resid itself

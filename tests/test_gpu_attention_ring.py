@@ -42,8 +42,8 @@ def test_attention_ring(env, H, hd, M, pos0, ps):
     cs, sn = torch.cos(new.double()[:, None] * inv)[:, None], torch.sin(new.double()[:, None] * inv)[:, None]
     rot = lambda x: torch.cat([x[..., :hd // 2] * cs - x[..., hd // 2:] * sn, x[..., hd // 2:] * cs + x[..., :hd // 2] * sn], -1)
     q, k, v = (qkv.double().reshape(M, 3, H, hd)[:, i] for i in range(3))
-    # the rows written: bf16 of the rotated k and of v (one ulp where the rounding of a float32 rotation falls the other way)
-    assert (K[pos0:] - rot(k)).abs().max() < 2 ** -8 * 8 and torch.equal(V[pos0:], v.to(torch.bfloat16).double())
+    # the rows written: bf16 of the rotated k (half a step of the element; the float32 rotation is good to 1e-5) and of v
+    assert ((K[pos0:] - rot(k)).abs() <= 1.01 * 2.0 ** -8 * rot(k).abs() + 1e-5).all() and torch.equal(V[pos0:], v.to(torch.bfloat16).double())
     S = torch.einsum("mhd,thd->hmt", rot(q), K) / hd ** 0.5
     S = S.masked_fill(torch.arange(T, device="cuda")[None, None] > new[None, :, None], float("-inf"))
     ref = torch.einsum("hmt,thd->mhd", torch.softmax(S, -1), V).reshape(M, d)

@@ -15,7 +15,7 @@ relative) differences of cache entries.  Measured maxima: 7B 6.5e-3 (logits) / 6
 confidences (and the 33B logits) do not meet the 1e-3 / 2e-2 of the 7B target, and the test output says by how much.
 
 Every trace is replayed twice: after the 16-row chunked prompt pass of the decode kernels (the figures above) and
-after the tensor-core prompt pass, the default for prompts of 32 tokens and more.  The two passes have the same
+after the tensor-core prompt pass, the default for prompts of more than 16 tokens.  The two passes have the same
 arithmetic per operator (bf16 hi + lo planes, fp32 accumulation, 1/rms applied after the product) but different
 summation orders, so they flip different cache entries; after the tensor-core pass the measured maxima are 7B
 1.1e-2 / 1.1e-3, 13B 1.2e-2 / 2.0e-3, 33B 2.7e-2 / 3.0e-3 to 4.2e-3 (which entries flip changes with any reordering of
