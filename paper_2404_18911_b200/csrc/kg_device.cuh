@@ -535,7 +535,13 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // Each of the 8 warps owns a fixed slice of the phase's k range; its B fragments are loaded once
 // per phase from the packed activation rows in global memory (L2) and stay in registers for every
 // row group, so the steady state touches shared memory only for the weights.  After a stage pair the 8 partial sums of each (weight row,
-// activation row) are added in warp order into the per-row accumulators in shared memory.
+// activation row) are added in warp order into the per-row accumulators in shared memory.  Operators of few stage pairs per phase and more than one
+// phase (O, down: d / 148 rows a CTA) leave that for the end: a warp's sums of a pair grow in place in shared memory, from phase to phase,
+// and no warp waits for another before the last phase is through.  The barrier and the cross-warp sum take 0.3 to 0.4 of a pair's 1400 to
+// 1800 clocks, and with two pairs between two fetches of fragments nothing hid them (7B, KV 512, 12 layers, verify pass of 1 row
+// 0.905 -> 0.897, of 4 rows 0.988 -> 0.960, of 7 rows 1.118 -> 1.077, of 11 rows 1.400 -> 1.364, of 16 rows 1.719 -> 1.634 ms).  With one
+// phase there is nothing to save (a model of four layers with d = 512: 1 % slower that way).  What does not fit the work area: QKV,
+// gate / up, the head.
 template <int V> struct LinGeom {
     static constexpr int NS = V == 16 ? 8 : 16;           // k16-steps per warp and stage
     static constexpr int PLEN = NS * 16 * NWARPS;         // k-elements per phase: 2048 or 1024
@@ -546,7 +552,10 @@ template <int V> struct LinGeom {
     // partial sums are double-buffered where the work area has room (V = 16: one buffer and one more barrier per pair);
     // partial sums and row accumulators together take the same space in every variant
     static constexpr int ACC_OFF = V == 16 ? NWARPS * RED_W : 2 * NWARPS * RED_W;
+    static constexpr int FEWP = V <= 8 ? 4 : (V == 12 ? 3 : 2);                // stage pairs per phase whose sums can be kept warp by warp
+    static constexpr int COLS = V == 4 ? 4 : (V == 8 ? 8 : MP);                // activation rows of a stage pair's sums
 };
+constexpr int FEW_ACC_OFF = 4608;                          // row accumulators behind the sums of few pairs
 constexpr int MP_MAX = 16;
 
 // First of the units (of N) that belong to CTA `cta`: even, so that a packed word has one writer.
@@ -642,6 +651,8 @@ constexpr int LW_HS = LW_PREG + 2 * PRE_NU;               // [M_MAX][3] LM head:
                                                           // in registers, which the fragments of the wide variants fill)
 constexpr int LW_END = LW_HS + M_MAX * 3;
 static_assert(LW_END * 4 <= WORK_BYTES, "linear work area too large");
+template <int V> constexpr bool FEW_FITS = LinGeom<V>::FEWP * NWARPS * LinGeom<V>::RED_W <= FEW_ACC_OFF && FEW_ACC_OFF + LinGeom<V>::FEWP * 16 * LinGeom<V>::MP <= LW_RS;
+static_assert(FEW_FITS<4> && FEW_FITS<8> && FEW_FITS<12> && FEW_FITS<16>, "sums of few pairs");
 static_assert(LinGeom<12>::ACC_OFF + SC_ROWS * LinGeom<12>::MP <= LW_RS && LinGeom<16>::ACC_OFF + SC_ROWS * 16 <= LW_RS && LinGeom<8>::ACC_OFF + SC_ROWS * 16 <= LW_RS,
               "partial sums and accumulators overlap what follows");
 
@@ -719,7 +730,6 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
 
     float* wk = reinterpret_cast<float*>(c.smem + WORK_OFF);
     float* red = wk + LW_RED;
-    float* acc_s = wk + G::ACC_OFF;
     float* rs = wk + LW_RS;
     const char* ring = c.smem + RING_OFF;
     Ctrl* ctl = c.ctl;
@@ -752,6 +762,8 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
         const int nu = sc1 - sc0;
         const int ngrp = (nu + ST_ROWS - 1) / ST_ROWS;
         const int nst = dual ? 2 * ngrp : ngrp;
+        const bool few = pl.nph > 1 && (nst + 1) >> 1 <= G::FEWP;
+        float* acc_s = wk + (few ? FEW_ACC_OFF : G::ACC_OFF);
         for (int ph = 0; ph < pl.nph; ++ph) {
             const int p0 = ph * pl.plen, len = min(pl.plen, K - p0);
             const int nsteps = len / 16;
@@ -852,31 +864,50 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                 slot = slot_b; phase = phase_b;
                 if (++slot == RING) { slot = 0; phase ^= 1u; }
                 // ---- add the k-slices in warp order into the row accumulators
-                if (V == 16) cta_sync();                     // single partial-sum buffer: the previous pair's sums have been read
-                float* r = red + (size_t)(V == 16 ? 0 : buf) * NWARPS * G::RED_W + (size_t)warp * G::RED_W;
+                if (V == 16 && !few) cta_sync();             // single partial-sum buffer: the previous pair's sums have been read
+                float* r = red + (size_t)((few ? si >> 1 : (V == 16 ? 0 : buf)) * NWARPS + warp) * G::RED_W;
+                // few pairs: onto the sums of the phases before (each word has one thread)
+                const bool add = few && ph != 0;
+                auto put = [&](float* q, float x, float y) {
+                    float2 o = make_float2(0.f, 0.f);
+                    if (add) o = *reinterpret_cast<const float2*>(q);
+                    *reinterpret_cast<float2*>(q) = make_float2(o.x + x, o.y + y);
+                };
                 if (V == 12) {
                     // acc[0], acc[1]: hi of rows 0-7 (even, odd steps), acc[4]: lo; acc[2], acc[3]: rows 8-11, hi in columns 0-3 and lo
                     // in columns 4-7, which sit two lanes further
-                    *reinterpret_cast<float2*>(r + g * MP + 2 * t) = make_float2(acc[0][0] + acc[1][0] + acc[4][0], acc[0][1] + acc[1][1] + acc[4][1]);
-                    *reinterpret_cast<float2*>(r + (g + 8) * MP + 2 * t) = make_float2(acc[0][2] + acc[1][2] + acc[4][2], acc[0][3] + acc[1][3] + acc[4][3]);
+                    put(r + g * MP + 2 * t, acc[0][0] + acc[1][0] + acc[4][0], acc[0][1] + acc[1][1] + acc[4][1]);
+                    put(r + (g + 8) * MP + 2 * t, acc[0][2] + acc[1][2] + acc[4][2], acc[0][3] + acc[1][3] + acc[4][3]);
                     float mx[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) { mx[i] = acc[2][i] + acc[3][i]; mx[i] += __shfl_xor_sync(0xffffffffu, mx[i], 2); }
                     if (t < 2) {
-                        *reinterpret_cast<float2*>(r + g * MP + 8 + 2 * t) = make_float2(mx[0], mx[1]);
-                        *reinterpret_cast<float2*>(r + (g + 8) * MP + 8 + 2 * t) = make_float2(mx[2], mx[3]);
+                        put(r + g * MP + 8 + 2 * t, mx[0], mx[1]);
+                        put(r + (g + 8) * MP + 8 + 2 * t, mx[2], mx[3]);
                     }
                 } else if (V == 16) {
                     // acc[0] / acc[1]: hi / lo of columns 0-7; acc[2] / acc[3]: hi / lo of columns 8-15
-                    *reinterpret_cast<float2*>(r + g * 8 + 2 * t) = make_float2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
-                    *reinterpret_cast<float2*>(r + (g + 8) * 8 + 2 * t) = make_float2(acc[0][2] + acc[1][2], acc[0][3] + acc[1][3]);
-                    *reinterpret_cast<float2*>(r + 128 + g * 8 + 2 * t) = make_float2(acc[2][0] + acc[3][0], acc[2][1] + acc[3][1]);
-                    *reinterpret_cast<float2*>(r + 128 + (g + 8) * 8 + 2 * t) = make_float2(acc[2][2] + acc[3][2], acc[2][3] + acc[3][3]);
+                    put(r + g * 8 + 2 * t, acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+                    put(r + (g + 8) * 8 + 2 * t, acc[0][2] + acc[1][2], acc[0][3] + acc[1][3]);
+                    put(r + 128 + g * 8 + 2 * t, acc[2][0] + acc[3][0], acc[2][1] + acc[3][1]);
+                    put(r + 128 + (g + 8) * 8 + 2 * t, acc[2][2] + acc[3][2], acc[2][3] + acc[3][3]);
                 } else {
-                    *reinterpret_cast<float2*>(r + g * 8 + 2 * t) =
-                        make_float2((acc[0][0] + acc[1][0]) + (acc[2][0] + acc[3][0]), (acc[0][1] + acc[1][1]) + (acc[2][1] + acc[3][1]));
-                    *reinterpret_cast<float2*>(r + (g + 8) * 8 + 2 * t) =
-                        make_float2((acc[0][2] + acc[1][2]) + (acc[2][2] + acc[3][2]), (acc[0][3] + acc[1][3]) + (acc[2][3] + acc[3][3]));
+                    put(r + g * 8 + 2 * t, (acc[0][0] + acc[1][0]) + (acc[2][0] + acc[3][0]), (acc[0][1] + acc[1][1]) + (acc[2][1] + acc[3][1]));
+                    put(r + (g + 8) * 8 + 2 * t, (acc[0][2] + acc[1][2]) + (acc[2][2] + acc[3][2]), (acc[0][3] + acc[1][3]) + (acc[2][3] + acc[3][3]));
+                }
+                if (few) {
+                    if (ph != pl.nph - 1 || si + 2 < nst) continue;
+                    cta_sync();
+                    constexpr int EL = 16 * G::COLS;         // sums of a pair
+                    for (int e = tid; e < ((nst + 1) >> 1) * EL; e += NTHREADS) {
+                        const int pr = e / EL, r16 = e % EL / G::COLS, m = e % G::COLS;
+                        const float* rb = red + (size_t)pr * NWARPS * G::RED_W + (V == 16 ? (m >> 3) * 128 + r16 * 8 + (m & 7) : r16 * (V == 12 ? 12 : 8) + m);
+                        float v = 0.f;
+#pragma unroll
+                        for (int w = 0; w < NWARPS; ++w) v += V == 4 ? rb[w * G::RED_W] + rb[w * G::RED_W + 4] : rb[w * G::RED_W];
+                        acc_s[(size_t)(pr * 16 + r16) * MP + m] = v;
+                    }
+                    continue;
                 }
                 cta_sync();
                 {

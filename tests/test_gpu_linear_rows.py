@@ -42,3 +42,11 @@ def test_rows(env, N, K, M):
     assert (z.double() - zr).abs().max() < 8 * bound
     assert torch.equal(tok.long(), z.argmax(-1))
     assert (p.double() - torch.softmax(zr, -1).max(-1).values).abs().max() < 1e-3
+
+
+# rows per CTA (of 148) at and behind the limits up to which a CTA keeps its warps' sums apart: 32 (M > 12), 48 (M > 8), 64; the pair of
+# matrices has twice as many
+@pytest.mark.parametrize("M", [1, 4, 8, 9, 12, 16])
+@pytest.mark.parametrize("N", [2368, 4736, 4738, 7104, 7300, 9472, 9474])
+def test_rows_per_cta(env, N, M):
+    test_rows(env, N, 2064, M)
