@@ -1025,6 +1025,7 @@ static int op_linear_common(int32_t dtype, LinArgs& a, unsigned char* xpk, int x
         if (a.K > xpk_k_max || nctas > 1024) return KG_E_LIMIT;
         pack_rows_kernel<<<nctas, 256, 0, s>>>(a.x, a.ldx, a.M, a.K, a.gain, xpk, a.K * 4, a.gain ? ssq : nullptr, nctas);
         a.xpk = xpk; a.ldpk = a.K * 4; a.ssq_in = a.gain ? ssq : nullptr; a.ld_ssq = nctas;
+        lin_phases(a);
     }
     int r;
     if (dtype == KG_F32) r = launch_plain<float>(a, nctas, s);
@@ -1384,6 +1385,7 @@ int prefill_tc(kg_model* m, int n) {
         a.xpk = D.hA_pk; a.ldpk = d * 4; a.ssq_in = D.ssq_hA; a.ld_ssq = m->nctas;
         a.epi = EPI_HEAD; a.scale = c.logit_scale; a.head_part = D.head_part;
         a.logits_dbg = c.debug_logits ? D.dbg_verify : nullptr; a.ld_dbg = c.vocab;
+        lin_phases(a);
         op_linear_kernel<WT, 4><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
         pf_finish_kernel<<<1, 32, 0, s>>>(D.head_part, m->nctas, D.st, D.out_tokens, n, err);
         CK(cudaGetLastError());

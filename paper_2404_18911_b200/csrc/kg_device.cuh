@@ -164,6 +164,7 @@ struct LinArgs {
     const void* W; const void* W2;   // [N, K]; W2 != null: SwiGLU pair (gate, up)
     int N, K;
     int M;                           // activation rows
+    int spw, nph;                    // streamed path: k16-steps per warp and phase, phases (lin_phases)
     const float* x; int ldx;         // plain path: fp32 rows (written earlier in this kernel)
     const float* gain; float eps;    // RMSNorm gain of the input (null: no norm)
     const unsigned char* xpk; int ldpk;   // streamed path: packed rows, already multiplied by the gain; bytes per row
@@ -518,7 +519,7 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // Work split.  The CTA owns a contiguous range of "units": output rows, or for the SwiGLU pair
 // gate/up feature pairs.  A stage of the ring holds 8 weight rows (for the pair: the 8 gate rows of
 // a feature group, then in the next stage the 8 up rows of the same features) times one k phase
-// (2048 k-elements when M <= 12, else 1024), i.e. one bulk copy of up to 4 KB per row: the copy
+// (at most 2048 k-elements when M <= 12, else 1024; lin_phases), i.e. one bulk copy of up to 4 KB per row: the copy
 // engine spends a fixed time per copy, and only copies of 2-4 KB and more keep HBM saturated.
 // The stages are visited superchunk (<= 256 accumulator rows) -> phase -> row group, in the same
 // order by the producer warp (which issues the copies) and the consumers.
@@ -544,7 +545,7 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // gate / up, the head.
 template <int V> struct LinGeom {
     static constexpr int NS = V == 16 ? 8 : 16;           // k16-steps per warp and stage
-    static constexpr int PLEN = NS * 16 * NWARPS;         // k-elements per phase: 2048 or 1024
+    static constexpr int PLEN = NS * 16 * NWARPS;         // most k-elements per phase: 2048 or 1024
     static constexpr int FR = V == 4 ? 2 : (V == 8 ? 4 : (V == 12 ? 6 : 8));   // B fragment registers per step
     static constexpr int NACC = V == 16 ? 2 : 1;          // column tiles
     static constexpr int RED_W = V == 16 ? 256 : (V == 12 ? 192 : 128);        // floats of one warp's partial sums of a stage pair
@@ -564,6 +565,17 @@ __device__ __forceinline__ int cta_unit(int N, int cta, int nctas) {
     return min(u, N);
 }
 
+// The phases of an operator: as many as the longest possible ones, and all (but the last) of the same length, a whole number of steps
+// for every warp.  With phases of the full length the last one may be short, and its copies with it: K = 6656 was 3 x 2048 + 512, now
+// 4 x 1664 (verify pass of one row, 33B widths, 8 layers 1.104 -> 1.023 ms, of 11 rows 1.493 -> 1.405; 13B, 12 layers, KV 2048
+// 1.370 -> 1.319; 7B, whose d is two full phases and whose F = 11008 leaves 88 steps of 120 instead of 48 of 128, 0.895 -> 0.894, 7 rows 1.072 -> 1.049).
+__host__ __device__ __forceinline__ void lin_phases(LinArgs& a) {
+    const unsigned steps = (unsigned)a.K >> 4, most = (unsigned)(a.M <= 12 ? LinGeom<12>::NS : LinGeom<16>::NS) * NWARPS;
+    const unsigned n = (steps + most - 1) / most;
+    a.spw = (int)(((steps + n - 1) / n + NWARPS - 1) / NWARPS);
+    a.nph = (int)((steps + a.spw * NWARPS - 1) / (a.spw * NWARPS));
+}
+
 struct LinPlan {
     int u0, u1;          // this CTA's units
     int sc_units;        // units per superchunk
@@ -575,8 +587,8 @@ __device__ __forceinline__ LinPlan make_plan(const LinArgs& a, int cta, int ncta
     p.u0 = cta_unit(a.N, cta, nctas);
     p.u1 = cta_unit(a.N, cta + 1, nctas);
     p.sc_units = a.W2 ? SC_ROWS / 2 : SC_ROWS;
-    p.plen = a.M <= 12 ? LinGeom<12>::PLEN : LinGeom<16>::PLEN;
-    p.nph = (a.K + p.plen - 1) / p.plen;
+    p.plen = a.spw * (16 * NWARPS);
+    p.nph = a.nph;
     return p;
 }
 
@@ -724,7 +736,7 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     constexpr int NS = G::NS, FR = G::FR, NACC = G::NACC, MP = G::MP;
     const int tid = tid_here(), lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const int M = a.M, K = a.K;
+    const int M = a.M, K = a.K, spw = a.spw;
     const bool dual = a.W2 != nullptr;
     const LinPlan pl = make_plan(a, c.cta, c.nctas);
 
@@ -772,20 +784,20 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
             // columns of the product are never read, and the columns of an MMA do not mix.  Steps past the end of the phase re-read
             // the last one and are skipped.
             unsigned fr[NS][FR];
-            const int last = nsteps - 1 - warp * NS;             // last valid step of this warp (< 0: none)
+            const int last = min(nsteps - 1 - warp * spw, spw - 1);      // last valid step of this warp (< 0: none)
             {
                 // this lane's rows of the packed input: V = 4: row g & 3 (hi for g < 4, lo for g >= 4); else row g and, mofs bytes
                 // away, V = 12: row 8 + (g & 3) (hi for g < 4, lo for g >= 4), V = 16: row 8 + g (M > 8 here, so that g < M)
                 const int xrow = V == 4 ? (g & 3) : g, mrow = 8 + (V == 12 ? (g & 3) : g);
                 const int mofs = ((mrow < M ? mrow : 0) - xrow) * a.ldpk + (V == 12 ? (g >> 2) * 8 : 0);
-                const unsigned char* pbase = a.xpk + (size_t)(xrow < M ? xrow : 0) * a.ldpk + (size_t)(p0 / 16 + warp * NS) * 64 + t * 16 + (V == 4 ? (g >> 2) * 8 : 0);
+                const unsigned char* pbase = a.xpk + (size_t)(xrow < M ? xrow : 0) * a.ldpk + (size_t)(p0 / 16 + warp * spw) * 64 + t * 16 + (V == 4 ? (g >> 2) * 8 : 0);
                 int lastv = last;
                 XchSpin sp; sp.spins = 0;
                 while (true) {
                     asm volatile("" : "+l"(pbase), "+r"(lastv));   // keeps the steps' addresses from being formed, and spilled, ahead of the loop
 #pragma unroll
                     for (int s = 0; s < NS; ++s) {
-                        const unsigned char* px = pbase + (size_t)max(min(s, lastv), -warp * NS) * 64;
+                        const unsigned char* px = pbase + (size_t)max(min(s, lastv), -warp * spw) * 64;
                         if (V == 4) {
                             const uint2 v = xch_ld2(px);
                             fr[s][0] = v.x; fr[s][1] = v.y;
@@ -815,7 +827,7 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
             }
             if (pre_pending) { pre_pending = false; epilogue_prefetch(); }
             // ---- the row groups of this phase, two stages (16 weight rows) at a time
-            const uint32_t a_lane = (uint32_t)((lane & 7) * ST_ROW_BYTES + (warp * NS * 16 + (lane >> 4) * 8) * 2);
+            const uint32_t a_lane = (uint32_t)((lane & 7) * ST_ROW_BYTES + (warp * spw * 16 + (lane >> 4) * 8) * 2);
             for (int si = 0; si < nst; si += 2) {
                 const bool two = si + 1 < nst;
                 const int slot_a = slot;

@@ -78,6 +78,7 @@ struct Sequencer {
         if (!o) return nullptr;
         LinArgs& a = o->lin;
         a.W = W; a.W2 = W2; a.N = N; a.K = K; a.M = M; a.eps = D.dm.eps;
+        if (streamed) lin_phases(a);
         a.gain = nullptr; a.ssq_in = nullptr; a.poll = 0; a.resid = nullptr; a.out = nullptr;
         a.pk[0] = PkOut{nullptr, nullptr}; a.pk[1] = PkOut{nullptr, nullptr}; a.ssq_out = nullptr;
         return &a;

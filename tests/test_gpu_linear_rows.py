@@ -50,3 +50,10 @@ def test_rows(env, N, K, M):
 @pytest.mark.parametrize("N", [2368, 4736, 4738, 7104, 7300, 9472, 9474])
 def test_rows_per_cta(env, N, M):
     test_rows(env, N, 2064, M)
+
+
+# row lengths around whole phases (2048 or 1024 elements) and those of the 33B and 7B shapes, whose phases are shorter
+@pytest.mark.parametrize("M", [1, 7, 12, 16])
+@pytest.mark.parametrize("K", [16, 1024, 1040, 2048, 2176, 4112, 6656, 11008])
+def test_phases(env, K, M):
+    test_rows(env, 300, K, M)
