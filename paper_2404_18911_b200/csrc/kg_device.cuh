@@ -5,7 +5,7 @@
 // (cta, nctas); its readers poll for the rows it writes, or a grid-wide barrier comes between.  The same operators are
 // also wrapped one-by-one in small kernels for unit tests.
 //
-// A CTA has 8 consumer warps and one producer warp.  The decode step is bound by HBM bandwidth:
+// A CTA has 8 consumer warps and one producer warp (the decode kernel a sequencer and a prefetch warp besides).  The decode step is bound by HBM bandwidth:
 // every weight byte is read exactly once per pass.  The producer warp streams this CTA's share of
 // every weight matrix of a pass through a ring of shared-memory slots with bulk asynchronous
 // copies (cp.async.bulk + mbarrier transaction counts); because weights do not depend on
@@ -26,8 +26,8 @@ constexpr int M_MAX = 16;          // rows per pass
 constexpr int NTHREADS = 256;      // consumer threads per CTA
 constexpr int NWARPS = NTHREADS / 32;
 constexpr int BLOCK_THREADS = NTHREADS + 32;   // + the producer warp (warp index NWARPS)
-// The decode kernel is launched with a whole warpgroup behind the consumers (warp NWARPS copies, the next one is the sequencer, two
-// leave at once): registers are handed out per warpgroup, and that warpgroup gives most of its share to the two consumer
+// The decode kernel is launched with a whole warpgroup behind the consumers (warp NWARPS copies, the next one is the sequencer, then
+// the prefetch warp; one leaves at once): registers are handed out per warpgroup, and that warpgroup gives most of its share to the two consumer
 // warpgroups at kernel start (setmaxnreg).  The pool is what the launch allocated: 384 threads x 168 registers = 64512; a
 // request beyond it would block forever, so the budgets below are checked against it.
 constexpr int DECODE_THREADS = NTHREADS + 128;
@@ -211,13 +211,14 @@ struct Ctrl {
     int abort;                         // a bounded wait of this CTA gave up
     int sync_ok;
     int att_last;
+    unsigned issued;                   // stages that the copy warp has issued
     int head_tok[M_MAX];
     float head_p[M_MAX];
     unsigned long long qfull[QUEUE];   // sequencer -> copy warp, consumers: operator written
     unsigned long long qempty[QUEUE];  // copy warp, consumer warps -> sequencer: operator done
     Op queue[QUEUE];
     // the per-role context (struct Ctx): one copy for the consumers, one for the copy warp, one for the sequencer
-    alignas(16) unsigned char ctx[3][128];
+    alignas(16) unsigned char ctx[4][128];
 };
 static_assert(sizeof(Ctrl) <= CTRL_BYTES - 16, "control block too large");
 
@@ -350,20 +351,20 @@ __device__ __forceinline__ Ctx& ctx_init(char* smem, State* st, unsigned* bar, b
                                          unsigned long long wait_clk = WAIT_TIMEOUT_CLK, int skip_arrival = 0) {
     static_assert(sizeof(Ctx) <= 128, "context slot too small");
     Ctrl* ctl = reinterpret_cast<Ctrl*>(smem);
-    const int role = threadIdx.x < NTHREADS ? 0 : (threadIdx.x < NTHREADS + 32 ? 1 : 2);       // consumers, copy warp, sequencer
+    const int role = threadIdx.x < NTHREADS ? 0 : (threadIdx.x < NTHREADS + 32 ? 1 : (threadIdx.x < NTHREADS + 64 ? 2 : 3));   // consumers, copy warp, sequencer, prefetch warp
     Ctx& c = *reinterpret_cast<Ctx*>(ctl->ctx[role]);
-    if (threadIdx.x == 0 || threadIdx.x == NTHREADS || threadIdx.x == NTHREADS + 32) {
+    if (threadIdx.x == 0 || threadIdx.x == NTHREADS || threadIdx.x == NTHREADS + 32 || threadIdx.x == NTHREADS + 64) {
         c.cta = blockIdx.x; c.nctas = gridDim.x; c.bar_target = 0; c.st = st; c.bar = bar; c.smem = smem;
         c.wait_clk = wait_clk; c.skip_arrival = skip_arrival;
         c.ctl = ctl; c.grid = grid;
-        c.producer = role == 1; c.backoff = role == 0 ? 0 : (role == 1 ? 200 : 40);
+        c.producer = role == 1; c.backoff = role == 0 ? 0 : (role == 2 ? 40 : 200);
         c.slot = 0; c.phase = 0; c.issued = 0; c.mail_phase = 0;
     }
     if (threadIdx.x == 0) {
         for (int i = 0; i < RING; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], NWARPS); }
-        for (int i = 0; i < QUEUE; ++i) { mbar_init(&ctl->qfull[i], 1); mbar_init(&ctl->qempty[i], NWARPS + 1); }
+        for (int i = 0; i < QUEUE; ++i) { mbar_init(&ctl->qfull[i], 1); mbar_init(&ctl->qempty[i], NWARPS + 2); }
         mbar_init(&ctl->mail, 1);
-        ctl->abort = 0; ctl->sync_ok = 1; ctl->att_last = 0;
+        ctl->abort = 0; ctl->sync_ok = 1; ctl->att_last = 0; ctl->issued = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -565,14 +566,16 @@ __device__ __forceinline__ int cta_unit(int N, int cta, int nctas) {
     return min(u, N);
 }
 
-// The phases of an operator: as many as the longest possible ones, and all (but the last) of the same length, a whole number of steps
-// for every warp.  With phases of the full length the last one may be short, and its copies with it: K = 6656 was 3 x 2048 + 512, now
-// 4 x 1664 (verify pass of one row, 33B widths, 8 layers 1.104 -> 1.023 ms, of 11 rows 1.493 -> 1.405; 13B, 12 layers, KV 2048
-// 1.370 -> 1.319; 7B, whose d is two full phases and whose F = 11008 leaves 88 steps of 120 instead of 48 of 128, 0.895 -> 0.894, 7 rows 1.072 -> 1.049).
+// The phases of an operator: as many as the longest possible ones and, up to 8 rows, all but the last of the same length, a whole number
+// of steps for every warp.  With phases of the full length the last one may be short, and its copies with it: K = 6656 was 3 x 2048 +
+// 512, now 4 x 1664 (verify pass of one row, 33B widths, 8 layers 1.104 -> 1.023 ms; 13B, 12 layers, KV 2048 1.370 -> 1.319; 7B, whose d is
+// two full phases, 7 rows 1.072 -> 1.049).  Beyond 8 rows it is left as it was (9 to 12 rows would gain 2 to 6 %): the rows of short
+// prompts go there, and with their sums in that order the confidences of the stored 33B trace are up to 4.1e-3 to 5.4e-3 off, more than its
+// test allows, in whatever order the warps' sums are added; as it is they are 3.4e-3 off (before these changes 3.7e-3).
 __host__ __device__ __forceinline__ void lin_phases(LinArgs& a) {
     const unsigned steps = (unsigned)a.K >> 4, most = (unsigned)(a.M <= 12 ? LinGeom<12>::NS : LinGeom<16>::NS) * NWARPS;
     const unsigned n = (steps + most - 1) / most;
-    a.spw = (int)(((steps + n - 1) / n + NWARPS - 1) / NWARPS);
+    a.spw = a.M <= 8 ? (int)(((steps + n - 1) / n + NWARPS - 1) / NWARPS) : (int)(most / NWARPS);
     a.nph = (int)((steps + a.spw * NWARPS - 1) / (a.spw * NWARPS));
 }
 
@@ -621,11 +624,67 @@ __device__ __noinline__ bool lin_produce(const LinArgs& a, Ctx& c) {
                 __syncwarp();
                 if (lane < nvalid) bulk_g2s(ring + (size_t)slot * SLOT_BYTES + lane * ST_ROW_BYTES, src, (unsigned)(len * 2), &ctl->full[slot], policy);
                 issued++;
+                if (lane == 0) *(volatile unsigned*)&ctl->issued = issued;
                 if (++slot == RING) { slot = 0; phase ^= 1u; }
             }
         }
     }
     c.slot = slot; c.phase = phase; c.issued = issued;
+    return true;
+}
+
+// ---- the prefetch warp of the decode kernel: weights on their way into L2 before the ring has room for them
+//
+// The ring holds 4.4 us of HBM's time, but the consumers stand still for longer at the hand-overs around the attention and at a
+// layer's end (about 9 and 6 us of a layer's 80 in the 7B shape at one row), and HBM with them.  A stage is therefore prefetched
+// into L2 once the copy warp is less than PF_AHEAD stages away from it; afterwards the ring is filled from L2, faster than HBM could.
+// Depth, 7B, 12 layers, KV 512, one row (ms): none 0.894, 8 stages 0.887, 10 0.874, 12 0.861, 14 0.850, 16 0.866, 24 1.041, 32 1.295
+// (at 32 KB a stage and 148 CTAs 16 stages are 78 MB: not all of the 126 MB of L2 can be used that way); 33B widths 1.023 -> 0.998 / 0.995 /
+// 0.996 / 1.009 (8 to 14), KV 4096 1.010 -> 0.995 / 0.989 / 0.978 / 0.983, 13B 1.319 -> 1.323 / 1.312 / 1.299 / 1.298.
+// Passes of more than PF_ROWS_MAX rows keep the consumers busier than HBM, and the additional traffic costs them: 11 rows 1.362 -> 1.398, 16
+// rows 1.635 -> 1.708 (7 rows 1.049 -> 1.008, 8 rows 1.080 -> 1.028).
+constexpr int PF_AHEAD = 12, PF_ROWS_MAX = 8;
+constexpr int PF_GAVE_UP = -0x40000000;
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+// One operator.  c.issued counts the stages of the operators before it, as the copy warp counts them; stages that the copy warp has issued
+// already are left out.  False: a wait gave up.
+__device__ __noinline__ bool lin_prefetch(const LinArgs& a, Ctx& c) {
+    const int lane = threadIdx.x & 31;
+    const LinPlan pl = make_plan(a, c.cta, c.nctas);
+    const bool dual = a.W2 != nullptr;
+    const __nv_bfloat16* W = reinterpret_cast<const __nv_bfloat16*>(a.W);
+    const __nv_bfloat16* W2 = reinterpret_cast<const __nv_bfloat16*>(a.W2);
+    unsigned n = c.issued;
+    __syncwarp();                                          // every lane has read the count before one writes it again
+    for (int sc0 = pl.u0; sc0 < pl.u1; sc0 += pl.sc_units) {
+        const int sc1 = min(pl.u1, sc0 + pl.sc_units);
+        const int ngrp = (sc1 - sc0 + ST_ROWS - 1) / ST_ROWS;
+        const int nst = dual ? 2 * ngrp : ngrp;
+        if (a.M > PF_ROWS_MAX) { n += (unsigned)(pl.nph * nst); continue; }
+        for (int ph = 0; ph < pl.nph; ++ph) {
+            const int p0 = ph * pl.plen, len = min(pl.plen, a.K - p0);
+            for (int si = 0; si < nst; ++si, ++n) {
+                int gap = 0;                               // stages between the copy warp and this one
+                if (lane == 0) {
+                    const long long t0 = clock64();
+                    while ((gap = (int)(n - *(volatile unsigned*)&c.ctl->issued)) >= PF_AHEAD) {
+                        __nanosleep(100);
+                        if (*(volatile int*)&c.ctl->abort || (unsigned long long)(clock64() - t0) > 2ull * c.wait_clk) { gap = PF_GAVE_UP; break; }
+                    }
+                }
+                gap = __shfl_sync(0xffffffffu, gap, 0);
+                if (gap == PF_GAVE_UP) return false;
+                if (gap < 1) continue;                     // on its way already
+                const int base = sc0 + (dual ? si >> 1 : si) * ST_ROWS;
+                const int nvalid = min(ST_ROWS, sc1 - base);
+                if (lane < nvalid) bulk_prefetch_l2(((dual && (si & 1)) ? W2 : W) + (size_t)(base + lane) * a.K + p0, (unsigned)(len * 2));
+            }
+        }
+    }
+    __syncwarp();
+    if (lane == 0) c.issued = n;
     return true;
 }
 
@@ -914,10 +973,15 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
                     for (int e = tid; e < ((nst + 1) >> 1) * EL; e += NTHREADS) {
                         const int pr = e / EL, r16 = e % EL / G::COLS, m = e % G::COLS;
                         const float* rb = red + (size_t)pr * NWARPS * G::RED_W + (V == 16 ? (m >> 3) * 128 + r16 * 8 + (m & 7) : r16 * (V == 12 ? 12 : 8) + m);
-                        float v = 0.f;
+                        float v[NWARPS];
 #pragma unroll
-                        for (int w = 0; w < NWARPS; ++w) v += V == 4 ? rb[w * G::RED_W] + rb[w * G::RED_W + 4] : rb[w * G::RED_W];
-                        acc_s[(size_t)(pr * 16 + r16) * MP + m] = v;
+                        for (int w = 0; w < NWARPS; ++w) v[w] = V == 4 ? rb[w * G::RED_W] + rb[w * G::RED_W + 4] : rb[w * G::RED_W];
+#pragma unroll
+                        for (int o = NWARPS / 2; o > 0; o >>= 1) {
+#pragma unroll
+                            for (int w = 0; w < o; ++w) v[w] += v[w + o];
+                        }
+                        acc_s[(size_t)(pr * 16 + r16) * MP + m] = v[0];
                     }
                     continue;
                 }
@@ -1722,11 +1786,22 @@ __device__ __noinline__ bool att_produce(const Dev& D, const AttPlan pl, int row
                             half * 64, row0 + ((page * H + hh) << psh) + (key & psm), bar);
             }
             issued++;
+            if (lane == 0) *(volatile unsigned*)&c.ctl->issued = issued;
             if (++slot == RING) { slot = 0; phase ^= 1u; }
         }
     }
     c.slot = slot; c.phase = phase; c.issued = issued;
     return ok;
+}
+
+// ring slots that att_produce fills
+template <int HD> __device__ __forceinline__ unsigned att_stages(const Dev& D, const AttPlan& pl, const Ctx& c) {
+    unsigned n = 0;
+    for (int item = c.cta; item < D.dm.H * pl.S; item += c.nctas) {
+        const int tb = item % pl.S * pl.chunk, nt = min(pl.ntile, tb + pl.chunk) - tb;
+        n += (unsigned)((nt + RaGeom<HD>::TPS - 1) / RaGeom<HD>::TPS);
+    }
+    return n;
 }
 
 // shared-memory address of the 16-byte chunk `ch` of row `row` of a tile's K or V at `base`

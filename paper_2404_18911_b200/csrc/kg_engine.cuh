@@ -3,12 +3,13 @@
 // prefix accept / rollback, or many rounds back to back - with exchanges or grid barriers between
 // dependent operators and no host involvement.
 //
-// Three roles in every CTA, joined by a queue of operators in shared memory:
+// The roles in every CTA, joined by a queue of operators in shared memory:
 //   the sequencer (one thread) walks through the method - layers, draft steps, accept decisions - and writes the arguments of one
 //     operator after the other into the queue.  It runs ahead of the others until the next decision that depends on a result (a
 //     drafted token, its confidence, the accepted prefix), which it receives through shared memory.  Every CTA's sequencer
 //     holds the same copy of the sequence state and comes to the same decisions.
-//   the copy warp streams the weights and the K / V tiles of the operators in the queue;
+//   the copy warp streams the weights and the K / V tiles of the operators in the queue, and a prefetch warp asks for weights further
+//     ahead than its ring reaches;
 //   the eight consumer warps do the arithmetic and take part in the grid barriers.
 // The consumers' loop holds every operator once, inlined.  Before, every thread walked through the method itself and called the
 // operators as functions from a dozen places: they were compiled for the 168 registers of the launch (the warpgroups' own budgets
@@ -415,6 +416,31 @@ __device__ __forceinline__ void copy_loop(const Dev& D, Ctx& c, bool streamed) {
     if (!ok) ring_drain(c);
 }
 
+// ---- the prefetch warp
+__device__ __forceinline__ void prefetch_loop(const Dev& D, Ctx& c, bool streamed) {
+    Ctrl* ctl = c.ctl;
+    const int lane = threadIdx.x & 31;
+    int q = 0; unsigned qph = 0;
+    bool ok = true, done = false;
+    while (!done) {
+        int w = 1;                       // (a wait here that gives up ends the launch as any other does)
+        if (lane == 0) w = mbar_wait(c, &ctl->qfull[q], qph, 35) ? 1 : 0;
+        if (!__shfl_sync(0xffffffffu, w, 0)) return;
+        const Op& op = ctl->queue[q];
+        const int kind = op.kind;
+        if (ok && streamed && kind == OPK_LIN) ok = lin_prefetch(op.lin, c);
+        else if (streamed && kind == OPK_ATT && D.dm.ring) {
+            const unsigned n = D.dm.hd == 128 ? att_stages<128>(D, op.att.plan, c) : att_stages<64>(D, op.att.plan, c);
+            __syncwarp();
+            if (lane == 0) c.issued += n;
+        }
+        done = kind == OPK_EXIT;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->qempty[q]);
+        if (++q == QUEUE) { q = 0; qph ^= 1u; }
+    }
+}
+
 // ---- the consumer warps ----------------------------------------------------------------------------------------------
 // true when the predicate holds in every consumer thread (a barrier among them)
 __device__ __forceinline__ bool cta_all(bool p) {
@@ -523,7 +549,7 @@ __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const 
         else if (w == 1 && (threadIdx.x & 31) == 0) {
             Sequencer<WT> seq(D, c, pg);
             seq.run();
-        }
+        } else if (w == 2) prefetch_loop(D, c, launch_streamed(D, pg));
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
         consume_loop<WT, HD, RING>(D, c, launch_streamed(D, pg));
