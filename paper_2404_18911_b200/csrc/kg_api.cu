@@ -1228,6 +1228,18 @@ int gemm_attributes() {
     return KG_OK;
 }
 
+template <int HD>
+int attention_tc_attributes() {
+    cudaFuncAttributes fa;
+    CK(cudaFuncGetAttributes(&fa, (const void*)pf_attention_tc_kernel<HD>));
+    if ((long long)fa.numRegs * FT_THREADS < 128LL * FT_CTRL_REGS + 32LL * FT_SOFT_WARPS * FT_SOFT_REGS) {
+        std::snprintf(g_cuda_err, sizeof(g_cuda_err), "attention kernel compiled with %d registers per thread: too few for its register budgets", fa.numRegs);
+        return KG_E_INTERNAL;
+    }
+    CK(cudaFuncSetAttribute((const void*)pf_attention_tc_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, FtSm<HD>::BYTES));
+    return KG_OK;
+}
+
 int prefill_tc_init(kg_model* m) {
     m->pf.ready = false;
     if (m->dev.dm.stream == 0 || !prefill_tc_shape(&m->cfg) || encode_tiled_fn() == nullptr) return KG_OK;
@@ -1253,6 +1265,7 @@ int prefill_tc_init(kg_model* m) {
     if ((r = gemm_attributes<PF_STORE>()) != KG_OK || (r = gemm_attributes<PF_QKV>()) != KG_OK || (r = gemm_attributes<PF_SWIGLU>()) != KG_OK) return r;
     CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<128>::BYTES));
     CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<64>::BYTES));
+    if ((r = attention_tc_attributes<128>()) != KG_OK || (r = attention_tc_attributes<64>()) != KG_OK) return r;
     CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
     CK(cudaMemsetAsync(A + m->lay.off_pf_cnt, 0, 4 * (size_t)m->nctas, m->stream));
     m->pf.ready = true;
@@ -1359,9 +1372,12 @@ int prefill_tc(kg_model* m, int n) {
             FaArgs fa;
             fa.qh = qh; fa.ql = ql; fa.kc = (const WT*)D.kcache + (size_t)i * lstride; fa.vc = (const WT*)D.vcache + (size_t)i * lstride;
             fa.oh = xh; fa.ol = xl; fa.page_table = D.page_table; fa.ps_shift = D.dm.ps_shift; fa.n_phys = D.dm.n_phys; fa.st = D.st;
-            fa.H = H; fa.pos0 = b0; fa.rows = rows;
+            fa.H = H; fa.pos0 = b0; fa.rows = rows; fa.row0 = i * D.dm.n_pages * H * c.page_size; fa.err = err;
             const int fgrid = (rows + FA_ROWS - 1) / FA_ROWS * H;
-            if (hd == 128) CK(launch_dependent(pf_attention_kernel<128>, dim3(fgrid), dim3(256), FaSm<128>::BYTES, s, fa));
+            if (D.dm.ring && b0 + rows > FT_MIN_KEYS) {
+                if (hd == 128) CK(launch_dependent(pf_attention_tc_kernel<128>, dim3(fgrid), dim3(FT_THREADS), FtSm<128>::BYTES, s, D.tmk, D.tmv, fa));
+                else CK(launch_dependent(pf_attention_tc_kernel<64>, dim3(fgrid), dim3(FT_THREADS), FtSm<64>::BYTES, s, D.tmk, D.tmv, fa));
+            } else if (hd == 128) CK(launch_dependent(pf_attention_kernel<128>, dim3(fgrid), dim3(256), FaSm<128>::BYTES, s, fa));
             else CK(launch_dependent(pf_attention_kernel<64>, dim3(fgrid), dim3(256), FaSm<64>::BYTES, s, fa));
             if ((r = resid(tm.o, d)) != KG_OK) return r;
             CK(norm(lw.g2));

@@ -611,6 +611,7 @@ struct FaArgs {
     __nv_bfloat16* oh; __nv_bfloat16* ol;                // [rows][d] planes of the output
     const int* page_table; int ps_shift, n_phys; State* st;
     int H, pos0, rows;
+    int row0; int* err;                                  // pf_attention_tc_kernel: first row of the layer in the caches' tensor maps; set to 1 when a bounded wait expired
 };
 
 template <int HD>
@@ -754,6 +755,303 @@ __global__ void __launch_bounds__(256, 1) pf_attention_kernel(const __grid_const
             *reinterpret_cast<unsigned*>(a.oh + (size_t)(wr0 + g + 8) * d + col) = hi;
             *reinterpret_cast<unsigned*>(a.ol + (size_t)(wr0 + g + 8) * d + col) = lo;
         }
+    }
+}
+
+// ---- the same on the 5th-generation tensor cores, for blocks of many rows and keys --------------------------------------
+// One CTA = 128 query rows of one head, one row per tensor-memory lane; key tiles of 128.  Warp 0 brings K and V tiles (TMA, pages of
+// the cache in boxes of up to 16 keys x 64 dims, two stages each), warp 1 issues the MMAs, eight warps do the softmax, two threads per
+// row (64 keys, and HD / 2 dims of the output each).  Tensor memory: two score tiles, each overwritten by its P in two planes (the A operand of the
+// second product), and the products of two tiles with V.  S(j + 1) is issued before P(j) V, so that the tensor cores work while tile
+// j's softmax runs; a product is read two tiles later, beside the scores, when nobody has to wait for it.
+//
+// Precision is that of the kernel above: q and P in two bf16 planes, softmax and the sum over the tiles in fp32.  The lo planes are
+// multiplied first, and a tile's P V starts from zero and is added to registers, so that fewer of the tensor core's truncations count.
+//
+// What bounds it: per tile 2048 clocks of MMAs (both planes) beside about as many of exponentials, splits and tensor-memory traffic.  7B, one layer
+// (us, the kernel above / this one): 512 rows 32.8 / 20.0, 1024 65 / 38, 1999 222 / 106; prompt pass of 1999 tokens 51.2 -> 47.9 ms.  At 1999
+// rows a tile takes about 5000 clocks: what bounds it is the latency of the softmax chain (issue slots 32 % busy) and, per CTA, its start
+// and end (about 5 us).
+constexpr int FT_ROWS = 128, FT_KEYS = 128, FT_THREADS = 384, FT_SOFT_WARPS = 8;
+constexpr int FT_MIN_KEYS = 128;                          // up to here the kernel above is the better one (us, 7B, one layer, the kernel above / this one: 64 keys 8.2 / 10.3, 128 12.7 / 13.5, 256
+                                                          // 19.3 / 15.4, 512 32.8 / 20.0)
+constexpr int FT_CTRL_REGS = 56, FT_SOFT_REGS = 216;
+static_assert(128 * FT_CTRL_REGS + 32 * FT_SOFT_WARPS * FT_SOFT_REGS <= FT_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
+template <int HD> struct FtSm {
+    static constexpr int PLANE = FT_ROWS * HD * 2, TILE = FT_KEYS * HD * 2;
+    static constexpr int KOFF = 2 * PLANE, VOFF = KOFF + 2 * TILE, CTRL = VOFF + 2 * TILE;
+    static constexpr int BYTES = 1024 + CTRL + 2048 + 256;               // alignment slack, operands, maxima / sums of the row halves, barriers
+};
+constexpr uint32_t FT_S = 0, FT_O = 256;                                 // tensor-memory columns: S [2][128], each overwritten by its P (hi, lo: 64 each); P V [2][128]
+
+__device__ __forceinline__ void umma_commit_one(unsigned long long* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate));
+}
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 db, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate));
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+
+template <int HD>
+__global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
+                                                                        const __grid_constant__ FaArgs a) {
+    extern __shared__ __align__(128) char smem_raw[];
+    using G = FtSm<HD>;
+    constexpr int HALVES = HD / 64;                        // 64-dim (128-byte) halves of a row
+    const uint32_t raw = smem_u32(smem_raw);
+    char* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);            // swizzled tiles sit on 1024-byte boundaries
+    float* part = reinterpret_cast<float*>(smem + G::CTRL);              // [2 turns][2 halves][128 rows]
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem + G::CTRL + 2048);
+    unsigned long long *k_full = bar, *k_empty = bar + 2, *v_full = bar + 4, *v_empty = bar + 6, *s_full = bar + 8, *o_full = bar + 10;
+    unsigned long long *p_full = bar + 12, *q_full = bar + 13;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 14);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nblk = (a.rows + FT_ROWS - 1) / FT_ROWS;
+    const int rb = nblk - 1 - blockIdx.x / a.H, hh = blockIdx.x % a.H;  // those with the most keys first
+    const int r0 = rb * FT_ROWS, rend = min(a.rows, r0 + FT_ROWS);
+    const int T = a.pos0 + rend;                           // keys any row of the block may see
+    const int ntile = (T + FT_KEYS - 1) / FT_KEYS;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 14; ++i) mbar_init(bar + i, i >= 12 ? FT_SOFT_WARPS : 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    grid_dependents_launch();
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FT_CTRL_REGS));
+        grid_dependency_wait();
+        if (warp == 0) {
+            // ---- K and V tiles; boxes without a valid key are left out
+            asm volatile("fence.proxy.async;" ::: "memory");
+            const int bsh = min(a.ps_shift, 4), psm = (1 << a.ps_shift) - 1;      // a box holds 2^bsh keys
+            bool ok = true;
+            auto load = [&](const CUtensorMap* tm, int j, uint32_t dst, unsigned long long* full) {
+                const int nbox = (min(FT_KEYS, T - j * FT_KEYS) + (1 << bsh) - 1) >> bsh;
+                if (lane == 0) mbar_arrive_expect_tx(full, (unsigned)(nbox * HALVES * (128 << bsh)));
+                __syncwarp();
+                for (int i = lane; i < nbox * HALVES; i += 32) {
+                    const int b = i / HALVES, half = i % HALVES, key = j * FT_KEYS + (b << bsh);
+                    const int page = checked_page(__ldg(a.page_table + (key >> a.ps_shift)), a.n_phys, a.st, 64);
+                    tma_load_2d(dst + (uint32_t)(half * (FT_KEYS * 128) + (b << (bsh + 7))), tm, half * 64, a.row0 + ((page * a.H + hh) << a.ps_shift) + (key & psm), smem_u32(full));
+                }
+                __syncwarp();
+            };
+            for (int j = 0; j < ntile && ok; ++j) {
+                const int s = j & 1; const unsigned par = ((unsigned)(j >> 1) & 1u) ^ 1u;
+                if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_empty[s], par, a.err)))) break;
+                load(&tmk, j, smem_u32(smem + G::KOFF + s * G::TILE), &k_full[s]);
+                if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_empty[s], par, a.err)))) break;
+                load(&tmv, j, smem_u32(smem + G::VOFF + s * G::TILE), &v_full[s]);
+            }
+            // every completion arrives in this CTA's shared memory before it may leave
+            for (int j = max(0, ntile - 2); j < ntile && ok; ++j)
+                ok = gm_wait(&k_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err) && gm_wait(&v_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err);
+        } else if (warp == 1) {
+            // ---- MMAs: S(j), then P(j - 1) V(j - 1).  S(j) overwrites P(j - 2), whose product must be complete
+            const uint32_t sbase = smem_u32(smem);
+            const uint32_t id_s = umma_idesc(FT_ROWS, FT_KEYS), id_o = umma_idesc(FT_ROWS, HD) | (1u << 16);       // V: dims are contiguous (MN-major)
+            bool ok = __all_sync(0xffffffffu, gm_wait(q_full, 0u, a.err));
+            for (int j = 0; j <= ntile && ok; ++j) {
+                if (j < ntile) {
+                    const int s = j & 1; const unsigned par = (unsigned)(j >> 1) & 1u;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_full[s], par, a.err) && (j < 2 || gm_wait(&o_full[s], par ^ 1u, a.err))))) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int pl = 1; pl >= 0; --pl) {              // lo, hi
+#pragma unroll
+                            for (int k = 0; k < HD / 16; ++k) {
+                                const uint32_t o = (uint32_t)((k >> 2) * (FT_KEYS * 128) + (k & 3) * 32);
+                                umma_ss(tmem + FT_S + 128u * s, umma_desc_lo(sbase + pl * G::PLANE + o), umma_desc_lo(sbase + G::KOFF + s * G::TILE + o), id_s, pl == 1 && k == 0 ? 0u : 1u);
+                            }
+                        }
+                        umma_commit_one(&k_empty[s]);
+                        umma_commit_one(&s_full[s]);
+                    }
+                    __syncwarp();
+                }
+                if (j > 0) {
+                    const int i = j - 1, s = i & 1;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_full[s], (unsigned)(i >> 1) & 1u, a.err)))) break;
+                    const int nv = T - i * FT_KEYS;                    // V rows without a key hold anything (0 * NaN would be NaN)
+                    if (nv < FT_KEYS) {
+                        for (int x = lane; x < (FT_KEYS - nv) * HALVES * 8; x += 32) {
+                            const int c = x & 7, half = (x >> 3) % HALVES, r = nv + (x >> 3) / HALVES;
+                            *reinterpret_cast<uint4*>(smem + G::VOFF + s * G::TILE + half * (FT_KEYS * 128) + r * 128 + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(p_full, (unsigned)i & 1u, a.err)))) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int pl = 1; pl >= 0; --pl) {
+#pragma unroll
+                            for (int k = 0; k < FT_KEYS / 16; ++k)
+                                umma_ts(tmem + FT_O + 128u * s, tmem + FT_S + 128u * s + 64u * pl + 8u * k,
+                                        (((sbase + G::VOFF + s * G::TILE + k * 2048) & 0x3FFFFu) >> 4) | ((uint32_t)(FT_KEYS * 128 / 16) << 16), id_o, pl == 1 && k == 0 ? 0u : 1u);
+                        }
+                        umma_commit_one(&v_empty[s]);
+                        umma_commit_one(&o_full[s]);
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FT_SOFT_REGS));
+        grid_dependency_wait();
+        const int d = a.H * HD;
+        {
+            // q planes -> shared memory, 128-byte swizzle (rows past the end repeat the last row and are not stored)
+            constexpr int CH = HD / 8;
+            const int tid = threadIdx.x - 128;
+#pragma unroll
+            for (int pl = 0; pl < 2; ++pl) {
+#pragma unroll
+                for (int i = 0; i < FT_ROWS * CH / 256; ++i) {
+                    const int id = tid + i * 256, r = id / CH, c = id % CH;
+                    const uint4 v = *reinterpret_cast<const uint4*>((pl ? a.ql : a.qh) + (size_t)min(r0 + r, a.rows - 1) * d + hh * HD + c * 8);
+                    *reinterpret_cast<uint4*>(smem + pl * G::PLANE + (c >> 3) * (FT_ROWS * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(q_full);
+        }
+        const int sw = warp - 4, q = sw & 3, half = sw >> 2, row = q * 32 + lane;
+        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);             // this warp's lanes
+        const int lim = min(a.pos0 + r0 + row, T - 1);                     // last key this row may see
+        constexpr int OC = HD / 2;                                         // dims of the output this thread keeps
+        float o[OC];
+#pragma unroll
+        for (int i = 0; i < OC; ++i) o[i] = 0.f;
+        float m = -INFINITY, l = 0.f;
+        bool ok = true;                    // after a wait that gave up the rest runs through without waiting, on values nobody will use
+        // the product of tile j, columns 32 c ..
+        auto request_o = [&](int j, int c, uint32_t (&v)[32]) { tmem_ld32(tl + FT_O + 128u * (j & 1) + (uint32_t)(half * OC + c * 32), v); };
+        auto wait_o = [&](int j) {
+            if (ok) ok = gm_wait(&o_full[j & 1], (unsigned)(j >> 1) & 1u, a.err);
+            __syncwarp();
+            tc_fence_after();
+        };
+        float cf = 1.f;                                                    // scale of the tile before, relative to the one before that
+        for (int j = 0; j < ntile; ++j) {
+            const int s = j & 1, key0 = j * FT_KEYS + half * 64;
+            if (ok) ok = gm_wait(&s_full[s], (unsigned)(j >> 1) & 1u, a.err);
+            __syncwarp();
+            tc_fence_after();
+            uint32_t w0[32], w1[32], v[32];
+            tmem_ld32(tl + FT_S + 128u * s + 64u * half, w0);
+            tmem_ld32(tl + FT_S + 128u * s + 64u * half + 32u, w1);
+            // (the product of tile j - 2 is complete: S(j) comes after it)
+            if (j > 1) {
+                wait_o(j - 2);
+                request_o(j - 2, 0, v);
+            }
+            tmem_ld_wait32(w0);
+            tmem_ld_wait32(w1);
+            float x[64];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { x[i] = __uint_as_float(w0[i]); x[32 + i] = __uint_as_float(w1[i]); }
+            if (j * FT_KEYS + FT_KEYS - 1 > a.pos0 + r0) {                 // the tile crosses the diagonal of the block
+#pragma unroll
+                for (int i = 0; i < 64; ++i) if (key0 + i > lim) x[i] = -INFINITY;
+            }
+            float mx[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+            for (int i = 4; i < 64; ++i) mx[i & 3] = fmaxf(mx[i & 3], x[i]);
+            mx[0] = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            part[(s * 2 + half) * FT_ROWS + row] = mx[0];
+            if (j > 1) {                                                   // while the other half's maximum is on its way
+                tmem_ld_wait32(v);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = (o[i] + __uint_as_float(v[i])) * cf;
+                if constexpr (OC > 32) request_o(j - 2, 1, v);
+            }
+            named_sync(1 + q, 64);                                         // the two warps of these rows
+            // key 0 is visible to every row, so the maxima are finite from the first tile on
+            const float mn = fmaxf(m, fmaxf(mx[0], part[(s * 2 + (half ^ 1)) * FT_ROWS + row]));
+            const float cf_new = ex2f(m - mn);
+            m = mn;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            uint32_t ph[32], pl[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const float p0 = ex2f(x[2 * i] - mn), p1 = ex2f(x[2 * i + 1] - mn);
+                sum[i & 3] += p0 + p1;
+                split_hi_lo(make_float2(p0, p1), ph[i], pl[i]);
+            }
+            l = l * cf_new + ((sum[0] + sum[1]) + (sum[2] + sum[3]));
+            if constexpr (OC > 32) {
+                if (j > 1) {
+                    tmem_ld_wait32(v);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[OC - 32 + i] = (o[OC - 32 + i] + __uint_as_float(v[i])) * cf;
+                }
+            }
+            cf = cf_new;
+            // (both halves of the scores have been read: the barrier above)
+            const uint32_t tp = tl + FT_S + 128u * s + 32u * half;
+            tmem_st16(tp, ph); tmem_st16(tp + 16u, ph + 16);
+            tmem_st16(tp + 64u, pl); tmem_st16(tp + 80u, pl + 16);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(p_full);
+        }
+        // the products of the last two tiles (the last but one at the scale before cf)
+        for (int j = max(0, ntile - 2); j < ntile; ++j) {
+            wait_o(j);
+#pragma unroll
+            for (int c = 0; c < OC / 32; ++c) {
+                uint32_t v[32];
+                request_o(j, c, v);
+                tmem_ld_wait32(v);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) { o[c * 32 + i] += __uint_as_float(v[i]); if (j < ntile - 1) o[c * 32 + i] *= cf; }
+            }
+        }
+        part[half * FT_ROWS + row] = l;                                    // (the last tile's maxima have been read, or lie in the other turn)
+        named_sync(1 + q, 64);
+        const float il = 1.0f / (l + part[(half ^ 1) * FT_ROWS + row]);
+        if (r0 + row < rend) {
+            const size_t at = (size_t)(r0 + row) * d + (size_t)hh * HD + half * OC;
+#pragma unroll
+            for (int i = 0; i < OC; i += 8) {
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = o[i + k] * il;
+                store8_planes(a.oh + at + i, a.ol + at + i, v);
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
 
