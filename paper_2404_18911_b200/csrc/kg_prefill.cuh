@@ -763,7 +763,9 @@ __global__ void __launch_bounds__(256, 1) pf_attention_kernel(const __grid_const
 // the cache in boxes of up to 16 keys x 64 dims, two stages each), warp 1 issues the MMAs, eight warps do the softmax, two threads per
 // row (64 keys, and HD / 2 dims of the output each).  Tensor memory: two score tiles, each overwritten by its P in two planes (the A operand of the
 // second product), and the products of two tiles with V.  S(j + 1) is issued before P(j) V, so that the tensor cores work while tile
-// j's softmax runs; a product is read two tiles later, beside the scores, when nobody has to wait for it.
+// j's softmax runs; a product is read two tiles later, beside the scores, when nobody has to wait for it.  The softmax warps of
+// different rows may therefore be a tile apart, and all of them a tile ahead of the MMAs, so that P has a barrier for each of the two
+// tiles: on one for all tiles, a fast warp's arrival for tile j + 1 would count for a slow one's for tile j.
 //
 // Precision is that of the kernel above: q and P in two bf16 planes, softmax and the sum over the tiles in fp32.  The lo planes are
 // multiplied first, and a tile's P V starts from zero and is added to registers, so that fewer of the tensor core's truncations count.
@@ -814,8 +816,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
     float* part = reinterpret_cast<float*>(smem + G::CTRL);              // [2 turns][2 halves][128 rows]
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem + G::CTRL + 2048);
     unsigned long long *k_full = bar, *k_empty = bar + 2, *v_full = bar + 4, *v_empty = bar + 6, *s_full = bar + 8, *o_full = bar + 10;
-    unsigned long long *p_full = bar + 12, *q_full = bar + 13;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 14);
+    unsigned long long *p_full = bar + 12, *q_full = bar + 14;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 15);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nblk = (a.rows + FT_ROWS - 1) / FT_ROWS;
     const int rb = nblk - 1 - blockIdx.x / a.H, hh = blockIdx.x % a.H;  // those with the most keys first
@@ -823,7 +825,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
     const int T = a.pos0 + rend;                           // keys any row of the block may see
     const int ntile = (T + FT_KEYS - 1) / FT_KEYS;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 14; ++i) mbar_init(bar + i, i >= 12 ? FT_SOFT_WARPS : 1);
+        for (int i = 0; i < 15; ++i) mbar_init(bar + i, i >= 12 ? FT_SOFT_WARPS : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -901,7 +903,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
                     }
-                    if (!(ok = __all_sync(0xffffffffu, gm_wait(p_full, (unsigned)i & 1u, a.err)))) break;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&p_full[s], (unsigned)(i >> 1) & 1u, a.err)))) break;
                     tc_fence_after();
                     if (elect_one()) {
 #pragma unroll
@@ -1018,7 +1020,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(p_full);
+            if (lane == 0) mbar_arrive(&p_full[s]);
         }
         // the products of the last two tiles (the last but one at the scale before cf)
         for (int j = max(0, ntile - 2); j < ntile; ++j) {
