@@ -190,6 +190,14 @@ int kg_debug_skip_barrier_arrival(kg_model* m, int cta);
  *   model is bf16 with head_dim 64 / 128 and d, F multiples of 128; 1: every prompt takes the 16-row chunked pass of
  *   the decode kernels (the two are compared with each other and with the oracle in the tests). */
 int kg_debug_set_prefill_mode(kg_model* m, int mode);
+/* kg_debug_prompt_attention: the attention of the tensor-core prompt pass by itself, on device buffers of the caller.  q_hi, q_lo and out_hi, out_lo are the
+ *   bf16 planes [rows][n_heads * head_dim] of the rotated q, times log2(e) / sqrt(head_dim), and of the result; rows (at most 2048) sit at positions pos0.., and
+ *   the caches [n_pages][n_heads][page_size][head_dim] (bf16) hold K and V of every position up to the last row's.  kernel: 0 the one that the prompt
+ *   pass takes, 1 mma.sync, 2 tcgen05.  *err_dev becomes 0, or not 0 when a wait gave up.  skip: -1; else (kernel 2) one softmax
+ *   warp of that CTA leaves out an arrival, so that the waits of the CTA run out (about 2 s): nothing faults, the kernel returns. */
+int kg_debug_prompt_attention(int32_t n_heads, int32_t head_dim, int32_t pos0, int32_t rows, const void* q_hi_dev, const void* q_lo_dev,
+                              const void* kcache_dev, const void* vcache_dev, const int32_t* page_table_dev, int32_t page_size,
+                              int32_t n_pages, int32_t kernel, int32_t skip, void* out_hi_dev, void* out_lo_dev, int32_t* err_dev, void* cuda_stream);
 
 /* ---- single operators on caller buffers (unit tests and microbenchmarks) ------------------------
  * All pointers are device pointers, 16-byte aligned (int32 arrays: 4-byte), else KG_E_ARG; `scratch_dev` must hold

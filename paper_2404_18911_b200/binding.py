@@ -25,7 +25,7 @@ EXPORTS = [
     "kg_debug_logits", "kg_read_weight", "kg_debug_fill_state", "kg_op_scratch_bytes", "kg_op_linear",
     "kg_op_lm_head", "kg_op_lm_head_noalloc", "kg_op_attention", "kg_strerror",
     "kg_last_cuda_error", "kg_debug_force_simple", "kg_debug_force_simple_ops", "kg_debug_set_wait_budget", "kg_debug_skip_barrier_arrival",
-    "kg_debug_set_prefill_mode", "kg_op_gemm",
+    "kg_debug_set_prefill_mode", "kg_debug_prompt_attention", "kg_op_gemm",
 ]
 
 
@@ -125,6 +125,7 @@ def load():
     lib.kg_debug_set_wait_budget.argtypes = [vp, C.c_double]
     lib.kg_debug_skip_barrier_arrival.argtypes = [vp, C.c_int]
     lib.kg_debug_set_prefill_mode.argtypes = [vp, C.c_int]
+    lib.kg_debug_prompt_attention.argtypes = [i32, i32, i32, i32, vp, vp, vp, vp, vp, i32, i32, i32, i32, vp, vp, vp, vp]
     _lib = lib
     return lib
 
@@ -415,3 +416,16 @@ def op_attention(qkv, pos0, n_heads, head_dim, rope_theta, kcache, vcache, page_
                                vcache.data_ptr(), page_table.data_ptr(), page_size, out.data_ptr(),
                                scratch.data_ptr(), _stream(torch)), "kg_op_attention")
     return out
+
+
+def debug_prompt_attention(q_hi, q_lo, pos0, n_heads, kcache, vcache, page_table, page_size, kernel=0, skip=-1):
+    """The prompt pass's attention by itself (kg_debug_prompt_attention): the planes of its output and the error word."""
+    import torch
+    lib = load()
+    rows, d = q_hi.shape
+    hi, lo = torch.empty_like(q_hi), torch.empty_like(q_lo)
+    err = torch.empty(1, dtype=torch.int32, device=q_hi.device)
+    _check(lib.kg_debug_prompt_attention(n_heads, d // n_heads, pos0, rows, q_hi.data_ptr(), q_lo.data_ptr(), kcache.data_ptr(), vcache.data_ptr(),
+                                         page_table.data_ptr(), page_size, kcache.shape[0], kernel, skip, hi.data_ptr(), lo.data_ptr(), err.data_ptr(),
+                                         _stream(torch)), "kg_debug_prompt_attention")
+    return hi, lo, err

@@ -1229,7 +1229,8 @@ int gemm_attributes() {
 }
 
 template <int HD>
-int attention_tc_attributes() {
+int attention_attributes() {
+    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<HD>::BYTES));
     cudaFuncAttributes fa;
     CK(cudaFuncGetAttributes(&fa, (const void*)pf_attention_tc_kernel<HD>));
     if ((long long)fa.numRegs * FT_THREADS < 128LL * FT_CTRL_REGS + 32LL * FT_SOFT_WARPS * FT_SOFT_REGS) {
@@ -1263,9 +1264,7 @@ int prefill_tc_init(kg_model* m) {
     if (!ok) return tmap_failed();
     int r;
     if ((r = gemm_attributes<PF_STORE>()) != KG_OK || (r = gemm_attributes<PF_QKV>()) != KG_OK || (r = gemm_attributes<PF_SWIGLU>()) != KG_OK) return r;
-    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<128>::BYTES));
-    CK(cudaFuncSetAttribute((const void*)pf_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FaSm<64>::BYTES));
-    if ((r = attention_tc_attributes<128>()) != KG_OK || (r = attention_tc_attributes<64>()) != KG_OK) return r;
+    if ((r = attention_attributes<128>()) != KG_OK || (r = attention_attributes<64>()) != KG_OK) return r;
     CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
     CK(cudaMemsetAsync(A + m->lay.off_pf_cnt, 0, 4 * (size_t)m->nctas, m->stream));
     m->pf.ready = true;
@@ -1273,11 +1272,11 @@ int prefill_tc_init(kg_model* m) {
 }
 
 // x_0 from the per-CTA LM-head partials; the sequence state after a prompt of n tokens (one warp)
-__global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* out_tokens, int n, const int* gemm_err) {
+__global__ void pf_finish_kernel(const float4* part, int nctas, State* st, int* out_tokens, int n, const int* err) {
     int tok; float p;
     head_final_warp(part, nctas, 0, tok, p);
     if (threadIdx.x == 0) {
-        if (*gemm_err) { atomicCAS(&st->status, 0, ST_TIMEOUT); st->timeout_where = 60; st->timed_out = 1; }      // a wait inside a GEMM gave up
+        if (*err) { atomicCAS(&st->status, 0, ST_TIMEOUT); st->timeout_where = *err == PF_ERR_ATT ? 61 : 60; st->timed_out = 1; }      // a wait inside the attention or a GEMM gave up
         st->P = n; st->len_A = n; st->x0 = tok; st->pending = 0; st->total = 1; st->rounds = 0;
         out_tokens[0] = tok;
     }
@@ -1316,6 +1315,19 @@ int gm_launch(GemmArgs& g, const CUtensorMap& hi, const CUtensorMap& lo, const C
     CK(launch_dependent(pf_gemm_kernel<EPI>, dim3(2 * used), dim3(GM_THREADS), GM_SMEM, s, hi, lo, w, w2, g));
     return KG_OK;
 }
+
+// The attention of a block of prompt rows; tc: on tcgen05.
+int launch_prompt_attention(const FaArgs& fa, int hd, bool tc, const CUtensorMap& tmk, const CUtensorMap& tmv, cudaStream_t s) {
+    const dim3 grid((fa.rows + FA_ROWS - 1) / FA_ROWS * fa.H);
+    static_assert(FA_ROWS == FT_ROWS, "rows of a CTA");
+    if (tc) {
+        if (hd == 128) CK(launch_dependent(pf_attention_tc_kernel<128>, grid, dim3(FT_THREADS), FtSm<128>::BYTES, s, tmk, tmv, fa));
+        else CK(launch_dependent(pf_attention_tc_kernel<64>, grid, dim3(FT_THREADS), FtSm<64>::BYTES, s, tmk, tmv, fa));
+    } else if (hd == 128) CK(launch_dependent(pf_attention_kernel<128>, grid, dim3(256), FaSm<128>::BYTES, s, fa));
+    else CK(launch_dependent(pf_attention_kernel<64>, grid, dim3(256), FaSm<64>::BYTES, s, fa));
+    return KG_OK;
+}
+bool prompt_attention_tc(const FaArgs& fa) { return fa.pos0 + fa.rows > FT_MIN_KEYS; }
 
 // The prompt in blocks of at most PF_ROWS rows of about equal size, each block through all layers (its K / V are in the
 // caches before the next block attends to them), the adapter's K / V after layer l, the LM head on the last row.
@@ -1372,13 +1384,8 @@ int prefill_tc(kg_model* m, int n) {
             FaArgs fa;
             fa.qh = qh; fa.ql = ql; fa.kc = (const WT*)D.kcache + (size_t)i * lstride; fa.vc = (const WT*)D.vcache + (size_t)i * lstride;
             fa.oh = xh; fa.ol = xl; fa.page_table = D.page_table; fa.ps_shift = D.dm.ps_shift; fa.n_phys = D.dm.n_phys; fa.st = D.st;
-            fa.H = H; fa.pos0 = b0; fa.rows = rows; fa.row0 = i * D.dm.n_pages * H * c.page_size; fa.err = err;
-            const int fgrid = (rows + FA_ROWS - 1) / FA_ROWS * H;
-            if (D.dm.ring && b0 + rows > FT_MIN_KEYS) {
-                if (hd == 128) CK(launch_dependent(pf_attention_tc_kernel<128>, dim3(fgrid), dim3(FT_THREADS), FtSm<128>::BYTES, s, D.tmk, D.tmv, fa));
-                else CK(launch_dependent(pf_attention_tc_kernel<64>, dim3(fgrid), dim3(FT_THREADS), FtSm<64>::BYTES, s, D.tmk, D.tmv, fa));
-            } else if (hd == 128) CK(launch_dependent(pf_attention_kernel<128>, dim3(fgrid), dim3(256), FaSm<128>::BYTES, s, fa));
-            else CK(launch_dependent(pf_attention_kernel<64>, dim3(fgrid), dim3(256), FaSm<64>::BYTES, s, fa));
+            fa.H = H; fa.pos0 = b0; fa.rows = rows; fa.row0 = i * D.dm.n_pages * H * c.page_size; fa.err = err; fa.skip = -1;
+            if ((r = launch_prompt_attention(fa, hd, D.dm.ring && prompt_attention_tc(fa), D.tmk, D.tmv, s)) != KG_OK) return r;
             if ((r = resid(tm.o, d)) != KG_OK) return r;
             CK(norm(lw.g2));
             GemmArgs g = base;
@@ -1415,6 +1422,31 @@ extern "C" int kg_debug_set_prefill_mode(kg_model* m, int mode) {
     if (!m || (mode != 0 && mode != 1)) return KG_E_ARG;
     m->prefill_mode = mode;
     return KG_OK;
+}
+
+extern "C" int kg_debug_prompt_attention(int32_t H, int32_t hd, int32_t pos0, int32_t rows, const void* qh, const void* ql, const void* kc, const void* vc,
+                                         const int32_t* page_table, int32_t page_size, int32_t n_pages, int32_t kernel, int32_t skip,
+                                         void* oh, void* ol, int32_t* err, void* stream) {
+    if (!qh || !ql || !kc || !vc || !page_table || !oh || !ol || !err) return KG_E_ARG;
+    for (const void* p : {qh, ql, kc, vc, (const void*)oh, (const void*)ol}) if (!aligned16(p)) return KG_E_ARG;
+    if ((reinterpret_cast<uintptr_t>(page_table) & 3u) || (reinterpret_cast<uintptr_t>(err) & 3u)) return KG_E_ARG;
+    if (H < 1 || H > 256 || (hd != 64 && hd != 128) || pos0 < 0 || rows < 1 || rows > PF_ROWS || pos0 > (1 << 24) || page_size < 1 || (page_size & (page_size - 1)) ||
+        n_pages < 1 || kernel < 0 || kernel > 2) return KG_E_ARG;
+    if ((long long)n_pages * H > 0x7fffffff / page_size) return KG_E_LIMIT;
+    typedef __nv_bfloat16 WT;
+    FaArgs fa;
+    fa.qh = (const WT*)qh; fa.ql = (const WT*)ql; fa.kc = (const WT*)kc; fa.vc = (const WT*)vc; fa.oh = (WT*)oh; fa.ol = (WT*)ol;
+    fa.page_table = page_table; fa.n_phys = n_pages; fa.st = nullptr; fa.H = H; fa.pos0 = pos0; fa.rows = rows; fa.row0 = 0; fa.err = err; fa.skip = skip;
+    for (fa.ps_shift = 0; (1 << fa.ps_shift) < page_size; ++fa.ps_shift) {}
+    CUtensorMap tmk, tmv;
+    const uint64_t crows = (uint64_t)n_pages * H * page_size;
+    const int box = page_size < 16 ? page_size : 16;
+    if (!make_tmap(&tmk, kc, crows, hd, box) || !make_tmap(&tmv, vc, crows, hd, box)) return tmap_failed();
+    int r = hd == 128 ? attention_attributes<128>() : attention_attributes<64>();
+    if (r != KG_OK) return r;
+    cudaStream_t s = (cudaStream_t)stream;
+    CK(cudaMemsetAsync(err, 0, 4, s));
+    return launch_prompt_attention(fa, hd, kernel == 2 || (kernel == 0 && prompt_attention_tc(fa)), tmk, tmv, s);
 }
 
 extern "C" int kg_op_gemm(const void* W, int32_t N, int32_t K, const float* x, int32_t M, const float* resid, float* out,

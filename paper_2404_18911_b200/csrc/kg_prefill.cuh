@@ -41,6 +41,8 @@ static_assert(GM_SMEM <= SMEM_TOTAL, "GEMM shared memory");
 constexpr int GM_CTRL_REGS = 56, GM_EPI_REGS = 216;
 static_assert(GM_THREADS == DECODE_THREADS && 128 * GM_CTRL_REGS + 32 * GM_EPI_WARPS * GM_EPI_REGS <= GM_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
 constexpr unsigned long long GM_WAIT_CLK = 4000000000ull;              // ~2 s: a wait that runs this long gives up
+constexpr unsigned long long GM_WAIT_CLK_FAILED = GM_WAIT_CLK / 64;    // ~30 ms: once another wait of the prompt pass gave up
+enum { PF_ERR_GEMM = 1, PF_ERR_ATT = 2 };                              // the error word: whose wait gave up first
 
 enum { PF_STORE = 0, PF_QKV = 1, PF_SWIGLU = 2 };                      // what the epilogue makes of the products
 
@@ -58,7 +60,7 @@ struct GemmArgs {
     __nv_bfloat16* kc; __nv_bfloat16* vc;
     float qscale;
     float* part; unsigned* cnt;         // partial sums of the cut tiles, arrival counters (left at zero)
-    int* err;                           // set to 1 when a bounded wait expired
+    int* err;                           // PF_ERR_GEMM when a bounded wait expired
 };
 
 // ---- TMA tile copy, tensor memory and tcgen05 MMA ----------------------------------------------------------------
@@ -129,15 +131,20 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) :: "memory");
 }
 
-// bounded wait on an mbarrier phase; on expiry the error word is set and false returned
-__device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity, int* err) {
+// Bounded wait on an mbarrier phase; on expiry the error word is set and false returned.  An error word that is set already does not end
+// a wait at once: the kernels behind a failed one run through as ever, and nobody leaves with copies or MMAs just issued.  It shortens
+// the limit, so that a pass in which every kernel fails ends within seconds.
+__device__ __forceinline__ bool gm_wait(unsigned long long* bar, unsigned parity, int* err, int code = PF_ERR_GEMM) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     unsigned spins = 0;
     while (!mbar_try_wait(bar, parity)) {
         if (((++spins) & 255u) == 0u) {
-            if (*(volatile int*)err) return false;
-            if ((unsigned long long)(clock64() - t0) > GM_WAIT_CLK) { *(volatile int*)err = 1; return false; }
+            const bool failed = *(volatile int*)err != 0;
+            if ((unsigned long long)(clock64() - t0) > (failed ? GM_WAIT_CLK_FAILED : GM_WAIT_CLK)) {
+                if (!failed) *(volatile int*)err = code;
+                return false;
+            }
         }
     }
     return true;
@@ -350,6 +357,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
     unsigned long long* acc_free = acc_full + GM_MAX_ACC;  // even CTA: both CTAs' epilogue warps have read the accumulator
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + GM_MAX_ACC);
     int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
+    unsigned long long* drained = acc_free + GM_MAX_ACC + 1;               // the MMAs issued before a wait gave up have completed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = blockIdx.x & 1, pair_id = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int stage_bytes = GM_A_BYTES + g.nt * 128;                       // weights, hi plane, lo plane
@@ -358,6 +366,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
     if (threadIdx.x == 0) {
         for (int i = 0; i < GM_MAX_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
         for (int i = 0; i < GM_MAX_ACC; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_free[i], 2 * GM_EPI_WARPS); }
+        mbar_init(drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -375,7 +384,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GM_CTRL_REGS));
         if (warp == 0) {
             // ---- TMA producer of this CTA's tiles (the warp stays together, one lane issues)
-            int s = 0; unsigned par = 1u;
+            int s = 0, issued = 0; unsigned par = 1u;
             const int hrow = g.nt >> 1;
             bool ok = true;
             // the weights do not come from the kernel before: those of the first stages are on their way while it ends
@@ -412,6 +421,7 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                     }
                     __syncwarp();
                     if (early > 0) --early;
+                    ++issued;
                     if (++s == nst) { s = 0; par ^= 1u; }
                 }
             }
@@ -420,6 +430,10 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                 ok = gm_wait(&empty[s], par, g.err);
                 if (++s == nst) { s = 0; par ^= 1u; }
             }
+            // after a wait that gave up: no MMA may come to empty the last stages, so the copies themselves are waited for.  Both CTAs'
+            // arrive at the even one's barriers, and the odd one stays until the even one leaves
+            if (!ok && rank == 0)
+                for (int i = max(0, issued - nst); i < issued; ++i) gm_wait(&full[i % nst], (unsigned)(i / nst) & 1u, g.err);
         } else if (warp == 1 && rank == 0) {
             // ---- MMA issuer of the pair.  The warp stays together and one elected lane issues: with a loop that only lane 0 ran,
             // issuing took 115 clocks per instruction, which made every tile of up to 192 columns issue-bound.
@@ -459,6 +473,12 @@ pf_gemm_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
                     }
                     if (++a == nacc) { a = 0; apar ^= 1u; }
                 }
+            }
+            if (!ok) {                     // tensor memory is given back after the MMAs that write it
+                __syncwarp();
+                if (elect_one()) umma_commit_pair(drained);
+                __syncwarp();
+                gm_wait(drained, 0u, g.err);
             }
         }
     } else {
@@ -611,7 +631,8 @@ struct FaArgs {
     __nv_bfloat16* oh; __nv_bfloat16* ol;                // [rows][d] planes of the output
     const int* page_table; int ps_shift, n_phys; State* st;
     int H, pos0, rows;
-    int row0; int* err;                                  // pf_attention_tc_kernel: first row of the layer in the caches' tensor maps; set to 1 when a bounded wait expired
+    int row0; int* err;                                  // pf_attention_tc_kernel: first row of the layer in the caches' tensor maps; PF_ERR_ATT when a bounded wait expired
+    int skip;                                            // test hook: this CTA's first softmax warp leaves out the arrival of its first tile (-1: none)
 };
 
 template <int HD>
@@ -817,7 +838,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem + G::CTRL + 2048);
     unsigned long long *k_full = bar, *k_empty = bar + 2, *v_full = bar + 4, *v_empty = bar + 6, *s_full = bar + 8, *o_full = bar + 10;
     unsigned long long *p_full = bar + 12, *q_full = bar + 14;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 15);
+    unsigned long long* drained = bar + 15;                // the MMAs issued before a wait gave up have completed
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 16);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nblk = (a.rows + FT_ROWS - 1) / FT_ROWS;
     const int rb = nblk - 1 - blockIdx.x / a.H, hh = blockIdx.x % a.H;  // those with the most keys first
@@ -825,7 +847,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
     const int T = a.pos0 + rend;                           // keys any row of the block may see
     const int ntile = (T + FT_KEYS - 1) / FT_KEYS;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 15; ++i) mbar_init(bar + i, i >= 12 ? FT_SOFT_WARPS : 1);
+        for (int i = 0; i < 16; ++i) mbar_init(bar + i, i >= 12 && i < 15 ? FT_SOFT_WARPS : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -846,6 +868,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
             asm volatile("fence.proxy.async;" ::: "memory");
             const int bsh = min(a.ps_shift, 4), psm = (1 << a.ps_shift) - 1;      // a box holds 2^bsh keys
             bool ok = true;
+            int nk = 0, nv = 0;                            // tiles on their way
             auto load = [&](const CUtensorMap* tm, int j, uint32_t dst, unsigned long long* full) {
                 const int nbox = (min(FT_KEYS, T - j * FT_KEYS) + (1 << bsh) - 1) >> bsh;
                 if (lane == 0) mbar_arrive_expect_tx(full, (unsigned)(nbox * HALVES * (128 << bsh)));
@@ -859,23 +882,27 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
             };
             for (int j = 0; j < ntile && ok; ++j) {
                 const int s = j & 1; const unsigned par = ((unsigned)(j >> 1) & 1u) ^ 1u;
-                if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_empty[s], par, a.err)))) break;
-                load(&tmk, j, smem_u32(smem + G::KOFF + s * G::TILE), &k_full[s]);
-                if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_empty[s], par, a.err)))) break;
-                load(&tmv, j, smem_u32(smem + G::VOFF + s * G::TILE), &v_full[s]);
+                if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_empty[s], par, a.err, PF_ERR_ATT)))) break;
+                load(&tmk, j, smem_u32(smem + G::KOFF + s * G::TILE), &k_full[s]); ++nk;
+                if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_empty[s], par, a.err, PF_ERR_ATT)))) break;
+                load(&tmv, j, smem_u32(smem + G::VOFF + s * G::TILE), &v_full[s]); ++nv;
             }
             // every completion arrives in this CTA's shared memory before it may leave
             for (int j = max(0, ntile - 2); j < ntile && ok; ++j)
-                ok = gm_wait(&k_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err) && gm_wait(&v_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err);
+                ok = gm_wait(&k_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT) && gm_wait(&v_empty[j & 1], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT);
+            if (!ok) {                                     // no MMA may come to empty the tiles, so the copies themselves are waited for
+                for (int j = max(0, nk - 2); j < nk; ++j) gm_wait(&k_full[j & 1], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT);
+                for (int j = max(0, nv - 2); j < nv; ++j) gm_wait(&v_full[j & 1], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT);
+            }
         } else if (warp == 1) {
             // ---- MMAs: S(j), then P(j - 1) V(j - 1).  S(j) overwrites P(j - 2), whose product must be complete
             const uint32_t sbase = smem_u32(smem);
             const uint32_t id_s = umma_idesc(FT_ROWS, FT_KEYS), id_o = umma_idesc(FT_ROWS, HD) | (1u << 16);       // V: dims are contiguous (MN-major)
-            bool ok = __all_sync(0xffffffffu, gm_wait(q_full, 0u, a.err));
+            bool ok = __all_sync(0xffffffffu, gm_wait(q_full, 0u, a.err, PF_ERR_ATT));
             for (int j = 0; j <= ntile && ok; ++j) {
                 if (j < ntile) {
                     const int s = j & 1; const unsigned par = (unsigned)(j >> 1) & 1u;
-                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_full[s], par, a.err) && (j < 2 || gm_wait(&o_full[s], par ^ 1u, a.err))))) break;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&k_full[s], par, a.err, PF_ERR_ATT) && (j < 2 || gm_wait(&o_full[s], par ^ 1u, a.err, PF_ERR_ATT))))) break;
                     tc_fence_after();
                     if (elect_one()) {
 #pragma unroll
@@ -893,7 +920,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
                 }
                 if (j > 0) {
                     const int i = j - 1, s = i & 1;
-                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_full[s], (unsigned)(i >> 1) & 1u, a.err)))) break;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&v_full[s], (unsigned)(i >> 1) & 1u, a.err, PF_ERR_ATT)))) break;
                     const int nv = T - i * FT_KEYS;                    // V rows without a key hold anything (0 * NaN would be NaN)
                     if (nv < FT_KEYS) {
                         for (int x = lane; x < (FT_KEYS - nv) * HALVES * 8; x += 32) {
@@ -903,7 +930,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
                     }
-                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&p_full[s], (unsigned)(i >> 1) & 1u, a.err)))) break;
+                    if (!(ok = __all_sync(0xffffffffu, gm_wait(&p_full[s], (unsigned)(i >> 1) & 1u, a.err, PF_ERR_ATT)))) break;
                     tc_fence_after();
                     if (elect_one()) {
 #pragma unroll
@@ -918,6 +945,12 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
                     }
                     __syncwarp();
                 }
+            }
+            if (!ok) {                                     // tensor memory is given back after the MMAs that write it
+                __syncwarp();
+                if (elect_one()) umma_commit_one(drained);
+                __syncwarp();
+                gm_wait(drained, 0u, a.err, PF_ERR_ATT);
             }
         }
     } else {
@@ -953,14 +986,15 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
         // the product of tile j, columns 32 c ..
         auto request_o = [&](int j, int c, uint32_t (&v)[32]) { tmem_ld32(tl + FT_O + 128u * (j & 1) + (uint32_t)(half * OC + c * 32), v); };
         auto wait_o = [&](int j) {
-            if (ok) ok = gm_wait(&o_full[j & 1], (unsigned)(j >> 1) & 1u, a.err);
+            if (ok) ok = gm_wait(&o_full[j & 1], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT);
             __syncwarp();
             tc_fence_after();
         };
+        const int skip = a.skip == (int)blockIdx.x && warp == 4 ? 0 : -1;
         float cf = 1.f;                                                    // scale of the tile before, relative to the one before that
         for (int j = 0; j < ntile; ++j) {
             const int s = j & 1, key0 = j * FT_KEYS + half * 64;
-            if (ok) ok = gm_wait(&s_full[s], (unsigned)(j >> 1) & 1u, a.err);
+            if (ok) ok = gm_wait(&s_full[s], (unsigned)(j >> 1) & 1u, a.err, PF_ERR_ATT);
             __syncwarp();
             tc_fence_after();
             uint32_t w0[32], w1[32], v[32];
@@ -1020,7 +1054,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) pf_attention_tc_kernel(const __
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&p_full[s]);
+            if (lane == 0 && j != skip) mbar_arrive(&p_full[s]);
         }
         // the products of the last two tiles (the last but one at the scale before cf)
         for (int j = max(0, ntile - 2); j < ntile; ++j) {

@@ -36,3 +36,41 @@ def test_tile_edges(binding, H, hd, page, n):
     print(f"n={n} H={H} hd={hd} page={page}: deviation {np.abs(z[1] - z[0]).max():.2e} of {np.abs(z[0]).max():.2f}")
     assert np.isfinite(z[1]).all()
     assert np.abs(z[1] - z[0]).max() < 2e-2
+
+
+def _operands(H, hd, pos0, rows, page, seed):
+    """Planes of q, a cache in shuffled pages with NaN behind the last key, and K and V by position."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    T = pos0 + rows
+    pages = (T + page - 1) // page + 2
+    q = torch.empty(rows, H * hd, device="cuda").normal_(0.0, 2.0 / np.log(2.0) / np.sqrt(hd), generator=g)
+    qh = q.bfloat16()
+    ql = (q - qh.float()).bfloat16()
+    k, v = (torch.empty(T, H, hd, device="cuda").normal_(generator=g).bfloat16() for _ in range(2))
+    table = torch.randperm(pages, generator=g, device="cuda").to(torch.int32)
+    kc, vc = (torch.full((pages, H, page, hd), float("nan"), device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    at = torch.arange(T, device="cuda")
+    pg, slot = table[at // page].long(), at % page
+    kc[pg, :, slot], vc[pg, :, slot] = k, v
+    return qh, ql, k, v, kc, vc, table
+
+
+def test_expired_wait_returns_and_leaves_the_gpu_usable(binding):
+    """One softmax warp of one block leaves out an arrival (test hook).  The block's waits run out, it waits for its copies and MMAs and
+    returns; the others' rows are complete, and the next call on the same buffers is as good as the one before."""
+    import time
+    import torch
+    H, hd, rows, page = 2, 128, 700, 16
+    qh, ql, _, _, kc, vc, table = _operands(H, hd, 0, rows, page, 1)
+    want = binding.debug_prompt_attention(qh, ql, 0, H, kc, vc, table, page, kernel=2)
+    assert want[2].item() == 0
+    t0 = time.time()
+    hi, lo, err = binding.debug_prompt_attention(qh, ql, 0, H, kc, vc, table, page, kernel=2, skip=0)
+    torch.cuda.synchronize()
+    assert err.item() != 0 and time.time() - t0 < 10
+    keep = torch.ones_like(hi, dtype=torch.bool)
+    keep[640:, :hd] = False                                           # block 0: the last rows of head 0
+    assert torch.equal(hi[keep], want[0][keep]) and torch.equal(lo[keep], want[1][keep])
+    again = binding.debug_prompt_attention(qh, ql, 0, H, kc, vc, table, page, kernel=2)
+    assert again[2].item() == 0 and torch.equal(again[0], want[0]) and torch.equal(again[1], want[1])
