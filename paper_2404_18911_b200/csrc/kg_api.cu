@@ -924,8 +924,8 @@ OpScratch op_layout() {
 }
 
 // One linear operator as a kernel of its own.  V: the row variant of the streamed tensor-core path (bf16 weights, K a multiple of
-// 16), 0: the plain path; compiled one by one, because all variants in one kernel spill at its 168 registers.
-template <typename WT, int V>
+// 16), 0: the plain path; compiled one by one, because all variants in one kernel spill at its 168 registers.  FEW: lin_few().
+template <typename WT, int V, bool FEW>
 __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(const __grid_constant__ LinArgs a) {
     extern __shared__ __align__(128) char smem[];
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
@@ -934,10 +934,10 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) op_linear_kernel(const __gri
         if (!c.producer) lin_simple<WT>(a, c);
     } else if (c.producer) {
         // launched while the kernel that packs the rows may still run: the copy warp starts on the weights at once
-        if (!lin_produce(a, c)) ring_drain(c);
+        if (!lin_produce<false>(a, c)) ring_drain(c);
     } else {
         grid_dependency_wait();
-        lin_consume<V>(a, c);
+        lin_consume<V, FEW>(a, c);
     }
 }
 // one warp per row (one thread per row took 60 us: a chain of a merge per CTA)
@@ -957,7 +957,7 @@ __global__ void __launch_bounds__(OP_ATT_THREADS<WT, HD>, 1) op_attention_kernel
     Ctx& c = ctx_init(smem, nullptr, nullptr, false);
     if constexpr (!RING_ATT<WT, HD>) attention_impl<WT, HD / 32, true>(D, a, a.plan, c);
     else if (!c.producer) attention_ring<HD, R, false>(D, a, c);
-    else if (!att_produce<HD>(D, a.plan, 0, c)) ring_drain(c);
+    else if (!att_produce<HD, false>(D, a.plan, 0, c)) ring_drain(c);
 }
 // The arrival counters of the splits.  The attention behind it starts at once and waits where it counts its first split.  (A
 // memset of the kilobyte cannot overlap the kernel behind it: 2 us a call.)
@@ -1001,16 +1001,28 @@ extern "C" size_t kg_op_scratch_bytes(void) { return op_layout().total; }
 
 extern "C" int kg_debug_force_simple_ops(int on) { g_force_simple_ops = on ? 1 : 0; return KG_OK; }
 
+// Whether the CTAs of a streamed operator have so few stage pairs that their warps' sums are kept apart.  The kernel without that code is the
+// faster one where it is not used (LM head 32000 x 4096, 16 rows, 78.6 -> 77.6 us; 12288 x 4096, 11 rows, 33.0 -> 32.0), and at 9 to 12 rows with two phases
+// (4096 x 4096, 12 rows, 18.4 -> 17.2 us; with three and more phases the sums kept apart win: 2368 x 8192 22.4 -> 20.9).
+template <int V>
+static bool lin_few(const LinArgs& a, int nctas) {
+    const int units = 2 * (((a.N + 1) / 2 + nctas - 1) / nctas), groups = (units + ST_ROWS - 1) / ST_ROWS;       // of a CTA, at most (cta_unit)
+    return a.nph > (V == 12 ? 2 : 1) && (a.W2 ? groups : (groups + 1) / 2) <= LinGeom<V>::FEWP;
+}
+template <int V, bool FEW>
+static int launch_streamed_linear(const LinArgs& a, int nctas, cudaStream_t s) {
+    if (set_smem<op_linear_kernel<__nv_bfloat16, V, FEW>>() != KG_OK) return KG_E_CUDA;
+    CK(launch_dependent(op_linear_kernel<__nv_bfloat16, V, FEW>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a));
+    return KG_OK;
+}
 template <int V>
 static int launch_linear(const LinArgs& a, int nctas, cudaStream_t s) {
-    if (set_smem<op_linear_kernel<__nv_bfloat16, V>>() != KG_OK) return KG_E_CUDA;
-    CK(launch_dependent(op_linear_kernel<__nv_bfloat16, V>, dim3(nctas), dim3(BLOCK_THREADS), SMEM_TOTAL, s, a));
-    return KG_OK;
+    return lin_few<V>(a, nctas) ? launch_streamed_linear<V, true>(a, nctas, s) : launch_streamed_linear<V, false>(a, nctas, s);
 }
 template <typename WT>
 static int launch_plain(const LinArgs& a, int nctas, cudaStream_t s) {
-    if (set_smem<op_linear_kernel<WT, 0>>() != KG_OK) return KG_E_CUDA;
-    op_linear_kernel<WT, 0><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
+    if (set_smem<op_linear_kernel<WT, 0, false>>() != KG_OK) return KG_E_CUDA;
+    op_linear_kernel<WT, 0, false><<<nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
     return KG_OK;
 }
 
@@ -1265,7 +1277,7 @@ int prefill_tc_init(kg_model* m) {
     int r;
     if ((r = gemm_attributes<PF_STORE>()) != KG_OK || (r = gemm_attributes<PF_QKV>()) != KG_OK || (r = gemm_attributes<PF_SWIGLU>()) != KG_OK) return r;
     if ((r = attention_attributes<128>()) != KG_OK || (r = attention_attributes<64>()) != KG_OK) return r;
-    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
+    CK(cudaFuncSetAttribute((const void*)op_linear_kernel<__nv_bfloat16, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL));
     CK(cudaMemsetAsync(A + m->lay.off_pf_cnt, 0, 4 * (size_t)m->nctas, m->stream));
     m->pf.ready = true;
     return KG_OK;
@@ -1409,7 +1421,7 @@ int prefill_tc(kg_model* m, int n) {
         a.epi = EPI_HEAD; a.scale = c.logit_scale; a.head_part = D.head_part;
         a.logits_dbg = c.debug_logits ? D.dbg_verify : nullptr; a.ld_dbg = c.vocab;
         lin_phases(a);
-        op_linear_kernel<WT, 4><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
+        op_linear_kernel<WT, 4, false><<<m->nctas, BLOCK_THREADS, SMEM_TOTAL, s>>>(a);
         pf_finish_kernel<<<1, 32, 0, s>>>(D.head_part, m->nctas, D.st, D.out_tokens, n, err);
         CK(cudaGetLastError());
     }

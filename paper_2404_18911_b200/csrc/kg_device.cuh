@@ -346,9 +346,9 @@ __device__ __forceinline__ bool arg_better(float za, int ia, float zb, int ib) {
 }
 
 // ------------------------------------------------------------------------------------ CTA set-up
-// Called by every thread of the CTA at kernel start; returns the context of the thread's role.
+// Called by every thread of the CTA at kernel start; returns the context of the thread's role.  prefetch: a prefetch warp reads the queue.
 __device__ __forceinline__ Ctx& ctx_init(char* smem, State* st, unsigned* bar, bool grid,
-                                         unsigned long long wait_clk = WAIT_TIMEOUT_CLK, int skip_arrival = 0) {
+                                         unsigned long long wait_clk = WAIT_TIMEOUT_CLK, int skip_arrival = 0, bool prefetch = false) {
     static_assert(sizeof(Ctx) <= 128, "context slot too small");
     Ctrl* ctl = reinterpret_cast<Ctrl*>(smem);
     const int role = threadIdx.x < NTHREADS ? 0 : (threadIdx.x < NTHREADS + 32 ? 1 : (threadIdx.x < NTHREADS + 64 ? 2 : 3));   // consumers, copy warp, sequencer, prefetch warp
@@ -362,7 +362,7 @@ __device__ __forceinline__ Ctx& ctx_init(char* smem, State* st, unsigned* bar, b
     }
     if (threadIdx.x == 0) {
         for (int i = 0; i < RING; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], NWARPS); }
-        for (int i = 0; i < QUEUE; ++i) { mbar_init(&ctl->qfull[i], 1); mbar_init(&ctl->qempty[i], NWARPS + 2); }
+        for (int i = 0; i < QUEUE; ++i) { mbar_init(&ctl->qfull[i], 1); mbar_init(&ctl->qempty[i], NWARPS + 1 + prefetch); }
         mbar_init(&ctl->mail, 1);
         ctl->abort = 0; ctl->sync_ok = 1; ctl->att_last = 0; ctl->issued = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -595,7 +595,8 @@ __device__ __forceinline__ LinPlan make_plan(const LinArgs& a, int cta, int ncta
     return p;
 }
 
-// Producer warp: issue the bulk copies of every stage of this operator.
+// Producer warp: issue the bulk copies of every stage of this operator.  PUBLISH: for a prefetch warp, which only the decode kernel has.
+template <bool PUBLISH>
 __device__ __noinline__ bool lin_produce(const LinArgs& a, Ctx& c) {
     const int lane = threadIdx.x & 31;
     const LinPlan pl = make_plan(a, c.cta, c.nctas);
@@ -624,7 +625,7 @@ __device__ __noinline__ bool lin_produce(const LinArgs& a, Ctx& c) {
                 __syncwarp();
                 if (lane < nvalid) bulk_g2s(ring + (size_t)slot * SLOT_BYTES + lane * ST_ROW_BYTES, src, (unsigned)(len * 2), &ctl->full[slot], policy);
                 issued++;
-                if (lane == 0) *(volatile unsigned*)&ctl->issued = issued;
+                if (PUBLISH && lane == 0) *(volatile unsigned*)&ctl->issued = issued;
                 if (++slot == RING) { slot = 0; phase ^= 1u; }
             }
         }
@@ -789,7 +790,8 @@ __device__ __forceinline__ void emit_rows(const LinArgs& a, float* wk, const flo
 // log2 of the threads that add the sums of squares of one of M rows
 __device__ __forceinline__ int sum_shift(int M) { return M <= 1 ? 8 : (M <= 2 ? 7 : (M <= 4 ? 6 : (M <= 8 ? 5 : 4))); }
 
-template <int V>
+// FEW: compiled with the sums of few pairs (a single operator that has no use for them is launched without).
+template <int V, bool FEW>
 __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
     using G = LinGeom<V>;
     constexpr int NS = G::NS, FR = G::FR, NACC = G::NACC, MP = G::MP;
@@ -833,7 +835,7 @@ __device__ __forceinline__ void lin_consume(const LinArgs& a, Ctx& c) {
         const int nu = sc1 - sc0;
         const int ngrp = (nu + ST_ROWS - 1) / ST_ROWS;
         const int nst = dual ? 2 * ngrp : ngrp;
-        const bool few = pl.nph > 1 && (nst + 1) >> 1 <= G::FEWP;
+        const bool few = FEW && pl.nph > 1 && (nst + 1) >> 1 <= G::FEWP;
         float* acc_s = wk + (few ? FEW_ACC_OFF : G::ACC_OFF);
         for (int ph = 0; ph < pl.nph; ++ph) {
             const int p0 = ph * pl.plen, len = min(pl.plen, K - p0);
@@ -1756,7 +1758,7 @@ static_assert(2 * RaGeom<128>::QG <= RaGeom<128>::NT_OFF && RaGeom<128>::TPS * R
 static_assert(RaGeom<128>::MB_OFF + NWARPS * ATT_RB * RaGeom<128>::ROW * 4 <= WORK_BYTES && WORK_OFF % 128 == 0 && SLOT_BYTES % 128 == 0, "attention buffers");
 
 // Copy warp: the old K / V tiles of this CTA's items.  row0: first row of this layer's cache in the tensor maps.
-template <int HD>
+template <int HD, bool PUBLISH>
 __device__ __noinline__ bool att_produce(const Dev& D, const AttPlan pl, int row0, Ctx& c) {
     using G = RaGeom<HD>;
     const int lane = threadIdx.x & 31;
@@ -1786,7 +1788,7 @@ __device__ __noinline__ bool att_produce(const Dev& D, const AttPlan pl, int row
                             half * 64, row0 + ((page * H + hh) << psh) + (key & psm), bar);
             }
             issued++;
-            if (lane == 0) *(volatile unsigned*)&c.ctl->issued = issued;
+            if (PUBLISH && lane == 0) *(volatile unsigned*)&c.ctl->issued = issued;
             if (++slot == RING) { slot = 0; phase ^= 1u; }
         }
     }
@@ -2159,7 +2161,7 @@ __device__ __forceinline__ void attention_ring(const Dev& D, const AttArgs& a, C
 template <typename WT, int HD> constexpr bool RING_ATT = sizeof(WT) == 2 && HD >= 64;
 
 __device__ __forceinline__ bool attention_producer(const Dev& D, const AttPlan& pl, int row0, Ctx& c) {
-    return D.dm.hd == 128 ? att_produce<128>(D, pl, row0, c) : att_produce<64>(D, pl, row0, c);
+    return D.dm.hd == 128 ? att_produce<128, true>(D, pl, row0, c) : att_produce<64, true>(D, pl, row0, c);
 }
 
 static_assert((M_MAX * HD_MAX + NWARPS * ATT_RB * ATT_MB_STRIDE + NWARPS * 40) * 4 <= WORK_BYTES, "attention buffers do not fit in the work area");

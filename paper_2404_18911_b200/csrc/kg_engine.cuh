@@ -406,7 +406,7 @@ __device__ __forceinline__ void copy_loop(const Dev& D, Ctx& c, bool streamed) {
         if (!ok) break;
         const Op& op = ctl->queue[q];
         const int kind = op.kind;
-        if (streamed && kind == OPK_LIN) ok = lin_produce(op.lin, c);
+        if (streamed && kind == OPK_LIN) ok = lin_produce<true>(op.lin, c);
         else if (streamed && kind == OPK_ATT && D.dm.ring) ok = attention_producer(D, op.att.plan, op.att.row0, c);
         done = kind == OPK_EXIT;
         __syncwarp();
@@ -416,8 +416,8 @@ __device__ __forceinline__ void copy_loop(const Dev& D, Ctx& c, bool streamed) {
     if (!ok) ring_drain(c);
 }
 
-// ---- the prefetch warp
-__device__ __forceinline__ void prefetch_loop(const Dev& D, Ctx& c, bool streamed) {
+// ---- the prefetch warp (of launches that stream weights: the others' queue is not held up by a reader that has nothing to do)
+__device__ __forceinline__ void prefetch_loop(const Dev& D, Ctx& c) {
     Ctrl* ctl = c.ctl;
     const int lane = threadIdx.x & 31;
     int q = 0; unsigned qph = 0;
@@ -428,8 +428,8 @@ __device__ __forceinline__ void prefetch_loop(const Dev& D, Ctx& c, bool streame
         if (!__shfl_sync(0xffffffffu, w, 0)) return;
         const Op& op = ctl->queue[q];
         const int kind = op.kind;
-        if (ok && streamed && kind == OPK_LIN) ok = lin_prefetch(op.lin, c);
-        else if (streamed && kind == OPK_ATT && D.dm.ring) {
+        if (ok && kind == OPK_LIN) ok = lin_prefetch(op.lin, c);
+        else if (kind == OPK_ATT && D.dm.ring) {
             const unsigned n = D.dm.hd == 128 ? att_stages<128>(D, op.att.plan, c) : att_stages<64>(D, op.att.plan, c);
             __syncwarp();
             if (lane == 0) c.issued += n;
@@ -487,7 +487,7 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
             const LinArgs& a = op.lin;
             if (!streamed) lin_simple<WT>(a, c);
             else if constexpr (sizeof(WT) == 2) {
-                if (a.M <= 4) lin_consume<4>(a, c); else if (a.M <= 8) lin_consume<8>(a, c); else if (a.M <= 12) lin_consume<12>(a, c); else lin_consume<16>(a, c);
+                if (a.M <= 4) lin_consume<4, true>(a, c); else if (a.M <= 8) lin_consume<8, true>(a, c); else if (a.M <= 12) lin_consume<12, true>(a, c); else lin_consume<16, true>(a, c);
             }
         } else if (kind == OPK_ATT) {
             const AttArgs& a = op.att;
@@ -540,7 +540,7 @@ __device__ __forceinline__ void consume_loop(const Dev& D, Ctx& c, bool streamed
 template <typename WT, int HD, bool RING>
 __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const __grid_constant__ Dev D, const __grid_constant__ Program pg) {
     extern __shared__ __align__(128) char smem[];
-    Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival);
+    Ctx& c = ctx_init(smem, D.st, D.bar, true, pg.wait_clk, pg.skip_arrival, sizeof(WT) == 2 && launch_streamed(D, pg));
     if (threadIdx.x >= NTHREADS) {
         // the third warpgroup: keeps what the copy loop and the sequencer need and returns the rest of its registers
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PRODUCER_REGS));
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(DECODE_THREADS, 1) kg_persistent_kernel(const 
         else if (w == 1 && (threadIdx.x & 31) == 0) {
             Sequencer<WT> seq(D, c, pg);
             seq.run();
-        } else if (w == 2) prefetch_loop(D, c, launch_streamed(D, pg));
+        } else if (sizeof(WT) == 2 && w == 2 && launch_streamed(D, pg)) prefetch_loop(D, c);
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CONSUMER_REGS));
         consume_loop<WT, HD, RING>(D, c, launch_streamed(D, pg));
