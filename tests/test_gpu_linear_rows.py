@@ -57,3 +57,10 @@ def test_rows_per_cta(env, N, M):
 @pytest.mark.parametrize("K", [16, 1024, 1040, 2048, 2176, 4112, 6656, 11008])
 def test_phases(env, K, M):
     test_rows(env, 300, K, M)
+
+
+# 9 to 12 rows keep the sums apart from three phases on
+@pytest.mark.parametrize("M", [9, 12])
+@pytest.mark.parametrize("N", [4738, 7104, 7300])
+def test_rows_per_cta_three_phases(env, N, M):
+    test_rows(env, N, 4112, M)
