@@ -211,13 +211,13 @@ struct Ctrl {
     int abort;                         // a bounded wait of this CTA gave up
     int sync_ok;
     int att_last;
-    unsigned issued;                   // stages that the copy warp has issued
+    unsigned issued;                   // stages that the copy warp has issued, for the prefetch warp
     int head_tok[M_MAX];
     float head_p[M_MAX];
-    unsigned long long qfull[QUEUE];   // sequencer -> copy warp, consumers: operator written
-    unsigned long long qempty[QUEUE];  // copy warp, consumer warps -> sequencer: operator done
+    unsigned long long qfull[QUEUE];   // sequencer -> copy warp, prefetch warp, consumers: operator written
+    unsigned long long qempty[QUEUE];  // copy warp, prefetch warp (of launches that have one), consumer warps -> sequencer: operator done
     Op queue[QUEUE];
-    // the per-role context (struct Ctx): one copy for the consumers, one for the copy warp, one for the sequencer
+    // the per-role context (struct Ctx): one copy each for the consumers, the copy warp, the sequencer and the prefetch warp
     alignas(16) unsigned char ctx[4][128];
 };
 static_assert(sizeof(Ctrl) <= CTRL_BYTES - 16, "control block too large");
@@ -545,8 +545,7 @@ __device__ __forceinline__ void head_merge(HeadStat& a, float zmax, float sum, i
 // phase there is nothing to save (a model of four layers with d = 512: 1 % slower that way).  What does not fit the work area: QKV,
 // gate / up, the head.
 template <int V> struct LinGeom {
-    static constexpr int NS = V == 16 ? 8 : 16;           // k16-steps per warp and stage
-    static constexpr int PLEN = NS * 16 * NWARPS;         // most k-elements per phase: 2048 or 1024
+    static constexpr int NS = V == 16 ? 8 : 16;           // most k16-steps per warp and phase: 2048 or 1024 k-elements of a CTA
     static constexpr int FR = V == 4 ? 2 : (V == 8 ? 4 : (V == 12 ? 6 : 8));   // B fragment registers per step
     static constexpr int NACC = V == 16 ? 2 : 1;          // column tiles
     static constexpr int RED_W = V == 16 ? 256 : (V == 12 ? 192 : 128);        // floats of one warp's partial sums of a stage pair
@@ -569,9 +568,11 @@ __device__ __forceinline__ int cta_unit(int N, int cta, int nctas) {
 // The phases of an operator: as many as the longest possible ones and, up to 8 rows, all but the last of the same length, a whole number
 // of steps for every warp.  With phases of the full length the last one may be short, and its copies with it: K = 6656 was 3 x 2048 +
 // 512, now 4 x 1664 (verify pass of one row, 33B widths, 8 layers 1.104 -> 1.023 ms; 13B, 12 layers, KV 2048 1.370 -> 1.319; 7B, whose d is
-// two full phases, 7 rows 1.072 -> 1.049).  Beyond 8 rows it is left as it was (9 to 12 rows would gain 2 to 6 %): the rows of short
-// prompts go there, and with their sums in that order the confidences of the stored 33B trace are up to 4.1e-3 to 5.4e-3 off, more than its
-// test allows, in whatever order the warps' sums are added; as it is they are 3.4e-3 off (before these changes 3.7e-3).
+// two full phases, 7 rows 1.072 -> 1.049).  The error stays what it was: linear operators of 2064 to 17920 k against float64 2.40e-6 to 2.51e-6 of the
+// norm both ways at every row count, bias at 6656 k -9.8e-8 -> -8.1e-8 (7 rows).  Beyond 8 rows the phases are left as they were.  It is not the error:
+// that is the same there too (9 to 12 rows of 6656 k 2.45e-6, bias -9.4e-8 and with equal phases -7.7e-8), and 9 to 12 rows would be 2 to 6 %
+// faster.  But rows of short prompts go there, and the largest deviation of a confidence in the stored 33B trace, which its test holds to 4e-3,
+// is anything from 3.4e-3 to 5.4e-3 with the order of the same sums (as it is 3.4e-3).
 __host__ __device__ __forceinline__ void lin_phases(LinArgs& a) {
     const unsigned steps = (unsigned)a.K >> 4, most = (unsigned)(a.M <= 12 ? LinGeom<12>::NS : LinGeom<16>::NS) * NWARPS;
     const unsigned n = (steps + most - 1) / most;
@@ -641,7 +642,7 @@ __device__ __noinline__ bool lin_produce(const LinArgs& a, Ctx& c) {
 // into L2 once the copy warp is less than PF_AHEAD stages away from it; afterwards the ring is filled from L2, faster than HBM could.
 // Depth, 7B, 12 layers, KV 512, one row (ms): none 0.894, 8 stages 0.887, 10 0.874, 12 0.861, 14 0.850, 16 0.866, 24 1.041, 32 1.295
 // (at 32 KB a stage and 148 CTAs 16 stages are 78 MB: not all of the 126 MB of L2 can be used that way); 33B widths 1.023 -> 0.998 / 0.995 /
-// 0.996 / 1.009 (8 to 14), KV 4096 1.010 -> 0.995 / 0.989 / 0.978 / 0.983, 13B 1.319 -> 1.323 / 1.312 / 1.299 / 1.298.
+// 0.996 / 1.009 (8 to 14; a stage of its phases is 26 KB), KV 4096 1.010 -> 0.995 / 0.989 / 0.978 / 0.983, 13B 1.319 -> 1.323 / 1.312 / 1.299 / 1.298.
 // Passes of more than PF_ROWS_MAX rows keep the consumers busier than HBM, and the additional traffic costs them: 11 rows 1.362 -> 1.398, 16
 // rows 1.635 -> 1.708 (7 rows 1.049 -> 1.008, 8 rows 1.080 -> 1.028).
 constexpr int PF_AHEAD = 12, PF_ROWS_MAX = 8;

@@ -775,16 +775,19 @@ __global__ void __launch_bounds__(256, 1) pf_attention_kernel(const __grid_const
 // different rows may therefore be a tile apart, and all of them a tile ahead of the MMAs, so that P has a barrier for each of the two
 // tiles: on one for all tiles, a fast warp's arrival for tile j + 1 would count for a slow one's for tile j.
 //
-// Precision is that of the kernel above: q and P in two bf16 planes, softmax and the sum over the tiles in fp32.  The lo planes are
-// multiplied first, and a tile's P V starts from zero and is added to registers, so that fewer of the tensor core's truncations count.
+// Precision: q and P in two bf16 planes, softmax and the sum over the tiles in fp32, as in the kernel above.  The lo planes are
+// multiplied first, and a tile's P V starts from zero and is added to registers, so that fewer of the tensor core's truncations count: rows against
+// float64, mean of the norm, the kernel above / this one, 300 rows 2.96e-6 / 2.88e-6, 1999 rows 4.2e-6 / 2.9e-6, 33 rows behind 2048 keys 6.1e-6 / 3.0e-6.
 //
 // What bounds it: per tile 2048 clocks of MMAs (both planes) beside about as many of exponentials, splits and tensor-memory traffic.  7B, one layer
-// (us, the kernel above / this one): 512 rows 32.8 / 20.0, 1024 65 / 38, 1999 222 / 106; prompt pass of 1999 tokens 51.2 -> 47.9 ms.  At 1999
-// rows a tile takes about 5000 clocks: what bounds it is the latency of the softmax chain (issue slots 32 % busy) and, per CTA, its start
-// and end (about 5 us).
+// (us, the kernel above / this one): 512 rows 32.9 / 20.5, 1000 62.7 / 37.6, 1999 211 / 102; prompt pass of 1999 tokens 51.2 -> 47.9 ms.  At 1999
+// rows a tile takes about 5000 clocks: what bounds it is the latency of the softmax chain (issue slots 35 % busy, tensor pipe 37 %) and, per CTA, its
+// start and end (about 5 us).
 constexpr int FT_ROWS = 128, FT_KEYS = 128, FT_THREADS = 384, FT_SOFT_WARPS = 8;
-constexpr int FT_MIN_KEYS = 128;                          // up to here the kernel above is the better one (us, 7B, one layer, the kernel above / this one: 64 keys 8.2 / 10.3, 128 12.7 / 13.5, 256
-                                                          // 19.3 / 15.4, 512 32.8 / 20.0)
+// Up to here the kernel above is the better one or as good (us, the kernel above / this one; 32 heads of 128: 33 rows 9.2 / 10.3, 64 10.3 / 12.3, 128 14.4 /
+// 14.4, 256 20.5 / 16.4; 64 heads of 64: 64 rows 8.2 / 10.3, 128 10.3 / 10.3, 256 14.4 / 12.3).  Rows do not matter beside the keys: 1 row behind 2048
+// keys 73 / 43, of 64 dims 43 / 33 (behind 128 keys of 64 dims up to 32 rows would be 1 to 2 us slower, but at least 1024 rows come before a block).
+constexpr int FT_MIN_KEYS = 128;
 constexpr int FT_CTRL_REGS = 56, FT_SOFT_REGS = 216;
 static_assert(128 * FT_CTRL_REGS + 32 * FT_SOFT_WARPS * FT_SOFT_REGS <= FT_THREADS * LAUNCH_REGS, "register budgets exceed the CTA's pool");
 template <int HD> struct FtSm {
